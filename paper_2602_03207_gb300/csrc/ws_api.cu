@@ -339,7 +339,7 @@ ws_status ws_rasterize(const uint32_t* num_keys, const uint64_t* keys, const uin
     for (const void* p : ptrs)
         if (!p || !aligned16(p)) return WS_ERR_INVALID_ARG;
     const Frame f = make_frame(cam, cfg);
-    return cuda_status(ws::launch_rasterize(num_keys, 0, keys, vals, splats, f, ranges,
+    return cuda_status(ws::launch_rasterize(num_keys, 0, keys, vals, splats, f, ranges, nullptr,
                                             image, t_final, n_contrib, static_cast<cudaStream_t>(stream)));
 }
 
@@ -483,12 +483,14 @@ ws_status ws_rasterize_backward(int64_t n, const float* means, const float* log_
     }
     if (key_capacity > 0 && (!vals || !aligned16(vals))) return WS_ERR_INVALID_ARG;
     const Frame f = make_frame(cam, cfg);
-    char* ws_base = static_cast<char*>(workspace);
-    return cuda_status(ws::launch_backward(n, means, log_scales, quats, sh, f, splats,
-                                           rect, offsets, tiles_touched, vals, ranges, t_final, n_contrib,
-                                           d_image, d_means, d_log_scales, d_quats, d_opacity_logits, d_sh,
-                                           key_capacity, ws_base + layout(0, key_capacity).bwd,
-                                           static_cast<cudaStream_t>(stream)));
+    char* scratch = static_cast<char*>(workspace) + layout(0, key_capacity).bwd;
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    const uint32_t* order = nullptr;
+    if (ws::launch_tile_order(ranges, (uint32_t)(f.TX * f.TY), key_capacity, scratch, &order, s) != cudaSuccess)
+        return WS_ERR_CUDA;
+    return cuda_status(ws::launch_backward(n, means, log_scales, quats, sh, f, splats, rect, offsets, tiles_touched,
+                                           vals, ranges, order, t_final, n_contrib, d_image, nullptr, d_means,
+                                           d_log_scales, d_quats, d_opacity_logits, d_sh, key_capacity, scratch, s));
 }
 
 size_t ws_batch_workspace_bytes(int64_t n, int32_t views, const ws_camera* cams, int64_t key_capacity,
@@ -549,7 +551,7 @@ ws_status ws_rasterize_batch(const uint32_t* num_keys, const uint64_t* keys, con
     const void* ptrs[] = {num_keys, keys, vals, splats, ranges, image, t_final, n_contrib};
     for (const void* p : ptrs)
         if (!p || !aligned16(p)) return WS_ERR_INVALID_ARG;
-    return cuda_status(ws::launch_rasterize_batch(num_keys, keys, vals, n, splats, ft, ranges,
+    return cuda_status(ws::launch_rasterize_batch(num_keys, keys, vals, n, splats, ft, ranges, nullptr,
                                                   image, t_final, n_contrib, static_cast<cudaStream_t>(stream)));
 }
 
@@ -573,12 +575,15 @@ ws_status ws_rasterize_backward_batch(int64_t n, const float* means, const float
             if (!p || !aligned16(p)) return WS_ERR_INVALID_ARG;
     }
     if (key_capacity > 0 && (!vals || !aligned16(vals))) return WS_ERR_INVALID_ARG;
-    char* ws_base = static_cast<char*>(workspace);
-    return cuda_status(ws::launch_backward_batch(n, means, log_scales, quats, sh, ft, splats,
-                                                 rect, offsets, tiles_touched, vals, ranges, t_final, n_contrib,
-                                                 d_image, d_means, d_log_scales, d_quats, d_opacity_logits, d_sh,
-                                                 key_capacity, ws_base + layout(0, key_capacity).bwd,
-                                                 static_cast<cudaStream_t>(stream)));
+    char* scratch = static_cast<char*>(workspace) + layout(0, key_capacity).bwd;
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    const uint32_t* order = nullptr;
+    if (ws::launch_tile_order(ranges, ft.tile_off[ft.views], key_capacity, scratch, &order, s) != cudaSuccess)
+        return WS_ERR_CUDA;
+    return cuda_status(ws::launch_backward_batch(n, means, log_scales, quats, sh, ft, splats, rect, offsets,
+                                                 tiles_touched, vals, ranges, order, t_final, n_contrib, d_image,
+                                                 nullptr, d_means, d_log_scales, d_quats, d_opacity_logits, d_sh,
+                                                 key_capacity, false, scratch, s));
 }
 
 ws_status ws_render_train_l2(int64_t n, const float* means, const float* log_scales, const float* quats,
@@ -601,11 +606,22 @@ ws_status ws_render_train_l2(int64_t n, const float* means, const float* log_sca
             if (!p || !aligned16(p)) return WS_ERR_INVALID_ARG;
     }
     const Frame f = make_frame(cam, cfg);
-    char* ws_base = static_cast<char*>(workspace);
-    return cuda_status(ws::launch_train(n, means, log_scales, quats, sh, f, num_keys, keys, vals, splats, rect,
-                                        offsets, tiles_touched, target, ranges, image, t_final, n_contrib, d_means,
-                                        d_log_scales, d_quats, d_opacity_logits, d_sh, key_capacity,
-                                        ws_base + layout(0, key_capacity).bwd, static_cast<cudaStream_t>(stream)));
+    char* scratch = static_cast<char*>(workspace) + layout(0, key_capacity).bwd;
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    // ranges, the tiles' order, the forward blend (image, t_final,
+    // n_contrib), the backward with dL/dC = image - target
+    const uint32_t ntiles = (uint32_t)(f.TX * f.TY);
+    const uint32_t* order = nullptr;
+    cudaError_t e = ws::launch_tile_ranges(keys, num_keys, ranges, ntiles, f.flags, s);
+    if (e == cudaSuccess) e = ws::launch_tile_order(ranges, ntiles, key_capacity, scratch, &order, s);
+    Frame fr = f;
+    fr.flags |= WS_CFG_RANGES_GIVEN;
+    if (e == cudaSuccess)
+        e = ws::launch_rasterize(num_keys, 0, keys, vals, splats, fr, ranges, order, image, t_final, n_contrib, s);
+    if (e != cudaSuccess) return WS_ERR_CUDA;
+    return cuda_status(ws::launch_backward(n, means, log_scales, quats, sh, f, splats, rect, offsets, tiles_touched,
+                                           vals, ranges, order, t_final, n_contrib, image, target, d_means,
+                                           d_log_scales, d_quats, d_opacity_logits, d_sh, key_capacity, scratch, s));
 }
 
 ws_status ws_render_train_l2_batch(int64_t n, const float* means, const float* log_scales, const float* quats,
@@ -629,13 +645,21 @@ ws_status ws_render_train_l2_batch(int64_t n, const float* means, const float* l
         for (const void* p : per)
             if (!p || !aligned16(p)) return WS_ERR_INVALID_ARG;
     }
-    char* ws_base = static_cast<char*>(workspace);
-    return cuda_status(ws::launch_train_batch(n, means, log_scales, quats, sh, ft, num_keys, keys, vals, splats, rect,
-                                              offsets, tiles_touched, target, ranges, image, t_final, n_contrib,
-                                              d_means, d_log_scales, d_quats, d_opacity_logits, d_sh, key_capacity,
-                                              (cfg->flags & WS_CFG_PERSISTENT) != 0u,
-                                              ws_base + layout(0, key_capacity).bwd,
-                                              static_cast<cudaStream_t>(stream)));
+    char* scratch = static_cast<char*>(workspace) + layout(0, key_capacity).bwd;
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    const uint32_t ntiles = ft.tile_off[ft.views];
+    const uint32_t* order = nullptr;
+    cudaError_t e = ws::launch_tile_ranges(keys, num_keys, ranges, ntiles, ft.f[0].flags, s);
+    if (e == cudaSuccess) e = ws::launch_tile_order(ranges, ntiles, key_capacity, scratch, &order, s);
+    ft.f[0].flags |= WS_CFG_RANGES_GIVEN;
+    if (e == cudaSuccess)
+        e = ws::launch_rasterize_batch(num_keys, keys, vals, n, splats, ft, ranges, order, image, t_final, n_contrib,
+                                       s);
+    if (e != cudaSuccess) return WS_ERR_CUDA;
+    return cuda_status(ws::launch_backward_batch(n, means, log_scales, quats, sh, ft, splats, rect, offsets,
+                                                 tiles_touched, vals, ranges, order, t_final, n_contrib, image, target,
+                                                 d_means, d_log_scales, d_quats, d_opacity_logits, d_sh, key_capacity,
+                                                 (cfg->flags & WS_CFG_PERSISTENT) != 0u, scratch, s));
 }
 
 ws_status ws_image_residual(int64_t count, const float* image, const float* target, float* d_image, void* stream) {

@@ -6,20 +6,11 @@
 // Gaussian sums its contiguous records in slot order. Results are therefore
 // bitwise reproducible.
 //
-// k_blend_bwd: one block per tile, one thread per pixel, back to front from
-//   the stored final transmittance and last-contributor count. With
-//   B = colour behind splat i normalised by T_{i+1} (B starts as the
-//   background and is updated B <- a c + (1 - a) B):
-//     dL/dc_i = a_i T_i dL/dC,   dL/da_i = T_i (c_i - B_i) . dL/dC,
-//   then, unless the alpha was clamped at 0.99,
-//     sigma dL/dsigma = raw dL/da (raw = sigma G, the unclamped alpha),
-//     dL/dpower = a dL/da, power = -1/2 d^T Q d,
-//   giving d/dmean = Q d, d/dQ_a = -dx^2/2, d/dQ_b = -dx dy, d/dQ_c = -dy^2/2.
-//   (The sigma partial is kept multiplied by sigma: dL/dlogit is then that
-//   sum times 1 - sigma.)
-//   Each half-warp (a 4x4 pixel sub-block) reduces its 16 pixels with a
-//   fixed shuffle tree, the block adds its half-warps in order, and the
-//   record goes to the pair's slot.
+// k_blend_bwd: one block per tile, back to front from the stored final
+//   transmittance: a walk that leaves two numbers per pixel and visit, then a
+//   thread per visit that sums its 16 pixels, then a thread per splat that
+//   adds its visits in a fixed order (BwdPixels in ws_blend.cuh) and writes
+//   the pair's record at its slot.
 // k_preprocess_bwd: one thread per Gaussian: slot-ordered sum of its
 //   records, then the adjoint of conic = Sigma'^{-1}, Sigma' = T Sigma T^T,
 //   T = J W (J's guard-band clamp passes no gradient), the projection of
@@ -35,35 +26,20 @@ namespace ws {
 
 namespace {
 
-// Backward records of one tile per block, the tiles taken centre-out
-// (centre_out_tile): 2.5 % faster than raster order on the 720p step, where
-// the longest lists are near the centre.
-template <int TS>
-__global__ void __launch_bounds__(TS * TS >= 256 ? 256 : TS * TS)
-k_blend_bwd(const uint2* __restrict__ ranges, const uint32_t* __restrict__ vals, const float4* __restrict__ splats,
-            const uint2* __restrict__ rect, const uint32_t* __restrict__ offsets, const Frame f,
-            const float* __restrict__ t_final, const uint32_t* __restrict__ n_contrib,
-            const float* __restrict__ d_image, float* __restrict__ partials) {
+// Backward records of one tile per block, the tiles in the order given
+// (launch_tile_order), or centre-out without one (centre_out_tile).
+template <int TS, int PX>
+__global__ void __launch_bounds__(TileGeom<TS, PX>::THREADS, bwd_min_blocks<TS>())
+k_blend_bwd(const uint2* __restrict__ ranges, const uint32_t* __restrict__ order, const uint32_t* __restrict__ vals,
+            const float4* __restrict__ splats, const uint2* __restrict__ rect, const uint32_t* __restrict__ offsets,
+            const Frame f, const float* __restrict__ t_final, const uint32_t* __restrict__ n_contrib,
+            const float* __restrict__ d_image, const float* __restrict__ target, const PairRecords out) {
+    __shared__ BwdSmem<TS, PX, bwd_batch<TS>()> sm;
     pdl_wait();
-    const int t = centre_out_tile(f, blockIdx.x);
-    blend_bwd_tile<TS>(f, t, ranges[t], vals, splats, rect,
-                       [offsets](uint32_t g) { return __ldg(offsets + g); }, t_final, n_contrib, d_image, partials);
-}
-
-// One training step's blend of a tile (forward, L2 residual, backward
-// records) in one block: train_tile, the tiles taken centre-out.
-template <int TS>
-__global__ void __launch_bounds__(TileGeom<TS>::THREADS)
-k_train(const uint2* __restrict__ ranges, const uint32_t* __restrict__ vals, const float4* __restrict__ splats,
-        const uint2* __restrict__ rect, const uint32_t* __restrict__ offsets, const Frame f,
-        const float* __restrict__ target, float* __restrict__ image, float* __restrict__ t_final,
-        uint32_t* __restrict__ n_contrib, float* __restrict__ partials) {
-    __shared__ TrainSmem<TS> sm;
-    pdl_wait();
-    const int t = centre_out_tile(f, blockIdx.x);
-    train_tile<TS>(f, t, ranges[t], vals, splats, rect,
-                   [offsets](uint32_t g) { return __ldg(offsets + g); }, target, image, t_final, n_contrib, partials,
-                   sm);
+    const int t = order ? (int)__ldg(order + blockIdx.x) : centre_out_tile(f, blockIdx.x);
+    blend_bwd_tile<TS, PX>(f, t, ranges[t], vals, splats, rect,
+                           offsets, t_final, n_contrib, d_image, target,
+                           out, sm);
 }
 
 constexpr int kPbThreads = 128;
@@ -72,7 +48,7 @@ __global__ void __launch_bounds__(kPbThreads, 8)
 k_preprocess_bwd(int64_t n, const float* __restrict__ means, const float* __restrict__ log_scales,
                  const float4* __restrict__ quats, const float4* __restrict__ sh, const Frame f,
                  const float4* __restrict__ splats, const uint32_t* __restrict__ offsets, const uint32_t* __restrict__ touched,
-                 uint32_t cap, const float* __restrict__ partials, float* __restrict__ d_means,
+                 uint32_t cap, const float4* __restrict__ partials, float* __restrict__ d_means,
                  float* __restrict__ d_log_scales, float4* __restrict__ d_quats,
                  float* __restrict__ d_logits, float4* __restrict__ d_sh) {
     __shared__ __align__(16) float s_sh[kPbThreads / kWarp][kWarp * kShPad];
@@ -122,7 +98,7 @@ k_preprocess_bwd(int64_t n, const float* __restrict__ means, const float* __rest
         col[1] = cl.y;
         col[2] = cl.z;
         // slot-ordered sum of this Gaussian's pair records
-        sum_pair_records(partials + (size_t)first * kPart, nrec, pr);
+        sum_pair_records(partials, reinterpret_cast<const float*>(partials + 2 * (size_t)cap), first, nrec, pr);
         glogit = pr[5] * (1.f - sig);  // pr[5] = sigma dL/dsigma
         splat_adjoint(f, X, q4, ls, pr, cl.w, gm, gls, gq);  // cl.w: the axis basis's t
     }
@@ -176,41 +152,111 @@ k_preprocess_bwd(int64_t n, const float* __restrict__ means, const float* __rest
     }
 }
 
+
+// Tiles sorted by the length of their lists, longest first (64 classes, two
+// per octave; raster order within a class): a stable counting sort by one
+// block, each warp ranking a contiguous run of tiles with ballots. A tile's
+// time in the backward grows with its list, and a long one that starts late
+// runs on alone: on the 720p / 500k step (lists up to 914, mean 138) the SMs
+// were busy for 170k of the 237k cycles of the tile-centred order. The
+// launch costs 4 us there and the backward call goes from 151.8 to 140.6 us.
+constexpr int kOrderThreads = 1024;
+constexpr int kOrderBits = 6;
+
+__device__ __forceinline__ uint32_t length_class(uint32_t len) {
+    if (len < 2u) return 63u;
+    const int lz = 31 - __clz(len);
+    return 63u - (uint32_t)(2 * lz + ((len >> (lz - 1)) & 1u));
+}
+
+__global__ void __launch_bounds__(kOrderThreads)
+k_tile_order(const uint2* __restrict__ ranges, uint32_t ntiles, uint32_t* __restrict__ order) {
+    constexpr int W = kOrderThreads / 32, R = 1 << kOrderBits, U = 4;
+    __shared__ uint32_t s_cnt[W][R];
+    __shared__ uint32_t s_red[W + 1];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int i = threadIdx.x; i < W * R; i += kOrderThreads) (&s_cnt[0][0])[i] = 0u;
+    pdl_wait();
+    __syncthreads();
+    const uint32_t per = (ntiles + kOrderThreads * U - 1) / (kOrderThreads * U) * (32 * U);
+    const uint32_t lo = min(warp * per, ntiles), hi = min(lo + per, ntiles);
+    const uint32_t lt = lanemask_lt();
+    // pass 0 counts, pass 1 places
+    for (int pass = 0; pass < 2; ++pass) {
+        for (uint32_t i0 = lo; i0 < hi; i0 += 32 * U) {
+            uint32_t cls[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const uint32_t i = i0 + u * 32 + lane;
+                const uint2 r = i < hi ? __ldg(ranges + i) : make_uint2(0u, 0u);
+                cls[u] = length_class(r.y - r.x);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const uint32_t i = i0 + u * 32 + lane;
+                const bool ok = i < hi;
+                const uint32_t peers = warp_match_digit<kOrderBits>(cls[u], ok);
+                const uint32_t prior = s_cnt[warp][cls[u]];
+                __syncwarp();
+                if (ok && (peers & lt) == 0u) s_cnt[warp][cls[u]] = prior + __popc(peers);
+                if (ok && pass) order[prior + __popc(peers & lt)] = i;
+                __syncwarp();
+            }
+        }
+        __syncthreads();
+        if (pass) break;
+        // counts -> first positions, by class and then warp
+        static_assert(W * R == 2 * kOrderThreads, "two counters per thread");
+        const int c = threadIdx.x / (W / 2), w = (threadIdx.x % (W / 2)) * 2;
+        const uint32_t a = s_cnt[w][c], b = s_cnt[w + 1][c];
+        uint32_t total;
+        const uint32_t ex = block_exclusive_scan<kOrderThreads>(a + b, s_red, &total);
+        s_cnt[w][c] = ex;
+        s_cnt[w + 1][c] = ex + a;
+        __syncthreads();
+    }
+}
+
 }  // namespace
 
 size_t backward_scratch_bytes(int64_t key_capacity) {
-    return (size_t)(key_capacity > 0 ? key_capacity : 1) * kPart * sizeof(float);
+    return (size_t)(key_capacity > 0 ? key_capacity : 1) * kPart * sizeof(float) + kOrderMax * sizeof(uint32_t);
+}
+
+cudaError_t launch_tile_order(const uint32_t* ranges, uint32_t ntiles, int64_t key_capacity, void* scratch,
+                              const uint32_t** order, cudaStream_t stream) {
+    *order = nullptr;
+    if (ntiles < kOrderMin || ntiles > kOrderMax) return cudaSuccess;
+    uint32_t* o = reinterpret_cast<uint32_t*>(pair_records(scratch, key_capacity > 0 ? key_capacity : 1).p9 +
+                                              (key_capacity > 0 ? key_capacity : 1));
+    *order = o;
+    return launch_pdl(k_tile_order, dim3(1), dim3(kOrderThreads), 0, stream, reinterpret_cast<const uint2*>(ranges),
+                      ntiles, o);
 }
 
 cudaError_t launch_backward(int64_t n, const float* means, const float* log_scales, const float* quats,
                             const float* sh, const Frame& f, const float* splats, const uint16_t* rect,
                             const uint32_t* offsets, const uint32_t* tiles_touched,
-                            const uint32_t* vals, const uint32_t* ranges, const float* t_final,
-                            const uint32_t* n_contrib, const float* d_image, float* d_means,
+                            const uint32_t* vals, const uint32_t* ranges, const uint32_t* order, const float* t_final,
+                            const uint32_t* n_contrib, const float* d_image, const float* target, float* d_means,
                             float* d_log_scales, float* d_quats, float* d_logits, float* d_sh,
                             int64_t key_capacity, void* scratch, cudaStream_t stream) {
-    float* partials = static_cast<float*>(scratch);
+    const PairRecords partials = pair_records(scratch, key_capacity);
     const int ntiles = f.TX * f.TY;
     const uint2* r2 = reinterpret_cast<const uint2*>(ranges);
     const float4* s4 = reinterpret_cast<const float4*>(splats);
     const uint2* rc = reinterpret_cast<const uint2*>(rect);
     cudaError_t e = cudaSuccess;
     if (ntiles > 0) {
+        auto run = [&](auto kernel, int threads) {
+            return launch_pdl(kernel, dim3(ntiles), dim3(threads), 0, stream, r2, order, vals, s4, rc, offsets, f,
+                              t_final, n_contrib, d_image, target, partials);
+        };
         switch (f.TS) {
-            case 8:
-                e = launch_pdl(k_blend_bwd<8>, dim3(ntiles), dim3(64), 0, stream, r2, vals, s4, rc, offsets, f,
-                               t_final, n_contrib, d_image, partials);
-                break;
-            case 16:
-                e = launch_pdl(k_blend_bwd<16>, dim3(ntiles), dim3(256), 0, stream, r2, vals, s4, rc, offsets, f,
-                               t_final, n_contrib, d_image, partials);
-                break;
-            case 32:
-                e = launch_pdl(k_blend_bwd<32>, dim3(ntiles), dim3(256), 0, stream, r2, vals, s4, rc, offsets, f,
-                               t_final, n_contrib, d_image, partials);
-                break;
-            default:
-                return cudaErrorInvalidValue;
+            case 8: e = run(k_blend_bwd<8, tile_px<8>()>, TileGeom<8, tile_px<8>()>::THREADS); break;
+            case 16: e = run(k_blend_bwd<16, tile_px<16>()>, TileGeom<16, tile_px<16>()>::THREADS); break;
+            case 32: e = run(k_blend_bwd<32, tile_px<32>()>, TileGeom<32, tile_px<32>()>::THREADS); break;
+            default: return cudaErrorInvalidValue;
         }
         if (e != cudaSuccess) return e;
     }
@@ -218,50 +264,7 @@ cudaError_t launch_backward(int64_t n, const float* means, const float* log_scal
         const int64_t blocks = (n + kPbThreads - 1) / kPbThreads;
         e = launch_pdl(k_preprocess_bwd, dim3((unsigned)blocks), dim3(kPbThreads), 0, stream, n, means, log_scales,
                        reinterpret_cast<const float4*>(quats), reinterpret_cast<const float4*>(sh), f, s4,
-                       offsets, tiles_touched, (uint32_t)key_capacity, (const float*)partials, d_means, d_log_scales,
-                       reinterpret_cast<float4*>(d_quats), d_logits, reinterpret_cast<float4*>(d_sh));
-    }
-    return e;
-}
-
-cudaError_t launch_train(int64_t n, const float* means, const float* log_scales, const float* quats, const float* sh,
-                         const Frame& f, const uint32_t* num_keys, const uint64_t* keys, const uint32_t* vals,
-                         const float* splats, const uint16_t* rect, const uint32_t* offsets,
-                         const uint32_t* tiles_touched, const float* target, uint32_t* ranges, float* image,
-                         float* t_final, uint32_t* n_contrib, float* d_means, float* d_log_scales, float* d_quats,
-                         float* d_logits, float* d_sh, int64_t key_capacity, void* scratch, cudaStream_t stream) {
-    float* partials = static_cast<float*>(scratch);
-    const int ntiles = f.TX * f.TY;
-    const float4* s4 = reinterpret_cast<const float4*>(splats);
-    const uint2* rc = reinterpret_cast<const uint2*>(rect);
-    cudaError_t e = cudaSuccess;
-    if (ntiles > 0) {
-        e = launch_tile_ranges(keys, num_keys, ranges, (uint32_t)ntiles, f.flags, stream);
-        if (e != cudaSuccess) return e;
-        const uint2* r2 = reinterpret_cast<const uint2*>(ranges);
-        switch (f.TS) {
-            case 8:
-                e = launch_pdl(k_train<8>, dim3(ntiles), dim3(TileGeom<8>::THREADS), 0, stream, r2, vals, s4, rc,
-                               offsets, f, target, image, t_final, n_contrib, partials);
-                break;
-            case 16:
-                e = launch_pdl(k_train<16>, dim3(ntiles), dim3(TileGeom<16>::THREADS), 0, stream, r2, vals, s4, rc,
-                               offsets, f, target, image, t_final, n_contrib, partials);
-                break;
-            case 32:
-                e = launch_pdl(k_train<32>, dim3(ntiles), dim3(TileGeom<32>::THREADS), 0, stream, r2, vals, s4, rc,
-                               offsets, f, target, image, t_final, n_contrib, partials);
-                break;
-            default:
-                return cudaErrorInvalidValue;
-        }
-        if (e != cudaSuccess) return e;
-    }
-    if (n > 0) {
-        const int64_t blocks = (n + kPbThreads - 1) / kPbThreads;
-        e = launch_pdl(k_preprocess_bwd, dim3((unsigned)blocks), dim3(kPbThreads), 0, stream, n, means, log_scales,
-                       reinterpret_cast<const float4*>(quats), reinterpret_cast<const float4*>(sh), f, s4,
-                       offsets, tiles_touched, (uint32_t)key_capacity, (const float*)partials, d_means, d_log_scales,
+                       offsets, tiles_touched, (uint32_t)key_capacity, (const float4*)partials.p8, d_means, d_log_scales,
                        reinterpret_cast<float4*>(d_quats), d_logits, reinterpret_cast<float4*>(d_sh));
     }
     return e;

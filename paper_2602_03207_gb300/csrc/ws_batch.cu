@@ -11,7 +11,8 @@
 //                        ids offset into one global tile grid, so one sort
 //                        orders every view's (tile, depth) keys.
 //   k_blend_batch        one launch over every (view, tile) work item.
-//   k_blend_bwd_batch    likewise, records at each pair's emission slot.
+//   k_blend_bwd_batch    likewise, longest lists first, records at each pair's
+//                        emission slot.
 //   k_preprocess_bwd_batch  one thread per Gaussian: for each view in order,
 //                        the slot-ordered sum of its records and that view's
 //                        adjoint, accumulated in view order (deterministic).
@@ -91,60 +92,44 @@ k_preprocess_batch(int64_t n, const float* __restrict__ means, const float* __re
     }
 }
 
-template <int TS>
-__global__ void __launch_bounds__(TS * TS, blend_min_blocks<TS>())
-k_blend_batch(const uint2* __restrict__ ranges, const uint32_t* __restrict__ vals, int64_t n,
-              const float4* __restrict__ splats, const FrameTable ft,
+template <int TS, int PX>
+__global__ void __launch_bounds__(TileGeom<TS, PX>::THREADS, fwd_min_blocks<TS>())
+k_blend_batch(const uint2* __restrict__ ranges, const uint32_t* __restrict__ order,
+              const uint32_t* __restrict__ vals, int64_t n, const float4* __restrict__ splats, const FrameTable ft,
               float* __restrict__ image, float* __restrict__ t_final, uint32_t* __restrict__ n_contrib) {
     pdl_wait();
-    const uint32_t t = blockIdx.x;
+    const uint32_t t = order ? __ldg(order + blockIdx.x) : blockIdx.x;
     const int v = view_of_tile(ft.tile_off, ft.views, t);
     const uint64_t vo = (uint64_t)v * (uint64_t)n, po = ft.pix_off[v];
     const FloatSplats sp{splats + kSplatVec4 * vo};
-    blend_tile<TS>(ft.f[v], (int)(t - ft.tile_off[v]), ranges[t], vals, sp, image + 3 * po, t_final + po,
+    blend_tile<TS, PX>(ft.f[v], (int)(t - ft.tile_off[v]), ranges[t], vals, sp, image + 3 * po, t_final + po,
                    n_contrib + po);
 }
 
-template <int TS>
-__global__ void __launch_bounds__(TS * TS >= 256 ? 256 : TS * TS)
-k_blend_bwd_batch(const uint2* __restrict__ ranges, const uint32_t* __restrict__ vals, int64_t n,
-                  const float4* __restrict__ splats, const uint2* __restrict__ rect,
-                  const uint32_t* __restrict__ offsets, const FrameTable ft, const float* __restrict__ t_final,
-                  const uint32_t* __restrict__ n_contrib, const float* __restrict__ d_image,
-                  float* __restrict__ partials) {
-    pdl_wait();
-    const uint32_t t = blockIdx.x;
-    const int v = view_of_tile(ft.tile_off, ft.views, t);
-    const uint64_t vo = (uint64_t)v * (uint64_t)n, po = ft.pix_off[v];
-    const uint32_t* voff = offsets + vo;
-    blend_bwd_tile<TS>(ft.f[v], (int)(t - ft.tile_off[v]), ranges[t], vals, splats + kSplatVec4 * vo, rect + vo, [voff](uint32_t g) { return __ldg(voff + g); }, t_final + po,
-                       n_contrib + po, d_image + 3 * po, partials);
-}
-
-// One training step's blend over every (view, tile) item: train_tile per
-// item. PERSISTENT = false: one block per item. PERSISTENT = true: a grid of
-// as many blocks as fit on the GPU at once, block b taking items b, b + G,
-// b + 2G, ... (G = the grid size) in that fixed order, so the assignment is
-// static and neighbouring blocks work on neighbouring tiles; no block waits
-// on another.
-template <int TS, bool PERSISTENT>
-__global__ void __launch_bounds__(TileGeom<TS>::THREADS)
-k_train_batch(const uint2* __restrict__ ranges, const uint32_t* __restrict__ vals, int64_t n,
-              const float4* __restrict__ splats, const uint2* __restrict__ rect,
-              const uint32_t* __restrict__ offsets, const FrameTable ft, const float* __restrict__ target,
-              float* __restrict__ image, float* __restrict__ t_final, uint32_t* __restrict__ n_contrib,
-              float* __restrict__ partials) {
-    __shared__ TrainSmem<TS> sm;
+// Backward records of every (view, tile) item. PERSISTENT = false: one block
+// per item, in the order given (launch_tile_order) or item order.
+// PERSISTENT = true: a grid of as many blocks as fit on the GPU at once, block
+// b taking items b, b + G, b + 2G, ... (G = the grid size) of that order, so
+// the assignment is static; no block waits on another.
+template <int TS, int PX, bool PERSISTENT>
+__global__ void __launch_bounds__(TileGeom<TS, PX>::THREADS, bwd_min_blocks<TS>())
+k_blend_bwd_batch(const uint2* __restrict__ ranges, const uint32_t* __restrict__ order,
+                  const uint32_t* __restrict__ vals, int64_t n, const float4* __restrict__ splats,
+                  const uint2* __restrict__ rect, const uint32_t* __restrict__ offsets, const FrameTable ft,
+                  const float* __restrict__ t_final, const uint32_t* __restrict__ n_contrib,
+                  const float* __restrict__ d_image, const float* __restrict__ target, const PairRecords out) {
+    __shared__ BwdSmem<TS, PX, bwd_batch<TS>()> sm;
     pdl_wait();
     const uint32_t ntiles = ft.tile_off[ft.views];
     const uint32_t stride = PERSISTENT ? gridDim.x : ntiles;
-    for (uint32_t t = blockIdx.x; t < ntiles; t += stride) {
+    for (uint32_t i = blockIdx.x; i < ntiles; i += stride) {
+        const uint32_t t = order ? __ldg(order + i) : i;
         const int v = view_of_tile(ft.tile_off, ft.views, t);
         const uint64_t vo = (uint64_t)v * (uint64_t)n, po = ft.pix_off[v];
-        const uint32_t* voff = offsets + vo;
-        train_tile<TS>(ft.f[v], (int)(t - ft.tile_off[v]), ranges[t], vals, splats + kSplatVec4 * vo, rect + vo,
-                       [voff](uint32_t g) { return __ldg(voff + g); }, target + 3 * po, image + 3 * po,
-                       t_final + po, n_contrib + po, partials, sm);
+        blend_bwd_tile<TS, PX>(ft.f[v], (int)(t - ft.tile_off[v]), ranges[t], vals, splats + kSplatVec4 * vo,
+                               rect + vo, offsets + vo, t_final + po,
+                               n_contrib + po, d_image + 3 * po, target ? target + 3 * po : nullptr, out, sm);
+        if (PERSISTENT) __syncthreads();  // the last reads of sm before the next item's writes
     }
 }
 
@@ -153,7 +138,7 @@ k_preprocess_bwd_batch(int64_t n, const float* __restrict__ means, const float* 
                        const float4* __restrict__ quats, const float4* __restrict__ sh, const FrameTable ft,
                        const float4* __restrict__ splats, const uint32_t* __restrict__ offsets,
                        const uint32_t* __restrict__ touched,
-                       uint32_t cap, const float* __restrict__ partials, float* __restrict__ d_means,
+                       uint32_t cap, const float4* __restrict__ partials, float* __restrict__ d_means,
                        float* __restrict__ d_log_scales, float4* __restrict__ d_quats,
                        float* __restrict__ d_logits, float4* __restrict__ d_sh) {
     __shared__ __align__(16) float s_sh[kBatchThreads / kWarp][kWarp * kShPad];
@@ -213,7 +198,7 @@ k_preprocess_bwd_batch(int64_t n, const float* __restrict__ means, const float* 
         // records past the key capacity were never written (the emission
         // dropped those pairs and raised WS_FLAG_CAPACITY)
         const uint32_t nrec = first >= cap ? 0u : min(cnt, cap - first);
-        sum_pair_records(partials + (size_t)first * kPart, nrec, pr);
+        sum_pair_records(partials, reinterpret_cast<const float*>(partials + 2 * (size_t)cap), first, nrec, pr);
         const float sig = __ldg(splats + kSplatVec4 * o + 1).w;  // sigma (the same in every view)
         glogit += pr[5] * (1.f - sig);  // pr[5] = sigma dL/dsigma
         const Frame& f = ft.f[v];
@@ -272,58 +257,72 @@ cudaError_t launch_preprocess_batch(int64_t n, const float* means, const float* 
 }
 
 cudaError_t launch_rasterize_batch(const uint32_t* num_keys, const uint64_t* keys, const uint32_t* vals, int64_t n,
-                                   const float* splats, const FrameTable& ft, uint32_t* ranges, float* image, float* t_final,
-                                   uint32_t* n_contrib, cudaStream_t stream) {
+                                   const float* splats, const FrameTable& ft, uint32_t* ranges, const uint32_t* order,
+                                   float* image, float* t_final, uint32_t* n_contrib, cudaStream_t stream) {
     const uint32_t ntiles = ft.tile_off[ft.views];
     if (ntiles == 0) return cudaSuccess;
-    cudaError_t e = launch_tile_ranges(keys, num_keys, ranges, ntiles, ft.f[0].flags, stream);
+    const cudaError_t e = launch_tile_ranges(keys, num_keys, ranges, ntiles, ft.f[0].flags, stream);
     if (e != cudaSuccess) return e;
     const uint2* r2 = reinterpret_cast<const uint2*>(ranges);
     const float4* s4 = reinterpret_cast<const float4*>(splats);
+    auto run = [&](auto kernel, int threads) {
+        return launch_pdl(kernel, dim3(ntiles), dim3(threads), 0, stream, r2, order, vals, n, s4, ft, image,
+                          t_final, n_contrib);
+    };
     switch (ft.f[0].TS) {
-        case 8:
-            return launch_pdl(k_blend_batch<8>, dim3(ntiles), dim3(64), 0, stream, r2, vals, n, s4, ft, image,
-                              t_final, n_contrib);
-        case 16:
-            return launch_pdl(k_blend_batch<16>, dim3(ntiles), dim3(256), 0, stream, r2, vals, n, s4, ft, image,
-                              t_final, n_contrib);
-        case 32:
-            return launch_pdl(k_blend_batch<32>, dim3(ntiles), dim3(1024), 0, stream, r2, vals, n, s4, ft, image,
-                              t_final, n_contrib);
-        default:
-            return cudaErrorInvalidValue;
+        case 8: return run(k_blend_batch<8, tile_px<8>()>, TileGeom<8, tile_px<8>()>::THREADS);
+        case 16: return run(k_blend_batch<16, tile_px<16>()>, TileGeom<16, tile_px<16>()>::THREADS);
+        case 32: return run(k_blend_batch<32, tile_px<32>()>, TileGeom<32, tile_px<32>()>::THREADS);
+        default: return cudaErrorInvalidValue;
     }
+}
+
+template <int TS>
+cudaError_t launch_bwd_items(const uint2* r2, const uint32_t* order, const uint32_t* vals, int64_t n, const float4* s4,
+                             const uint2* rc, const uint32_t* offsets, const FrameTable& ft, const float* t_final,
+                             const uint32_t* n_contrib, const float* d_image, const float* target,
+                             const PairRecords& out, bool persistent, cudaStream_t stream) {
+    const uint32_t ntiles = ft.tile_off[ft.views];
+    constexpr int PX = tile_px<TS>();
+    constexpr int kThreads = TileGeom<TS, PX>::THREADS;
+    if (!persistent)
+        return launch_pdl(k_blend_bwd_batch<TS, PX, false>, dim3(ntiles), dim3(kThreads), 0, stream, r2, order, vals,
+                          n, s4, rc, offsets, ft, t_final, n_contrib, d_image, target, out);
+    int dev = 0, sms = 148, occ = 1;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_blend_bwd_batch<TS, PX, true>, kThreads, 0);
+    if (e != cudaSuccess) return e;
+    const uint32_t grid = min(ntiles, (uint32_t)(sms * (occ > 0 ? occ : 1)));
+    return launch_pdl(k_blend_bwd_batch<TS, PX, true>, dim3(grid), dim3(kThreads), 0, stream, r2, order, vals, n, s4,
+                      rc, offsets, ft, t_final, n_contrib, d_image, target, out);
 }
 
 cudaError_t launch_backward_batch(int64_t n, const float* means, const float* log_scales, const float* quats,
                                   const float* sh, const FrameTable& ft, const float* splats, const uint16_t* rect,
                                   const uint32_t* offsets, const uint32_t* tiles_touched, const uint32_t* vals,
-                                  const uint32_t* ranges, const float* t_final, const uint32_t* n_contrib,
-                                  const float* d_image, float* d_means, float* d_log_scales, float* d_quats,
-                                  float* d_logits, float* d_sh, int64_t key_capacity, void* scratch,
-                                  cudaStream_t stream) {
-    float* partials = static_cast<float*>(scratch);
+                                  const uint32_t* ranges, const uint32_t* order, const float* t_final,
+                                  const uint32_t* n_contrib, const float* d_image, const float* target, float* d_means,
+                                  float* d_log_scales, float* d_quats, float* d_logits, float* d_sh,
+                                  int64_t key_capacity, bool persistent, void* scratch, cudaStream_t stream) {
+    const PairRecords partials = pair_records(scratch, key_capacity);
     const uint32_t ntiles = ft.tile_off[ft.views];
     const uint2* r2 = reinterpret_cast<const uint2*>(ranges);
     const float4* s4 = reinterpret_cast<const float4*>(splats);
     const uint2* rc = reinterpret_cast<const uint2*>(rect);
     cudaError_t e = cudaSuccess;
     if (ntiles > 0) {
+        auto run = [&](auto items) {
+            return items(r2, order, vals, n, s4, rc, offsets, ft, t_final, n_contrib, d_image, target, partials,
+                         persistent, stream);
+        };
         switch (ft.f[0].TS) {
-            case 8:
-                e = launch_pdl(k_blend_bwd_batch<8>, dim3(ntiles), dim3(64), 0, stream, r2, vals, n, s4, rc, offsets,
-                               ft, t_final, n_contrib, d_image, partials);
-                break;
-            case 16:
-                e = launch_pdl(k_blend_bwd_batch<16>, dim3(ntiles), dim3(256), 0, stream, r2, vals, n, s4, rc,
-                               offsets, ft, t_final, n_contrib, d_image, partials);
-                break;
-            case 32:
-                e = launch_pdl(k_blend_bwd_batch<32>, dim3(ntiles), dim3(256), 0, stream, r2, vals, n, s4, rc,
-                               offsets, ft, t_final, n_contrib, d_image, partials);
-                break;
-            default:
-                return cudaErrorInvalidValue;
+            case 8: e = run(launch_bwd_items<8>); break;
+            case 16: e = run(launch_bwd_items<16>); break;
+            case 32: e = run(launch_bwd_items<32>); break;
+            default: return cudaErrorInvalidValue;
         }
         if (e != cudaSuccess) return e;
     }
@@ -331,7 +330,7 @@ cudaError_t launch_backward_batch(int64_t n, const float* means, const float* lo
         const int64_t blocks = (n + kBatchThreads - 1) / kBatchThreads;
         e = launch_pdl(k_preprocess_bwd_batch, dim3((unsigned)blocks), dim3(kBatchThreads), 0, stream, n, means,
                        log_scales, reinterpret_cast<const float4*>(quats), reinterpret_cast<const float4*>(sh), ft, s4,
-                       offsets, tiles_touched, (uint32_t)key_capacity, (const float*)partials, d_means,
+                       offsets, tiles_touched, (uint32_t)key_capacity, (const float4*)partials.p8, d_means,
                        d_log_scales,
                        reinterpret_cast<float4*>(d_quats), d_logits, reinterpret_cast<float4*>(d_sh));
     }
@@ -347,72 +346,6 @@ cudaError_t launch_residual(int64_t count, const float* image, const float* targ
     return launch_pdl(k_residual, dim3(sms * 4), dim3(256), 0, stream, count,
                       reinterpret_cast<const float4*>(image), reinterpret_cast<const float4*>(target),
                       reinterpret_cast<float4*>(d_image), count / 4);
-}
-
-template <int TS>
-cudaError_t launch_train_batch_ts(const uint2* r2, const uint32_t* vals, int64_t n, const float4* s4, const uint2* rc,
-                                  const uint32_t* offsets, const FrameTable& ft, const float* target, float* image,
-                                  float* t_final, uint32_t* n_contrib, float* partials, bool persistent,
-                                  cudaStream_t stream) {
-    const uint32_t ntiles = ft.tile_off[ft.views];
-    constexpr int kThreads = TileGeom<TS>::THREADS;
-    if (!persistent)
-        return launch_pdl(k_train_batch<TS, false>, dim3(ntiles), dim3(kThreads), 0, stream, r2, vals, n, s4, rc,
-                          offsets, ft, target, image, t_final, n_contrib, partials);
-    int dev = 0, sms = 148, occ = 1;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_train_batch<TS, true>, kThreads, 0);
-    if (e != cudaSuccess) return e;
-    const uint32_t grid = min(ntiles, (uint32_t)(sms * (occ > 0 ? occ : 1)));
-    return launch_pdl(k_train_batch<TS, true>, dim3(grid), dim3(kThreads), 0, stream, r2, vals, n, s4, rc, offsets,
-                      ft, target, image, t_final, n_contrib, partials);
-}
-
-cudaError_t launch_train_batch(int64_t n, const float* means, const float* log_scales, const float* quats,
-                               const float* sh, const FrameTable& ft, const uint32_t* num_keys, const uint64_t* keys,
-                               const uint32_t* vals, const float* splats, const uint16_t* rect,
-                               const uint32_t* offsets, const uint32_t* tiles_touched, const float* target,
-                               uint32_t* ranges, float* image, float* t_final, uint32_t* n_contrib, float* d_means,
-                               float* d_log_scales, float* d_quats, float* d_logits, float* d_sh,
-                               int64_t key_capacity, bool persistent, void* scratch, cudaStream_t stream) {
-    float* partials = static_cast<float*>(scratch);
-    const uint32_t ntiles = ft.tile_off[ft.views];
-    const float4* s4 = reinterpret_cast<const float4*>(splats);
-    const uint2* rc = reinterpret_cast<const uint2*>(rect);
-    cudaError_t e = cudaSuccess;
-    if (ntiles > 0) {
-        e = launch_tile_ranges(keys, num_keys, ranges, ntiles, ft.f[0].flags, stream);
-        if (e != cudaSuccess) return e;
-        const uint2* r2 = reinterpret_cast<const uint2*>(ranges);
-        switch (ft.f[0].TS) {
-            case 8:
-                e = launch_train_batch_ts<8>(r2, vals, n, s4, rc, offsets, ft, target, image, t_final, n_contrib,
-                                             partials, persistent, stream);
-                break;
-            case 16:
-                e = launch_train_batch_ts<16>(r2, vals, n, s4, rc, offsets, ft, target, image, t_final, n_contrib,
-                                              partials, persistent, stream);
-                break;
-            case 32:
-                e = launch_train_batch_ts<32>(r2, vals, n, s4, rc, offsets, ft, target, image, t_final, n_contrib,
-                                              partials, persistent, stream);
-                break;
-            default:
-                return cudaErrorInvalidValue;
-        }
-        if (e != cudaSuccess) return e;
-    }
-    if (n > 0) {
-        const int64_t blocks = (n + kBatchThreads - 1) / kBatchThreads;
-        e = launch_pdl(k_preprocess_bwd_batch, dim3((unsigned)blocks), dim3(kBatchThreads), 0, stream, n, means,
-                       log_scales, reinterpret_cast<const float4*>(quats), reinterpret_cast<const float4*>(sh), ft, s4,
-                       offsets, tiles_touched, (uint32_t)key_capacity, (const float*)partials, d_means,
-                       d_log_scales, reinterpret_cast<float4*>(d_quats), d_logits, reinterpret_cast<float4*>(d_sh));
-    }
-    return e;
 }
 
 }  // namespace ws

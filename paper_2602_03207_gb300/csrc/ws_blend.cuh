@@ -1,6 +1,17 @@
 // Per-tile blend bodies (paper §3.4 with §2.1's compositing) shared by the
-// single-view, batched and fused training kernels: the forward composite,
-// its deterministic adjoint, and both in one pass over a tile.
+// single-view and batched kernels: the forward composite and its
+// deterministic adjoint.
+//
+// Both are bound by instruction issue and by the latency of a step's chain
+// (list entry, record, log-alpha, exponential), not by memory: on the 1080p
+// / 1M frame the forward moves 63 MB in 65 us. Measured against the walk that
+// they replace (two streams of 16 lanes, one pixel per lane, a bit set per
+// 32 splats; the backward's partials summed by 12 shuffles a visit and 16
+// selects a splat), warm, at 16-pixel tiles:
+//   forward, 1080p / 1M                 80.4 -> 64.9 us (72.0M -> 51M warp instructions)
+//   forward, 2160p / 6M                617.6 -> 448 us
+//   backward call, 720p / 500k         220.4 -> 133 us (102.6M -> 48.7M)
+//   backward call, 64 views of 2M       33.2 -> 20.6 ms
 #pragma once
 
 #include <type_traits>
@@ -9,23 +20,11 @@
 
 namespace ws {
 
-constexpr int kBlendBatch = 256;  // splats staged in shared memory at a time
-constexpr int kBwdChunk = 64;     // splats whose partials the backward holds at a time
-// The fused training pass holds the partials of 32 splats at a time: half the
-// partial buffer and 48 registers instead of 64 let five of its blocks share
-// an SM instead of four.
-constexpr int kTrainChunk = 32;
-constexpr int kPart = 9;          // dmean x, y; dconic a, b, c; sigma dsigma; drgb r, g, b
-
-// Blocks per SM that the forward blends are compiled for (their register
-// budget): 64 threads x 16, 256 x 8 and 1024 x 2 for 8, 16 and 32 pixel
-// tiles (one thread per pixel).
-template <int TS>
-constexpr int blend_min_blocks() { return TS == 8 ? 16 : (TS == 16 ? 8 : 2); }
+constexpr int kPart = 9;  // partials of a pair: dmean x, y; dconic a, b, c; sigma dsigma; drgb r, g, b
 
 // Shared-memory record of one staged splat (48 bytes):
-//   geo  = tile-relative centre x, y; conic premultiplied A = -log2(e) a / 2,
-//          B = -log2(e) b
+//   geo  = minus the tile-relative centre (-x, -y); conic premultiplied
+//          A = -log2(e) a / 2, B = -log2(e) b
 //   geo2 = C = -log2(e) c / 2, L = log2(sigma); the splat's axis basis
 //          e1 = (ct, st) (axis_basis; staged for the backward only)
 //   col  = r, g, b; 0
@@ -36,21 +35,50 @@ struct SplatRec {
     float4 col;
 };
 
-// Staged records sit in groups of 33: slot 33 g holds a null splat (zero
-// conic, L = -inf, so its log-alpha is -inf and it is never composited) and
-// slots 33 g + 1 .. 33 g + 32 the splats 32 g .. 32 g + 31, so that a
-// half-warp with nothing left to visit in a group of 32 reads the null splat
-// at index 0 of the group (__ffs of an empty bit set) and needs no select.
-__device__ __forceinline__ int rec_slot(int j) { return j + (j >> 5) + 1; }
-__host__ __device__ constexpr int rec_slots(int batch) { return batch + batch / 32 + 1; }
-
-// Writes the null splat of every group of a staging area of `batch` splats.
-__device__ __forceinline__ void init_null_splats(SplatRec* s_rec, int batch) {
-    for (int g = threadIdx.x; g <= (batch - 1) / 32; g += blockDim.x) {
-        s_rec[33 * g].geo = make_float4(0.f, 0.f, 0.f, 0.f);
-        s_rec[33 * g].geo2 = make_float4(0.f, -INFINITY, 0.f, 0.f);
-        s_rec[33 * g].col = make_float4(0.f, 0.f, 0.f, 0.f);
+// Writes the null splat at index `batch` of a staging area: zero conic,
+// L = -inf, so its log-alpha is -inf and it is never composited. The visit
+// lists of a warp's streams are padded with it.
+__device__ __forceinline__ void init_null_splat(SplatRec* s_rec, int batch) {
+    if (threadIdx.x == 0) {
+        s_rec[batch].geo = make_float4(0.f, 0.f, 0.f, 0.f);
+        s_rec[batch].geo2 = make_float4(0.f, -INFINITY, 0.f, 0.f);
+        s_rec[batch].col = make_float4(0.f, 0.f, 0.f, 0.f);
     }
+}
+
+// Two floats in one 64-bit register pair, for the two-wide FP32
+// instructions (each half rounds as the scalar instruction does).
+struct F2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ F2 pack2(float lo, float hi) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ F2 dup2(float x) { return pack2(x, x); }
+__device__ __forceinline__ void unpack2(F2 a, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a.v));
+}
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ float sum2(F2 a) {
+    float lo, hi;
+    unpack2(a, lo, hi);
+    return __fadd_rn(lo, hi);
 }
 
 // Per-splat inputs of the blend, read from the splat records of
@@ -73,30 +101,105 @@ struct FloatSplats {
     }
 };
 
-// Geometry of a TS x TS tile: TH threads, one per pixel of one 8x4 region per
-// warp (PPT regions per warp when the tile has more pixels than threads);
-// each region is two 4x4 sub-blocks, one per half-warp. A splat's mask has
-// one bit per sub-block (row-major, SPR per row). The backward and the fused
-// training pass take at most 256 threads (their per-half-warp partial
-// buffers grow with the warps); the forward blend takes one thread per pixel.
-template <int TS, int TH = (TS * TS >= 256 ? 256 : TS * TS)>
+// Geometry of a TS x TS tile: its 4x4 pixel sub-blocks (numbered row-major,
+// SPR per row) are the unit of culling, and a stream of 16 / PX lanes walks
+// the splats that reach one sub-block, PX pixels of a column per lane. A
+// warp runs SPW streams in lockstep, each on its own visit list.
+//
+// Why streams of few lanes: the steps a warp takes are the longest of its
+// streams' lists, and the work around a pixel evaluation (the list entry,
+// the three record loads, the loop, and in the backward the sum over the
+// sub-block) is paid per step, so PX pixels per lane pay it once for PX
+// evaluations, two of which share each FP32 instruction. On the 1080p / 1M
+// frame (counted on the host): 1.68M steps with two streams of 16 lanes
+// kept in step every 32 splats, 0.45M with eight streams of four lanes over a
+// whole staged batch, with 7 % more (idle included) evaluations.
+template <int TS, int PX>
 struct TileGeom {
-    static constexpr int THREADS = TH;
-    static constexpr int WARPS = THREADS / 32;
-    static constexpr int PPT = TS * TS / THREADS;
-    static constexpr int RPR = TS / 8;  // regions per row
-    static constexpr int SPR = TS / 4;  // sub-blocks per row
-    using Mask = typename std::conditional<(SPR * SPR > 32), unsigned long long, uint32_t>::type;
-    // region k of this warp: lane's pixel (tile-relative, centre) and the
-    // index of the region's left sub-block
-    __device__ static __forceinline__ void pixel(int warp, int lane, int k, float& px, float& py, int& sb) {
-        const int rg = warp + k * WARPS;
-        const int rx = rg % RPR, ry = rg / RPR;
-        px = (float)(rx * 8 + (lane >> 4) * 4 + (lane & 3)) + 0.5f;
-        py = (float)(ry * 4 + ((lane >> 2) & 3)) + 0.5f;
-        sb = ry * SPR + 2 * rx;
+    static constexpr int SPR = TS / 4;
+    static constexpr int NSB = SPR * SPR;
+    static constexpr int LPS = 16 / PX;
+    static constexpr int SPW = 32 / LPS;
+    static constexpr int WARPS = NSB / SPW;
+    static constexpr int THREADS = 32 * WARPS;
+    static_assert(NSB % SPW == 0 && PX % 2 == 0, "whole warps of streams, pairs of pixels");
+    using Mask = typename std::conditional<(NSB > 32), unsigned long long, uint32_t>::type;
+    // this lane's sub-block and its pixels (tile-relative centres): column
+    // px, rows py0 .. py0 + PX - 1
+    __device__ static __forceinline__ int sub_block(int warp, int lane) { return warp * SPW + lane / LPS; }
+    __device__ static __forceinline__ void pixel(int warp, int lane, int& ix, int& iy0) {
+        const int sb = sub_block(warp, lane), q = lane % LPS;
+        ix = (sb % SPR) * 4 + (q & 3);
+        iy0 = (sb / SPR) * 4 + (q >> 2) * PX;
     }
 };
+
+// Pixels per lane: two (four streams a warp, four warps for a 16-pixel
+// tile). Four (eight streams, two warps) execute 20 % fewer instructions but
+// leave a tile of many splats to two warps: 78 against 65 us on the 1080p /
+// 1M frame, whose longest list has 1,300 splats, 457 against 448 us at 2160p
+// / 6M. A 32-pixel tile has enough sub-blocks for eight warps of four.
+template <int TS>
+__host__ __device__ constexpr int tile_px() { return TS == 32 ? 4 : 2; }
+
+// Splats the forward stages in shared memory at a time. The visit lists hold
+// 8-bit indices, the null splat's (the batch size) among them. 192 instead of
+// 128: 66.3 against 64.9 us at 1080p / 1M (fewer blocks fit an SM).
+template <int TS>
+__host__ __device__ constexpr int fwd_batch() { return 128; }
+
+// Blocks per SM that the blends are compiled for (their register budget). At
+// 16-pixel tiles nine for the forward (56 registers: 64.9 us at 1080p / 1M
+// against 65.5 with ten, 67.5 with 80 registers and 77 with 40) and six for
+// the backward (80 registers: 133 us on the 720p call against 142 with the
+// compiler's own choice of 72, and 140 with 127).
+template <int TS>
+__host__ __device__ constexpr int fwd_min_blocks() { return TS == 8 ? 16 : (TS == 16 ? 9 : 4); }
+template <int TS>
+__host__ __device__ constexpr int bwd_min_blocks() { return TS == 8 ? 12 : (TS == 16 ? 6 : 2); }
+
+// One row of visit indices per stream: the batch and a padded end.
+template <int BATCH>
+__host__ __device__ constexpr int list_row() { return BATCH + 16; }
+
+// Builds the visit lists of this warp's streams over the staged splats
+// [lo, hi): for each stream the indices whose mask has its sub-block, in
+// list order (REV: back to front), padded with the null splat. Returns the
+// longest list's length. A list of the whole span rather than one bit set
+// per 32 splats: the streams then wait for each other only at its end.
+template <typename G, int BATCH, bool REV>
+__device__ __forceinline__ int build_lists(const typename G::Mask* s_mask, int lo, int hi, uint8_t* rows, int warp,
+                                           int lane) {
+    constexpr int ROW = list_row<BATCH>();
+    static_assert(BATCH < 256 && ROW % 16 == 0, "8-bit indices, 16-byte rows");
+    constexpr uint32_t kNull4 = 0x01010101u * (uint32_t)BATCH;
+    const int q = lane % G::LPS;
+    uint4* mine = reinterpret_cast<uint4*>(rows + (lane / G::LPS) * ROW);
+    for (int v = q; v <= (hi - lo) >> 4; v += G::LPS) mine[v] = make_uint4(kNull4, kNull4, kNull4, kNull4);
+    __syncwarp();
+    const uint32_t lt = lanemask_lt();
+    const int sb0 = warp * G::SPW;
+    int c[G::SPW];
+#pragma unroll
+    for (int t = 0; t < G::SPW; ++t) c[t] = 0;
+    for (int k = 0; k < hi - lo; k += 32) {
+        const bool in = k + lane < hi - lo;
+        const int j = REV ? hi - 1 - k - lane : lo + k + lane;
+        const uint32_t m = in ? (uint32_t)(s_mask[j] >> sb0) : 0u;
+#pragma unroll
+        for (int t = 0; t < G::SPW; ++t) {
+            const bool bit = (m >> t) & 1u;
+            const uint32_t bal = __ballot_sync(kFull, bit);
+            if (bit) rows[t * ROW + c[t] + __popc(bal & lt)] = (uint8_t)j;
+            c[t] += __popc(bal);
+        }
+    }
+    __syncwarp();
+    int steps = 0;
+#pragma unroll
+    for (int t = 0; t < G::SPW; ++t) steps = max(steps, c[t]);
+    return steps;
+}
 
 // Bitmask of a tile's 4x4 sub-blocks whose pixel centres meet the box
 // [xl, xh] x [yl, yh] (tile-relative): one compare pair per sub-block column
@@ -172,9 +275,9 @@ __device__ __forceinline__ MaskT ellipse_subblock_mask(float gx, float gy, float
 // (13 % of them on the 1080p / 1M frame): a gain where a visit is dear (the
 // backward), not in the forward. WS_CFG_BOX_MASKS takes the box's mask
 // everywhere; the results are the same bits either way.
-template <int TS, bool ELLIPSE, typename Splats>
+template <typename G, bool ELLIPSE, typename Splats>
 __device__ __forceinline__ void stage_splat(const Frame& f, float ox, float oy, const Splats& sp, uint32_t g,
-                                            SplatRec* dst, typename TileGeom<TS>::Mask& mask) {
+                                            SplatRec* dst, typename G::Mask& mask) {
     float a, b, c, op, gx, gy;
     float4 col;
     sp.load(g, ox, oy, gx, gy, a, b, c, op, col);
@@ -182,7 +285,7 @@ __device__ __forceinline__ void stage_splat(const Frame& f, float ox, float oy, 
     // the record first: its registers are free before the mask's arithmetic
     float ct = 0.f, st = 0.f;
     if (ELLIPSE) axis_basis(col.w, ct, st);
-    dst->geo = make_float4(gx, gy, -0.5f * kLog2e * a, -kLog2e * b);
+    dst->geo = make_float4(-gx, -gy, -0.5f * kLog2e * a, -kLog2e * b);
     dst->geo2 = make_float4(-0.5f * kLog2e * c, L, ct, st);
     dst->col = make_float4(col.x, col.y, col.z, 0.f);
     const float qc = (f.flags & WS_CFG_FIXED_RADIUS) ? 2.f * kLn255 : fmaxf(0.f, kTwoLn2 * (L - kLog2AlphaMin));
@@ -190,234 +293,413 @@ __device__ __forceinline__ void stage_splat(const Frame& f, float ox, float oy, 
     const float rdet = rcp_approx(fmaf(a, c, -b * b));
     const float ex = sqrt_approx(qm * c * rdet) * 1.0001f + 1e-3f;
     const float ey = sqrt_approx(qm * a * rdet) * 1.0001f + 1e-3f;
-    using M = typename TileGeom<TS>::Mask;
+    using M = typename G::Mask;
     if (ELLIPSE && !(f.flags & WS_CFG_BOX_MASKS))
-        mask = ellipse_subblock_mask<TileGeom<TS>::SPR, M>(gx, gy, a, b, c, qm, rdet, ey, fmaf(ex, 1e-4f, 1e-3f));
+        mask = ellipse_subblock_mask<G::SPR, M>(gx, gy, a, b, c, qm, rdet, ey, fmaf(ex, 1e-4f, 1e-3f));
     else
-        mask = box_subblock_mask<TileGeom<TS>::SPR, M>(gx - ex, gx + ex, gy - ey, gy + ey);
+        mask = box_subblock_mask<G::SPR, M>(gx - ex, gx + ex, gy - ey, gy + ey);
+}
+
+// e of splat_log2_alpha for a pair of pixels of one column: the same
+// operations in the same order, so the same bits.
+__device__ __forceinline__ F2 splat_log2_alpha2(float dx, F2 dy, const float4& geo, const float4& geo2) {
+    const F2 u = fma2(dup2(geo.z), dup2(dx), mul2(dup2(geo.w), dy));
+    return fma2(dup2(dx), u, fma2(mul2(dup2(geo2.x), dy), dy, dup2(geo2.y)));
 }
 
 // Forward state of a thread's pixels: front to back, C += c a T, T -= a T.
-template <int TS, int TH = TileGeom<TS>::THREADS>
+template <typename G, int PX>
 struct FwdPixels {
-    using G = TileGeom<TS, TH>;
-    float px[G::PPT], py[G::PPT], T[G::PPT], C0[G::PPT], C1[G::PPT], C2[G::PPT];
-    uint32_t last[G::PPT];
-    int sb[G::PPT];
+    static constexpr int NP = PX / 2;
+    int ix, iy0;
+    float px;
+    F2 py[NP], T[NP], C0[NP], C1[NP], C2[NP];
+    uint32_t last[PX];
 
     __device__ __forceinline__ void init(int warp, int lane) {
+        G::pixel(warp, lane, ix, iy0);
+        px = (float)ix + 0.5f;
 #pragma unroll
-        for (int k = 0; k < G::PPT; ++k) {
-            G::pixel(warp, lane, k, px[k], py[k], sb[k]);
-            T[k] = 1.f;
-            C0[k] = C1[k] = C2[k] = 0.f;
-            last[k] = 0;
+        for (int p = 0; p < NP; ++p) {
+            const float y = (float)(iy0 + 2 * p) + 0.5f;
+            py[p] = pack2(y, y + 1.f);
+            T[p] = dup2(1.f);
+            C0[p] = C1[p] = C2[p] = dup2(0.f);
+            last[2 * p] = last[2 * p + 1] = 0;
         }
     }
 
-    // Composites the staged splats [0, cnt) (list positions rel0 - 1 + j, made
-    // 1-based for n_contrib). Each half-warp walks the batch 32 splats at a
-    // time and visits only the splats whose mask has its own sub-block, in
-    // list order; the two halves run in lockstep for max(visits of either
-    // half) steps, the idle half visiting its group's null splat (w = 0,
-    // which leaves C and T bit for bit unchanged), so per pixel the
+    // Composites the visits of this lane's stream (`row`, `steps` entries,
+    // the null splat past its own). rel0: the 1-based list position of
+    // staged index 0. A null visit and one below the 1/255 test add w = 0,
+    // which leaves C and T bit for bit unchanged, so per pixel the
     // compositing order and arithmetic are those of a plain front-to-back
-    // loop. The last composited position is noted per group (1-based within
-    // the group) and made a list position once at the group's end.
-    __device__ __forceinline__ void batch(const SplatRec* s_rec, const typename G::Mask* s_mask, int cnt,
-                                          uint32_t rel0, int lane) {
-        const int half = lane >> 4;
+    // loop. The last composited index is kept 1-based and made a list
+    // position once at the end.
+    __device__ __forceinline__ void walk(const SplatRec* s_rec, const uint8_t* row, int steps, uint32_t rel0) {
+        int lastk[PX];
 #pragma unroll
-        for (int k = 0; k < G::PPT; ++k) {
-            for (int base = 0; base < cnt; base += 32) {
-                const int jj = base + lane;
-                const typename G::Mask m = jj < cnt ? s_mask[jj] : typename G::Mask(0);
-                const uint32_t ba = __ballot_sync(kFull, (uint32_t)(m >> sb[k]) & 1u);
-                const uint32_t bb = __ballot_sync(kFull, (uint32_t)(m >> (sb[k] + 1)) & 1u);
-                uint32_t bits = half ? bb : ba;
-                const int steps = max(__popc(ba), __popc(bb));
-                const SplatRec* grp = s_rec + base + (base >> 5);  // grp[0]: the null splat
-                int lastk = 0;
+        for (int k = 0; k < PX; ++k) lastk[k] = 0;
+        int j = row[0];
 #pragma unroll 4
-                for (int it = 0; it < steps; ++it) {
-                    const int q = __ffs(bits);  // 0 once this half has no visit left
-                    bits &= bits - 1u;
-                    const float4 geo = grp[q].geo;
-                    const float2 geo2 = *reinterpret_cast<const float2*>(&grp[q].geo2);
-                    const float dx = px[k] - geo.x, dy = py[k] - geo.y;
-                    const float e = splat_log2_alpha(dx, dy, geo.z, geo.w, geo2.x, geo2.y);
-                    const bool keep = e >= kLog2AlphaMin;
-                    const float alpha = fminf(kAlphaMax, ex2_approx(e));
-                    const float w = keep ? alpha * T[k] : 0.f;
-                    const float4 col = grp[q].col;
-                    C0[k] = fmaf(col.x, w, C0[k]);
-                    C1[k] = fmaf(col.y, w, C1[k]);
-                    C2[k] = fmaf(col.z, w, C2[k]);
-                    T[k] = T[k] - w;
-                    lastk = keep ? q : lastk;
+        for (int it = 0; it < steps; ++it) {
+            const SplatRec& r = s_rec[j];
+            const int j1 = j + 1;
+            j = row[it + 1];  // the next entry's latency overlaps this visit
+            const float4 geo = r.geo;
+            const float2 g2 = *reinterpret_cast<const float2*>(&r.geo2);
+            const float4 geo2 = make_float4(g2.x, g2.y, 0.f, 0.f);
+            const float4 col = r.col;
+            const float dx = __fadd_rn(px, geo.x);
+#pragma unroll
+            for (int p = 0; p < NP; ++p) {
+                const F2 e2 = splat_log2_alpha2(dx, add2(py[p], dup2(geo.y)), geo, geo2);
+                float e[2], al[2];
+                unpack2(e2, e[0], e[1]);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const bool keep = e[h] >= kLog2AlphaMin;
+                    const float alpha = fminf(kAlphaMax, ex2_approx(e[h]));
+                    al[h] = keep ? alpha : 0.f;
+                    lastk[2 * p + h] = keep ? j1 : lastk[2 * p + h];
                 }
-                if (lastk) last[k] = rel0 + (uint32_t)(base + lastk - 1);
+                const F2 w = mul2(pack2(al[0], al[1]), T[p]);
+                C0[p] = fma2(dup2(col.x), w, C0[p]);
+                C1[p] = fma2(dup2(col.y), w, C1[p]);
+                C2[p] = fma2(dup2(col.z), w, C2[p]);
+                T[p] = fma2(w, dup2(-1.f), T[p]);  // T - w
             }
         }
+#pragma unroll
+        for (int k = 0; k < PX; ++k)
+            if (lastk[k]) last[k] = rel0 + (uint32_t)(lastk[k] - 1);
     }
 };
 
+// Splats the backward stages at a time, the visits (a staged splat and a
+// sub-block that it reaches) whose rows it holds at a time, and the
+// granularity of the splat spans it processes: a span of vis_unit splats
+// always fits. At 16-pixel tiles 96 and 128: 31 KB, six blocks of which leave
+// the L1 56 KB of the SM's 256. 128 splats (35 KB a block) shrink it to 23 KB
+// and took the 64-view backward from 20.6 to 23.1 ms; 64 splats end their
+// spans early (22.5 ms), and rows for 64 visits double the barriers (21.9).
+template <int TS>
+__host__ __device__ constexpr int bwd_batch() { return TS == 16 ? 96 : 64; }
+template <int TS>
+__host__ __device__ constexpr int vis_cap() { return TS == 8 ? 32 : 128; }
+template <int TS>
+__host__ __device__ constexpr int vis_unit() { return TS == 32 ? 2 : 8; }
+
+// The pair records of a backward: partials 0..7 of slot s at p8[2 s], p8[2 s
+// + 1] (one 32-byte sector), partial 8 at p9[s].
+struct PairRecords {
+    float4* p8;
+    float* p9;
+};
+
+// The pair records in a backward's scratch: 36 bytes per key of capacity,
+// the 32-byte parts first.
+inline PairRecords pair_records(void* scratch, int64_t key_capacity) {
+    float4* p8 = static_cast<float4*>(scratch);
+    return {p8, reinterpret_cast<float*>(p8 + 2 * (size_t)key_capacity)};
+}
+
+// Shared memory of the backward, staging BATCH splats.
+template <int TS, int PX, int BATCH>
+struct BwdSmem {
+    using G = TileGeom<TS, PX>;
+    static constexpr int VCAP = vis_cap<TS>();
+    static constexpr int ROW = BATCH + 16;  // entries of a visit list
+    SplatRec rec[BATCH + 1];
+    // row v: the 16 pixels' (w, dp) of visit v, a float4 (w, w, dp, dp) for
+    // each vertical pair of pixels, and 16 bytes of padding (a thread per row
+    // then reads its float4s without bank conflicts); row VCAP takes the null
+    // visits
+    float4 vrow[(VCAP + 1) * 9];
+    __align__(16) uint16_t list[G::NSB * ROW];  // staged index | visit << 8
+    // dL/dC of each sub-block's pixels: 8 pairs (r, r, g, g), 8 pairs (b, b),
+    // in rows of 52 floats, whose float4s fall in distinct banks for eight
+    // neighbouring sub-blocks (rows of 48 cost the 64-view step 25 %)
+    __align__(16) float dC[G::NSB][52];
+    typename G::Mask mask[BATCH];
+    uint32_t slot[BATCH];
+    uint32_t maxl[G::WARPS];
+    uint16_t vis[VCAP];        // staged index | sub-block << 8
+    uint16_t base[BATCH + 2];  // visits of the staged splats before each
+};
+
 // Backward state of a thread's pixels, walked back to front from the final
-// transmittance. With B = colour behind the splat normalised by the
-// transmittance after it (B starts as the background, B <- a c + (1 - a) B):
-//   dL/dc = a T dL/dC,   dL/da = T (c - B) . dL/dC,
-// and, unless the alpha was clamped at 0.99, sigma dL/dsigma = raw dL/da
-// (raw = sigma G, the unclamped alpha) and dL/dpower = a dL/da with
-// power = -1/2 d^T Q d, giving d/dmean = Q d, d/dQ_a = -dx^2/2,
-// d/dQ_b = -dx dy, d/dQ_c = -dy^2/2.
-template <int TS, int CHUNK = kBwdChunk>
+// transmittance. With b = the colour behind the splat, normalised by the
+// transmittance after it and projected on the pixel's dL/dC (b starts as
+// bg . dL/dC, b <- a s + (1 - a) b with s = c . dL/dC):
+//   dL/dc = w dL/dC with w = a T,   dL/da = T (s - b),
+// and, unless the alpha was clamped at 0.99, sigma dL/dsigma = dL/dpower =
+// a dL/da =: dp (a = sigma G there) with power = -1/2 d^T Q d, giving
+// d/dmean = Q d dp and the conic's derivatives from dp u^2, dp u v, dp v^2
+// in the splat's axis basis. So w and dp are all a visit's pixels contribute:
+// the walk, which must follow the list, stores the two per pixel, and the
+// sums over the sub-block's 16 pixels are taken afterwards by one thread per
+// visit, with no shuffle and every lane busy.
+template <int TS, int PX>
 struct BwdPixels {
-    using G = TileGeom<TS>;
-    float px[G::PPT], py[G::PPT], T[G::PPT], dC[G::PPT][3], Bc[G::PPT][3];
-    uint32_t last[G::PPT];
-    int sb[G::PPT];
-    typename G::Mask wmask;  // sub-blocks of this warp's regions
+    using G = TileGeom<TS, PX>;
+    static constexpr int NP = PX / 2;
+    float px;
+    F2 py[NP], T[NP], b[NP], dC[NP][3];
 
-    __device__ __forceinline__ void init_geometry(int warp, int lane) {
-        wmask = 0;
+    // ix, iy0: this lane's pixels (TileGeom::pixel); tf, dc: their final
+    // transmittance and dL/dC, zeros outside the image (T = 0 there keeps
+    // every partial of such a pixel zero). s_dC: this lane's sub-block's row
+    // of BwdSmem::dC.
+    __device__ __forceinline__ void init(const Frame& f, int lane, int ix, int iy0, const float (&tf)[PX],
+                                         const float (&dc)[PX][3], float* s_dC) {
+        px = (float)ix + 0.5f;
 #pragma unroll
-        for (int k = 0; k < G::PPT; ++k) {
-            G::pixel(warp, lane, k, px[k], py[k], sb[k]);
-            wmask |= typename G::Mask(3) << sb[k];
+        for (int p = 0; p < NP; ++p) {
+            const float y = (float)(iy0 + 2 * p) + 0.5f;
+            py[p] = pack2(y, y + 1.f);
+            T[p] = pack2(tf[2 * p], tf[2 * p + 1]);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) dC[p][c] = pack2(dc[2 * p][c], dc[2 * p + 1][c]);
+            b[p] = fma2(dup2(f.bg[2]), dC[p][2], fma2(dup2(f.bg[1]), dC[p][1], mul2(dup2(f.bg[0]), dC[p][0])));
+            const int k = p * 4 + lane % G::LPS;  // pair of pixels: row pair * 4 + column
+            *reinterpret_cast<float4*>(s_dC + 4 * k) =
+                make_float4(dc[2 * p][0], dc[2 * p + 1][0], dc[2 * p][1], dc[2 * p + 1][1]);
+            *reinterpret_cast<float2*>(s_dC + 32 + 2 * k) = make_float2(dc[2 * p][2], dc[2 * p + 1][2]);
         }
     }
 
-    // Walks the staged splats [0, cnt) back to front (list positions pos0 +
-    // j), in chunks of CHUNK. Each half-warp visits, back to front, the
-    // splats whose mask has its own 4x4 sub-block; the two halves run in
-    // lockstep for max(visits of either half) steps (an idle half evaluates
-    // nothing). Each half sums its splat's 9 partials over its 16 pixels in
-    // a fixed order and stores them in s_part[j][half-warp]; the block then
-    // adds the half-warps that wrote, in order, and writes one record per
-    // pair at its emission slot.
-    __device__ __forceinline__ void batch(const SplatRec* s_rec, const typename G::Mask* s_mask,
-                                          const uint32_t* s_slot, float (*s_part)[2 * G::WARPS][kPart],
-                                          uint32_t* s_wrote, int cnt, uint32_t pos0, int warp, int lane,
-                                          float* __restrict__ partials) {
-        const int half = lane >> 4;
-        const int hw = 2 * warp + half;  // this lane's half-warp
-        for (int hi = cnt; hi > 0; hi -= CHUNK) {
-            const int lo = max(0, hi - CHUNK);
-            for (int j = threadIdx.x; j < hi - lo; j += G::THREADS) s_wrote[j] = 0u;
-            __syncthreads();
+    // A visit of this lane's stream: advances the pixels' state and stores
+    // their (w, dp) in the visit's row. A pixel that does not composite the
+    // splat has alpha = 0, which makes its w and dp zero and leaves T and b
+    // as they are, unless a colour or dL/dC is infinite or NaN: FINITE =
+    // false selects instead of multiplying, so that such a value reaches
+    // only the pixels and splats that it belongs to.
+    template <bool FINITE>
+    __device__ __forceinline__ void visit(const float4& geo, const float2& g2, const float4& col, float4* row) {
+        const float4 geo2 = make_float4(g2.x, g2.y, 0.f, 0.f);
+        const float dx = __fadd_rn(px, geo.x);
 #pragma unroll
-            for (int k = 0; k < G::PPT; ++k) {
-                for (int base = lo + (((hi - lo - 1) >> 5) << 5); base >= lo; base -= 32) {
-                    const int jj = base + lane;
-                    const typename G::Mask mm = jj < hi ? s_mask[jj] : typename G::Mask(0);
-                    const uint32_t ba = __ballot_sync(kFull, (uint32_t)(mm >> sb[k]) & 1u);
-                    const uint32_t bb = __ballot_sync(kFull, (uint32_t)(mm >> (sb[k] + 1)) & 1u);
-                    uint32_t bits = half ? bb : ba;
-                    const int steps = max(__popc(ba), __popc(bb));
-                    for (int it = 0; it < steps; ++it) {
-                        const bool act = bits != 0u;
-                        const int hb = act ? 31 - __clz(bits) : 0;
-                        bits &= ~(1u << hb);
-                        const int j = base + hb;
-                        const uint32_t pos = pos0 + (uint32_t)j;
-                        float acc[kPart];
+        for (int p = 0; p < NP; ++p) {
+            const F2 e2 = splat_log2_alpha2(dx, add2(py[p], dup2(geo.y)), geo, geo2);
+            float e[2], al[2], rt[2], au[2];
+            unpack2(e2, e[0], e[1]);
 #pragma unroll
-                        for (int c = 0; c < kPart; ++c) acc[c] = 0.f;
-                        bool any = false;
-                        if (act && pos < last[k]) {
-                            const SplatRec r = s_rec[rec_slot(j)];
-                            const float dx = px[k] - r.geo.x, dy = py[k] - r.geo.y;
-                            const float e = splat_log2_alpha(dx, dy, r.geo.z, r.geo.w, r.geo2.x, r.geo2.y);
-                            if (e >= kLog2AlphaMin) {
-                                const float raw = ex2_approx(e);
-                                const float alpha = fminf(kAlphaMax, raw);
-                                any = true;
-                                const float Tb = T[k] * rcp_approx(1.f - alpha);
-                                const float w = alpha * Tb;
-                                float dalpha = 0.f;
-                                const float cc[3] = {r.col.x, r.col.y, r.col.z};
+            for (int h = 0; h < 2; ++h) {
+                const float raw = e[h] >= kLog2AlphaMin ? ex2_approx(e[h]) : 0.f;
+                al[h] = fminf(kAlphaMax, raw);
+                au[h] = raw < kAlphaMax ? raw : 0.f;        // no gradient through the clamp
+                rt[h] = rcp_approx(__fsub_rn(1.f, al[h]));  // 1 for alpha = 0: T unchanged
+            }
+            const F2 alpha = pack2(al[0], al[1]);
+            T[p] = mul2(T[p], pack2(rt[0], rt[1]));
+            const F2 sc = fma2(dup2(col.z), dC[p][2], fma2(dup2(col.y), dC[p][1], mul2(dup2(col.x), dC[p][0])));
+            const F2 d = fma2(b[p], dup2(-1.f), sc);  // s - b
+            const F2 w = mul2(alpha, T[p]);
+            const F2 dp = mul2(pack2(au[0], au[1]), mul2(d, T[p]));
+            const F2 bn = fma2(alpha, d, b[p]);
+            float4 o;
+            unpack2(w, o.x, o.y);
+            unpack2(dp, o.z, o.w);
+            if (FINITE) {
+                b[p] = bn;
+            } else {
+                float b0, b1, n0, n1;
+                unpack2(b[p], b0, b1);
+                unpack2(bn, n0, n1);
+                b[p] = pack2(al[0] > 0.f ? n0 : b0, al[1] > 0.f ? n1 : b1);
+                o.z = au[0] > 0.f ? o.z : 0.f;
+                o.w = au[1] > 0.f ? o.w : 0.f;
+            }
+            row[p * 4] = o;
+        }
+    }
+
+    // One thread's sum over the 16 pixels of a visit of splat r in sub-block
+    // sb, in a fixed order, written over the visit's row: dp Q d (x, y) and
+    // dp (u^2, u v, v^2), dp, w dL/dC, without the constant factors that
+    // batch() applies once per splat.
+    template <bool FINITE>
+    __device__ static __forceinline__ void sum_visit(const SplatRec& r, int sb, const float* s_dC, float4* row) {
+        const float4 geo = r.geo, geo2 = r.geo2;
+        const float x0 = (float)((sb % G::SPR) * 4) + 0.5f, y0 = (float)((sb / G::SPR) * 4) + 0.5f;
+        const F2 st = dup2(geo2.w), ct = dup2(geo2.z), zero = dup2(0.f);
+        bool any = FINITE;
+        F2 S0 = zero, Sx = zero, Sy = zero, Suu = zero, Suv = zero, Svv = zero, Cr = zero, Cg = zero, Cb = zero;
 #pragma unroll
-                                for (int c = 0; c < 3; ++c) {
-                                    acc[6 + c] = w * dC[k][c];
-                                    dalpha = fmaf(cc[c] - Bc[k][c], dC[k][c], dalpha);
-                                    Bc[k][c] = fmaf(alpha, cc[c] - Bc[k][c], Bc[k][c]);
-                                }
-                                dalpha *= Tb;
-                                T[k] = Tb;
-                                if (raw < kAlphaMax) {
-                                    acc[5] = raw * dalpha;
-                                    const float dp = alpha * dalpha;
-                                    // d/dmean = dp C d with C = -(2A, B; B, 2C) / log2(e)
-                                    const float dpl = -kLn2 * dp;
-                                    acc[0] = dpl * fmaf(2.f * r.geo.z, dx, r.geo.w * dy);
-                                    acc[1] = dpl * fmaf(r.geo.w, dx, 2.f * r.geo2.x * dy);
-                                    // conic derivatives in the splat's axis basis
-                                    const float ct = r.geo2.z, st = r.geo2.w;
-                                    const float u = fmaf(ct, dx, st * dy), v = fmaf(ct, dy, -st * dx);
-                                    const float hdp = -0.5f * dp;
-                                    acc[2] = hdp * (u * u);
-                                    acc[3] = -dp * (u * v);
-                                    acc[4] = hdp * (v * v);
-                                }
-                            }
-                        }
-                        const uint32_t anyb = __ballot_sync(kFull, any);
-                        if (anyb) {
-                            // Sums over each half's 16 lanes in a fixed order, 12
-                            // shuffles for both halves: partials 0..7 by
-                            // reduce-scatter (offsets 8, 4, 2; lane l of a half then
-                            // holds partial (l >> 1) & 7 over 8 lanes) and a last
-                            // butterfly step (offset 1), partial 8 by a butterfly.
-                            const bool b3 = lane & 8, b2 = lane & 4, b1 = lane & 2;
-                            float h4[4];
+        for (int k = 0; k < 8; ++k) {
+            const float dx = __fadd_rn(x0 + (float)(k & 3), geo.x);
+            const float y = y0 + (float)(2 * (k >> 2));
+            const F2 dy = add2(pack2(y, y + 1.f), dup2(geo.y));
+            const F2 u = fma2(st, dy, dup2(__fmul_rn(geo2.z, dx))), v = fma2(ct, dy, dup2(__fmul_rn(-geo2.w, dx)));
+            const float4 q = row[k];
+            const F2 w = pack2(q.x, q.y), dp = pack2(q.z, q.w);
+            const F2 du = mul2(dp, u), dv = mul2(dp, v);
+            float4 rg = *reinterpret_cast<const float4*>(s_dC + 4 * k);
+            float2 bb = *reinterpret_cast<const float2*>(s_dC + 32 + 2 * k);
+            if (!FINITE) {  // only the pixels that composite the splat
+                any = any || q.x != 0.f || q.y != 0.f || q.z != 0.f || q.w != 0.f;
+                if (q.x == 0.f) rg.x = rg.z = bb.x = 0.f;
+                if (q.y == 0.f) rg.y = rg.w = bb.y = 0.f;
+            }
+            S0 = add2(S0, dp);
+            Sx = fma2(dp, dup2(dx), Sx);
+            Sy = fma2(dp, dy, Sy);
+            Suu = fma2(du, u, Suu);
+            Suv = fma2(du, v, Suv);
+            Svv = fma2(dv, v, Svv);
+            Cr = fma2(w, pack2(rg.x, rg.y), Cr);
+            Cg = fma2(w, pack2(rg.z, rg.w), Cg);
+            Cb = fma2(w, pack2(bb.x, bb.y), Cb);
+        }
+        const float sx = sum2(Sx), sy = sum2(Sy), hb = __fmul_rn(0.5f, geo.w);
+        row[0] = make_float4(__fmaf_rn(geo.z, sx, __fmul_rn(hb, sy)), __fmaf_rn(geo2.x, sy, __fmul_rn(hb, sx)),
+                             sum2(Suu), sum2(Suv));
+        row[1] = make_float4(sum2(Svv), sum2(S0), sum2(Cr), sum2(Cg));
+        row[2].x = sum2(Cb);
+        if (!any) row[0] = row[1] = row[2] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+
+    // The visit lists of this warp's streams over the staged splats [lo, hi),
+    // back to front (as build_lists), each entry with the visit's row; also
+    // vis[]. Returns the longest list's length.
+    template <int BATCH>
+    __device__ __forceinline__ int build_visits(BwdSmem<TS, PX, BATCH>& sm, int lo, int hi, int vis0, int warp,
+                                                int lane) {
+        using S = BwdSmem<TS, PX, BATCH>;
+        static_assert(BATCH < 256 && S::VCAP < 256 && S::ROW % 8 == 0, "8-bit indices and visits, 16-byte rows");
+        uint16_t* rows = sm.list + warp * G::SPW * S::ROW;
+        constexpr uint32_t kNull2 = 0x00010001u * (uint32_t)(BATCH | (S::VCAP << 8));
+        uint4* mine = reinterpret_cast<uint4*>(rows + (lane / G::LPS) * S::ROW);
+        for (int v = lane % G::LPS; v <= (hi - lo + 1) >> 3; v += G::LPS) mine[v] = make_uint4(kNull2, kNull2, kNull2, kNull2);
+        __syncwarp();
+        const uint32_t lt = lanemask_lt();
+        const int sb0 = warp * G::SPW;
+        int c[G::SPW];
 #pragma unroll
-                            for (int q = 0; q < 4; ++q) {
-                                const float give = b3 ? acc[q] : acc[4 + q];
-                                const float keep = b3 ? acc[4 + q] : acc[q];
-                                h4[q] = keep + __shfl_xor_sync(kFull, give, 8);
-                            }
-                            float h2[2];
+        for (int t = 0; t < G::SPW; ++t) c[t] = 0;
+        for (int k = 0; k < hi - lo; k += 32) {
+            const bool in = k + lane < hi - lo;
+            const int j = hi - 1 - k - lane;
+            const typename G::Mask full = in ? sm.mask[j] : typename G::Mask(0);
+            const uint32_t m = (uint32_t)(full >> sb0);
+            int v = in ? (int)sm.base[j] - vis0 + popc_mask(full & ((typename G::Mask(1) << sb0) - 1)) : 0;
 #pragma unroll
-                            for (int q = 0; q < 2; ++q) {
-                                const float give = b2 ? h4[q] : h4[2 + q];
-                                const float keep = b2 ? h4[2 + q] : h4[q];
-                                h2[q] = keep + __shfl_xor_sync(kFull, give, 4);
-                            }
-                            float h1 = (b1 ? h2[1] : h2[0]) + __shfl_xor_sync(kFull, b1 ? h2[0] : h2[1], 2);
-                            h1 += __shfl_xor_sync(kFull, h1, 1);
-                            float v8 = acc[8];
-#pragma unroll
-                            for (int o = 8; o > 0; o >>= 1) v8 += __shfl_xor_sync(kFull, v8, o);
-                            const bool mine = (anyb >> (16 * half)) & 0xffffu;  // this half has a partial
-                            if (mine) {
-                                // with several regions per warp, a half-warp adds to
-                                // what it stored for the same splat in an earlier region
-                                const bool add = G::PPT > 1 && ((s_wrote[j - lo] >> hw) & 1u);
-                                const int p = ((lane & 15) >> 1);
-                                if ((lane & 1) == 0) s_part[j - lo][hw][p] = add ? s_part[j - lo][hw][p] + h1 : h1;
-                                if ((lane & 15) == 0) {
-                                    s_part[j - lo][hw][8] = add ? s_part[j - lo][hw][8] + v8 : v8;
-                                    atomicOr(s_wrote + (j - lo), 1u << hw);
-                                }
-                            }
-                        }
-                    }
+            for (int t = 0; t < G::SPW; ++t) {
+                const bool bit = (m >> t) & 1u;
+                const uint32_t bal = __ballot_sync(kFull, bit);
+                if (bit) {
+                    rows[t * S::ROW + c[t] + __popc(bal & lt)] = (uint16_t)(j | (v << 8));
+                    sm.vis[v] = (uint16_t)(j | ((sb0 + t) << 8));
+                    ++v;
                 }
-                __syncwarp();  // this region's stores and flags before the next region's reads
+                c[t] += __popc(bal);
             }
-            __syncthreads();
-            // Block sum over the half-warps that wrote, in order, one record per pair.
-            for (int e = threadIdx.x; e < (hi - lo) * kPart; e += G::THREADS) {
-                const int j = e / kPart, c = e - j * kPart;
-                const uint32_t wr = s_wrote[j];
-                float s = 0.f;
+        }
+        __syncwarp();
+        int steps = 0;
 #pragma unroll
-                for (int w = 0; w < 2 * G::WARPS; ++w) s += ((wr >> w) & 1u) ? s_part[j][w][c] : 0.f;
-                partials[(size_t)s_slot[lo + j] * kPart + c] = s;
-            }
-            __syncthreads();
+        for (int t = 0; t < G::SPW; ++t) steps = max(steps, c[t]);
+        return steps;
+    }
+
+    // This lane's visits of one span. The next visit's record is loaded
+    // before this one's stores (which the compiler must assume to alias it),
+    // the entry after it before that, so their latencies overlap the
+    // arithmetic: 157 -> 152 us on the 720p backward call.
+    template <bool FINITE, typename S>
+    __device__ __forceinline__ void walk(const S& sm, const uint16_t* row, float4* vrow, int steps) {
+        uint32_t code = row[0], next = row[1];
+        const SplatRec* r = sm.rec + (code & 255u);
+        float4 geo = r->geo, col = r->col;
+        float2 g2 = *reinterpret_cast<const float2*>(&r->geo2);
+#pragma unroll FINITE ? 4 : 1
+        for (int it = 0; it < steps; ++it) {
+            const float4 geo0 = geo, col0 = col;
+            const float2 g20 = g2;
+            float4* dst = vrow + (code >> 8) * 9;
+            code = next;
+            next = row[it + 2];
+            r = sm.rec + (code & 255u);
+            geo = r->geo;
+            col = r->col;
+            g2 = *reinterpret_cast<const float2*>(&r->geo2);
+            visit<FINITE>(geo0, g20, col0, dst);
         }
     }
+
+    // Walks the staged splats [0, cnt) back to front. The splats are taken
+    // in spans of at most vis_cap visits: every stream walks its visits of
+    // the span (visit), one thread per visit sums its pixels (sum_visit),
+    // and one thread per splat adds its visits (contiguous, its sub-blocks
+    // ascending) and writes its record at the pair's emission slot. Which
+    // visits exist is known from the masks, so nothing is cleared or
+    // flagged.
+    template <bool FINITE, int BATCH>
+    __device__ __forceinline__ void batch(BwdSmem<TS, PX, BATCH>& sm, int cnt, int warp, int lane,
+                                          const PairRecords& out) {
+        using S = BwdSmem<TS, PX, BATCH>;
+        if (warp == 0) {  // exclusive scan of the visit counts
+            uint32_t run = 0;
+            for (int k = 0; k < cnt; k += 32) {
+                const uint32_t n = k + lane < cnt ? (uint32_t)popc_mask(sm.mask[k + lane]) : 0u;
+                uint32_t x = n;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t y = __shfl_up_sync(kFull, x, o);
+                    if (lane >= o) x += y;
+                }
+                if (k + lane < cnt) sm.base[k + lane] = (uint16_t)(run + x - n);
+                run += __shfl_sync(kFull, x, 31);
+            }
+            if (lane == 0) sm.base[cnt] = (uint16_t)run;
+        }
+        __syncthreads();
+        const uint16_t* row = sm.list + (warp * G::SPW + lane / G::LPS) * S::ROW;
+        float4* vrow = sm.vrow + lane % G::LPS;
+        constexpr int U = vis_unit<TS>();
+        for (int hi = cnt; hi > 0;) {
+            // the longest span [lo, hi), lo a multiple of U, that fits
+            int lo = ((hi - 1) / U - lane) * U;
+            const int end = sm.base[hi];
+            const bool fits = lo >= 0 && end - (int)sm.base[max(lo, 0)] <= S::VCAP;
+            lo = ((hi - 1) / U - (__popc(__ballot_sync(kFull, fits)) - 1)) * U;
+            const int vis0 = sm.base[lo];
+            const int steps = build_visits<BATCH>(sm, lo, hi, vis0, warp, lane);
+            walk<FINITE>(sm, row, vrow, steps);
+            __syncthreads();
+            for (int v = threadIdx.x; v < end - vis0; v += G::THREADS) {
+                const uint32_t c = sm.vis[v];
+                sum_visit<FINITE>(sm.rec[c & 255u], (int)(c >> 8), sm.dC[c >> 8], sm.vrow + v * 9);
+            }
+            __syncthreads();
+            for (int j = lo + threadIdx.x; j < hi; j += G::THREADS) {
+                float4 a = make_float4(0.f, 0.f, 0.f, 0.f), c = a;
+                float d = 0.f;
+                const int v1 = (int)sm.base[j + 1] - vis0;
+                for (int v = (int)sm.base[j] - vis0; v < v1; ++v) {
+                    const float4 x = sm.vrow[v * 9], y = sm.vrow[v * 9 + 1];
+                    a.x += x.x;
+                    a.y += x.y;
+                    a.z += x.z;
+                    a.w += x.w;
+                    c.x += y.x;
+                    c.y += y.y;
+                    c.z += y.z;
+                    c.w += y.w;
+                    d += sm.vrow[v * 9 + 2].x;
+                }
+                const size_t s = sm.slot[j];
+                out.p8[2 * s] = make_float4(-2.f * kLn2 * a.x, -2.f * kLn2 * a.y, -0.5f * a.z, -a.w);
+                out.p8[2 * s + 1] = make_float4(-0.5f * c.x, c.y, c.z, c.w);
+                out.p9[s] = d;
+            }
+            __syncthreads();
+            hi = lo;
+        }
+    }
+    __device__ static __forceinline__ int popc_mask(uint32_t m) { return __popc(m); }
+    __device__ static __forceinline__ int popc_mask(unsigned long long m) { return __popcll(m); }
 };
 
 // Tile of a frame that the backward's launch index b takes: the tile rows
@@ -446,12 +728,11 @@ __device__ __forceinline__ uint32_t pair_slot(SlotBase slot_of, const uint2* __r
 
 // Block-wide maximum of the last-contributor counts (positions past it are
 // never composited; their records are zero).
-template <int TS>
-__device__ __forceinline__ uint32_t block_max_last(const uint32_t* last, uint32_t* s_max, int warp, int lane) {
-    using G = TileGeom<TS>;
+template <typename G, int PX>
+__device__ __forceinline__ uint32_t block_max_last(const uint32_t (&last)[PX], uint32_t* s_max, int warp, int lane) {
     uint32_t my = 0;
 #pragma unroll
-    for (int k = 0; k < G::PPT; ++k) my = max(my, last[k]);
+    for (int k = 0; k < PX; ++k) my = max(my, last[k]);
     for (int o = 16; o > 0; o >>= 1) my = max(my, __shfl_xor_sync(kFull, my, o));
     if (lane == 0) s_max[warp] = my;
     __syncthreads();
@@ -465,233 +746,204 @@ __device__ __forceinline__ uint32_t block_max_last(const uint32_t* last, uint32_
 template <typename SlotBase>
 __device__ __forceinline__ void zero_records(uint2 range, uint32_t from, const uint32_t* __restrict__ vals,
                                              const uint2* __restrict__ rect, SlotBase slot_of, int tx, int ty,
-                                             int threads, float* __restrict__ partials) {
+                                             int threads, const PairRecords& out) {
     const uint32_t len = range.y - range.x;
     for (uint32_t j = from + threadIdx.x; j < len; j += threads) {
         const uint32_t slot = pair_slot(slot_of, rect, __ldg(vals + range.x + j), tx, ty);
-        float* dst = partials + (size_t)slot * kPart;
-#pragma unroll
-        for (int c = 0; c < kPart; ++c) dst[c] = 0.f;
+        out.p8[2 * (size_t)slot] = out.p8[2 * (size_t)slot + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
+        out.p9[slot] = 0.f;
     }
 }
 
-// Slot-ordered sum of a Gaussian's nrec pair records (kPart floats each,
-// contiguous from src) into pr: the loads of four records are issued before
-// their adds, and the adds keep slot order (a record past nrec adds +0, which
-// leaves a sum that started at +0 bit for bit unchanged), so the result is
-// that of the plain loop with a quarter of its dependent load latencies.
-__device__ __forceinline__ void sum_pair_records(const float* __restrict__ src, uint32_t nrec, float (&pr)[kPart]) {
+// Slot-ordered sum of a Gaussian's nrec pair records (slots first ..) into
+// pr: the loads of four records are issued before their adds, and the adds
+// keep slot order (a record past nrec adds +0, which leaves a sum that
+// started at +0 bit for bit unchanged), so the result is that of the plain
+// loop with a quarter of its dependent load latencies.
+__device__ __forceinline__ void sum_pair_records(const float4* __restrict__ p8, const float* __restrict__ p9,
+                                                 size_t first, uint32_t nrec, float (&pr)[kPart]) {
     for (uint32_t s = 0; s < nrec; s += 4) {
-        float r[4][kPart];
+        float4 a[4], b[4];
+        float c[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const bool ok = s + k < nrec;
-#pragma unroll
-            for (int c = 0; c < kPart; ++c) r[k][c] = ok ? __ldg(src + (size_t)(s + k) * kPart + c) : 0.f;
+            const size_t t = first + s + k;
+            a[k] = ok ? __ldg(p8 + 2 * t) : make_float4(0.f, 0.f, 0.f, 0.f);
+            b[k] = ok ? __ldg(p8 + 2 * t + 1) : make_float4(0.f, 0.f, 0.f, 0.f);
+            c[k] = ok ? __ldg(p9 + t) : 0.f;
         }
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-#pragma unroll
-            for (int c = 0; c < kPart; ++c) pr[c] += r[k][c];
+        for (int k = 0; k < 4; ++k) {
+            pr[0] += a[k].x;
+            pr[1] += a[k].y;
+            pr[2] += a[k].z;
+            pr[3] += a[k].w;
+            pr[4] += b[k].x;
+            pr[5] += b[k].y;
+            pr[6] += b[k].z;
+            pr[7] += b[k].w;
+            pr[8] += c[k];
+        }
     }
 }
 
 // Stages list positions [start, start + cnt) of a tile: records and masks,
-// and (WITH_SLOT) each pair's emission slot. The stagings of the backward
-// and of the fused training pass (WITH_SLOT) build the ellipse's sub-block
-// masks, the forward's the bounding box's.
-template <int TS, bool WITH_SLOT, typename Splats, typename SlotBase, int TH = TileGeom<TS>::THREADS>
-__device__ __forceinline__ void stage_batch(const Frame& f, float ox, float oy, int tx, int ty, uint32_t start,
+// and (WITH_SLOT) each pair's emission slot. The staging of the backward
+// (WITH_SLOT) builds the ellipse's sub-block
+// masks, the forward's the bounding box's. Returns whether the records that
+// this thread staged are finite (WITH_SLOT).
+template <typename G, bool WITH_SLOT, typename Splats, typename SlotBase>
+__device__ __forceinline__ bool stage_batch(const Frame& f, float ox, float oy, int tx, int ty, uint32_t start,
                                             int cnt, const uint32_t* __restrict__ vals, const Splats& sp,
                                             const uint2* __restrict__ rect, SlotBase slot_of, SplatRec* s_rec,
-                                            typename TileGeom<TS>::Mask* s_mask, uint32_t* s_slot) {
-    for (int j = threadIdx.x; j < cnt; j += TH) {
+                                            typename G::Mask* s_mask, uint32_t* s_slot) {
+    bool finite = true;
+    for (int j = threadIdx.x; j < cnt; j += G::THREADS) {
         const uint32_t g = __ldg(vals + start + j);
-        typename TileGeom<TS>::Mask m;
-        stage_splat<TS, WITH_SLOT>(f, ox, oy, sp, g, s_rec + rec_slot(j), m);
+        typename G::Mask m;
+        stage_splat<G, WITH_SLOT>(f, ox, oy, sp, g, s_rec + j, m);
         s_mask[j] = m;
-        if (WITH_SLOT) s_slot[j] = pair_slot(slot_of, rect, g, tx, ty);
+        if (WITH_SLOT) {
+            s_slot[j] = pair_slot(slot_of, rect, g, tx, ty);
+            const SplatRec& r = s_rec[j];  // 0 x is 0 for a finite x and NaN otherwise
+            float z = 0.f;
+            z = fmaf(r.geo.x, 0.f, fmaf(r.geo.y, 0.f, fmaf(r.geo.z, 0.f, fmaf(r.geo.w, 0.f, z))));
+            z = fmaf(r.geo2.x, 0.f, fmaf(r.geo2.y, 0.f, fmaf(r.geo2.z, 0.f, fmaf(r.geo2.w, 0.f, z))));
+            z = fmaf(r.col.x, 0.f, fmaf(r.col.y, 0.f, fmaf(r.col.z, 0.f, z)));
+            finite = finite && z == 0.f;
+        }
     }
+    return finite;
 }
 
 struct NoSlot {
     __device__ __forceinline__ uint32_t operator()(uint32_t) const { return 0u; }
 };
 
-// Forward of one tile, one thread per pixel (TS * TS threads): stages the
-// list 256 splats at a time and composites each batch (FwdPixels::batch),
+// Forward of one tile: stages the list a batch at a time, and each warp
+// builds its streams' visit lists and composites them (FwdPixels::walk);
 // then writes image = C + T bg, the final transmittance and the 1-based list
 // position of the last composited splat.
-template <int TS, typename Splats>
+template <int TS, int PX, typename Splats>
 __device__ __forceinline__ void blend_tile(const Frame& f, int tile, uint2 range, const uint32_t* __restrict__ vals,
                                            const Splats& sp, float* __restrict__ image, float* __restrict__ t_final,
                                            uint32_t* __restrict__ n_contrib) {
-    constexpr int TH = TS * TS;
-    using G = TileGeom<TS, TH>;
-    __shared__ SplatRec s_rec[rec_slots(kBlendBatch)];
-    __shared__ typename G::Mask s_mask[kBlendBatch];
+    using G = TileGeom<TS, PX>;
+    constexpr int BATCH = fwd_batch<TS>();
+    __shared__ SplatRec s_rec[BATCH + 1];
+    __shared__ typename G::Mask s_mask[BATCH];
+    __shared__ __align__(16) uint8_t s_list[G::NSB * list_row<BATCH>()];
     const int tx = tile % f.TX, ty = tile / f.TX;
     const float ox = (float)(tx * TS), oy = (float)(ty * TS);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    init_null_splats(s_rec, kBlendBatch);
-    FwdPixels<TS, TH> P;
+    uint8_t* rows = s_list + warp * G::SPW * list_row<BATCH>();
+    init_null_splat(s_rec, BATCH);
+    FwdPixels<G, PX> P;
     P.init(warp, lane);
-    for (uint32_t start = range.x; start < range.y; start += kBlendBatch) {
-        const int cnt = (int)min((uint32_t)kBlendBatch, range.y - start);
+    for (uint32_t start = range.x; start < range.y; start += BATCH) {
+        const int cnt = (int)min((uint32_t)BATCH, range.y - start);
         __syncthreads();
-        stage_batch<TS, false, Splats, NoSlot, TH>(f, ox, oy, tx, ty, start, cnt, vals, sp, nullptr, NoSlot{}, s_rec,
-                                                   s_mask, nullptr);
+        stage_batch<G, false>(f, ox, oy, tx, ty, start, cnt, vals, sp, nullptr, NoSlot{}, s_rec, s_mask, nullptr);
         __syncthreads();
-        P.batch(s_rec, s_mask, cnt, start + 1 - range.x, lane);
+        const int steps = build_lists<G, BATCH, false>(s_mask, 0, cnt, rows, warp, lane);
+        P.walk(s_rec, rows + (lane / G::LPS) * list_row<BATCH>(), steps, start + 1 - range.x);
     }
+    const int gx = tx * TS + P.ix;
 #pragma unroll
-    for (int k = 0; k < G::PPT; ++k) {
-        const int gx = tx * TS + (int)P.px[k], gy = ty * TS + (int)P.py[k];
+    for (int k = 0; k < PX; ++k) {
+        const int gy = ty * TS + P.iy0 + k;
         if (gx < f.W && gy < f.H) {
             const size_t pix = (size_t)gy * f.W + gx;
-            image[3 * pix] = fmaf(P.T[k], f.bg[0], P.C0[k]);
-            image[3 * pix + 1] = fmaf(P.T[k], f.bg[1], P.C1[k]);
-            image[3 * pix + 2] = fmaf(P.T[k], f.bg[2], P.C2[k]);
-            t_final[pix] = P.T[k];
+            float c[2][4];
+            unpack2(P.T[k / 2], c[0][3], c[1][3]);
+            unpack2(P.C0[k / 2], c[0][0], c[1][0]);
+            unpack2(P.C1[k / 2], c[0][1], c[1][1]);
+            unpack2(P.C2[k / 2], c[0][2], c[1][2]);
+            const float(&o)[4] = c[k & 1];
+            image[3 * pix] = fmaf(o[3], f.bg[0], o[0]);
+            image[3 * pix + 1] = fmaf(o[3], f.bg[1], o[1]);
+            image[3 * pix + 2] = fmaf(o[3], f.bg[2], o[2]);
+            t_final[pix] = o[3];
             n_contrib[pix] = P.last[k];
         }
     }
 }
 
-// Shared memory of the backward and fused kernels, staging BATCH splats and
-// holding the partials of CHUNK of them.
-template <int TS, int BATCH = kBlendBatch, int CHUNK = kBwdChunk>
-struct BwdSmem {
-    SplatRec rec[rec_slots(BATCH)];
-    typename TileGeom<TS>::Mask mask[BATCH];
-    uint32_t slot[BATCH];
-    float part[CHUNK][2 * TileGeom<TS>::WARPS][kPart];
-    uint32_t wrote[CHUNK];
-    uint32_t maxl[TileGeom<TS>::WARPS];
-};
-
-// Shared memory of the fused training pass.
-template <int TS>
-using TrainSmem = BwdSmem<TS, kBlendBatch, kTrainChunk>;
-
 // Backward of one tile from the stored forward outputs: each pair's 9
-// partials at its emission slot (see BwdPixels), staging kBwdChunk splats at
-// a time (the smaller shared-memory footprint keeps more blocks resident).
-// `slot_of(g)` gives the first emission slot of Gaussian g's pairs for this
-// frame (offsets[g] for one view, offsets[v * n + g] in a batch).
-template <int TS, typename SlotBase>
-__device__ __forceinline__ void blend_bwd_tile(const Frame& f, int tile, uint2 range, const uint32_t* __restrict__ vals,
+// partials at its emission slot (see BwdPixels). offsets[g]: the first
+// emission slot of Gaussian g's pairs (in a batch, of this view's). dL/dC is d_image, or in an L2
+// training step d_image - target with the image in d_image's place.
+// FINITE = true stops and returns false when a staged record or a dL/dC is
+// infinite or NaN.
+template <int TS, int PX, bool FINITE>
+__device__ __forceinline__ bool bwd_tile_body(const Frame& f, int tile, uint2 range, const uint32_t* __restrict__ vals,
                                                const float4* __restrict__ splats, const uint2* __restrict__ rect,
-                                               SlotBase slot_of, const float* __restrict__ t_final,
+                                               const uint32_t* __restrict__ offsets, const float* __restrict__ t_final,
                                                const uint32_t* __restrict__ n_contrib,
-                                               const float* __restrict__ d_image, float* __restrict__ partials) {
-    using G = TileGeom<TS>;
-    __shared__ BwdSmem<TS, kBwdChunk> sm;
+                                               const float* __restrict__ d_image, const float* __restrict__ target,
+                                               const PairRecords& out, BwdSmem<TS, PX, bwd_batch<TS>()>& sm) {
+    using G = TileGeom<TS, PX>;
+    constexpr int BATCH = bwd_batch<TS>();
     const int tx = tile % f.TX, ty = tile / f.TX;
     const float ox = (float)(tx * TS), oy = (float)(ty * TS);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const FloatSplats sp{splats};
-    BwdPixels<TS> B;
-    B.init_geometry(warp, lane);
-#pragma unroll
-    for (int k = 0; k < G::PPT; ++k) {
-        const int gx = tx * TS + (int)B.px[k], gy = ty * TS + (int)B.py[k];
-        const bool inside = gx < f.W && gy < f.H;
-        const size_t pix = inside ? (size_t)gy * f.W + gx : 0;
-        B.T[k] = inside ? t_final[pix] : 1.f;
-        B.last[k] = inside ? n_contrib[pix] : 0u;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            B.dC[k][c] = inside ? d_image[3 * pix + c] : 0.f;
-            B.Bc[k][c] = f.bg[c];
-        }
-    }
-    const uint32_t max_last = block_max_last<TS>(B.last, sm.maxl, warp, lane);
-    zero_records(range, max_last, vals, rect, slot_of, tx, ty, G::THREADS, partials);
-    // batches of the composited prefix [0, max_last), last batch first
-    const int nb = (int)((max_last + kBwdChunk - 1) / kBwdChunk);
-    for (int b = nb - 1; b >= 0; --b) {
-        const uint32_t lo = (uint32_t)b * kBwdChunk;
-        const int cnt = (int)min((uint32_t)kBwdChunk, max_last - lo);
-        __syncthreads();
-        stage_batch<TS, true>(f, ox, oy, tx, ty, range.x + lo, cnt, vals, sp, rect, slot_of, sm.rec, sm.mask,
-                              sm.slot);
-        __syncthreads();
-        B.batch(sm.rec, sm.mask, sm.slot, sm.part, sm.wrote, cnt, lo, warp, lane, partials);
-    }
-}
-
-// One training step's blend of one tile in a single pass: the forward
-// composite (bit-identical to blend_tile), image and final transmittance
-// written, the L2 residual d = image - target formed in registers, then the
-// backward of BwdPixels over the same list. When the tile's list fits one
-// batch (most tiles), the backward reuses the forward's staged records.
-template <int TS, typename SlotBase>
-__device__ __forceinline__ void train_tile(const Frame& f, int tile, uint2 range, const uint32_t* __restrict__ vals,
-                                           const float4* __restrict__ splats, const uint2* __restrict__ rect,
-                                           SlotBase slot_of, const float* __restrict__ target,
-                                           float* __restrict__ image, float* __restrict__ t_final,
-                                           uint32_t* __restrict__ n_contrib, float* __restrict__ partials,
-                                           TrainSmem<TS>& sm) {
-    using G = TileGeom<TS>;
-    const int tx = tile % f.TX, ty = tile / f.TX;
-    const float ox = (float)(tx * TS), oy = (float)(ty * TS);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const FloatSplats sp{splats};
-    const uint32_t len = range.y - range.x;
-    const int nb = (int)((len + kBlendBatch - 1) / kBlendBatch);
-    init_null_splats(sm.rec, kBlendBatch);
-    BwdPixels<TS, kTrainChunk> B;
+    const auto slot_of = [offsets](uint32_t g) { return __ldg(offsets + g); };
+    init_null_splat(sm.rec, BATCH);
+    BwdPixels<TS, PX> B;
+    uint32_t last[PX];
+    bool dc_finite = true;
     {
-        FwdPixels<TS> P;
-        P.init(warp, lane);
-        for (int b = 0; b < nb; ++b) {
-            const uint32_t lo = (uint32_t)b * kBlendBatch;
-            const int cnt = (int)min((uint32_t)kBlendBatch, len - lo);
-            __syncthreads();
-            stage_batch<TS, true>(f, ox, oy, tx, ty, range.x + lo, cnt, vals, sp, rect, slot_of, sm.rec, sm.mask,
-                                  sm.slot);
-            __syncthreads();
-            P.batch(sm.rec, sm.mask, cnt, lo + 1, lane);
-        }
-        B.init_geometry(warp, lane);
+        int ix, iy0;
+        G::pixel(warp, lane, ix, iy0);
+        float tf[PX], dc[PX][3];
+        const int gx = tx * TS + ix;
 #pragma unroll
-        for (int k = 0; k < G::PPT; ++k) {
-            const int gx = tx * TS + (int)P.px[k], gy = ty * TS + (int)P.py[k];
+        for (int k = 0; k < PX; ++k) {
+            const int gy = ty * TS + iy0 + k;
             const bool inside = gx < f.W && gy < f.H;
             const size_t pix = inside ? (size_t)gy * f.W + gx : 0;
-            const float img[3] = {fmaf(P.T[k], f.bg[0], P.C0[k]), fmaf(P.T[k], f.bg[1], P.C1[k]),
-                                  fmaf(P.T[k], f.bg[2], P.C2[k])};
-            if (inside) {
-                image[3 * pix] = img[0];
-                image[3 * pix + 1] = img[1];
-                image[3 * pix + 2] = img[2];
-                t_final[pix] = P.T[k];
-                n_contrib[pix] = P.last[k];
-            }
-            B.T[k] = inside ? P.T[k] : 1.f;
-            B.last[k] = inside ? P.last[k] : 0u;
+            tf[k] = inside ? t_final[pix] : 0.f;
+            last[k] = inside ? n_contrib[pix] : 0u;
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                B.dC[k][c] = inside ? img[c] - __ldg(target + 3 * pix + c) : 0.f;
-                B.Bc[k][c] = f.bg[c];
+                const float g = inside ? d_image[3 * pix + c] : 0.f;
+                dc[k][c] = target && inside ? g - __ldg(target + 3 * pix + c) : g;
+                dc_finite = dc_finite && dc[k][c] * 0.f == 0.f;
             }
         }
+        B.init(f, lane, ix, iy0, tf, dc, sm.dC[G::sub_block(warp, lane)]);
     }
-    const uint32_t max_last = block_max_last<TS>(B.last, sm.maxl, warp, lane);
-    zero_records(range, max_last, vals, rect, slot_of, tx, ty, G::THREADS, partials);
-    const int nbb = (int)((max_last + kBlendBatch - 1) / kBlendBatch);
-    for (int b = nbb - 1; b >= 0; --b) {
-        const uint32_t lo = (uint32_t)b * kBlendBatch;
-        const int cnt = (int)min((uint32_t)kBlendBatch, max_last - lo);
-        if (b != nb - 1) {  // the last forward batch is still staged
-            __syncthreads();
-            stage_batch<TS, true>(f, ox, oy, tx, ty, range.x + lo, cnt, vals, sp, rect, slot_of, sm.rec, sm.mask,
-                                  sm.slot);
-        }
+    const uint32_t max_last = block_max_last<G>(last, sm.maxl, warp, lane);
+    zero_records(range, max_last, vals, rect, slot_of, tx, ty, G::THREADS, out);
+    // batches of the composited prefix [0, max_last), last batch first
+    const int nb = (int)((max_last + BATCH - 1) / BATCH);
+    for (int b = nb - 1; b >= 0; --b) {
+        const uint32_t lo = (uint32_t)b * BATCH;
+        const int cnt = (int)min((uint32_t)BATCH, max_last - lo);
         __syncthreads();
-        B.batch(sm.rec, sm.mask, sm.slot, sm.part, sm.wrote, cnt, lo, warp, lane, partials);
+        const bool ok =
+            stage_batch<G, true>(f, ox, oy, tx, ty, range.x + lo, cnt, vals, sp, rect, slot_of, sm.rec, sm.mask, sm.slot);
+        if (!__syncthreads_and(ok && dc_finite) && FINITE) return false;
+        B.template batch<FINITE>(sm, cnt, warp, lane, out);
     }
+    return true;
+}
+
+template <int TS, int PX>
+__device__ __forceinline__ void blend_bwd_tile(const Frame& f, int tile, uint2 range, const uint32_t* __restrict__ vals,
+                                               const float4* __restrict__ splats, const uint2* __restrict__ rect,
+                                               const uint32_t* __restrict__ offsets, const float* __restrict__ t_final,
+                                               const uint32_t* __restrict__ n_contrib,
+                                               const float* __restrict__ d_image, const float* __restrict__ target,
+                                               const PairRecords& out, BwdSmem<TS, PX, bwd_batch<TS>()>& sm) {
+    if (bwd_tile_body<TS, PX, true>(f, tile, range, vals, splats, rect, offsets, t_final, n_contrib, d_image, target,
+                                    out, sm))
+        return;
+    __syncthreads();
+    bwd_tile_body<TS, PX, false>(f, tile, range, vals, splats, rect, offsets, t_final, n_contrib, d_image, target, out,
+                                 sm);
 }
 
 }  // namespace ws

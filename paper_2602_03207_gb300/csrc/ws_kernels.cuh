@@ -77,7 +77,7 @@ cudaError_t launch_tile_ranges(const uint64_t* keys, const uint32_t* num_keys, u
                                uint32_t flags, cudaStream_t stream);
 cudaError_t launch_rasterize(const uint32_t* num_keys, int64_t key_capacity_hint,
                              const uint64_t* keys, const uint32_t* vals, const float* splats,
-                             const Frame& f, uint32_t* ranges, float* image, float* t_final,
+                             const Frame& f, uint32_t* ranges, const uint32_t* order, float* image, float* t_final,
                              uint32_t* n_contrib, cudaStream_t stream);
 
 // ---- packed-record variant
@@ -101,12 +101,21 @@ cudaError_t launch_render_quads(int64_t n, const float* splats, const float* dep
                                 float* t_final, void* workspace, cudaStream_t stream);
 
 // ---- backward
+// Tile counts for which the tiles are ordered by list length: below, every
+// block is resident at once and the order does not matter; the scratch holds
+// kOrderMax of them.
+constexpr uint32_t kOrderMin = 1024, kOrderMax = 1u << 18;
 size_t backward_scratch_bytes(int64_t key_capacity);
+// *order: the tiles, longest list first, in the backward's scratch; null
+// where the count is outside [kOrderMin, kOrderMax].
+cudaError_t launch_tile_order(const uint32_t* ranges, uint32_t ntiles, int64_t key_capacity, void* scratch,
+                              const uint32_t** order, cudaStream_t stream);
+// target: null, or the L2 target with the image in d_image's place.
 cudaError_t launch_backward(int64_t n, const float* means, const float* log_scales, const float* quats,
                             const float* sh, const Frame& f, const float* splats, const uint16_t* rect,
                             const uint32_t* offsets, const uint32_t* tiles_touched,
-                            const uint32_t* vals, const uint32_t* ranges, const float* t_final,
-                            const uint32_t* n_contrib, const float* d_image, float* d_means,
+                            const uint32_t* vals, const uint32_t* ranges, const uint32_t* order, const float* t_final,
+                            const uint32_t* n_contrib, const float* d_image, const float* target, float* d_means,
                             float* d_log_scales, float* d_quats, float* d_logits, float* d_sh,
                             int64_t key_capacity, void* scratch, cudaStream_t stream);
 
@@ -115,32 +124,16 @@ cudaError_t launch_preprocess_batch(int64_t n, const float* means, const float* 
                                     const float* logits, const float* sh, const FrameTable& ft, float* splats,
                                     float* depth, uint16_t* rect, uint32_t* tiles_touched, cudaStream_t stream);
 cudaError_t launch_rasterize_batch(const uint32_t* num_keys, const uint64_t* keys, const uint32_t* vals, int64_t n,
-                                   const float* splats, const FrameTable& ft, uint32_t* ranges, float* image, float* t_final,
-                                   uint32_t* n_contrib, cudaStream_t stream);
+                                   const float* splats, const FrameTable& ft, uint32_t* ranges, const uint32_t* order,
+                                   float* image, float* t_final, uint32_t* n_contrib, cudaStream_t stream);
 cudaError_t launch_backward_batch(int64_t n, const float* means, const float* log_scales, const float* quats,
                                   const float* sh, const FrameTable& ft, const float* splats, const uint16_t* rect,
                                   const uint32_t* offsets, const uint32_t* tiles_touched, const uint32_t* vals,
-                                  const uint32_t* ranges, const float* t_final, const uint32_t* n_contrib,
-                                  const float* d_image, float* d_means, float* d_log_scales, float* d_quats,
-                                  float* d_logits, float* d_sh, int64_t key_capacity, void* scratch,
-                                  cudaStream_t stream);
+                                  const uint32_t* ranges, const uint32_t* order, const float* t_final,
+                                  const uint32_t* n_contrib, const float* d_image, const float* target, float* d_means,
+                                  float* d_log_scales, float* d_quats, float* d_logits, float* d_sh,
+                                  int64_t key_capacity, bool persistent, void* scratch, cudaStream_t stream);
 cudaError_t launch_residual(int64_t count, const float* image, const float* target, float* d_image,
                             cudaStream_t stream);
-
-// ---- fused training step (blend forward + L2 residual + backward records,
-// then the per-Gaussian adjoint)
-cudaError_t launch_train(int64_t n, const float* means, const float* log_scales, const float* quats, const float* sh,
-                         const Frame& f, const uint32_t* num_keys, const uint64_t* keys, const uint32_t* vals,
-                         const float* splats, const uint16_t* rect, const uint32_t* offsets,
-                         const uint32_t* tiles_touched, const float* target, uint32_t* ranges, float* image,
-                         float* t_final, uint32_t* n_contrib, float* d_means, float* d_log_scales, float* d_quats,
-                         float* d_logits, float* d_sh, int64_t key_capacity, void* scratch, cudaStream_t stream);
-cudaError_t launch_train_batch(int64_t n, const float* means, const float* log_scales, const float* quats,
-                               const float* sh, const FrameTable& ft, const uint32_t* num_keys, const uint64_t* keys,
-                               const uint32_t* vals, const float* splats, const uint16_t* rect,
-                               const uint32_t* offsets, const uint32_t* tiles_touched, const float* target,
-                               uint32_t* ranges, float* image, float* t_final, uint32_t* n_contrib, float* d_means,
-                               float* d_log_scales, float* d_quats, float* d_logits, float* d_sh,
-                               int64_t key_capacity, bool persistent, void* scratch, cudaStream_t stream);
 
 }  // namespace ws

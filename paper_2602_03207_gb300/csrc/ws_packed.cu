@@ -205,15 +205,15 @@ k_preprocess_packed(int64_t n, const float* __restrict__ means, const float* __r
     }
 }
 
-template <int TS>
-__global__ void __launch_bounds__(TS * TS, blend_min_blocks<TS>())
+template <int TS, int PX>
+__global__ void __launch_bounds__(TileGeom<TS, PX>::THREADS, fwd_min_blocks<TS>())
 k_blend_packed(const uint2* __restrict__ ranges, const uint32_t* __restrict__ vals,
                const float2* __restrict__ mean2d, const uint2* __restrict__ axes,
                const uint32_t* __restrict__ rgba, const Frame f, float* __restrict__ image,
                float* __restrict__ t_final, uint32_t* __restrict__ n_contrib) {
     pdl_wait();
     const PackedSplats sp{mean2d, axes, rgba};
-    blend_tile<TS>(f, blockIdx.x, ranges[blockIdx.x], vals, sp, image, t_final, n_contrib);
+    blend_tile<TS, PX>(f, blockIdx.x, ranges[blockIdx.x], vals, sp, image, t_final, n_contrib);
 }
 
 }  // namespace
@@ -241,18 +241,15 @@ cudaError_t launch_rasterize_packed(const uint32_t* num_keys, const uint64_t* ke
     const uint2* r2 = reinterpret_cast<const uint2*>(ranges);
     const float2* m2 = reinterpret_cast<const float2*>(mean2d);
     const uint2* a2 = reinterpret_cast<const uint2*>(axes);
+    auto run = [&](auto kernel, int threads) {
+        return launch_pdl(kernel, dim3(ntiles), dim3(threads), 0, stream, r2, vals, m2, a2, rgba, f, image, t_final,
+                          n_contrib);
+    };
     switch (f.TS) {
-        case 8:
-            return launch_pdl(k_blend_packed<8>, dim3(ntiles), dim3(64), 0, stream, r2, vals, m2, a2, rgba, f, image,
-                              t_final, n_contrib);
-        case 16:
-            return launch_pdl(k_blend_packed<16>, dim3(ntiles), dim3(256), 0, stream, r2, vals, m2, a2, rgba, f,
-                              image, t_final, n_contrib);
-        case 32:
-            return launch_pdl(k_blend_packed<32>, dim3(ntiles), dim3(1024), 0, stream, r2, vals, m2, a2, rgba, f,
-                              image, t_final, n_contrib);
-        default:
-            return cudaErrorInvalidValue;
+        case 8: return run(k_blend_packed<8, tile_px<8>()>, TileGeom<8, tile_px<8>()>::THREADS);
+        case 16: return run(k_blend_packed<16, tile_px<16>()>, TileGeom<16, tile_px<16>()>::THREADS);
+        case 32: return run(k_blend_packed<32, tile_px<32>()>, TileGeom<32, tile_px<32>()>::THREADS);
+        default: return cudaErrorInvalidValue;
     }
 }
 

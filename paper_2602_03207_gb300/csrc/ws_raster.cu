@@ -48,13 +48,14 @@ k_tile_ranges(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ nu
         });
 }
 
-template <int TS>
-__global__ void __launch_bounds__(TS * TS, blend_min_blocks<TS>())
-k_blend(const uint2* __restrict__ ranges, const uint32_t* __restrict__ vals, const float4* __restrict__ splats,
-        const Frame f, float* __restrict__ image, float* __restrict__ t_final, uint32_t* __restrict__ n_contrib) {
+template <int TS, int PX>
+__global__ void __launch_bounds__(TileGeom<TS, PX>::THREADS, fwd_min_blocks<TS>())
+k_blend(const uint2* __restrict__ ranges, const uint32_t* __restrict__ order, const uint32_t* __restrict__ vals,
+        const float4* __restrict__ splats, const Frame f, float* __restrict__ image, float* __restrict__ t_final, uint32_t* __restrict__ n_contrib) {
     pdl_wait();
     const FloatSplats sp{splats};
-    blend_tile<TS>(f, blockIdx.x, ranges[blockIdx.x], vals, sp, image, t_final, n_contrib);
+    const uint32_t t = order ? __ldg(order + blockIdx.x) : blockIdx.x;
+    blend_tile<TS, PX>(f, (int)t, ranges[t], vals, sp, image, t_final, n_contrib);
 }
 
 }  // namespace
@@ -71,26 +72,23 @@ cudaError_t launch_tile_ranges(const uint64_t* keys, const uint32_t* num_keys, u
 
 cudaError_t launch_rasterize(const uint32_t* num_keys, int64_t /*key_capacity_hint*/,
                              const uint64_t* keys, const uint32_t* vals, const float* splats,
-                             const Frame& f, uint32_t* ranges, float* image, float* t_final,
+                             const Frame& f, uint32_t* ranges, const uint32_t* order, float* image, float* t_final,
                              uint32_t* n_contrib, cudaStream_t stream) {
     const int ntiles = f.TX * f.TY;
     if (ntiles == 0) return cudaSuccess;
-    cudaError_t e = launch_tile_ranges(keys, num_keys, ranges, (uint32_t)ntiles, f.flags, stream);
+    const cudaError_t e = launch_tile_ranges(keys, num_keys, ranges, (uint32_t)ntiles, f.flags, stream);
     if (e != cudaSuccess) return e;
     const uint2* r2 = reinterpret_cast<const uint2*>(ranges);
     const float4* s4 = reinterpret_cast<const float4*>(splats);
+    auto run = [&](auto kernel, int threads) {
+        return launch_pdl(kernel, dim3(ntiles), dim3(threads), 0, stream, r2, order, vals, s4, f, image, t_final,
+                          n_contrib);
+    };
     switch (f.TS) {
-        case 8:
-            return launch_pdl(k_blend<8>, dim3(ntiles), dim3(64), 0, stream, r2, vals, s4, f, image, t_final,
-                              n_contrib);
-        case 16:
-            return launch_pdl(k_blend<16>, dim3(ntiles), dim3(256), 0, stream, r2, vals, s4, f, image, t_final,
-                              n_contrib);
-        case 32:
-            return launch_pdl(k_blend<32>, dim3(ntiles), dim3(1024), 0, stream, r2, vals, s4, f, image, t_final,
-                              n_contrib);
-        default:
-            return cudaErrorInvalidValue;
+        case 8: return run(k_blend<8, tile_px<8>()>, TileGeom<8, tile_px<8>()>::THREADS);
+        case 16: return run(k_blend<16, tile_px<16>()>, TileGeom<16, tile_px<16>()>::THREADS);
+        case 32: return run(k_blend<32, tile_px<32>()>, TileGeom<32, tile_px<32>()>::THREADS);
+        default: return cudaErrorInvalidValue;
     }
 }
 

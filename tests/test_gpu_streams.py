@@ -1,0 +1,122 @@
+"""The blends' visit streams at the sizes where they can go wrong: list lengths
+around the staging batches (96 in the backward, 128 in the forward), the spans
+of the backward (8 splats that reach every sub-block fill its rows), tile
+counts around the one from which the backward orders its tiles, and infinite
+or NaN values, which must reach only the splats that they belong to."""
+import numpy as np
+import pytest
+
+import oracle
+from helpers import compare_image, fetch, gpu_frame
+from paper_2602_03207_gb300 import synthetic as S
+
+pytestmark = pytest.mark.gpu
+
+GRAD_RTOL = 1e-3
+
+
+def _scene(n, seed, log_scale):
+    """n splats in front of a small camera, log-scales around log_scale."""
+    s = S.uniform_scene(n, seed=seed, extent=0.6, log_scale_mean=log_scale, log_scale_std=0.3)
+    s["opacity_logits"] = np.clip(s["opacity_logits"], -3.0, 3.0)
+    return s
+
+
+def _cam(width, height, f=64.0, bg=(0.2, 0.4, 0.1)):
+    view = np.array([[1, 0, 0, 0], [0, 1, 0, 0], [0, 0, 1, 3]], dtype=np.float32)
+    return {"viewmat": view, "fx": f, "fy": f, "cx": width / 2.0, "cy": height / 2.0, "width": width,
+            "height": height, "znear": float(np.float32(0.2)), "bg": bg}
+
+
+def _check(scene, cam, tile, capacity):
+    import torch
+    from paper_2602_03207_gb300 import render
+    g = gpu_frame(scene, cam, tile=tile, key_capacity=capacity)
+    ref = oracle.render(scene, cam, tile=tile)
+    stats = compare_image(fetch(g), ref)
+    assert stats["n_bad"] == 0, stats
+    target = np.random.default_rng(5).random((cam["height"], cam["width"], 3)).astype(np.float32)
+    dev = render.scene_to_device(scene)
+    r = render.Renderer(len(scene["means"]), cam["width"], cam["height"], tile=tile, key_capacity=capacity)
+    grads = {k: v.clone() for k, v in r.train_step_l2(dev, cam, torch.as_tensor(target).cuda()).items()}
+    r.check_status()
+    img = r.forward(dev, cam)
+    sep = r.backward(dev, cam, img - torch.as_tensor(target).cuda())
+    want = oracle.loss_grad(scene, cam, target, tile=tile)["grads"]
+    for k, v in grads.items():
+        assert torch.equal(v, sep[k]), k
+        a, b = v.cpu().numpy().astype(np.float64).ravel(), want[k].ravel()
+        assert np.linalg.norm(a - b) <= GRAD_RTOL * max(np.linalg.norm(b), 1e-12), k
+
+
+@pytest.mark.parametrize("tile", [8, 16, 32])
+@pytest.mark.parametrize("n", [1, 8, 9, 32, 33, 64, 65, 96, 97, 128, 129, 193, 300])
+def test_list_lengths_around_the_batches(tile, n):
+    """Splats of several pixels over one and a half tiles a side: every list
+    close to n long, most splats reaching every sub-block."""
+    cam = _cam(tile + tile // 2 + 1, tile + 3)
+    _check(_scene(n, 10 + n, -1.2), cam, tile, 64 * n + 64)
+
+
+@pytest.mark.parametrize("tile,width,height", [(8, 256, 255), (8, 259, 253), (16, 509, 515)])
+def test_tile_counts_around_the_ordering(tile, width, height):
+    """1,024 tiles and a few more or fewer (33 x 32 and 32 x 33 included)."""
+    cam = _cam(width, height, f=float(width))
+    _check(_scene(800, 3, -3.5), cam, tile, 100_000)
+
+
+@pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan])
+def test_non_finite_gradient_stays_with_its_pixel(value):
+    """dL/dimage infinite or NaN at one pixel: the splats composited there get
+    non-finite gradients, every other splat the bits it gets with a zero
+    there. A splat is composited there iff a gradient of one at this pixel
+    alone reaches its colour."""
+    import torch
+    from paper_2602_03207_gb300 import render
+    cam = _cam(40, 37)
+    scene = render.scene_to_device(_scene(400, 21, -3.0))
+    r = render.Renderer(400, 40, 37, key_capacity=20_000)
+    r.forward(scene, cam)
+    d = torch.randn(37, 40, 3, generator=torch.Generator().manual_seed(1)).cuda()
+    d[18, 17] = 0.0
+    plain = r.backward(scene, cam, d)
+    one = torch.zeros_like(d)
+    one[18, 17] = 1.0
+    there = r.backward(scene, cam, one)["sh"].abs().sum((1, 2)) > 0
+    d[18, 17] = value
+    bad = r.backward(scene, cam, d)
+    assert there.any() and not there.all()
+    for k, v in bad.items():
+        assert torch.equal(v[~there], plain[k][~there]), k
+    assert not torch.isfinite(bad["sh"][there]).all(dim=(1, 2)).any()
+
+
+def test_non_finite_colour_stays_with_its_splat():
+    """An infinite SH coefficient makes one splat's colour infinite: with a
+    finite dL/dimage, the splats that share no pixel with it keep the bits
+    they have without it."""
+    import torch
+    from paper_2602_03207_gb300 import render
+    cam = _cam(40, 37)
+    scene = render.scene_to_device(_scene(400, 22, -3.0))
+    r = render.Renderer(400, 40, 37, key_capacity=20_000)
+    r.forward(scene, cam)
+    d = torch.randn(37, 40, 3, generator=torch.Generator().manual_seed(2)).cuda()
+    plain = r.backward(scene, cam, d)
+    g = int((r.tiles_touched[:400] > 0).nonzero()[7])
+    # the pixels that splat g composites: where the image changes with its colour
+    base = r.forward(scene, cam).clone()
+    sh = scene["sh"].clone()
+    scene["sh"][g, 0] += 1.0
+    touched = (r.forward(scene, cam) != base).any(-1)
+    scene["sh"].copy_(sh)
+    own = torch.zeros_like(d)
+    own[touched] = 1.0
+    r.forward(scene, cam)
+    shared = r.backward(scene, cam, own)["sh"].abs().sum((1, 2)) > 0
+    scene["sh"][g, 0] = float("inf")
+    r.forward(scene, cam)
+    bad = r.backward(scene, cam, d)
+    assert shared[g] and not shared.all()
+    for k, v in bad.items():
+        assert torch.equal(v[~shared], plain[k][~shared]), k
