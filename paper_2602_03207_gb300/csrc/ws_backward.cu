@@ -154,8 +154,9 @@ k_preprocess_bwd(int64_t n, const float* __restrict__ means, const float* __rest
 
 
 // Tiles sorted by the length of their lists, longest first (64 classes, two
-// per octave; raster order within a class): a stable counting sort by one
-// block, each warp ranking a contiguous run of tiles with ballots. A tile's
+// per octave): a counting sort by one block, with integer atomics in shared
+// memory, so that the order within a class and warp is not fixed; no result
+// depends on the order that the tiles are taken in. A tile's
 // time in the backward grows with its list, and a long one that starts late
 // runs on alone: on the 720p / 500k step (lists up to 914, mean 138) the SMs
 // were busy for 170k of the 237k cycles of the tile-centred order. The
@@ -180,27 +181,22 @@ k_tile_order(const uint2* __restrict__ ranges, uint32_t ntiles, uint32_t* __rest
     __syncthreads();
     const uint32_t per = (ntiles + kOrderThreads * U - 1) / (kOrderThreads * U) * (32 * U);
     const uint32_t lo = min(warp * per, ntiles), hi = min(lo + per, ntiles);
-    const uint32_t lt = lanemask_lt();
     // pass 0 counts, pass 1 places
     for (int pass = 0; pass < 2; ++pass) {
         for (uint32_t i0 = lo; i0 < hi; i0 += 32 * U) {
-            uint32_t cls[U];
+            uint32_t len[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const uint32_t i = i0 + u * 32 + lane;
                 const uint2 r = i < hi ? __ldg(ranges + i) : make_uint2(0u, 0u);
-                cls[u] = length_class(r.y - r.x);
+                len[u] = r.y - r.x;
             }
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const uint32_t i = i0 + u * 32 + lane;
-                const bool ok = i < hi;
-                const uint32_t peers = warp_match_digit<kOrderBits>(cls[u], ok);
-                const uint32_t prior = s_cnt[warp][cls[u]];
-                __syncwarp();
-                if (ok && (peers & lt) == 0u) s_cnt[warp][cls[u]] = prior + __popc(peers);
-                if (ok && pass) order[prior + __popc(peers & lt)] = i;
-                __syncwarp();
+                if (i >= hi) break;
+                const uint32_t at = atomicAdd(&s_cnt[warp][length_class(len[u])], 1u);
+                if (pass) order[at] = i;
             }
         }
         __syncthreads();
