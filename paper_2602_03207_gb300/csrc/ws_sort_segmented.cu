@@ -7,19 +7,28 @@
 //      bits [31, end_bit) only. Being stable, they leave each segment's keys
 //      in input order.
 //   2. bounds:    start[s] = first position whose segment id is >= s, for
-//      every s in [0, 2^(end_bit - 31)], from adjacent-key comparisons.
+//      every s in [0, 2^(end_bit - 31)], by searches of the partitioned keys.
 //   3. local:     every segment is sorted by its sub-key bits [begin_bit, 31)
-//      on chip. A warp sorts a segment of at most 256 keys with a bitonic
-//      network in registers over (sub-key << 32 | input index), whose
-//      values are unique, so ties keep their input order. A block of its
-//      own sorts a segment of at most 2048 keys in shared memory, and one
-//      of more keys with chunked passes over global memory; both use stable
-//      8-bit counting passes ranked with warp ballots, skipping a pass whose
-//      digit is the same for every key of the segment.
+//      on chip, as 32-bit words: the sub-key's distance from the segment's
+//      smallest, cut to the leading bits that fit, above the position in the
+//      segment. The words are distinct and positions break ties, so equal
+//      sub-keys keep their input order; where bits were cut off, a check of
+//      neighbours by the whole sub-key puts right what they would have
+//      decided (fix_order). A warp sorts a segment of at most 512 keys with a
+//      bitonic network in registers, a block one of at most 2,048 (256 threads)
+//      or 8,192 (1,024 threads) with three 7-bit counting passes in shared memory, and one of more
+//      keys with chunked 8-bit passes over global memory, ranked with warp
+//      ballots, skipping a pass whose digit is the same for every key.
 // A stable partition by the high bits followed by a stable sort of each
 // segment by the low bits orders the pairs exactly as the full-key LSD
 // sort does, ties included. There are no global atomics and no block waits
 // on another: each segment belongs to one block.
+//
+// The local sorts are bound by instruction issue: 64-bit words (the whole
+// sub-key above the position) took the network two shuffles, a two-part
+// comparison and two selects an element and stage against a shuffle and a
+// minimum or maximum, and a block's passes four rounds of 12-byte pairs against
+// three of 4-byte words.
 #include "ws_common.cuh"
 #include "ws_kernels.cuh"
 
@@ -27,37 +36,63 @@ namespace ws {
 
 namespace {
 
-constexpr int kSegThreads = 256;
+constexpr int kSegThreads = 256;      // a block of segments, or of one segment of at most 2,048 keys
+constexpr int kHugeThreads = 1024;     // a block of one larger segment
 constexpr int kSegWarps = kSegThreads / kWarp;
 constexpr int kSegItems = 8;
-constexpr int kWarpCap = kWarp * kSegItems;       // keys a warp sorts alone
-constexpr int kCtaCap = kSegThreads * kSegItems;  // keys the block sorts in shared memory
+constexpr int kWarpItems = 16;
+constexpr int kWarpCap = kWarp * kWarpItems;      // keys a warp sorts alone
+// keys that a block of THREADS sorts in shared memory, or takes at a time of a
+// larger segment
+template <int THREADS>
+__host__ __device__ constexpr int block_cap() { return THREADS * kSegItems; }
 constexpr int kLocalBits = 8;
 constexpr int kLocalRadix = 1 << kLocalBits;
 constexpr int kSplitBit = 31;                     // segment id above, sub-key below
 constexpr int kMaxSegBits = 24;
 
-// start[s] for s in (seg(i-1), seg(i)]: the first position of every segment,
-// empty ones included; start[nseg] = n (scan_boundaries over positions 0..n).
+// start[s], the first position whose segment is >= s, for s in [0, nseg], and
+// the same boundaries as [start, end) per tile (the local sort keeps every
+// segment in place). Eight lanes search one boundary, each round splitting
+// the remaining range in nine: seven rounds of dependent loads for 1M keys
+// whatever their distribution, and only the probed sectors are read. A pass
+// over all keys that compares neighbours read 8.9 MB and took 9.5 us on the
+// 1080p / 1M frame.
+constexpr int kBoundLanes = 8;
+
 __global__ void __launch_bounds__(256)
 k_seg_bounds(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ num_keys, uint32_t cap,
              uint32_t seg_mask, uint32_t nseg, uint32_t* __restrict__ start, uint2* __restrict__ ranges,
              uint32_t ntiles) {
     pdl_wait();
-    const int lane = threadIdx.x & 31;
-    const int64_t nt = ranges ? (int64_t)ntiles : 0;
-    scan_boundaries<4>(
-        keys, min(*num_keys, cap), (int64_t)nseg,
-        [seg_mask](uint64_t k) { return (int64_t)((uint32_t)(k >> kSplitBit) & seg_mask); },
-        [&](int64_t lo, int64_t hi, uint32_t pos) {
-            for (int64_t s = lo + 1 + lane; s <= hi; s += kWarp) start[s] = pos;
-            // the same boundaries as [start, end) per segment: a local sort
-            // keeps every segment in place
-            for (int64_t t = lo + lane; t <= hi && t < nt; t += kWarp) {
-                if (t >= 0 && t < hi) ranges[t].y = pos;
-                if (t > lo) ranges[t].x = pos;
-            }
-        });
+    const uint32_t s = (blockIdx.x * 256u + threadIdx.x) / kBoundLanes;
+    const uint32_t lane = threadIdx.x % kBoundLanes;
+    const uint32_t gshift = threadIdx.x & 31u & ~(kBoundLanes - 1u);
+    const uint32_t n = min(*num_keys, cap);
+    // the answer lies in [lo, hi]; keys before lo are < s, keys from hi on >= s
+    uint32_t lo = 0, hi = s == 0 ? 0u : n;
+    if (s > nseg) lo = hi = 0;
+    while (__any_sync(kFull, lo < hi)) {
+        const uint32_t len = hi - lo;
+        // probes lo + k len / 9 for k = 1 .. 8 (all below hi when lo < hi)
+        const uint32_t pos = lo + (uint32_t)(((uint64_t)len * (lane + 1u)) / (kBoundLanes + 1u));
+        const bool below = lo < hi && ((uint32_t)(__ldg(keys + pos) >> kSplitBit) & seg_mask) < s;
+        const uint32_t c = __popc((__ballot_sync(kFull, below) >> gshift) & ((1u << kBoundLanes) - 1u));
+        if (lo < hi) {
+            const uint32_t nlo = c == 0 ? lo : lo + (uint32_t)(((uint64_t)len * c) / (kBoundLanes + 1u)) + 1u;
+            const uint32_t nhi = c == kBoundLanes ? hi : lo + (uint32_t)(((uint64_t)len * (c + 1u)) / (kBoundLanes + 1u));
+            lo = nlo;
+            hi = nhi;
+        }
+    }
+    if (lane == 0 && s <= nseg) {
+        start[s] = s == nseg ? n : lo;
+        const uint32_t p = s == nseg ? n : lo;
+        if (ranges) {
+            if (s < ntiles) ranges[s].x = p;
+            if (s >= 1 && s - 1 < ntiles) ranges[s - 1].y = p;
+        }
+    }
 }
 
 __device__ __forceinline__ uint32_t sub_key(uint64_t k, int begin_bit, uint32_t sub_mask) {
@@ -96,99 +131,139 @@ __device__ __forceinline__ void warp_rank(const uint64_t (&key)[kSegItems], int 
     }
 }
 
-__device__ __forceinline__ uint64_t shfl_xor64(uint64_t v, int m) {
-    const uint32_t lo = __shfl_xor_sync(kFull, (uint32_t)v, m);
-    const uint32_t hi = __shfl_xor_sync(kFull, (uint32_t)(v >> 32), m);
-    return ((uint64_t)hi << 32) | lo;
+// Sort word of the element at position `idx` of its segment: its sub-key less
+// the segment's smallest, without the lowest `cut` bits, above the position.
+__device__ __forceinline__ uint32_t sort_word(uint32_t sub, uint32_t least, int cut, int idx_bits, uint32_t idx) {
+    return (((sub - least) >> cut) << idx_bits) | idx;
 }
 
-// Bitonic sorting network over the warp's 32*K values, element e = lane*K + k
-// in register k of lane `lane`; ascending on return. The values are
-// distinct (the sort key carries the input index), so each compare-exchange
-// is one 64-bit comparison whose outcome, xor the direction, picks the
-// element to keep. For the stages whose partner is in another lane
-// (j >= K), the direction depends on the lane only: bits j and `size` of
-// e = lane*K + k are those of lane*K, since k < K <= j.
+// Bits to cut off so that `range` (largest less smallest sub-key) fits above
+// idx_bits of position.
+__device__ __forceinline__ int cut_bits(uint32_t range, int idx_bits) {
+    return max(0, 32 - __clz(range) - (32 - idx_bits));
+}
+
+// Bitonic sorting network over the warp's 32*K distinct words, element
+// e = lane*K + k in register k of lane `lane`; ascending on return. In the
+// phase of runs of `size`, the lanes of descending runs hold their words
+// complemented, so that every exchange is an ascending one.
 template <int K>
-__device__ __forceinline__ void warp_bitonic(uint64_t (&v)[K]) {
+__device__ __forceinline__ void warp_bitonic(uint32_t (&v)[K]) {
     const int lane = threadIdx.x & 31;
     const int lk = lane * K;
     constexpr int N = kWarp * K;
 #pragma unroll
     for (int size = 2; size <= N; size <<= 1) {
+        // complement where the run's direction differs from the last phase's
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const bool down = ((lk + k) & size) != 0;
+            const bool was = size > 2 && ((lk + k) & (size >> 1)) != 0;
+            v[k] ^= down != was ? ~0u : 0u;
+        }
 #pragma unroll
         for (int j = size >> 1; j > 0; j >>= 1) {
             if (j < K) {  // partner in the same lane
 #pragma unroll
                 for (int k = 0; k < K; ++k) {
                     if (k & j) continue;
-                    const bool up = ((lk + k) & size) == 0;
-                    const uint64_t x = v[k], y = v[k | j];
-                    const bool swap = (x > y) == up;
-                    v[k] = swap ? y : x;
-                    v[k | j] = swap ? x : y;
+                    const uint32_t x = v[k], y = v[k | j];
+                    v[k] = min(x, y);
+                    v[k | j] = max(x, y);
                 }
             } else {  // partner in lane ^ (j / K), same register
-                const bool keep_min = ((lk & j) == 0) == ((lk & size) == 0);
+                const bool low = (lk & j) == 0;
 #pragma unroll
                 for (int k = 0; k < K; ++k) {
-                    const uint64_t o = shfl_xor64(v[k], j / K);
-                    v[k] = ((o < v[k]) == keep_min) ? o : v[k];
+                    const uint32_t o = __shfl_xor_sync(kFull, v[k], j / K);
+                    v[k] = low ? min(v[k], o) : max(v[k], o);
                 }
             }
         }
     }
 }
 
-// Index of element e in a warp's staging slice: one padding element after
-// every 8, so the transposing accesses (lane l touching element l*K + k)
-// fall in distinct banks: word 9l + k for K = 8.
-__device__ __forceinline__ int spad(int e) { return e + (e >> 3); }
+// Index of element e in a warp's list of sorted positions: one padding entry
+// after every 16, so that lane l's entries l*K .. l*K + K - 1 and the
+// consecutive entries of the way back fall in few banks.
+__device__ __forceinline__ int spad(int e) { return e + (e >> 4); }
 
-// One warp sorts n <= 32*K pairs [b, b + n) of (kin, vin) into (kout, vout):
-// the pairs are staged in the warp's slice of shared memory (keys and sort
-// indices padded, see spad), the network sorts (sub-key << 32 | input index)
-// -- unique values, so equal sub-keys keep their input order -- and the pairs
-// are written out in that order.
+// Puts a list of positions right where the cut bits would have decided:
+// odd-even exchanges of neighbours by (sub-key, position) until none is out of
+// order. The list is sorted but for runs of equal sort words, so a round or
+// two will do on all but contrived inputs. any(x): the vote of `threads`
+// threads, of which this is number t, and a barrier between them.
+template <typename Order, typename Vote>
+__device__ __forceinline__ void fix_order(uint16_t* list, int n, int t, int threads, Order sub_of, Vote any) {
+    for (;;) {
+        bool swapped = false;
+        for (int odd = 0; odd < 2; ++odd) {
+            for (int q = 2 * t + odd; q + 1 < n; q += 2 * threads) {
+                const uint16_t a = list[spad(q)], b = list[spad(q + 1)];
+                const uint32_t sa = sub_of(a), sb = sub_of(b);
+                if (sa > sb || (sa == sb && a > b)) {
+                    list[spad(q)] = b;
+                    list[spad(q + 1)] = a;
+                    swapped = true;
+                }
+            }
+            any(false);
+        }
+        if (!any(swapped)) return;
+    }
+}
+
+// One warp sorts n <= 32*K pairs [b, b + n) of (kin, vin) into (kout, vout).
 template <int K>
-__device__ void warp_sort(const uint64_t* kin, const uint32_t* vin, uint64_t* kout, uint32_t* vout, uint32_t b,
-                          int n, int begin_bit, uint64_t* buf_k, uint32_t* buf_v, uint32_t* buf_i) {
+__device__ __forceinline__ void warp_sort(const uint64_t* kin, const uint32_t* vin, uint64_t* kout, uint32_t* vout,
+                                          uint32_t b, int n, int begin_bit, uint16_t* list) {
     const int lane = threadIdx.x & 31;
     const uint32_t sub_mask = (1u << (kSplitBit - begin_bit)) - 1u;
+    constexpr int idx_bits = K == 1 ? 5 : (K == 2 ? 6 : (K == 4 ? 7 : (K == 8 ? 8 : 9)));
+    uint32_t v[K];
+    uint32_t least = ~0u, most = 0u;
 #pragma unroll
     for (int k = 0; k < K; ++k) {
         const int idx = k * kWarp + lane;
+        v[k] = idx < n ? sub_key(__ldg(kin + b + idx), begin_bit, sub_mask) : 0u;
         if (idx < n) {
-            buf_k[spad(idx)] = __ldg(kin + b + idx);
-            buf_v[idx] = __ldg(vin + b + idx);
+            least = min(least, v[k]);
+            most = max(most, v[k]);
         }
     }
-    __syncwarp();
-    uint64_t v[K];
+    least = __reduce_min_sync(kFull, least);
+    most = __reduce_max_sync(kFull, most);
+    const int cut = cut_bits(most - least, idx_bits);
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-        const int e = lane * K + k;
-        v[k] = e < n ? ((uint64_t)sub_key(buf_k[spad(e)], begin_bit, sub_mask) << 32) | (uint32_t)e : ~0ull;
+        const int idx = k * kWarp + lane;
+        // past the end: the largest words (the position makes them distinct)
+        v[k] = idx < n ? sort_word(v[k], least, cut, idx_bits, (uint32_t)idx) : (~0u << idx_bits) | (uint32_t)idx;
     }
     warp_bitonic<K>(v);
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const int e = lane * K + k;
-        if (e < n) buf_i[spad(e)] = (uint32_t)v[k];
-    }
+    for (int k = 0; k < K; ++k) list[spad(lane * K + k)] = (uint16_t)(v[k] & ((1u << idx_bits) - 1u));
     __syncwarp();
+    if (cut > 0)
+        fix_order(
+            list, n, lane, kWarp, [&](uint16_t i) { return sub_key(__ldg(kin + b + i), begin_bit, sub_mask); },
+            [](bool x) {
+                __syncwarp();  // the exchanges before the next reads
+                return __any_sync(kFull, x) != 0;
+            });
 #pragma unroll
     for (int k = 0; k < K; ++k) {
         const int p = k * kWarp + lane;
         if (p < n) {
-            const uint32_t src = buf_i[spad(p)];
-            kout[b + p] = buf_k[spad((int)src)];
-            vout[b + p] = buf_v[src];
+            const uint32_t src = list[spad(p)];
+            kout[b + p] = __ldg(kin + b + src);
+            vout[b + p] = __ldg(vin + b + src);
         }
     }
 }
 
 // Block-wide AND / OR of one value per thread.
+template <int THREADS>
 __device__ __forceinline__ uint32_t block_varying(uint32_t a, uint32_t o, uint32_t* red) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     a = warp_and(a);
@@ -201,119 +276,158 @@ __device__ __forceinline__ uint32_t block_varying(uint32_t a, uint32_t o, uint32
     __syncthreads();
     uint32_t ra = ~0u, ro = 0u;
 #pragma unroll
-    for (int w = 0; w < kSegWarps; ++w) {
+    for (int w = 0; w < THREADS / kWarp; ++w) {
         ra &= red[2 * w];
         ro |= red[2 * w + 1];
     }
     return ra ^ ro;
 }
 
-// After warp_rank by every warp: turns cnt[w][d] (warp counts) into the
-// warp's first position for digit d within this chunk (digit start + the
-// counts of earlier warps) and returns the chunk's count of digit
-// d = threadIdx.x in *total. Threads are digits (256 threads, 256 digits).
-__device__ __forceinline__ uint32_t chunk_offsets(uint32_t (*cnt)[kLocalRadix], uint32_t* red, uint32_t* total) {
-    const int d = threadIdx.x;
-    uint32_t run = 0;
-#pragma unroll
-    for (int w = 0; w < kSegWarps; ++w) {
-        const uint32_t c = cnt[w][d];
-        cnt[w][d] = run;
-        run += c;
-    }
-    uint32_t all;
-    const uint32_t start = block_exclusive_scan<kSegThreads>(run, red, &all);
-#pragma unroll
-    for (int w = 0; w < kSegWarps; ++w) cnt[w][d] += start;
-    *total = run;
-    return start;
-}
+// The block sorts n <= 8 THREADS pairs by their sort words (log2 of that many
+// bits of position, 21 or 19 of sub-key) with three stable 7-bit LSD passes
+// over the sub-key's part; with kn = ceil(n / THREADS), element w*32*kn + k*32
+// + lane lives in lane `lane` of warp w, item k. s_word: a word per key
+// (reused for the list of positions); s_cnt: THREADS / 32 rows of 128
+// counters.
+constexpr int kCtaDigit = 7;
+constexpr int kCtaRadix = 1 << kCtaDigit;
 
-// The block sorts 256 < n <= 2048 pairs in shared memory with 8-bit LSD
-// passes; with kn = ceil(n / 256), element w*32*kn + k*32 + lane lives in
-// lane `lane` of warp w, item k.
-__device__ void block_sort_smem(const uint64_t* kin, const uint32_t* vin, uint64_t* kout, uint32_t* vout,
-                                uint32_t b, int n, int begin_bit, uint64_t* s_key, uint32_t* s_val,
-                                uint32_t (*cnt)[kLocalRadix], uint32_t* red) {
+template <int THREADS>
+__device__ __forceinline__ void block_sort_smem(const uint64_t* kin, const uint32_t* vin, uint64_t* kout,
+                                                uint32_t* vout, uint32_t b, int n, int begin_bit, uint32_t* s_word,
+                                                uint16_t* s_cnt, uint32_t* red) {
+    constexpr int kCap = block_cap<THREADS>();
+    constexpr int kIdxBits = THREADS == 1024 ? 13 : 11;
+    static_assert((1 << kIdxBits) == kCap && kIdxBits + 3 * kCtaDigit >= 32, "position bits and passes");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // every warp takes kn consecutive runs of 32 (input order = warp, item, lane)
-    const int kn = (n + kSegThreads - 1) / kSegThreads;
+    const int kn = (n + THREADS - 1) / THREADS;
     const int wbase = warp * kWarp * kn;
     const uint32_t sub_mask = (1u << (kSplitBit - begin_bit)) - 1u;
-    uint64_t key[kSegItems];
-    uint32_t val[kSegItems];
-    uint32_t all_and = ~0u, all_or = 0u;
+    uint32_t word[kSegItems];
+    uint32_t least = ~0u, most = 0u;
 #pragma unroll
     for (int k = 0; k < kSegItems; ++k) {
-        key[k] = 0;
-        val[k] = 0;
+        word[k] = 0;
         const int idx = wbase + k * kWarp + lane;
         if (k < kn && idx < n) {
-            key[k] = __ldg(kin + b + idx);
-            val[k] = __ldg(vin + b + idx);
-            const uint32_t s = sub_key(key[k], begin_bit, sub_mask);
-            all_and &= s;
-            all_or |= s;
+            word[k] = sub_key(__ldg(kin + b + idx), begin_bit, sub_mask);
+            least = min(least, word[k]);
+            most = max(most, word[k]);
         }
     }
-    const uint32_t varying = block_varying(all_and, all_or, red);
-    for (int shift = begin_bit; shift < kSplitBit; shift += kLocalBits) {
-        const int bits = kSplitBit - shift < kLocalBits ? kSplitBit - shift : kLocalBits;
-        const uint32_t mask = (1u << bits) - 1u;
-        if (((varying >> (shift - begin_bit)) & mask) == 0u) continue;
-        for (int i = threadIdx.x; i < kSegWarps * kLocalRadix; i += kSegThreads) (&cnt[0][0])[i] = 0u;
-        __syncthreads();
+    least = __reduce_min_sync(kFull, least);
+    most = __reduce_max_sync(kFull, most);
+    if (lane == 0) {
+        red[2 * warp] = least;
+        red[2 * warp + 1] = most;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < THREADS / kWarp; ++w) {
+        least = min(least, red[2 * w]);
+        most = max(most, red[2 * w + 1]);
+    }
+    const uint32_t range = most - least;
+    const int cut = cut_bits(range, kIdxBits);
+#pragma unroll
+    for (int k = 0; k < kSegItems; ++k)
+        word[k] = sort_word(word[k], least, cut, kIdxBits, (uint32_t)(wbase + k * kWarp + lane));
+    const int top = 32 - __clz((range >> cut) | 1u);  // bits of sub-key in the words
+    const uint32_t lt = lanemask_lt();
+    uint16_t* cnt = s_cnt + warp * kCtaRadix;
+    for (int shift = kIdxBits; shift < kIdxBits + top; shift += kCtaDigit) {
+        __syncthreads();  // the last pass's reads of the words and counters
+        reinterpret_cast<uint2*>(cnt)[lane] = make_uint2(0u, 0u);
+        __syncwarp();
         uint32_t rnk[kSegItems];
-        warp_rank(key, kn, wbase, n, shift, mask, cnt[warp], rnk);
+#pragma unroll
+        for (int k = 0; k < kSegItems; ++k) {
+            if (k >= kn) break;
+            const bool ok = wbase + k * kWarp + lane < n;
+            const uint32_t dg = (word[k] >> shift) & (kCtaRadix - 1);
+            const uint32_t peers = warp_match_digit<kCtaDigit>(dg, ok);
+            const uint32_t prior = cnt[dg];
+            rnk[k] = prior + __popc(peers & lt);
+            __syncwarp();
+            if (ok && (peers & lt) == 0u) cnt[dg] = (uint16_t)(prior + __popc(peers));
+            __syncwarp();
+        }
         __syncthreads();
-        uint32_t total;
-        chunk_offsets(cnt, red, &total);
+        // counts -> first positions, by digit and then warp: thread t owns
+        // digit t of the first 128 threads
+        uint32_t run = 0;
+        if (threadIdx.x < kCtaRadix)
+            for (int w = 0; w < THREADS / kWarp; ++w) run += s_cnt[w * kCtaRadix + threadIdx.x];
+        uint32_t all;
+        uint32_t first = block_exclusive_scan<THREADS>(run, red, &all);
+        if (threadIdx.x < kCtaRadix) {
+            for (int w = 0; w < THREADS / kWarp; ++w) {
+                const uint32_t c = s_cnt[w * kCtaRadix + threadIdx.x];
+                s_cnt[w * kCtaRadix + threadIdx.x] = (uint16_t)first;
+                first += c;
+            }
+        }
         __syncthreads();
 #pragma unroll
         for (int k = 0; k < kSegItems; ++k) {
             if (k >= kn) break;
-            if (wbase + k * kWarp + lane < n) {
-                const uint32_t pos = cnt[warp][(uint32_t)(key[k] >> shift) & mask] + rnk[k];
-                s_key[pos] = key[k];
-                s_val[pos] = val[k];
-            }
+            if (wbase + k * kWarp + lane < n) s_word[cnt[(word[k] >> shift) & (kCtaRadix - 1)] + rnk[k]] = word[k];
         }
         __syncthreads();
 #pragma unroll
         for (int k = 0; k < kSegItems; ++k) {
             if (k >= kn) break;
             const int idx = wbase + k * kWarp + lane;
-            if (idx < n) {
-                key[k] = s_key[idx];
-                val[k] = s_val[idx];
-            }
+            if (idx < n) word[k] = s_word[idx];
+        }
+    }
+    if (cut > 0) {
+        uint16_t* list = reinterpret_cast<uint16_t*>(s_word);
+        __syncthreads();  // the words are in registers
+#pragma unroll
+        for (int k = 0; k < kSegItems; ++k) {
+            const int idx = wbase + k * kWarp + lane;
+            if (k < kn && idx < n) list[spad(idx)] = (uint16_t)(word[k] & (kCap - 1));
         }
         __syncthreads();
+        fix_order(
+            list, n, threadIdx.x, THREADS,
+            [&](uint16_t i) { return sub_key(__ldg(kin + b + i), begin_bit, sub_mask); },
+            [](bool x) { return __syncthreads_or(x) != 0; });
+#pragma unroll
+        for (int k = 0; k < kSegItems; ++k) {
+            const int idx = wbase + k * kWarp + lane;
+            if (k < kn && idx < n) word[k] = list[spad(idx)];
+        }
     }
 #pragma unroll
     for (int k = 0; k < kSegItems; ++k) {
         if (k >= kn) break;
         const int idx = wbase + k * kWarp + lane;
         if (idx < n) {
-            kout[b + idx] = key[k];
-            vout[b + idx] = val[k];
+            const uint32_t src = word[k] & (kCap - 1);
+            kout[b + idx] = __ldg(kin + b + src);
+            vout[b + idx] = __ldg(vin + b + src);
         }
     }
 }
 
-// The block sorts n > 2048 pairs through global memory, 2048 at a time:
+// The block sorts any number of pairs through global memory, 8 THREADS at a
+// time:
 // per pass a histogram sweep, then chunks in order, each scattered to its
 // digit's running offset. Ping-pongs between the two buffers' [b, b + n);
 // the result ends in (kout, vout). Loads here are plain (not read-only
 // cache): the block reads what it wrote, ordered by __syncthreads.
+template <int THREADS>
 __device__ void block_sort_global(uint64_t* kin, uint32_t* vin, uint64_t* kout, uint32_t* vout, uint32_t b,
                                   uint32_t n, int begin_bit, uint32_t (*cnt)[kLocalRadix], uint32_t* off,
                                   uint32_t* red) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int wbase = warp * kWarpCap;
+    const int wbase = warp * kWarp * kSegItems;
     const uint32_t sub_mask = (1u << (kSplitBit - begin_bit)) - 1u;
     uint32_t all_and = ~0u, all_or = 0u;
-    for (uint32_t c0 = 0; c0 < n; c0 += kCtaCap) {
+    for (uint32_t c0 = 0; c0 < n; c0 += block_cap<THREADS>()) {
 #pragma unroll
         for (int k = 0; k < kSegItems; ++k) {
             const uint32_t idx = c0 + wbase + k * kWarp + lane;
@@ -324,7 +438,7 @@ __device__ void block_sort_global(uint64_t* kin, uint32_t* vin, uint64_t* kout, 
             }
         }
     }
-    const uint32_t varying = block_varying(all_and, all_or, red);
+    const uint32_t varying = block_varying<THREADS>(all_and, all_or, red);
     uint64_t* sk = kin + b;
     uint32_t* sv = vin + b;
     uint64_t* dk = kout + b;
@@ -335,10 +449,10 @@ __device__ void block_sort_global(uint64_t* kin, uint32_t* vin, uint64_t* kout, 
         const uint32_t mask = (1u << bits) - 1u;
         if (((varying >> (shift - begin_bit)) & mask) == 0u) continue;
         // digit totals of the segment -> running offsets
-        for (int i = threadIdx.x; i < kSegWarps * kLocalRadix; i += kSegThreads) (&cnt[0][0])[i] = 0u;
+        for (int i = threadIdx.x; i < (THREADS / kWarp) * kLocalRadix; i += THREADS) (&cnt[0][0])[i] = 0u;
         __syncthreads();
-        for (uint32_t c0 = 0; c0 < n; c0 += kCtaCap) {
-            const int rem = (int)(n - c0 < (uint32_t)kCtaCap ? n - c0 : (uint32_t)kCtaCap);
+        for (uint32_t c0 = 0; c0 < n; c0 += block_cap<THREADS>()) {
+            const int rem = (int)(n - c0 < (uint32_t)block_cap<THREADS>() ? n - c0 : (uint32_t)block_cap<THREADS>());
             uint64_t key[kSegItems];
             const int kn = rem > wbase ? ((rem - wbase + kWarp - 1) / kWarp < kSegItems
                                               ? (rem - wbase + kWarp - 1) / kWarp
@@ -354,21 +468,24 @@ __device__ void block_sort_global(uint64_t* kin, uint32_t* vin, uint64_t* kout, 
         }
         __syncthreads();
         {
-            const int d = threadIdx.x;
+            const int d = threadIdx.x;  // the first 256 threads are the digits
             uint32_t t = 0;
+            if (d < kLocalRadix) {
 #pragma unroll
-            for (int w = 0; w < kSegWarps; ++w) t += cnt[w][d];
+                for (int w = 0; w < (THREADS / kWarp); ++w) t += cnt[w][d];
+            }
             uint32_t all;
-            off[d] = block_exclusive_scan<kSegThreads>(t, red, &all);
+            t = block_exclusive_scan<THREADS>(t, red, &all);
+            if (d < kLocalRadix) off[d] = t;
         }
         __syncthreads();
-        for (uint32_t c0 = 0; c0 < n; c0 += kCtaCap) {
-            const int rem = (int)(n - c0 < (uint32_t)kCtaCap ? n - c0 : (uint32_t)kCtaCap);
+        for (uint32_t c0 = 0; c0 < n; c0 += block_cap<THREADS>()) {
+            const int rem = (int)(n - c0 < (uint32_t)block_cap<THREADS>() ? n - c0 : (uint32_t)block_cap<THREADS>());
             const int kn = rem > wbase ? ((rem - wbase + kWarp - 1) / kWarp < kSegItems
                                               ? (rem - wbase + kWarp - 1) / kWarp
                                               : kSegItems)
                                        : 0;
-            for (int i = threadIdx.x; i < kSegWarps * kLocalRadix; i += kSegThreads) (&cnt[0][0])[i] = 0u;
+            for (int i = threadIdx.x; i < (THREADS / kWarp) * kLocalRadix; i += THREADS) (&cnt[0][0])[i] = 0u;
             __syncthreads();
             uint64_t key[kSegItems];
             uint32_t val[kSegItems];
@@ -386,11 +503,13 @@ __device__ void block_sort_global(uint64_t* kin, uint32_t* vin, uint64_t* kout, 
             // running offsets place the chunk)
             const int d = threadIdx.x;
             uint32_t run = 0;
+            if (d < kLocalRadix) {
 #pragma unroll
-            for (int w = 0; w < kSegWarps; ++w) {
-                const uint32_t c = cnt[w][d];
-                cnt[w][d] = run;
-                run += c;
+                for (int w = 0; w < (THREADS / kWarp); ++w) {
+                    const uint32_t c = cnt[w][d];
+                    cnt[w][d] = run;
+                    run += c;
+                }
             }
             __syncthreads();
 #pragma unroll
@@ -404,7 +523,7 @@ __device__ void block_sort_global(uint64_t* kin, uint32_t* vin, uint64_t* kout, 
                 }
             }
             __syncthreads();
-            off[d] += run;
+            if (d < kLocalRadix) off[d] += run;
         }
         __syncthreads();
         uint64_t* tk = sk; sk = dk; dk = tk;
@@ -412,70 +531,133 @@ __device__ void block_sort_global(uint64_t* kin, uint32_t* vin, uint64_t* kout, 
         in_out = !in_out;
     }
     if (!in_out) {  // an even number of passes ran: copy into (kout, vout)
-        for (uint32_t i = threadIdx.x; i < n; i += kSegThreads) {
+        for (uint32_t i = threadIdx.x; i < n; i += THREADS) {
             kout[b + i] = kin[b + i];
             vout[b + i] = vin[b + i];
         }
     }
 }
 
-// Blocks [0, nseg) sort one segment each when it holds more than 256 keys
-// (and return at once otherwise); blocks nseg + g, g >= 0, give warp w the
-// segment 8g + w when it holds 1 to 256 keys. The large segments come first
-// in launch order so their longer sorts start early.
+// Shared memory of a block that sorts one segment: the words and counters of
+// the passes over words, or the counters of the passes over global memory.
+template <int THREADS>
+struct SegSmem {
+    static constexpr int kWordBytes = block_cap<THREADS>() * 4;
+    static constexpr int kBytes = kWordBytes + (THREADS / kWarp) * kCtaRadix * 2;
+    static constexpr int kGlobalBytes = (THREADS / kWarp) * kLocalRadix * 4;
+    static constexpr int kRaw = kBytes > kGlobalBytes ? kBytes : kGlobalBytes;
+};
+
+// The block sorts one segment [b, b + n).
+template <int THREADS>
+__device__ __forceinline__ void block_sort(uint64_t* kin, uint32_t* vin, uint64_t* kout, uint32_t* vout, uint32_t b,
+                                           uint32_t n, int begin_bit, unsigned char* raw, uint32_t* off,
+                                           uint32_t* red) {
+    if (n <= (uint32_t)block_cap<THREADS>())
+        block_sort_smem<THREADS>(kin, vin, kout, vout, b, (int)n, begin_bit, reinterpret_cast<uint32_t*>(raw),
+                                 reinterpret_cast<uint16_t*>(raw + SegSmem<THREADS>::kWordBytes), red);
+    else
+        block_sort_global<THREADS>(kin, vin, kout, vout, b, n, begin_bit,
+                                   reinterpret_cast<uint32_t (*)[kLocalRadix]>(raw), off, red);
+}
+
+// Segment s as [b, e), clamped into [0, n].
+__device__ __forceinline__ void seg_bounds(const uint32_t* __restrict__ start, uint32_t s, uint32_t n, uint32_t& b,
+                                           uint32_t& e) {
+    e = min(__ldg(start + s + 1), n);
+    b = min(__ldg(start + s), e);
+}
+
+// The segments i, i + nblocks, i + 2 nblocks, ... (32 at most) of block i, of
+// more than `above` and at most `most` keys, one after another.
+template <int THREADS>
+__device__ __forceinline__ void sort_own_segments(uint64_t* kin, uint32_t* vin, uint64_t* kout, uint32_t* vout,
+                                                  const uint32_t* __restrict__ start, uint32_t n_all, uint32_t nseg,
+                                                  uint32_t nblocks, uint32_t above, uint32_t most, int begin_bit,
+                                                  unsigned char* raw, uint32_t* off, uint32_t* red) {
+    uint32_t b0 = 0, e0 = 0;  // bounds of the lane's segment (every warp alike)
+    const uint32_t s0 = blockIdx.x + (threadIdx.x & 31u) * nblocks;
+    if (s0 < nseg) seg_bounds(start, s0, n_all, b0, e0);
+    uint32_t todo = __ballot_sync(kFull, e0 - b0 > above && e0 - b0 <= most);
+    while (todo) {
+        const int src = __ffs(todo) - 1;
+        todo &= todo - 1;
+        const uint32_t b = __shfl_sync(kFull, b0, src), n = __shfl_sync(kFull, e0, src) - b;
+        block_sort<THREADS>(kin, vin, kout, vout, b, n, begin_bit, raw, off, red);
+        __syncthreads();  // shared memory is free for the next segment
+    }
+}
+
+// Blocks [0, nbig) sort the segments of more than 512 and at most `most` keys:
+// block i those among i, i + nbig, i + 2 nbig, ..., found by one look at their
+// bounds. Blocks nbig + g, g >= 0, give warp w the segment 8g + w when it
+// holds 1 to 512 keys. The large segments come first in launch order so their
+// longer sorts start early.
+// nbig (big_blocks): every segment its own block up to 2,048 of them, then
+// 2,048 blocks and more segments each: a block that finds nothing to do still
+// costs its launch (8,192 of them 13 us of the 1080p / 1M frame's 34 us local
+// sort), while a block with many large segments sorts them one after another
+// (with 256 blocks for 8,192 segments of 514 keys on average, 311 us instead
+// of 209 for the whole sort).
+uint32_t big_blocks(uint32_t nseg) {
+    const uint32_t per = nseg <= 2048u ? 1u : (nseg / 2048u < 32u ? nseg / 2048u : 32u);
+    return (nseg + per - 1) / per;
+}
+
 __global__ void __launch_bounds__(kSegThreads, 4)
 k_seg_sort(uint64_t* kin, uint32_t* vin, uint64_t* kout, uint32_t* vout, const uint32_t* __restrict__ start,
-           const uint32_t* __restrict__ num_keys, uint32_t cap, uint32_t nseg, int begin_bit) {
-    // One buffer, carved two ways: the block paths' key / value / digit
-    // count arrays, or each warp's padded staging slice (keys, values, sort
-    // indices) for the warp path.
-    constexpr int kPadCap = kWarpCap + kWarpCap / 8;
-    constexpr int kWarpBytes = kPadCap * 8 + kWarpCap * 4 + kPadCap * 4;
-    constexpr int kBlockBytes = kCtaCap * 8 + kCtaCap * 4 + kSegWarps * kLocalRadix * 4;
-    constexpr int kRawBytes = kSegWarps * kWarpBytes > kBlockBytes ? kSegWarps * kWarpBytes : kBlockBytes;
-    __shared__ __align__(16) unsigned char s_raw[kRawBytes];
-    uint64_t* s_key = reinterpret_cast<uint64_t*>(s_raw);
-    uint32_t* s_val = reinterpret_cast<uint32_t*>(s_raw + kCtaCap * 8);
-    auto s_cnt = reinterpret_cast<uint32_t (*)[kLocalRadix]>(s_raw + kCtaCap * 12);
+           const uint32_t* __restrict__ num_keys, uint32_t cap, uint32_t nseg, uint32_t nbig, uint32_t most,
+           int begin_bit) {
+    // One buffer, carved two ways: a block's segment, or each warp's list.
+    constexpr int kListLen = kWarpCap + kWarpCap / 16;
+    constexpr int kListBytes = kSegWarps * kListLen * 2;
+    constexpr int kRaw = SegSmem<kSegThreads>::kRaw > kListBytes ? SegSmem<kSegThreads>::kRaw : kListBytes;
+    __shared__ __align__(16) unsigned char s_raw[kRaw];
     __shared__ uint32_t s_off[kLocalRadix];
     __shared__ uint32_t s_red[2 * kSegWarps + 2];
     const int warp = threadIdx.x >> 5;
     pdl_wait();
     const uint32_t n_all = min(*num_keys, cap);
-    // segment s as [b, e), clamped into [0, n]
-    auto bounds = [&](uint32_t s, uint32_t& b, uint32_t& e) {
-        e = min(__ldg(start + s + 1), n_all);
-        b = min(__ldg(start + s), e);
-    };
-    if (blockIdx.x < nseg) {
-        uint32_t b, e;
-        bounds(blockIdx.x, b, e);
-        const uint32_t n = e - b;
-        if (n <= (uint32_t)kWarpCap) return;  // uniform over the block
-        if (n <= (uint32_t)kCtaCap)
-            block_sort_smem(kin, vin, kout, vout, b, (int)n, begin_bit, s_key, s_val, s_cnt, s_red);
-        else
-            block_sort_global(kin, vin, kout, vout, b, n, begin_bit, s_cnt, s_off, s_red);
+    if (blockIdx.x < nbig) {
+        sort_own_segments<kSegThreads>(kin, vin, kout, vout, start, n_all, nseg, nbig, (uint32_t)kWarpCap, most,
+                                       begin_bit, s_raw, s_off, s_red);
         return;
     }
-    const uint32_t s = (blockIdx.x - nseg) * kSegWarps + warp;
+    const uint32_t s = (blockIdx.x - nbig) * kSegWarps + warp;
     if (s >= nseg) return;
     uint32_t b, e;
-    bounds(s, b, e);
+    seg_bounds(start, s, n_all, b, e);
     const int n = (int)(e - b);
     if (n == 0 || n > kWarpCap) return;
-    unsigned char* wraw = s_raw + warp * kWarpBytes;
-    uint64_t* bk = reinterpret_cast<uint64_t*>(wraw);
-    uint32_t* bv = reinterpret_cast<uint32_t*>(wraw + kPadCap * 8);
-    uint32_t* bi = reinterpret_cast<uint32_t*>(wraw + kPadCap * 8 + kWarpCap * 4);
+    uint16_t* list = reinterpret_cast<uint16_t*>(s_raw) + warp * kListLen;
     if (n <= 32)
-        warp_sort<1>(kin, vin, kout, vout, b, n, begin_bit, bk, bv, bi);
+        warp_sort<1>(kin, vin, kout, vout, b, n, begin_bit, list);
     else if (n <= 64)
-        warp_sort<2>(kin, vin, kout, vout, b, n, begin_bit, bk, bv, bi);
+        warp_sort<2>(kin, vin, kout, vout, b, n, begin_bit, list);
     else if (n <= 128)
-        warp_sort<4>(kin, vin, kout, vout, b, n, begin_bit, bk, bv, bi);
+        warp_sort<4>(kin, vin, kout, vout, b, n, begin_bit, list);
+    else if (n <= 256)
+        warp_sort<8>(kin, vin, kout, vout, b, n, begin_bit, list);
     else
-        warp_sort<8>(kin, vin, kout, vout, b, n, begin_bit, bk, bv, bi);
+        warp_sort<16>(kin, vin, kout, vout, b, n, begin_bit, list);
+}
+
+// The segments of more than 2,048 keys, 1,024 threads each (up to 8,192 keys
+// in shared memory). Launched where the capacity allows such segments to be
+// common, kHugeMean keys or more a segment: the launch costs 3 us, and the
+// 256-thread blocks of k_seg_sort, which take them otherwise, 8 passes over
+// global memory.
+constexpr uint32_t kHugeMean = 600;
+__global__ void __launch_bounds__(kHugeThreads, 1)
+k_seg_sort_huge(uint64_t* kin, uint32_t* vin, uint64_t* kout, uint32_t* vout, const uint32_t* __restrict__ start,
+                const uint32_t* __restrict__ num_keys, uint32_t cap, uint32_t nseg, int begin_bit) {
+    __shared__ __align__(16) unsigned char s_raw[SegSmem<kHugeThreads>::kRaw];
+    __shared__ uint32_t s_off[kLocalRadix];
+    __shared__ uint32_t s_red[2 * kHugeThreads / kWarp + 2];
+    pdl_wait();
+    const uint32_t n_all = min(*num_keys, cap);
+    sort_own_segments<kHugeThreads>(kin, vin, kout, vout, start, n_all, nseg, gridDim.x,
+                                    (uint32_t)block_cap<kSegThreads>(), ~0u, begin_bit, s_raw, s_off, s_red);
 }
 
 // Scratch: [partition histograms, sized for 11-bit digits | segment starts].
@@ -533,16 +715,22 @@ cudaError_t launch_sort_segmented(const uint32_t* num_keys, int64_t key_capacity
     uint32_t* ov = part_alt ? vals : vals_alt;
     uint32_t* start = static_cast<uint32_t*>(scratch) + seg_start_offset_words(key_capacity);
     const uint32_t nseg = 1u << seg_bits;
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t spans = (key_capacity + 1 + 1023) / 1024;
-    e = launch_pdl(k_seg_bounds, dim3((unsigned)(spans < sms * 8 ? spans : sms * 8)), dim3(256), 0, stream,
-                   (const uint64_t*)pk, num_keys, (uint32_t)key_capacity, nseg - 1u, nseg, start,
-                   reinterpret_cast<uint2*>(ranges), ntiles);
+    const uint32_t bound_blocks = (uint32_t)(((uint64_t)(nseg + 1u) * kBoundLanes + 255u) / 256u);
+    e = launch_pdl(k_seg_bounds, dim3(bound_blocks), dim3(256), 0, stream, (const uint64_t*)pk, num_keys,
+                   (uint32_t)key_capacity, nseg - 1u, nseg, start, reinterpret_cast<uint2*>(ranges), ntiles);
     if (e != cudaSuccess) return e;
-    e = launch_pdl(k_seg_sort, dim3(nseg + (nseg + kSegWarps - 1) / kSegWarps), dim3(kSegThreads), 0, stream, pk, pv,
-                   ok, ov, (const uint32_t*)start, num_keys, (uint32_t)key_capacity, nseg, begin_bit);
+    const bool huge = (uint64_t)key_capacity >= (uint64_t)kHugeMean * nseg &&
+                      key_capacity > (int64_t)block_cap<kSegThreads>();
+    if (huge) {
+        e = launch_pdl(k_seg_sort_huge, dim3(nseg <= 512u ? nseg : (nseg / 32u < 512u ? 512u : (nseg + 31u) / 32u)),
+                       dim3(kHugeThreads), 0, stream, pk, pv, ok, ov, (const uint32_t*)start, num_keys,
+                       (uint32_t)key_capacity, nseg, begin_bit);
+        if (e != cudaSuccess) return e;
+    }
+    const uint32_t nbig = big_blocks(nseg);
+    e = launch_pdl(k_seg_sort, dim3(nbig + (nseg + kSegWarps - 1) / kSegWarps), dim3(kSegThreads), 0, stream, pk, pv,
+                   ok, ov, (const uint32_t*)start, num_keys, (uint32_t)key_capacity, nseg, nbig,
+                   huge ? (uint32_t)block_cap<kSegThreads>() : ~0u, begin_bit);
     if (e != cudaSuccess) return e;
     *in_alt = !part_alt;
     return cudaGetLastError();

@@ -325,3 +325,72 @@ def test_sort_tiles_rejects_what_the_segmented_sort_cannot_take():
     with pytest.raises(capi.WsError) as e:
         capi.ws_sort_tiles(num, 16, 31, k, v, k, v, cfg, ws, ranges, 1)
     assert e.value.status == capi.WS_ERR_UNSUPPORTED
+
+
+def _segments(lengths, kind, rng):
+    """Keys of segments of the given lengths, shuffled: depths spread over one
+    octave (their sort words hold them whole), over all positive floats (the
+    words drop bits), in runs that differ in the dropped bits only, or equal."""
+    keys = []
+    for s, n in enumerate(lengths):
+        if kind == "octave":
+            d = rng.uniform(1.0, 2.0, n).astype(np.float32).view(np.uint32)
+        elif kind == "wide":
+            d = rng.integers(0, 1 << 31, n, dtype=np.uint32)
+        elif kind == "runs":  # 30 clusters far apart, each within 64 values
+            d = (rng.integers(0, 30, n).astype(np.uint32) << np.uint32(26)) + rng.integers(0, 64, n, dtype=np.uint32)
+        else:
+            d = np.full(n, 12345, np.uint32)
+        keys.append((np.uint64(s) << np.uint64(31)) | d.astype(np.uint64))
+    keys = np.concatenate(keys)
+    return keys[rng.permutation(keys.size)]
+
+
+@pytest.mark.parametrize("kind", ["octave", "wide", "runs", "equal"])
+@pytest.mark.parametrize("lengths", [
+    [1, 2, 31, 32, 33, 64, 65, 128, 129, 256, 257],        # a warp, every width of its network
+    [511, 512, 513, 0, 700, 2047, 2048, 2049],             # warp / 256 threads / past them
+    [4095, 8191, 8192, 8193, 3, 20000],                    # 1,024 threads / global memory
+])
+@pytest.mark.parametrize("room", [1, 40])
+def test_segment_lengths_at_the_edges_of_each_path(lengths, kind, room):
+    """Segmented sort against the stable sort. room = 40 gives the capacity of
+    600 keys a segment from which the larger segments get blocks of their own."""
+    from paper_2602_03207_gb300 import capi
+    rng = np.random.default_rng(len(lengths) + len(kind))
+    keys = _segments(lengths, kind, rng)
+    vals = rng.permutation(keys.size).astype(np.uint32)
+    end_bit = 31 + max(1, int(np.ceil(np.log2(len(lengths)))))
+    cap = max(keys.size, room * 600 * (1 << (end_bit - 31)) // 40)
+    for begin_bit in (0, 5):
+        k, v = gpu_sort(keys, vals, digit_bits=8, begin_bit=begin_bit, end_bit=end_bit, capacity=cap,
+                        flags=capi.WS_CFG_SORT_SEGMENTED)
+        perm = np.argsort(keys >> np.uint64(begin_bit), kind="stable")
+        np.testing.assert_array_equal(k, keys[perm])
+        np.testing.assert_array_equal(v, vals[perm])
+
+
+@pytest.mark.parametrize("tiles", [2, 7, 300, 4095])
+def test_tile_ranges_of_sparse_tiles(tiles):
+    """ws_sort_tiles' ranges against the bounds of the sorted tile ids: empty
+    tiles first, last and in runs."""
+    import torch
+    from paper_2602_03207_gb300 import capi
+    rng = np.random.default_rng(tiles)
+    used = rng.choice(tiles, size=max(1, tiles // 3), replace=False)
+    tile = rng.choice(used, size=5000).astype(np.uint64)
+    keys = (tile << np.uint64(31)) | rng.integers(1, 1 << 30, 5000, dtype=np.uint64)
+    for n in (0, 1, 4999):
+        kt = torch.zeros(8192, dtype=torch.int64, device="cuda")
+        kt[:5000] = torch.from_numpy(keys.view(np.int64))
+        vt = torch.arange(8192, dtype=torch.int32, device="cuda")
+        ka, va = torch.empty_like(kt), torch.empty_like(vt)
+        num = torch.tensor([n, 0, 0, 0], dtype=torch.int32, device="cuda")
+        ranges = torch.full((tiles, 2), -1, dtype=torch.int32, device="cuda")
+        cfg = capi.config(flags=capi.WS_CFG_SORT_SEGMENTED)
+        cam = capi.camera(S.small_forward()[1])
+        ws = torch.zeros(capi.ws_workspace_bytes(0, 8192, cam, cfg), dtype=torch.uint8, device="cuda")
+        capi.ws_sort_tiles(num, 8192, 31 + int(np.ceil(np.log2(tiles))), kt, vt, ka, va, cfg, ws, ranges, tiles)
+        t = np.sort(tile[:n]).astype(np.int64)
+        want = np.stack([np.searchsorted(t, np.arange(tiles), "left"), np.searchsorted(t, np.arange(tiles), "right")], 1)
+        np.testing.assert_array_equal(ranges.cpu().numpy(), want)
