@@ -15,6 +15,7 @@
 // the pixel centre inside |p_x|, |p_y| <= r; a = min(0.99, sigma e^{-p.p}), and
 // fragments with a < 1/255 are skipped as in the tile path, so both
 // paths produce the same image.
+#include "ws_blend.cuh"
 #include "ws_common.cuh"
 #include "ws_kernels.cuh"
 
@@ -23,7 +24,7 @@ namespace ws {
 namespace {
 
 constexpr int kQuadThreads = 256;
-constexpr int kQuadBatch = 256;
+constexpr int kQuadBatch = 128;
 
 // Per-splat quad: p = M d maps a pixel offset d from the centre to the local
 // coordinate; r is the E8 radius; the tile rectangle covers the quad's box.
@@ -121,107 +122,121 @@ k_quad_bin_items(int64_t n, const uint32_t* __restrict__ num_vis, const uint32_t
 }
 
 struct QuadStage {
-    float cx, cy;          // tile-relative centre
-    float m00, m01, m10, m11;
-    float r, l2s;          // E8 radius, log2(sigma)
-    float cr, cg, cb, pad;
+    float4 geo;   // minus the tile-relative centre; m00, m01
+    float4 geo2;  // m10, m11; r (E8), log2(sigma)
+    float4 col;   // colour; 0
 };
 
-// One block per tile, one thread per pixel (TS = 16: 256 pixels), the tile's
-// quads back to front (highest rank first) in batches staged in shared
-// memory; a warp skips a quad whose box misses its 8x4 pixel block.
-template <int TS>
-__global__ void __launch_bounds__(TS * TS >= 256 ? 256 : TS * TS)
+// One block per tile, the tile's quads back to front (highest rank first) in
+// batches staged in shared memory. Each 4x4 sub-block's lanes walk the quads
+// whose box reaches it (the visit lists and the geometry of the tile path's
+// blend, reversed), two pixels a lane with paired FP32 instructions. Against
+// a warp per 8x4 block, one pixel a lane, that visited every quad reaching
+// the block: 313 -> 263 us on the whole 1080p / 1M frame. Bound by
+// instruction issue, as the tile path's blend.
+template <int TS, int PX>
+__global__ void __launch_bounds__(TileGeom<TS, PX>::THREADS, fwd_min_blocks<TS>())
 k_blend_quads(const uint2* __restrict__ ranges, const uint32_t* __restrict__ ranks,
               const uint32_t* __restrict__ order, const float4* __restrict__ splats,
               const QuadRec* __restrict__ quad, const Frame f, float* __restrict__ image, float* __restrict__ t_final) {
-    constexpr int THREADS = TS * TS >= 256 ? 256 : TS * TS;
-    constexpr int WARPS = THREADS / 32;
-    constexpr int PPT = TS * TS / THREADS;
-    constexpr int BW = 8, BH = 4, BPR = TS / BW, BROWS = TS / BH;
-    __shared__ QuadStage s_q[kQuadBatch];
-    __shared__ uint32_t s_mask[kQuadBatch];
+    using G = TileGeom<TS, PX>;
+    constexpr int NP = PX / 2;
+    constexpr int ROW = list_row<kQuadBatch>();
+    __shared__ QuadStage s_q[kQuadBatch + 1];
+    __shared__ typename G::Mask s_mask[kQuadBatch];
+    __shared__ __align__(16) uint8_t s_list[G::NSB * ROW];
     pdl_wait();
     const int tile = blockIdx.x;
     const uint2 range = ranges[tile];
     const int tx = tile % f.TX, ty = tile / f.TX;
     const float ox = (float)(tx * TS), oy = (float)(ty * TS);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint8_t* rows = s_list + warp * G::SPW * ROW;
+    const uint8_t* row = rows + (lane / G::LPS) * ROW;
 
-    float px[PPT], py[PPT], T[PPT], C0[PPT], C1[PPT], C2[PPT];
+    if (threadIdx.x == 0) {  // the null quad: log2(sigma) = -inf, never drawn
+        s_q[kQuadBatch].geo = s_q[kQuadBatch].col = make_float4(0.f, 0.f, 0.f, 0.f);
+        s_q[kQuadBatch].geo2 = make_float4(0.f, 0.f, 0.f, -INFINITY);
+    }
+    int ix, iy0;
+    G::pixel(warp, lane, ix, iy0);
+    const float px = (float)ix + 0.5f;
+    F2 py[NP], T[NP], C0[NP], C1[NP], C2[NP];
 #pragma unroll
-    for (int k = 0; k < PPT; ++k) {
-        const int b = warp + k * WARPS;
-        px[k] = (float)((b % BPR) * BW + (lane & 7)) + 0.5f;
-        py[k] = (float)((b / BPR) * BH + (lane >> 3)) + 0.5f;
-        T[k] = 1.f;
-        C0[k] = f.bg[0];
-        C1[k] = f.bg[1];
-        C2[k] = f.bg[2];
+    for (int p = 0; p < NP; ++p) {
+        const float y = (float)(iy0 + 2 * p) + 0.5f;
+        py[p] = pack2(y, y + 1.f);
+        T[p] = dup2(1.f);
+        C0[p] = dup2(f.bg[0]);
+        C1[p] = dup2(f.bg[1]);
+        C2[p] = dup2(f.bg[2]);
     }
     for (int end = (int)(range.y - range.x); end > 0; end -= kQuadBatch) {
         const int lo = max(0, end - kQuadBatch);
         const int cnt = end - lo;
         __syncthreads();
-        for (int j = threadIdx.x; j < cnt; j += THREADS) {
+        for (int j = threadIdx.x; j < cnt; j += G::THREADS) {
             const uint32_t g = __ldg(order + __ldg(ranks + range.x + lo + j));
             const float4 m = __ldg(splats + kSplatVec4 * g);
             const float op = __ldg(splats + kSplatVec4 * g + 1).w;
             const float4 cl = __ldg(splats + kSplatVec4 * g + 2);
             const QuadRec q = quad[g];
-            QuadStage st;
-            st.cx = __fadd_rn(__fsub_rn(m.x, ox), m.z);
-            st.cy = __fadd_rn(__fsub_rn(m.y, oy), m.w);
-            st.m00 = q.m00;
-            st.m01 = q.m01;
-            st.m10 = q.m10;
-            st.m11 = q.m11;
-            st.r = q.r;
-            st.l2s = log2f(op);
-            st.cr = cl.x;
-            st.cg = cl.y;
-            st.cb = cl.z;
-            st.pad = 0.f;
-            s_q[j] = st;
-            s_mask[j] = box_block_mask<BW, BH, BPR, BROWS>(st.cx - q.hx, st.cx + q.hx, st.cy - q.hy, st.cy + q.hy);
+            const float cx = __fadd_rn(__fsub_rn(m.x, ox), m.z), cy = __fadd_rn(__fsub_rn(m.y, oy), m.w);
+            s_q[j].geo = make_float4(-cx, -cy, q.m00, q.m01);
+            s_q[j].geo2 = make_float4(q.m10, q.m11, q.r, log2f(op));
+            s_q[j].col = make_float4(cl.x, cl.y, cl.z, 0.f);
+            s_mask[j] = box_subblock_mask<G::SPR, typename G::Mask>(cx - q.hx, cx + q.hx, cy - q.hy, cy + q.hy);
         }
         __syncthreads();
+        const int steps = build_lists<G, kQuadBatch, true>(s_mask, 0, cnt, rows, warp, lane);
+        int j = row[0];
+#pragma unroll 4
+        for (int it = 0; it < steps; ++it) {
+            const QuadStage& st = s_q[j];
+            j = row[it + 1];  // the next entry's latency overlaps this visit
+            const float4 geo = st.geo, geo2 = st.geo2, col = st.col;
+            const F2 dx = dup2(__fadd_rn(px, geo.x));
 #pragma unroll
-        for (int k = 0; k < PPT; ++k) {
-            const int blk = warp + k * WARPS;
-            for (int base = ((cnt - 1) >> 5) << 5; base >= 0; base -= 32) {
-                const int jj = base + lane;
-                uint32_t bits = __ballot_sync(kFull, jj < cnt && ((s_mask[jj] >> blk) & 1u));
-                while (bits) {  // back to front: highest position first
-                    const int hb = 31 - __clz(bits);
-                    bits &= ~(1u << hb);
-                    const QuadStage& st = s_q[base + hb];
-                    const float dx = px[k] - st.cx, dy = py[k] - st.cy;
-                    // E9: local coordinate, a = p . p, fragment inside the quad
-                    const float p0 = fmaf(st.m00, dx, st.m01 * dy), p1 = fmaf(st.m10, dx, st.m11 * dy);
-                    const float a = fmaf(p0, p0, p1 * p1);
-                    const bool inside = fabsf(p0) <= st.r && fabsf(p1) <= st.r;
-                    const float e = fmaf(-kLog2e, a, st.l2s);  // log2(sigma e^{-a})
-                    const bool keep = inside && e >= kLog2AlphaMin;
-                    const float alpha = keep ? fminf(kAlphaMax, ex2_approx(e)) : 0.f;
-                    // "over": C = a c + (1 - a) C
-                    C0[k] = fmaf(alpha, st.cr - C0[k], C0[k]);
-                    C1[k] = fmaf(alpha, st.cg - C1[k], C1[k]);
-                    C2[k] = fmaf(alpha, st.cb - C2[k], C2[k]);
-                    T[k] = T[k] - alpha * T[k];
+            for (int p = 0; p < NP; ++p) {
+                // E9: local coordinate, a = p . p, fragment inside the quad
+                const F2 dy = add2(py[p], dup2(geo.y));
+                const F2 p0 = fma2(dup2(geo.z), dx, mul2(dup2(geo.w), dy));
+                const F2 p1 = fma2(dup2(geo2.x), dx, mul2(dup2(geo2.y), dy));
+                const F2 a = fma2(p0, p0, mul2(p1, p1));
+                const F2 e2 = fma2(dup2(-kLog2e), a, dup2(geo2.w));  // log2(sigma e^{-a})
+                float u0[2], u1[2], e[2], al[2];
+                unpack2(p0, u0[0], u0[1]);
+                unpack2(p1, u1[0], u1[1]);
+                unpack2(e2, e[0], e[1]);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const bool inside = fabsf(u0[h]) <= geo2.z && fabsf(u1[h]) <= geo2.z;
+                    al[h] = inside && e[h] >= kLog2AlphaMin ? fminf(kAlphaMax, ex2_approx(e[h])) : 0.f;
                 }
+                // "over": C = a c + (1 - a) C
+                const F2 alpha = pack2(al[0], al[1]), minus = dup2(-1.f);
+                C0[p] = fma2(alpha, fma2(C0[p], minus, dup2(col.x)), C0[p]);
+                C1[p] = fma2(alpha, fma2(C1[p], minus, dup2(col.y)), C1[p]);
+                C2[p] = fma2(alpha, fma2(C2[p], minus, dup2(col.z)), C2[p]);
+                T[p] = fma2(mul2(alpha, T[p]), minus, T[p]);
             }
         }
     }
+    const int gx = tx * TS + ix;
 #pragma unroll
-    for (int k = 0; k < PPT; ++k) {
-        const int gx = tx * TS + (int)px[k], gy = ty * TS + (int)py[k];
+    for (int k = 0; k < PX; ++k) {
+        const int gy = ty * TS + iy0 + k;
         if (gx < f.W && gy < f.H) {
             const size_t pix = (size_t)gy * f.W + gx;
-            image[3 * pix] = C0[k];
-            image[3 * pix + 1] = C1[k];
-            image[3 * pix + 2] = C2[k];
-            t_final[pix] = T[k];
+            float c[2][4];
+            unpack2(T[k / 2], c[0][3], c[1][3]);
+            unpack2(C0[k / 2], c[0][0], c[1][0]);
+            unpack2(C1[k / 2], c[0][1], c[1][1]);
+            unpack2(C2[k / 2], c[0][2], c[1][2]);
+            image[3 * pix] = c[k & 1][0];
+            image[3 * pix + 1] = c[k & 1][1];
+            image[3 * pix + 2] = c[k & 1][2];
+            t_final[pix] = c[k & 1][3];
         }
     }
 }
@@ -311,18 +326,15 @@ cudaError_t launch_render_quads(int64_t n, const float* splats, const float* dep
     e = launch_tile_ranges(pk, num_keys, reinterpret_cast<uint32_t*>(ranges), (uint32_t)ntiles, 0u, stream);
     if (e != cudaSuccess) return e;
     // 4. back-to-front quads per tile
+    auto run = [&](auto kernel, int threads) {
+        return launch_pdl(kernel, dim3((unsigned)ntiles), dim3(threads), 0, stream, (const uint2*)ranges, pv, order, s4,
+                          (const QuadRec*)quad, f, image, t_final);
+    };
     switch (f.TS) {
-        case 8:
-            return launch_pdl(k_blend_quads<8>, dim3((unsigned)ntiles), dim3(64), 0, stream, (const uint2*)ranges, pv,
-                              order, s4, (const QuadRec*)quad, f, image, t_final);
-        case 16:
-            return launch_pdl(k_blend_quads<16>, dim3((unsigned)ntiles), dim3(256), 0, stream, (const uint2*)ranges,
-                              pv, order, s4, (const QuadRec*)quad, f, image, t_final);
-        case 32:
-            return launch_pdl(k_blend_quads<32>, dim3((unsigned)ntiles), dim3(256), 0, stream, (const uint2*)ranges,
-                              pv, order, s4, (const QuadRec*)quad, f, image, t_final);
-        default:
-            return cudaErrorInvalidValue;
+        case 8: return run(k_blend_quads<8, tile_px<8>()>, TileGeom<8, tile_px<8>()>::THREADS);
+        case 16: return run(k_blend_quads<16, tile_px<16>()>, TileGeom<16, tile_px<16>()>::THREADS);
+        case 32: return run(k_blend_quads<32, tile_px<32>()>, TileGeom<32, tile_px<32>()>::THREADS);
+        default: return cudaErrorInvalidValue;
     }
 }
 
