@@ -100,7 +100,10 @@ k_preprocess_bwd(int64_t n, const float* __restrict__ means, const float* __rest
         // slot-ordered sum of this Gaussian's pair records
         sum_pair_records(partials, reinterpret_cast<const float*>(partials + 2 * (size_t)cap), first, nrec, pr);
         glogit = pr[5] * (1.f - sig);  // pr[5] = sigma dL/dsigma
-        splat_adjoint(f, X, q4, ls, pr, cl.w, gm, gls, gq);  // cl.w: the axis basis's t
+        float M[9], gM[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        gaussian_shape(q4, ls[0], ls[1], ls[2], M);
+        splat_adjoint(f, X, M, pr, cl.w, gm, gM);  // cl.w: the axis basis's t
+        shape_adjoint(q4, ls, gM, gls, gq);
     }
 
     // SH colour adjoint; gradients staged back through shared memory for
@@ -115,7 +118,7 @@ k_preprocess_bwd(int64_t n, const float* __restrict__ means, const float* __rest
     if (vis) {
         // the SH gradients overwrite this lane's staged coefficients in place
         // (sh_adjoint reads every coefficient before it writes a gradient)
-        sh_adjoint(f, X, mine, col, pr, gm, mine, false);
+        sh_adjoint<false>(f, X, mine, col, pr, gm, mine);
     } else if (need) {
 #pragma unroll
         for (int k = 0; k < 48; ++k) mine[k] = 0.f;

@@ -66,6 +66,10 @@ k_preprocess_batch(int64_t n, const float* __restrict__ means, const float* __re
         asm volatile("cp.async.wait_group 0;" ::: "memory");
         __syncwarp();
     }
+    // what the views share (the configuration's flags are every view's)
+    float M[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, sigma = 0.f, qc = 0.f;
+    const bool drawable = opaque_enough && gaussian_shape(q, l0, l1, l2, M);
+    if (drawable) qc = opacity_extent(ft.f[0], logit, sigma);
     for (int v = 0; v < ft.views; ++v) {
         const Frame& f = ft.f[v];
         const int64_t o = (int64_t)v * n + i;
@@ -74,8 +78,7 @@ k_preprocess_batch(int64_t n, const float* __restrict__ means, const float* __re
         if (valid) {
             const float d = view_depth(f, x, y, z);
             depth[o] = d;
-            vis = opaque_enough && d > f.znear;
-            if (vis) vis = project_splat(f, x, y, z, q, l0, l1, l2, logit, P);
+            vis = drawable && d > f.znear && project_splat(f, x, y, z, M, sigma, qc, P);
         }
         float3 c3 = make_float3(0.f, 0.f, 0.f);
         if (vis) {
@@ -179,7 +182,10 @@ k_preprocess_bwd_batch(int64_t n, const float* __restrict__ means, const float* 
         for (int k = 0; k < 48; ++k) gsh[k] = 0.f;
         __syncwarp();
     }
-    float gm[3] = {0.f, 0.f, 0.f}, gls[3] = {0.f, 0.f, 0.f}, gq[4] = {0.f, 0.f, 0.f, 0.f}, glogit = 0.f;
+    float gm[3] = {0.f, 0.f, 0.f}, glogit = 0.f;
+    float M[9], gM[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (valid) gaussian_shape(q4, ls[0], ls[1], ls[2], M);
+    bool seen = false;  // in some view
     // The next view's pair count and first slot are loaded one view ahead, so
     // their latency overlaps this view's adjoint.
     uint32_t cnt_next = valid ? __ldg(touched + i) : 0u;
@@ -192,6 +198,7 @@ k_preprocess_bwd_batch(int64_t n, const float* __restrict__ means, const float* 
             off_next = __ldg(offsets + o + n);
         }
         if (cnt == 0) continue;
+        seen = true;
         float pr[kPart];
 #pragma unroll
         for (int c = 0; c < kPart; ++c) pr[c] = 0.f;
@@ -203,10 +210,12 @@ k_preprocess_bwd_batch(int64_t n, const float* __restrict__ means, const float* 
         glogit += pr[5] * (1.f - sig);  // pr[5] = sigma dL/dsigma
         const Frame& f = ft.f[v];
         const float4 cl = __ldg(splats + kSplatVec4 * o + 2);  // colour and the axis basis's t
-        splat_adjoint(f, X, q4, ls, pr, cl.w, gm, gls, gq);
+        splat_adjoint(f, X, M, pr, cl.w, gm, gM);
         const float col[3] = {cl.x, cl.y, cl.z};
-        sh_adjoint(f, X, stage + lane * kShPad, col, pr, gm, gsh, true);
+        sh_adjoint<true>(f, X, stage + lane * kShPad, col, pr, gm, gsh);
     }
+    float gls[3] = {0.f, 0.f, 0.f}, gq[4] = {0.f, 0.f, 0.f, 0.f};
+    if (seen) shape_adjoint(q4, ls, gM, gls, gq);
     __syncwarp();
     float4* dst = d_sh + warp_first * 12;
     const float* gstage = s_gsh[warp];

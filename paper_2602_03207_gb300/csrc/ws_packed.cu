@@ -154,7 +154,8 @@ k_preprocess_packed(int64_t n, const float* __restrict__ means, const float* __r
         depth[i] = d;
         vis = opaque_enough && d > f.znear;
         float sxx, sxy, syy;
-        if (vis) vis = project_core(f, x, y, z, q, l0, l1, l2, P, sxx, sxy, syy);
+        float M[9];
+        vis = vis && gaussian_shape(q, l0, l1, l2, M) && project_core(f, x, y, z, M, P, sxx, sxy, syy);
         if (vis) {
             // pack: opacity on 8 bits, ellipse as binary16 axes
             a8 = quant8(1.f / (1.f + expf(-logit)));

@@ -71,7 +71,14 @@ k_preprocess(int64_t n, const float* __restrict__ means, const float* __restrict
     if (valid) {
         depth[i] = d;
         vis = opaque_enough && d > f.znear;
-        if (vis) vis = project_splat(f, x, y, z, q, l0, l1, l2, logit, P);
+        if (vis) {
+            float M[9], sigma;
+            vis = gaussian_shape(q, l0, l1, l2, M);
+            if (vis) {
+                const float qc = opacity_extent(f, logit, sigma);
+                vis = project_splat(f, x, y, z, M, sigma, qc, P);
+            }
+        }
     }
     const uint32_t late = __ballot_sync(kFull, vis && !likely);
     if (late) {

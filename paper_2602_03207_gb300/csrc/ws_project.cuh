@@ -139,14 +139,10 @@ __device__ __forceinline__ float sigma2d_det(const float V0[3], const float V1[3
     return fmaf(dil, sxx + syy - dil, cross2);
 }
 
-// Projection of one Gaussian that passed the opacity and near-plane tests:
-// Sigma = M M^T with M = R(q) diag(exp(log_scale)) (§2.1); the centre through
-// the pinhole in double-float; Sigma' = V V^T + dilation I with V = J W M
-// (EWA Jacobian J with the guard-band clamp) returned in sxx, sxy, syy;
-// conic = Sigma'^{-1}. Returns false when the quaternion is zero or Sigma' is
-// degenerate.
-__device__ __forceinline__ bool project_core(const Frame& f, float x, float y, float z, float4 q, float l0, float l1,
-                                             float l2, Projection& P, float& sxx, float& sxy, float& syy) {
+// What a Gaussian's projections to any camera share: M = R(q) diag(exp(
+// log_scale)), row-major (§2.1; Sigma = M M^T). Returns false when the
+// quaternion is zero. The batched kernels evaluate it once for all views.
+__device__ __forceinline__ bool gaussian_shape(float4 q, float l0, float l1, float l2, float (&M)[9]) {
     const float qn2 = q.x * q.x + q.y * q.y + q.z * q.z + q.w * q.w;
     if (qn2 == 0.f) return false;
     const float inv = rsqrtf(qn2);
@@ -155,8 +151,31 @@ __device__ __forceinline__ bool project_core(const Frame& f, float x, float y, f
                         2.f * (qx * qy + w * qz), 1.f - 2.f * (qx * qx + qz * qz), 2.f * (qy * qz - w * qx),
                         2.f * (qx * qz - w * qy), 2.f * (qy * qz + w * qx), 1.f - 2.f * (qx * qx + qy * qy)};
     const float s0 = expf(l0), s1 = expf(l1), s2 = expf(l2);
-    const float M[9] = {R[0] * s0, R[1] * s1, R[2] * s2, R[3] * s0, R[4] * s1,
-                        R[5] * s2, R[6] * s0, R[7] * s1, R[8] * s2};
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        M[3 * a] = R[3 * a] * s0;
+        M[3 * a + 1] = R[3 * a + 1] * s1;
+        M[3 * a + 2] = R[3 * a + 2] * s2;
+    }
+    return true;
+}
+
+// sigma and the opacity-aware extent (§3.4): q_c = 2 ln(255 sigma), or under
+// WS_CFG_FIXED_RADIUS (ablation) the extent every splat would need at
+// sigma = 1, independent of its opacity (conservative, only larger).
+__device__ __forceinline__ float opacity_extent(const Frame& f, float logit, float& sigma) {
+    const float en = expf(-logit);
+    sigma = 1.f / (1.f + en);
+    return (f.flags & WS_CFG_FIXED_RADIUS) ? 2.f * kLn255 : fmaxf(0.f, 2.f * (kLn255 - log1pf(en)));
+}
+
+// Projection of one Gaussian that passed the opacity and near-plane tests
+// (M from gaussian_shape): the centre through
+// the pinhole in double-float; Sigma' = V V^T + dilation I with V = J W M
+// (EWA Jacobian J with the guard-band clamp) returned in sxx, sxy, syy;
+// conic = Sigma'^{-1}. Returns false when Sigma' is degenerate.
+__device__ __forceinline__ bool project_core(const Frame& f, float x, float y, float z, const float (&M)[9],
+                                             Projection& P, float& sxx, float& sxy, float& syy) {
     // Camera-space centre in double-float, then the projected centre.
     const DF tx = df_affine3(f.R[0], f.R[1], f.R[2], x, y, z, f.t[0]);
     const DF ty = df_affine3(f.R[3], f.R[4], f.R[5], x, y, z, f.t[1]);
@@ -209,18 +228,13 @@ __device__ __forceinline__ bool splat_rect(const Frame& f, float mxh, float mxl,
     return true;
 }
 
-// project_core, then sigma and the opacity-aware extent
-// e = sqrt(2 ln(255 sigma) diag Sigma') (§3.4) and splat_rect.
-__device__ __forceinline__ bool project_splat(const Frame& f, float x, float y, float z, float4 q, float l0,
-                                              float l1, float l2, float logit, Projection& P) {
+// project_core, then the extent e = sqrt(q_c diag Sigma') (opacity_extent's
+// q_c and sigma) and splat_rect.
+__device__ __forceinline__ bool project_splat(const Frame& f, float x, float y, float z, const float (&M)[9],
+                                              float sigma, float qc, Projection& P) {
     float sxx, sxy, syy;
-    if (!project_core(f, x, y, z, q, l0, l1, l2, P, sxx, sxy, syy)) return false;
-    // sigma and the opacity-aware extent (§3.4): q_c = 2 ln(255 sigma)
-    const float en = expf(-logit);
-    P.sigma = 1.f / (1.f + en);
-    // WS_CFG_FIXED_RADIUS (ablation): the box every splat would need at
-    // sigma = 1, independent of its opacity (conservative, only larger).
-    const float qc = (f.flags & WS_CFG_FIXED_RADIUS) ? 2.f * kLn255 : fmaxf(0.f, 2.f * (kLn255 - log1pf(en)));
+    if (!project_core(f, x, y, z, M, P, sxx, sxy, syy)) return false;
+    P.sigma = sigma;
     const float ex = sqrtf(qc * sxx), ey = sqrtf(qc * syy);
     return splat_rect(f, P.m4.x, P.m4.z, P.m4.y, P.m4.w, ex, ey, P);
 }
@@ -229,50 +243,14 @@ __device__ __forceinline__ bool project_splat(const Frame& f, float x, float y, 
 // float4 reads of 32 consecutive records are bank-conflict free.
 constexpr int kShPad = 52;
 
-// Real SH basis of degree 3 (Condon-Shortley phase, index l*l + l + m) and
-// its gradient with respect to the (unit) direction.
-__device__ __forceinline__ void sh_basis_grad(float x, float y, float z, float* Y, float (*dY)[3]) {
-    const float k0 = 0.28209479177387814f, k1 = 0.4886025119029199f;
-    const float k2a = 1.0925484305920792f, k2b = 0.31539156525252005f, k2c = 0.5462742152960396f;
-    const float k3a = 0.5900435899266435f, k3b = 2.890611442640554f, k3c = 0.4570457994644658f;
-    const float k3d = 0.3731763325901154f, k3e = 1.445305721320277f;
-    const float xx = x * x, yy = y * y, zz = z * z;
-    Y[0] = k0;
-    dY[0][0] = dY[0][1] = dY[0][2] = 0.f;
-    Y[1] = -k1 * y;  dY[1][0] = 0.f; dY[1][1] = -k1; dY[1][2] = 0.f;
-    Y[2] = k1 * z;   dY[2][0] = 0.f; dY[2][1] = 0.f; dY[2][2] = k1;
-    Y[3] = -k1 * x;  dY[3][0] = -k1; dY[3][1] = 0.f; dY[3][2] = 0.f;
-    Y[4] = k2a * x * y;  dY[4][0] = k2a * y; dY[4][1] = k2a * x; dY[4][2] = 0.f;
-    Y[5] = -k2a * y * z; dY[5][0] = 0.f; dY[5][1] = -k2a * z; dY[5][2] = -k2a * y;
-    Y[6] = k2b * (2.f * zz - xx - yy);
-    dY[6][0] = -2.f * k2b * x; dY[6][1] = -2.f * k2b * y; dY[6][2] = 4.f * k2b * z;
-    Y[7] = -k2a * x * z; dY[7][0] = -k2a * z; dY[7][1] = 0.f; dY[7][2] = -k2a * x;
-    Y[8] = k2c * (xx - yy); dY[8][0] = 2.f * k2c * x; dY[8][1] = -2.f * k2c * y; dY[8][2] = 0.f;
-    Y[9] = -k3a * y * (3.f * xx - yy);
-    dY[9][0] = -6.f * k3a * x * y; dY[9][1] = -3.f * k3a * (xx - yy); dY[9][2] = 0.f;
-    Y[10] = k3b * x * y * z;
-    dY[10][0] = k3b * y * z; dY[10][1] = k3b * x * z; dY[10][2] = k3b * x * y;
-    Y[11] = -k3c * y * (4.f * zz - xx - yy);
-    dY[11][0] = 2.f * k3c * x * y; dY[11][1] = -k3c * (4.f * zz - xx - 3.f * yy); dY[11][2] = -8.f * k3c * y * z;
-    Y[12] = k3d * z * (2.f * zz - 3.f * xx - 3.f * yy);
-    dY[12][0] = -6.f * k3d * x * z; dY[12][1] = -6.f * k3d * y * z; dY[12][2] = k3d * (6.f * zz - 3.f * xx - 3.f * yy);
-    Y[13] = -k3c * x * (4.f * zz - xx - yy);
-    dY[13][0] = -k3c * (4.f * zz - 3.f * xx - yy); dY[13][1] = 2.f * k3c * x * y; dY[13][2] = -8.f * k3c * x * z;
-    Y[14] = k3e * z * (xx - yy);
-    dY[14][0] = 2.f * k3e * x * z; dY[14][1] = -2.f * k3e * y * z; dY[14][2] = k3e * (xx - yy);
-    Y[15] = -k3a * x * (xx - 3.f * yy);
-    dY[15][0] = -3.f * k3a * (xx - yy); dY[15][1] = 6.f * k3a * x * y; dY[15][2] = 0.f;
-}
-
-
 // Adjoint of project_splat's geometry for one view: given the summed pair
 // derivatives pr[0..1] = dL/d(centre x, y) and pr[2..4] = dL/d(alpha, beta,
 // gamma), the conic in the splat's axis basis (axis_basis(axis_t): q = alpha u^2 +
-// 2 beta u v + gamma v^2 with u = e1 . d, v = e2 . d), ADDS dL/dmeans,
-// dL/dlog_scales and dL/dquats into gm, gls, gq. The chain: conic =
+// 2 beta u v + gamma v^2 with u = e1 . d, v = e2 . d), ADDS dL/dmeans into gm
+// and dL/dM into gM (M from gaussian_shape, row-major). The chain: conic =
 // Sigma'^{-1}, Sigma' = V V^T + dilation I, V = J W M (the guard-band clamp of
-// J passes no gradient), M = R(q) diag(exp(log_scale)), q normalised, and the
-// pinhole projection of the centre.
+// J passes no gradient) and the pinhole projection of the centre. dL/dM is
+// linear in the views, so a batch adds it up and takes shape_adjoint once.
 //
 // Why the axis basis: for an elongated splat (Sigma' eigenvalues 1e4 and 0.3
 // px^2, say) the pixels far along its major axis give conic derivatives of
@@ -282,21 +260,13 @@ __device__ __forceinline__ void sh_basis_grad(float x, float y, float z, float* 
 // gradient of the major axis's scale comes out wrong by several times its
 // size; summed and transformed in the axis basis, each part keeps its own
 // relative precision.
-__device__ __forceinline__ void splat_adjoint(const Frame& f, const float X[3], float4 q4, const float ls[3],
-                                              const float pr[9], float axis_t, float gm[3], float gls[3], float gq[4]) {
-    // forward quantities
-    const float qn2 = q4.x * q4.x + q4.y * q4.y + q4.z * q4.z + q4.w * q4.w;
-    const float qinv = rsqrtf(qn2);
-    const float w = q4.x * qinv, x = q4.y * qinv, y = q4.z * qinv, z = q4.w * qinv;
-    const float R[3][3] = {{1.f - 2.f * (y * y + z * z), 2.f * (x * y - w * z), 2.f * (x * z + w * y)},
-                           {2.f * (x * y + w * z), 1.f - 2.f * (x * x + z * z), 2.f * (y * z - w * x)},
-                           {2.f * (x * z - w * y), 2.f * (y * z + w * x), 1.f - 2.f * (x * x + y * y)}};
-    const float s[3] = {expf(ls[0]), expf(ls[1]), expf(ls[2])};
+__device__ __forceinline__ void splat_adjoint(const Frame& f, const float X[3], const float (&Ms)[9],
+                                              const float pr[9], float axis_t, float gm[3], float (&gM)[9]) {
     float M[3][3];
 #pragma unroll
     for (int a = 0; a < 3; ++a)
 #pragma unroll
-        for (int b = 0; b < 3; ++b) M[a][b] = R[a][b] * s[b];
+        for (int b = 0; b < 3; ++b) M[a][b] = Ms[3 * a + b];
     float t[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) t[a] = f.R[3 * a] * X[0] + f.R[3 * a + 1] * X[1] + f.R[3 * a + 2] * X[2] + f.t[a];
@@ -374,18 +344,35 @@ __device__ __forceinline__ void splat_adjoint(const Frame& f, const float X[3], 
     gt[2] -= (pr[0] * f.fx * t[0] + pr[1] * f.fy * t[1]) * rz2;
 #pragma unroll
     for (int a = 0; a < 3; ++a) gm[a] += f.R[a] * gt[0] + f.R[3 + a] * gt[1] + f.R[6 + a] * gt[2];
-    // M = R diag(s): dM = Tm^T dV
+    // V = Tm M: dM = Tm^T dV
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) gM[3 * a + b] += Tm[0][a] * dV[0][b] + Tm[1][a] * dV[1][b];
+}
+
+// Adjoint of gaussian_shape: dL/dlog_scales and dL/dquats (through the
+// quaternion's normalisation) from gM = dL/dM.
+__device__ __forceinline__ void shape_adjoint(float4 q4, const float ls[3], const float (&gM)[9], float (&gls)[3],
+                                              float (&gq)[4]) {
+    const float qn2 = q4.x * q4.x + q4.y * q4.y + q4.z * q4.z + q4.w * q4.w;
+    const float qinv = rsqrtf(qn2);
+    const float w = q4.x * qinv, x = q4.y * qinv, y = q4.z * qinv, z = q4.w * qinv;
+    const float R[3][3] = {{1.f - 2.f * (y * y + z * z), 2.f * (x * y - w * z), 2.f * (x * z + w * y)},
+                           {2.f * (x * y + w * z), 1.f - 2.f * (x * x + z * z), 2.f * (y * z - w * x)},
+                           {2.f * (x * z - w * y), 2.f * (y * z + w * x), 1.f - 2.f * (x * x + y * y)}};
+    const float s[3] = {expf(ls[0]), expf(ls[1]), expf(ls[2])};
+    // M = R diag(s)
     float GR[3][3];
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
         float dsb = 0.f;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            const float gma = Tm[0][a] * dV[0][b] + Tm[1][a] * dV[1][b];
-            dsb = fmaf(gma, R[a][b], dsb);
-            GR[a][b] = gma * s[b];
+            dsb = fmaf(gM[3 * a + b], R[a][b], dsb);
+            GR[a][b] = gM[3 * a + b] * s[b];
         }
-        gls[b] += dsb * s[b];
+        gls[b] = dsb * s[b];
     }
     float gqh[4];
     gqh[0] = 2.f * (-z * GR[0][1] + y * GR[0][2] + z * GR[1][0] - x * GR[1][2] - y * GR[2][0] + x * GR[2][1]);
@@ -398,41 +385,92 @@ __device__ __forceinline__ void splat_adjoint(const Frame& f, const float X[3], 
     const float qh[4] = {w, x, y, z};
     const float qd = gqh[0] * w + gqh[1] * x + gqh[2] * y + gqh[3] * z;
 #pragma unroll
-    for (int a = 0; a < 4; ++a) gq[a] += (gqh[a] - qd * qh[a]) * qinv;
+    for (int a = 0; a < 4; ++a) gq[a] = (gqh[a] - qd * qh[a]) * qinv;
 }
 
 // Adjoint of the SH colour for one view: pr[6..8] = dL/drgb (zeroed where the
 // channel was clamped at 0, detected from the stored colour), `coef` the 48
 // coefficients (16-byte aligned). ADDS the direction term into gm and writes
-// dL/dcoef into gsh[48] (or adds to it when accumulate is true).
+// dL/dcoef into gsh[48] (or adds to it when ACCUMULATE). Four coefficients (12
+// floats, three 16-byte accesses of shared memory) at a time; every
+// coefficient is read before a gradient is written (gsh may be coef). The
+// direction's gradient is taken from h_k = coef_k . dL/drgb and the nonzero
+// derivatives of the basis: 81 multiply-adds where the full Jacobian per
+// channel took 192.
+template <bool ACCUMULATE>
 __device__ __forceinline__ void sh_adjoint(const Frame& f, const float X[3], const float* coef, const float rgb[3],
-                                           const float pr[9], float gm[3], float* gsh, bool accumulate) {
+                                           const float pr[9], float gm[3], float* gsh) {
     const float dx = X[0] - f.campos[0], dy = X[1] - f.campos[1], dz = X[2] - f.campos[2];
     const float invn = rsqrtf(dx * dx + dy * dy + dz * dz);
-    const float d[3] = {dx * invn, dy * invn, dz * invn};
-    float Y[16], dY[16][3];
-    sh_basis_grad(d[0], d[1], d[2], Y, dY);
-    float gd[3] = {0.f, 0.f, 0.f};
-    float gcol[3];
+    const float x = dx * invn, y = dy * invn, z = dz * invn;
+    float g[3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) gcol[c] = rgb[c] > 0.f ? pr[6 + c] : 0.f;
+    for (int c = 0; c < 3; ++c) g[c] = rgb[c] > 0.f ? pr[6 + c] : 0.f;
+    float h[16];
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const float cf = coef[3 * k + c];
-            gd[0] = fmaf(cf * gcol[c], dY[k][0], gd[0]);
-            gd[1] = fmaf(cf * gcol[c], dY[k][1], gd[1]);
-            gd[2] = fmaf(cf * gcol[c], dY[k][2], gd[2]);
-        }
+    for (int r = 0; r < 4; ++r) {
+        const float4 a = reinterpret_cast<const float4*>(coef)[3 * r];
+        const float4 b = reinterpret_cast<const float4*>(coef)[3 * r + 1];
+        const float4 c = reinterpret_cast<const float4*>(coef)[3 * r + 2];
+        h[4 * r] = fmaf(a.z, g[2], fmaf(a.y, g[1], a.x * g[0]));
+        h[4 * r + 1] = fmaf(b.y, g[2], fmaf(b.x, g[1], a.w * g[0]));
+        h[4 * r + 2] = fmaf(c.x, g[2], fmaf(b.w, g[1], b.z * g[0]));
+        h[4 * r + 3] = fmaf(c.w, g[2], fmaf(c.z, g[1], c.y * g[0]));
     }
+    const float k0 = 0.28209479177387814f, k1 = 0.4886025119029199f;
+    const float k2a = 1.0925484305920792f, k2b = 0.31539156525252005f, k2c = 0.5462742152960396f;
+    const float k3a = 0.5900435899266435f, k3b = 2.890611442640554f, k3c = 0.4570457994644658f;
+    const float k3d = 0.3731763325901154f, k3e = 1.445305721320277f;
+    const float xx = x * x, yy = y * y, zz = z * z, xy = x * y, xz = x * z, yz = y * z;
+    // (d/dx, d/dy, d/dz) of sum_k h_k Y_k
+    const float dif = xx - yy;
+    float gd[3];
+    gd[0] = -k1 * h[3];
+    gd[1] = -k1 * h[1];
+    gd[2] = k1 * h[2];
+    gd[0] = fmaf(k2a, fmaf(y, h[4], -z * h[7]), gd[0]);
+    gd[1] = fmaf(k2a, fmaf(x, h[4], -z * h[5]), gd[1]);
+    gd[2] = fmaf(-k2a, fmaf(y, h[5], x * h[7]), gd[2]);
+    gd[0] = fmaf(2.f * x, fmaf(k2c, h[8], -k2b * h[6]), gd[0]);
+    gd[1] = fmaf(-2.f * y, fmaf(k2c, h[8], k2b * h[6]), gd[1]);
+    gd[2] = fmaf(4.f * k2b * z, h[6], gd[2]);
+    gd[0] = fmaf(-3.f * k3a, fmaf(2.f * xy, h[9], dif * h[15]), gd[0]);
+    gd[1] = fmaf(-3.f * k3a, fmaf(dif, h[9], -2.f * xy * h[15]), gd[1]);
+    gd[0] = fmaf(k3b * yz, h[10], gd[0]);
+    gd[1] = fmaf(k3b * xz, h[10], gd[1]);
+    gd[2] = fmaf(k3b * xy, h[10], gd[2]);
+    gd[0] = fmaf(k3c, fmaf(2.f * xy, h[11], -(4.f * zz - 3.f * xx - yy) * h[13]), gd[0]);
+    gd[1] = fmaf(k3c, fmaf(2.f * xy, h[13], -(4.f * zz - xx - 3.f * yy) * h[11]), gd[1]);
+    gd[2] = fmaf(-8.f * k3c, fmaf(yz, h[11], xz * h[13]), gd[2]);
+    gd[0] = fmaf(xz, fmaf(2.f * k3e, h[14], -6.f * k3d * h[12]), gd[0]);
+    gd[1] = fmaf(-yz, fmaf(2.f * k3e, h[14], 6.f * k3d * h[12]), gd[1]);
+    gd[2] = fmaf(3.f * k3d * (2.f * zz - xx - yy), h[12], fmaf(k3e * dif, h[14], gd[2]));
+    const float Y[16] = {k0, -k1 * y, k1 * z, -k1 * x, k2a * xy, -k2a * yz, k2b * (2.f * zz - xx - yy), -k2a * xz,
+                         k2c * dif, -k3a * y * (3.f * xx - yy), k3b * xy * z, -k3c * y * (4.f * zz - xx - yy),
+                         k3d * z * (2.f * zz - 3.f * xx - 3.f * yy), -k3c * x * (4.f * zz - xx - yy), k3e * z * dif,
+                         -k3a * x * (xx - 3.f * yy)};
 #pragma unroll
-    for (int k = 0; k < 16; ++k)
+    for (int r = 0; r < 12; ++r) {
+        float4* o = reinterpret_cast<float4*>(gsh) + r;
+        float v[4] = {0.f, 0.f, 0.f, 0.f};
+        if (ACCUMULATE) {
+            const float4 t = *o;
+            v[0] = t.x;
+            v[1] = t.y;
+            v[2] = t.z;
+            v[3] = t.w;
+        }
 #pragma unroll
-        for (int c = 0; c < 3; ++c) gsh[3 * k + c] = accumulate ? gsh[3 * k + c] + Y[k] * gcol[c] : Y[k] * gcol[c];
-    const float dd = gd[0] * d[0] + gd[1] * d[1] + gd[2] * d[2];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) gm[a] += (gd[a] - dd * d[a]) * invn;
+        for (int c = 0; c < 4; ++c) {
+            const int e = 4 * r + c;
+            v[c] = ACCUMULATE ? fmaf(Y[e / 3], g[e % 3], v[c]) : Y[e / 3] * g[e % 3];
+        }
+        *o = make_float4(v[0], v[1], v[2], v[3]);
+    }
+    const float dd = gd[0] * x + gd[1] * y + gd[2] * z;
+    gm[0] += (gd[0] - dd * x) * invn;
+    gm[1] += (gd[1] - dd * y) * invn;
+    gm[2] += (gd[2] - dd * z) * invn;
 }
 
 }  // namespace ws
