@@ -485,8 +485,8 @@ ws_status ws_rasterize_backward(int64_t n, const float* means, const float* log_
     const Frame f = make_frame(cam, cfg);
     char* scratch = static_cast<char*>(workspace) + layout(0, key_capacity).bwd;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const uint32_t* order = nullptr;
-    if (ws::launch_tile_order(ranges, (uint32_t)(f.TX * f.TY), key_capacity, scratch, &order, s) != cudaSuccess)
+    ws::TileOrder order;
+    if (ws::launch_tile_order(ranges, (uint32_t)(f.TX * f.TY), f.TS, key_capacity, scratch, &order, s) != cudaSuccess)
         return WS_ERR_CUDA;
     return cuda_status(ws::launch_backward(n, means, log_scales, quats, sh, f, splats, rect, offsets, tiles_touched,
                                            vals, ranges, order, t_final, n_contrib, d_image, nullptr, d_means,
@@ -577,8 +577,9 @@ ws_status ws_rasterize_backward_batch(int64_t n, const float* means, const float
     if (key_capacity > 0 && (!vals || !aligned16(vals))) return WS_ERR_INVALID_ARG;
     char* scratch = static_cast<char*>(workspace) + layout(0, key_capacity).bwd;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const uint32_t* order = nullptr;
-    if (ws::launch_tile_order(ranges, ft.tile_off[ft.views], key_capacity, scratch, &order, s) != cudaSuccess)
+    ws::TileOrder order;
+    if (ws::launch_tile_order(ranges, ft.tile_off[ft.views], ft.f[0].TS, key_capacity, scratch, &order, s) !=
+        cudaSuccess)
         return WS_ERR_CUDA;
     return cuda_status(ws::launch_backward_batch(n, means, log_scales, quats, sh, ft, splats, rect, offsets,
                                                  tiles_touched, vals, ranges, order, t_final, n_contrib, d_image,
@@ -611,13 +612,13 @@ ws_status ws_render_train_l2(int64_t n, const float* means, const float* log_sca
     // ranges, the tiles' order, the forward blend (image, t_final,
     // n_contrib), the backward with dL/dC = image - target
     const uint32_t ntiles = (uint32_t)(f.TX * f.TY);
-    const uint32_t* order = nullptr;
+    ws::TileOrder order;
     cudaError_t e = ws::launch_tile_ranges(keys, num_keys, ranges, ntiles, f.flags, s);
-    if (e == cudaSuccess) e = ws::launch_tile_order(ranges, ntiles, key_capacity, scratch, &order, s);
+    if (e == cudaSuccess) e = ws::launch_tile_order(ranges, ntiles, f.TS, key_capacity, scratch, &order, s);
     Frame fr = f;
     fr.flags |= WS_CFG_RANGES_GIVEN;
     if (e == cudaSuccess)
-        e = ws::launch_rasterize(num_keys, 0, keys, vals, splats, fr, ranges, order, image, t_final, n_contrib, s);
+        e = ws::launch_rasterize(num_keys, 0, keys, vals, splats, fr, ranges, order.order, image, t_final, n_contrib, s);
     if (e != cudaSuccess) return WS_ERR_CUDA;
     return cuda_status(ws::launch_backward(n, means, log_scales, quats, sh, f, splats, rect, offsets, tiles_touched,
                                            vals, ranges, order, t_final, n_contrib, image, target, d_means,
@@ -648,13 +649,13 @@ ws_status ws_render_train_l2_batch(int64_t n, const float* means, const float* l
     char* scratch = static_cast<char*>(workspace) + layout(0, key_capacity).bwd;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const uint32_t ntiles = ft.tile_off[ft.views];
-    const uint32_t* order = nullptr;
+    ws::TileOrder order;
     cudaError_t e = ws::launch_tile_ranges(keys, num_keys, ranges, ntiles, ft.f[0].flags, s);
-    if (e == cudaSuccess) e = ws::launch_tile_order(ranges, ntiles, key_capacity, scratch, &order, s);
+    if (e == cudaSuccess) e = ws::launch_tile_order(ranges, ntiles, ft.f[0].TS, key_capacity, scratch, &order, s);
     ft.f[0].flags |= WS_CFG_RANGES_GIVEN;
     if (e == cudaSuccess)
-        e = ws::launch_rasterize_batch(num_keys, keys, vals, n, splats, ft, ranges, order, image, t_final, n_contrib,
-                                       s);
+        e = ws::launch_rasterize_batch(num_keys, keys, vals, n, splats, ft, ranges, order.order, image, t_final,
+                                       n_contrib, s);
     if (e != cudaSuccess) return WS_ERR_CUDA;
     return cuda_status(ws::launch_backward_batch(n, means, log_scales, quats, sh, ft, splats, rect, offsets,
                                                  tiles_touched, vals, ranges, order, t_final, n_contrib, image, target,

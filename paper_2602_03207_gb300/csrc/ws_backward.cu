@@ -26,20 +26,49 @@ namespace ws {
 
 namespace {
 
-// Backward records of one tile per block, the tiles in the order given
-// (launch_tile_order), or centre-out without one (centre_out_tile).
+// Backward records of one item per block: a segment of a long list, or a tile
+// in the order given (launch_tile_order); without an order the tiles
+// centre-out (centre_out_tile).
 template <int TS, int PX>
 __global__ void __launch_bounds__(TileGeom<TS, PX>::THREADS, bwd_min_blocks<TS>())
-k_blend_bwd(const uint2* __restrict__ ranges, const uint32_t* __restrict__ order, const uint32_t* __restrict__ vals,
+k_blend_bwd(const uint2* __restrict__ ranges, const TileOrder order, const uint32_t* __restrict__ vals,
             const float4* __restrict__ splats, const uint2* __restrict__ rect, const uint32_t* __restrict__ offsets,
-            const Frame f, const float* __restrict__ t_final, const uint32_t* __restrict__ n_contrib,
-            const float* __restrict__ d_image, const float* __restrict__ target, const PairRecords out) {
+            const Frame f, const float* __restrict__ t_final, const float* __restrict__ d_image,
+            const float* __restrict__ target, const PairRecords out) {
     __shared__ BwdSmem<TS, PX, bwd_batch<TS>()> sm;
     pdl_wait();
-    const int t = order ? (int)__ldg(order + blockIdx.x) : centre_out_tile(f, blockIdx.x);
-    blend_bwd_tile<TS, PX>(f, t, ranges[t], vals, splats, rect,
-                           offsets, t_final, n_contrib, d_image, target,
-                           out, sm);
+    const auto item = [&](uint32_t& t, uint32_t& first, BwdSpan& span) {
+        if (order.order) return bwd_item(order, ranges, blockIdx.x, TS * TS, t, first, span);
+        t = (uint32_t)centre_out_tile(f, blockIdx.x);
+        const uint2 range = ranges[t];
+        first = range.x;
+        span = BwdSpan{0u, range.y - range.x, nullptr, 0u, 1u};
+        return true;
+    };
+    uint32_t t, first;
+    BwdSpan span;
+    if (!item(t, first, span)) return;
+    if (bwd_tile_body<TS, PX, true>(f, (int)t, first, span, vals, splats, rect, offsets, t_final, d_image, target, out,
+                                    sm))
+        return;
+    // an infinite or NaN value: the whole item again with the selecting walk
+    __syncthreads();
+    item(t, first, span);
+    bwd_tile_body<TS, PX, false>(f, (int)t, first, span, vals, splats, rect, offsets, t_final, d_image, target, out, sm);
+}
+
+// The states of the long lists' segments, one per block (segment_state).
+template <int TS, int PX>
+__global__ void __launch_bounds__(TileGeom<TS, PX>::THREADS, fwd_min_blocks<TS>())
+k_seg_state(const uint2* __restrict__ ranges, const TileOrder order, const uint32_t* __restrict__ vals,
+            const float4* __restrict__ splats, const Frame f, const float* __restrict__ d_image,
+            const float* __restrict__ target) {
+    pdl_wait();
+    uint32_t t, first;
+    BwdSpan span;
+    if (!bwd_item(order, ranges, blockIdx.x, TS * TS, t, first, span)) return;
+    segment_state<TS, PX>(f, (int)t, first + span.lo, first + span.hi, vals, splats, d_image, target,
+                          order.states + (size_t)blockIdx.x * (TS * TS));
 }
 
 constexpr int kPbThreads = 128;
@@ -173,15 +202,28 @@ __device__ __forceinline__ uint32_t length_class(uint32_t len) {
     return 63u - (uint32_t)(2 * lz + ((len >> (lz - 1)) & 1u));
 }
 
+// Lists of more than head[1] positions are cut into segments of that length
+// (max_split > 0): the shortest for which max_split segments are enough, as 2
+// total / max_split positions each give at most total / head[1] + (lists cut)
+// of them.
 __global__ void __launch_bounds__(kOrderThreads)
-k_tile_order(const uint2* __restrict__ ranges, uint32_t ntiles, uint32_t* __restrict__ order) {
+k_tile_order(const uint2* __restrict__ ranges, uint32_t ntiles, uint32_t* __restrict__ order,
+             uint32_t* __restrict__ head, uint2* __restrict__ split, uint32_t max_split) {
     constexpr int W = kOrderThreads / 32, R = 1 << kOrderBits, U = 4;
     __shared__ uint32_t s_cnt[W][R];
     __shared__ uint32_t s_red[W + 1];
+    __shared__ uint32_t s_split;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < W * R; i += kOrderThreads) (&s_cnt[0][0])[i] = 0u;
+    if (threadIdx.x == 0) s_split = 0u;
     pdl_wait();
     __syncthreads();
+    uint32_t seg_len = ~0u;
+    if (max_split) {
+        const uint32_t total = __ldg(ranges + ntiles - 1).y;  // pairs of all lists
+        const uint32_t need = (uint32_t)((2ull * total + max_split - 1) / max_split);
+        seg_len = max(kSplitLeast, (need + kSplitUnit - 1) / kSplitUnit * kSplitUnit);
+    }
     const uint32_t per = (ntiles + kOrderThreads * U - 1) / (kOrderThreads * U) * (32 * U);
     const uint32_t lo = min(warp * per, ntiles), hi = min(lo + per, ntiles);
     // pass 0 counts, pass 1 places
@@ -200,6 +242,12 @@ k_tile_order(const uint2* __restrict__ ranges, uint32_t ntiles, uint32_t* __rest
                 if (i >= hi) break;
                 const uint32_t at = atomicAdd(&s_cnt[warp][length_class(len[u])], 1u);
                 if (pass) order[at] = i;
+                if (pass && len[u] > seg_len) {
+                    const uint32_t nseg = (len[u] + seg_len - 1) / seg_len;
+                    const uint32_t base = atomicAdd(&s_split, nseg);
+                    for (uint32_t k = 0; k < nseg && base + k < max_split; ++k)
+                        split[base + k] = make_uint2(i | (k << kSplitTileBits), base);
+                }
             }
         }
         __syncthreads();
@@ -214,32 +262,55 @@ k_tile_order(const uint2* __restrict__ ranges, uint32_t ntiles, uint32_t* __rest
         s_cnt[w + 1][c] = ex + a;
         __syncthreads();
     }
+    if (max_split && threadIdx.x == 0) {
+        head[0] = s_split;
+        head[1] = seg_len;
+    }
 }
 
 }  // namespace
 
+// Scratch: [pair records, 36 B per key | tile order | head | split | states],
+// the last three from kSplitMinCapacity on.
 size_t backward_scratch_bytes(int64_t key_capacity) {
-    return (size_t)(key_capacity > 0 ? key_capacity : 1) * kPart * sizeof(float) + kOrderMax * sizeof(uint32_t);
+    const int64_t cap = key_capacity > 0 ? key_capacity : 1;
+    size_t bytes = (size_t)cap * kPart * sizeof(float) + 256 + kOrderMax * sizeof(uint32_t);
+    if (cap >= kSplitMinCapacity) bytes += 256 + kSplitMost * sizeof(uint2) + kSplitStateBytes;
+    return bytes;
 }
 
-cudaError_t launch_tile_order(const uint32_t* ranges, uint32_t ntiles, int64_t key_capacity, void* scratch,
-                              const uint32_t** order, cudaStream_t stream) {
-    *order = nullptr;
-    if (ntiles < kOrderMin || ntiles > kOrderMax) return cudaSuccess;
-    uint32_t* o = reinterpret_cast<uint32_t*>(pair_records(scratch, key_capacity > 0 ? key_capacity : 1).p9 +
-                                              (key_capacity > 0 ? key_capacity : 1));
-    *order = o;
+cudaError_t launch_tile_order(const uint32_t* ranges, uint32_t ntiles, int side, int64_t key_capacity, void* scratch,
+                              TileOrder* o, cudaStream_t stream) {
+    *o = TileOrder{nullptr, nullptr, nullptr, nullptr, 0u};
+    const int64_t cap = key_capacity > 0 ? key_capacity : 1;
+    const bool cut = cap >= kSplitMinCapacity &&
+                     (cap >= kSplitAnyCapacity || cap >= (int64_t)kSplitMean * (int64_t)ntiles);
+    if (ntiles == 0 || ntiles > kOrderMax || (ntiles < kOrderMin && !cut)) return cudaSuccess;
+    char* base = static_cast<char*>(scratch) + (((size_t)cap * kPart * sizeof(float) + 255) & ~size_t(255));
+    uint32_t* order = reinterpret_cast<uint32_t*>(base);
+    uint32_t* head = order + kOrderMax;
+    uint2* split = reinterpret_cast<uint2*>(head + 64);
+    o->order = order;
+    if (cut) {
+        o->head = head;
+        o->split = split;
+        o->states = reinterpret_cast<float2*>(split + kSplitMost);
+        const size_t states = kSplitStateBytes / ((size_t)side * side * sizeof(float2));
+        const uint32_t most = ntiles < kOrderMin ? kSplitMost : kSplitMost / 2;
+        o->max_split = states < most ? (uint32_t)states : most;
+    }
     return launch_pdl(k_tile_order, dim3(1), dim3(kOrderThreads), 0, stream, reinterpret_cast<const uint2*>(ranges),
-                      ntiles, o);
+                      ntiles, order, head, split, o->max_split);
 }
 
 cudaError_t launch_backward(int64_t n, const float* means, const float* log_scales, const float* quats,
                             const float* sh, const Frame& f, const float* splats, const uint16_t* rect,
                             const uint32_t* offsets, const uint32_t* tiles_touched,
-                            const uint32_t* vals, const uint32_t* ranges, const uint32_t* order, const float* t_final,
+                            const uint32_t* vals, const uint32_t* ranges, const TileOrder& order, const float* t_final,
                             const uint32_t* n_contrib, const float* d_image, const float* target, float* d_means,
                             float* d_log_scales, float* d_quats, float* d_logits, float* d_sh,
                             int64_t key_capacity, void* scratch, cudaStream_t stream) {
+    (void)n_contrib;  // the walk finds for itself what each pixel composites
     const PairRecords partials = pair_records(scratch, key_capacity);
     const int ntiles = f.TX * f.TY;
     const uint2* r2 = reinterpret_cast<const uint2*>(ranges);
@@ -247,14 +318,20 @@ cudaError_t launch_backward(int64_t n, const float* means, const float* log_scal
     const uint2* rc = reinterpret_cast<const uint2*>(rect);
     cudaError_t e = cudaSuccess;
     if (ntiles > 0) {
-        auto run = [&](auto kernel, int threads) {
-            return launch_pdl(kernel, dim3(ntiles), dim3(threads), 0, stream, r2, order, vals, s4, rc, offsets, f,
-                              t_final, n_contrib, d_image, target, partials);
+        auto run = [&](auto states, auto kernel, int threads) {
+            if (order.max_split) {
+                const cudaError_t se = launch_pdl(states, dim3(order.max_split), dim3(threads), 0, stream, r2, order,
+                                                  vals, s4, f, d_image, target);
+                if (se != cudaSuccess) return se;
+            }
+            return launch_pdl(kernel, dim3(ntiles + order.max_split), dim3(threads), 0, stream, r2, order, vals, s4,
+                              rc, offsets, f, t_final, d_image, target, partials);
         };
+        constexpr int P8 = tile_px<8>(), P16 = tile_px<16>(), P32 = tile_px<32>();
         switch (f.TS) {
-            case 8: e = run(k_blend_bwd<8, tile_px<8>()>, TileGeom<8, tile_px<8>()>::THREADS); break;
-            case 16: e = run(k_blend_bwd<16, tile_px<16>()>, TileGeom<16, tile_px<16>()>::THREADS); break;
-            case 32: e = run(k_blend_bwd<32, tile_px<32>()>, TileGeom<32, tile_px<32>()>::THREADS); break;
+            case 8: e = run(k_seg_state<8, P8>, k_blend_bwd<8, P8>, TileGeom<8, P8>::THREADS); break;
+            case 16: e = run(k_seg_state<16, P16>, k_blend_bwd<16, P16>, TileGeom<16, P16>::THREADS); break;
+            case 32: e = run(k_seg_state<32, P32>, k_blend_bwd<32, P32>, TileGeom<32, P32>::THREADS); break;
             default: return cudaErrorInvalidValue;
         }
         if (e != cudaSuccess) return e;

@@ -109,31 +109,55 @@ k_blend_batch(const uint2* __restrict__ ranges, const uint32_t* __restrict__ ord
                    n_contrib + po);
 }
 
-// Backward records of every (view, tile) item. PERSISTENT = false: one block
-// per item, in the order given (launch_tile_order) or item order.
-// PERSISTENT = true: a grid of as many blocks as fit on the GPU at once, block
-// b taking items b, b + G, b + 2G, ... (G = the grid size) of that order, so
-// the assignment is static; no block waits on another.
+// Backward records of every item (a segment of a long list, or a tile of a
+// view: bwd_item). PERSISTENT = false: one block per item. PERSISTENT = true: a
+// grid of as many blocks as fit on the GPU at once, block b taking items b, b +
+// G, b + 2G, ... (G = the grid size), so the assignment is static; no block
+// waits on another.
 template <int TS, int PX, bool PERSISTENT>
 __global__ void __launch_bounds__(TileGeom<TS, PX>::THREADS, bwd_min_blocks<TS>())
-k_blend_bwd_batch(const uint2* __restrict__ ranges, const uint32_t* __restrict__ order,
-                  const uint32_t* __restrict__ vals, int64_t n, const float4* __restrict__ splats,
-                  const uint2* __restrict__ rect, const uint32_t* __restrict__ offsets, const FrameTable ft,
-                  const float* __restrict__ t_final, const uint32_t* __restrict__ n_contrib,
+k_blend_bwd_batch(const uint2* __restrict__ ranges, const TileOrder order, const uint32_t* __restrict__ vals,
+                  int64_t n, const float4* __restrict__ splats, const uint2* __restrict__ rect,
+                  const uint32_t* __restrict__ offsets, const FrameTable ft, const float* __restrict__ t_final,
                   const float* __restrict__ d_image, const float* __restrict__ target, const PairRecords out) {
     __shared__ BwdSmem<TS, PX, bwd_batch<TS>()> sm;
     pdl_wait();
-    const uint32_t ntiles = ft.tile_off[ft.views];
-    const uint32_t stride = PERSISTENT ? gridDim.x : ntiles;
-    for (uint32_t i = blockIdx.x; i < ntiles; i += stride) {
-        const uint32_t t = order ? __ldg(order + i) : i;
-        const int v = view_of_tile(ft.tile_off, ft.views, t);
-        const uint64_t vo = (uint64_t)v * (uint64_t)n, po = ft.pix_off[v];
-        blend_bwd_tile<TS, PX>(ft.f[v], (int)(t - ft.tile_off[v]), ranges[t], vals, splats + kSplatVec4 * vo,
-                               rect + vo, offsets + vo, t_final + po,
-                               n_contrib + po, d_image + 3 * po, target ? target + 3 * po : nullptr, out, sm);
+    const uint32_t items = ft.tile_off[ft.views] + order.max_split;
+    const uint32_t stride = PERSISTENT ? gridDim.x : items;
+    for (uint32_t i = blockIdx.x; i < items; i += stride) {
+        const auto walk = [&](auto finite) {
+            uint32_t t, first;
+            BwdSpan span;
+            if (!bwd_item(order, ranges, i, TS * TS, t, first, span)) return true;
+            const int v = view_of_tile(ft.tile_off, ft.views, t);
+            const uint64_t vo = (uint64_t)v * (uint64_t)n, po = ft.pix_off[v];
+            return bwd_tile_body<TS, PX, decltype(finite)::value>(
+                ft.f[v], (int)(t - ft.tile_off[v]), first, span, vals, splats + kSplatVec4 * vo, rect + vo,
+                offsets + vo, t_final + po, d_image + 3 * po, target ? target + 3 * po : nullptr, out, sm);
+        };
+        if (!walk(std::true_type{})) {  // an infinite or NaN value: the item again with the selecting walk
+            __syncthreads();
+            walk(std::false_type{});
+        }
         if (PERSISTENT) __syncthreads();  // the last reads of sm before the next item's writes
     }
+}
+
+// The states of the long lists' segments, one per block (segment_state).
+template <int TS, int PX>
+__global__ void __launch_bounds__(TileGeom<TS, PX>::THREADS, fwd_min_blocks<TS>())
+k_seg_state_batch(const uint2* __restrict__ ranges, const TileOrder order, const uint32_t* __restrict__ vals,
+                  int64_t n, const float4* __restrict__ splats, const FrameTable ft,
+                  const float* __restrict__ d_image, const float* __restrict__ target) {
+    pdl_wait();
+    uint32_t t, first;
+    BwdSpan span;
+    if (!bwd_item(order, ranges, blockIdx.x, TS * TS, t, first, span)) return;
+    const int v = view_of_tile(ft.tile_off, ft.views, t);
+    const uint64_t vo = (uint64_t)v * (uint64_t)n, po = ft.pix_off[v];
+    segment_state<TS, PX>(ft.f[v], (int)(t - ft.tile_off[v]), first + span.lo, first + span.hi, vals,
+                          splats + kSplatVec4 * vo, d_image + 3 * po, target ? target + 3 * po : nullptr,
+                          order.states + (size_t)blockIdx.x * (TS * TS));
 }
 
 __global__ void __launch_bounds__(kBatchThreads)
@@ -182,10 +206,10 @@ k_preprocess_bwd_batch(int64_t n, const float* __restrict__ means, const float* 
         for (int k = 0; k < 48; ++k) gsh[k] = 0.f;
         __syncwarp();
     }
-    float gm[3] = {0.f, 0.f, 0.f}, glogit = 0.f;
+    float gm[3] = {0.f, 0.f, 0.f}, gsig = 0.f;
     float M[9], gM[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (valid) gaussian_shape(q4, ls[0], ls[1], ls[2], M);
-    bool seen = false;  // in some view
+    int64_t last_seen = -1;  // this Gaussian in the last view that sees it
     // The next view's pair count and first slot are loaded one view ahead, so
     // their latency overlaps this view's adjoint.
     uint32_t cnt_next = valid ? __ldg(touched + i) : 0u;
@@ -198,7 +222,7 @@ k_preprocess_bwd_batch(int64_t n, const float* __restrict__ means, const float* 
             off_next = __ldg(offsets + o + n);
         }
         if (cnt == 0) continue;
-        seen = true;
+        last_seen = o;
         float pr[kPart];
 #pragma unroll
         for (int c = 0; c < kPart; ++c) pr[c] = 0.f;
@@ -206,8 +230,7 @@ k_preprocess_bwd_batch(int64_t n, const float* __restrict__ means, const float* 
         // dropped those pairs and raised WS_FLAG_CAPACITY)
         const uint32_t nrec = first >= cap ? 0u : min(cnt, cap - first);
         sum_pair_records(partials, reinterpret_cast<const float*>(partials + 2 * (size_t)cap), first, nrec, pr);
-        const float sig = __ldg(splats + kSplatVec4 * o + 1).w;  // sigma (the same in every view)
-        glogit += pr[5] * (1.f - sig);  // pr[5] = sigma dL/dsigma
+        gsig += pr[5];  // sigma dL/dsigma
         const Frame& f = ft.f[v];
         const float4 cl = __ldg(splats + kSplatVec4 * o + 2);  // colour and the axis basis's t
         splat_adjoint(f, X, M, pr, cl.w, gm, gM);
@@ -215,7 +238,11 @@ k_preprocess_bwd_batch(int64_t n, const float* __restrict__ means, const float* 
         sh_adjoint<true>(f, X, stage + lane * kShPad, col, pr, gm, gsh);
     }
     float gls[3] = {0.f, 0.f, 0.f}, gq[4] = {0.f, 0.f, 0.f, 0.f};
-    if (seen) shape_adjoint(q4, ls, gM, gls, gq);
+    float glogit = 0.f;
+    if (last_seen >= 0) {
+        shape_adjoint(q4, ls, gM, gls, gq);
+        glogit = gsig * (1.f - __ldg(splats + kSplatVec4 * last_seen + 1).w);  // sigma: the same in every view
+    }
     __syncwarp();
     float4* dst = d_sh + warp_first * 12;
     const float* gstage = s_gsh[warp];
@@ -287,35 +314,41 @@ cudaError_t launch_rasterize_batch(const uint32_t* num_keys, const uint64_t* key
 }
 
 template <int TS>
-cudaError_t launch_bwd_items(const uint2* r2, const uint32_t* order, const uint32_t* vals, int64_t n, const float4* s4,
+cudaError_t launch_bwd_items(const uint2* r2, const TileOrder& order, const uint32_t* vals, int64_t n, const float4* s4,
                              const uint2* rc, const uint32_t* offsets, const FrameTable& ft, const float* t_final,
-                             const uint32_t* n_contrib, const float* d_image, const float* target,
-                             const PairRecords& out, bool persistent, cudaStream_t stream) {
-    const uint32_t ntiles = ft.tile_off[ft.views];
+                             const float* d_image, const float* target, const PairRecords& out, bool persistent, cudaStream_t stream) {
+    const uint32_t items = ft.tile_off[ft.views] + order.max_split;
     constexpr int PX = tile_px<TS>();
     constexpr int kThreads = TileGeom<TS, PX>::THREADS;
+    cudaError_t e = cudaSuccess;
+    if (order.max_split) {
+        e = launch_pdl(k_seg_state_batch<TS, PX>, dim3(order.max_split), dim3(kThreads), 0, stream, r2, order, vals, n,
+                       s4, ft, d_image, target);
+        if (e != cudaSuccess) return e;
+    }
     if (!persistent)
-        return launch_pdl(k_blend_bwd_batch<TS, PX, false>, dim3(ntiles), dim3(kThreads), 0, stream, r2, order, vals,
-                          n, s4, rc, offsets, ft, t_final, n_contrib, d_image, target, out);
+        return launch_pdl(k_blend_bwd_batch<TS, PX, false>, dim3(items), dim3(kThreads), 0, stream, r2, order, vals, n,
+                          s4, rc, offsets, ft, t_final, d_image, target, out);
     int dev = 0, sms = 148, occ = 1;
-    cudaError_t e = cudaGetDevice(&dev);
+    e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_blend_bwd_batch<TS, PX, true>, kThreads, 0);
     if (e != cudaSuccess) return e;
-    const uint32_t grid = min(ntiles, (uint32_t)(sms * (occ > 0 ? occ : 1)));
+    const uint32_t grid = min(items, (uint32_t)(sms * (occ > 0 ? occ : 1)));
     return launch_pdl(k_blend_bwd_batch<TS, PX, true>, dim3(grid), dim3(kThreads), 0, stream, r2, order, vals, n, s4,
-                      rc, offsets, ft, t_final, n_contrib, d_image, target, out);
+                      rc, offsets, ft, t_final, d_image, target, out);
 }
 
 cudaError_t launch_backward_batch(int64_t n, const float* means, const float* log_scales, const float* quats,
                                   const float* sh, const FrameTable& ft, const float* splats, const uint16_t* rect,
                                   const uint32_t* offsets, const uint32_t* tiles_touched, const uint32_t* vals,
-                                  const uint32_t* ranges, const uint32_t* order, const float* t_final,
+                                  const uint32_t* ranges, const TileOrder& order, const float* t_final,
                                   const uint32_t* n_contrib, const float* d_image, const float* target, float* d_means,
                                   float* d_log_scales, float* d_quats, float* d_logits, float* d_sh,
                                   int64_t key_capacity, bool persistent, void* scratch, cudaStream_t stream) {
+    (void)n_contrib;  // the walk finds for itself what each pixel composites
     const PairRecords partials = pair_records(scratch, key_capacity);
     const uint32_t ntiles = ft.tile_off[ft.views];
     const uint2* r2 = reinterpret_cast<const uint2*>(ranges);
@@ -324,7 +357,7 @@ cudaError_t launch_backward_batch(int64_t n, const float* means, const float* lo
     cudaError_t e = cudaSuccess;
     if (ntiles > 0) {
         auto run = [&](auto items) {
-            return items(r2, order, vals, n, s4, rc, offsets, ft, t_final, n_contrib, d_image, target, partials,
+            return items(r2, order, vals, n, s4, rc, offsets, ft, t_final, d_image, target, partials,
                          persistent, stream);
         };
         switch (ft.f[0].TS) {

@@ -423,7 +423,6 @@ struct BwdSmem {
     __align__(16) float dC[G::NSB][52];
     typename G::Mask mask[BATCH];
     uint32_t slot[BATCH];
-    uint32_t maxl[G::WARPS];
     uint16_t vis[VCAP];        // staged index | sub-block << 8
     uint16_t base[BATCH + 2];  // visits of the staged splats before each
 };
@@ -447,21 +446,22 @@ struct BwdPixels {
     float px;
     F2 py[NP], T[NP], b[NP], dC[NP][3];
 
-    // ix, iy0: this lane's pixels (TileGeom::pixel); tf, dc: their final
-    // transmittance and dL/dC, zeros outside the image (T = 0 there keeps
-    // every partial of such a pixel zero). s_dC: this lane's sub-block's row
-    // of BwdSmem::dC.
-    __device__ __forceinline__ void init(const Frame& f, int lane, int ix, int iy0, const float (&tf)[PX],
-                                         const float (&dc)[PX][3], float* s_dC) {
+    // ix, iy0: this lane's pixels (TileGeom::pixel); tf, bf, dc: the
+    // transmittance and b behind the span walked (the whole list's: t_final
+    // and bg . dL/dC) and dL/dC, zeros outside the image; inside: pixels past
+    // the image's edge have no position (NaN), so that nothing composites
+    // there. s_dC: this lane's sub-block's row of BwdSmem::dC.
+    __device__ __forceinline__ void init(int lane, int ix, int iy0, const bool (&inside)[PX], const float (&tf)[PX],
+                                         const float (&bf)[PX], const float (&dc)[PX][3], float* s_dC) {
         px = (float)ix + 0.5f;
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
             const float y = (float)(iy0 + 2 * p) + 0.5f;
-            py[p] = pack2(y, y + 1.f);
+            py[p] = pack2(inside[2 * p] ? y : NAN, inside[2 * p + 1] ? y + 1.f : NAN);
             T[p] = pack2(tf[2 * p], tf[2 * p + 1]);
 #pragma unroll
             for (int c = 0; c < 3; ++c) dC[p][c] = pack2(dc[2 * p][c], dc[2 * p + 1][c]);
-            b[p] = fma2(dup2(f.bg[2]), dC[p][2], fma2(dup2(f.bg[1]), dC[p][1], mul2(dup2(f.bg[0]), dC[p][0])));
+            b[p] = pack2(bf[2 * p], bf[2 * p + 1]);
             const int k = p * 4 + lane % G::LPS;  // pair of pixels: row pair * 4 + column
             *reinterpret_cast<float4*>(s_dC + 4 * k) =
                 make_float4(dc[2 * p][0], dc[2 * p + 1][0], dc[2 * p][1], dc[2 * p + 1][1]);
@@ -726,35 +726,6 @@ __device__ __forceinline__ uint32_t pair_slot(SlotBase slot_of, const uint2* __r
     return slot_of(g) + (ty - y0) * (x1 - x0 + 1) + (tx - x0);
 }
 
-// Block-wide maximum of the last-contributor counts (positions past it are
-// never composited; their records are zero).
-template <typename G, int PX>
-__device__ __forceinline__ uint32_t block_max_last(const uint32_t (&last)[PX], uint32_t* s_max, int warp, int lane) {
-    uint32_t my = 0;
-#pragma unroll
-    for (int k = 0; k < PX; ++k) my = max(my, last[k]);
-    for (int o = 16; o > 0; o >>= 1) my = max(my, __shfl_xor_sync(kFull, my, o));
-    if (lane == 0) s_max[warp] = my;
-    __syncthreads();
-    uint32_t m = 0;
-#pragma unroll
-    for (int w = 0; w < G::WARPS; ++w) m = max(m, s_max[w]);
-    return m;
-}
-
-// Zero records for list positions [from, len) that no pixel composited.
-template <typename SlotBase>
-__device__ __forceinline__ void zero_records(uint2 range, uint32_t from, const uint32_t* __restrict__ vals,
-                                             const uint2* __restrict__ rect, SlotBase slot_of, int tx, int ty,
-                                             int threads, const PairRecords& out) {
-    const uint32_t len = range.y - range.x;
-    for (uint32_t j = from + threadIdx.x; j < len; j += threads) {
-        const uint32_t slot = pair_slot(slot_of, rect, __ldg(vals + range.x + j), tx, ty);
-        out.p8[2 * (size_t)slot] = out.p8[2 * (size_t)slot + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
-        out.p9[slot] = 0.f;
-    }
-}
-
 // Slot-ordered sum of a Gaussian's nrec pair records (slots first ..) into
 // pr: the loads of four records are issued before their adds, and the adds
 // keep slot order (a record past nrec adds +0, which leaves a sum that
@@ -791,16 +762,17 @@ __device__ __forceinline__ void sum_pair_records(const float4* __restrict__ p8, 
 // Stages list positions [start, start + cnt) of a tile: records and masks,
 // and (WITH_SLOT) each pair's emission slot. The staging of the backward
 // (WITH_SLOT) builds the ellipse's sub-block
-// masks, the forward's the bounding box's. Returns whether the records that
-// this thread staged are finite (WITH_SLOT).
+// masks, the forward's the bounding box's. g0: vals[start + threadIdx.x], which
+// the caller has loaded. Returns whether the records that this thread staged
+// are finite (WITH_SLOT).
 template <typename G, bool WITH_SLOT, typename Splats, typename SlotBase>
 __device__ __forceinline__ bool stage_batch(const Frame& f, float ox, float oy, int tx, int ty, uint32_t start,
-                                            int cnt, const uint32_t* __restrict__ vals, const Splats& sp,
-                                            const uint2* __restrict__ rect, SlotBase slot_of, SplatRec* s_rec,
-                                            typename G::Mask* s_mask, uint32_t* s_slot) {
+                                            int cnt, uint32_t g0, const uint32_t* __restrict__ vals,
+                                            const Splats& sp, const uint2* __restrict__ rect, SlotBase slot_of,
+                                            SplatRec* s_rec, typename G::Mask* s_mask, uint32_t* s_slot) {
     bool finite = true;
     for (int j = threadIdx.x; j < cnt; j += G::THREADS) {
-        const uint32_t g = __ldg(vals + start + j);
+        const uint32_t g = j == (int)threadIdx.x ? g0 : __ldg(vals + start + j);
         typename G::Mask m;
         stage_splat<G, WITH_SLOT>(f, ox, oy, sp, g, s_rec + j, m);
         s_mask[j] = m;
@@ -815,6 +787,14 @@ __device__ __forceinline__ bool stage_batch(const Frame& f, float ox, float oy, 
         }
     }
     return finite;
+}
+
+// vals[start + threadIdx.x] for the threads that stage it of a batch of the list
+// [.., end), loaded a batch ahead: the records' addresses are then known when
+// their turn comes.
+template <typename G, int BATCH>
+__device__ __forceinline__ uint32_t first_value(const uint32_t* __restrict__ vals, uint32_t start, uint32_t end) {
+    return threadIdx.x < BATCH && start + threadIdx.x < end ? __ldg(vals + start + threadIdx.x) : 0u;
 }
 
 struct NoSlot {
@@ -841,10 +821,12 @@ __device__ __forceinline__ void blend_tile(const Frame& f, int tile, uint2 range
     init_null_splat(s_rec, BATCH);
     FwdPixels<G, PX> P;
     P.init(warp, lane);
+    uint32_t g0 = first_value<G, BATCH>(vals, range.x, range.y);
     for (uint32_t start = range.x; start < range.y; start += BATCH) {
         const int cnt = (int)min((uint32_t)BATCH, range.y - start);
         __syncthreads();
-        stage_batch<G, false>(f, ox, oy, tx, ty, start, cnt, vals, sp, nullptr, NoSlot{}, s_rec, s_mask, nullptr);
+        stage_batch<G, false>(f, ox, oy, tx, ty, start, cnt, g0, vals, sp, nullptr, NoSlot{}, s_rec, s_mask, nullptr);
+        g0 = first_value<G, BATCH>(vals, start + BATCH, range.y);
         __syncthreads();
         const int steps = build_lists<G, BATCH, false>(s_mask, 0, cnt, rows, warp, lane);
         P.walk(s_rec, rows + (lane / G::LPS) * list_row<BATCH>(), steps, start + 1 - range.x);
@@ -870,19 +852,140 @@ __device__ __forceinline__ void blend_tile(const Frame& f, int tile, uint2 range
     }
 }
 
-// Backward of one tile from the stored forward outputs: each pair's 9
-// partials at its emission slot (see BwdPixels). offsets[g]: the first
-// emission slot of Gaussian g's pairs (in a batch, of this view's). dL/dC is d_image, or in an L2
-// training step d_image - target with the image in d_image's place.
-// FINITE = true stops and returns false when a staged record or a dL/dC is
-// infinite or NaN.
+// dL/dC of this lane's pixels, zeros outside the image: d_image, or in an L2
+// training step d_image - target with the image in d_image's place. Returns
+// whether they are finite.
+template <int PX>
+__device__ __forceinline__ bool load_dc(const Frame& f, int gx, int gy0, const float* __restrict__ d_image,
+                                        const float* __restrict__ target, float (&dc)[PX][3]) {
+    bool finite = true;
+#pragma unroll
+    for (int k = 0; k < PX; ++k) {
+        const int gy = gy0 + k;
+        const bool inside = gx < f.W && gy < f.H;
+        const size_t pix = inside ? (size_t)gy * f.W + gx : 0;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const float g = inside ? d_image[3 * pix + c] : 0.f;
+            dc[k][c] = target && inside ? g - __ldg(target + 3 * pix + c) : g;
+            finite = finite && dc[k][c] * 0.f == 0.f;
+        }
+    }
+    return finite;
+}
+
+__device__ __forceinline__ float dot3(const float* a, const float (&d)[3]) {
+    return fmaf(a[2], d[2], fmaf(a[1], d[1], a[0] * d[0]));
+}
+
+// Long lists are cut into segments that the backward walks at the same time
+// (launch_tile_order): one tile of the 6-view step has 4,819 of its 1.9M
+// pairs, and its walk alone, about 100 ns a splat, took as long as all
+// others together. segment_state finds, for one segment, what the segments in
+// front of it have to know: its transmittance T (from 1 at its front) and its
+// colour D, composited from T = 1 and projected on dL/dC. Segment k then starts
+// from T = T_0 ... T_k and b = D_{k+1} + T_{k+1} (D_{k+2} + ... T_last bg . dL/dC):
+// sums of non-negative weights, nothing subtracted.
+template <int TS, int PX>
+__device__ __forceinline__ void segment_state(const Frame& f, int tile, uint32_t first, uint32_t last,
+                                              const uint32_t* __restrict__ vals, const float4* __restrict__ splats,
+                                              const float* __restrict__ d_image, const float* __restrict__ target,
+                                              float2* __restrict__ state) {
+    using G = TileGeom<TS, PX>;
+    constexpr int BATCH = fwd_batch<TS>();
+    constexpr int NP = PX / 2;
+    __shared__ SplatRec s_rec[BATCH + 1];
+    __shared__ typename G::Mask s_mask[BATCH];
+    __shared__ __align__(16) uint8_t s_list[G::NSB * list_row<BATCH>()];
+    const int tx = tile % f.TX, ty = tile / f.TX;
+    const float ox = (float)(tx * TS), oy = (float)(ty * TS);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint8_t* rows = s_list + warp * G::SPW * list_row<BATCH>();
+    const uint8_t* row = rows + (lane / G::LPS) * list_row<BATCH>();
+    const FloatSplats sp{splats};
+    init_null_splat(s_rec, BATCH);
+    int ix, iy0;
+    G::pixel(warp, lane, ix, iy0);
+    float dc[PX][3];
+    load_dc<PX>(f, tx * TS + ix, ty * TS + iy0, d_image, target, dc);
+    const float px = (float)ix + 0.5f;
+    F2 py[NP], T[NP];
+    float D[PX];
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+        const int gy = ty * TS + iy0 + 2 * p;  // (pixels past the image's edge have no position)
+        const float y = (float)(iy0 + 2 * p) + 0.5f;
+        const bool col_in = tx * TS + ix < f.W;
+        py[p] = pack2(col_in && gy < f.H ? y : NAN, col_in && gy + 1 < f.H ? y + 1.f : NAN);
+        T[p] = dup2(1.f);
+        D[2 * p] = D[2 * p + 1] = 0.f;
+    }
+    uint32_t g0 = first_value<G, BATCH>(vals, first, last);
+    for (uint32_t start = first; start < last; start += BATCH) {
+        const int cnt = (int)min((uint32_t)BATCH, last - start);
+        __syncthreads();
+        stage_batch<G, false>(f, ox, oy, tx, ty, start, cnt, g0, vals, sp, nullptr, NoSlot{}, s_rec, s_mask, nullptr);
+        g0 = first_value<G, BATCH>(vals, start + BATCH, last);
+        __syncthreads();
+        const int steps = build_lists<G, BATCH, false>(s_mask, 0, cnt, rows, warp, lane);
+        int j = row[0];
+#pragma unroll 4
+        for (int it = 0; it < steps; ++it) {
+            const SplatRec& r = s_rec[j];
+            j = row[it + 1];
+            const float4 geo = r.geo, col = r.col;
+            const float2 g2 = *reinterpret_cast<const float2*>(&r.geo2);
+            const float4 geo2 = make_float4(g2.x, g2.y, 0.f, 0.f);
+            const float dx = __fadd_rn(px, geo.x);
+#pragma unroll
+            for (int p = 0; p < NP; ++p) {
+                const F2 e2 = splat_log2_alpha2(dx, add2(py[p], dup2(geo.y)), geo, geo2);
+                float e[2], w[2];
+                unpack2(e2, e[0], e[1]);
+                F2 al = pack2(e[0] >= kLog2AlphaMin ? fminf(kAlphaMax, ex2_approx(e[0])) : 0.f,
+                              e[1] >= kLog2AlphaMin ? fminf(kAlphaMax, ex2_approx(e[1])) : 0.f);
+                al = mul2(al, T[p]);
+                T[p] = fma2(al, dup2(-1.f), T[p]);
+                unpack2(al, w[0], w[1]);
+                const float cc[3] = {col.x, col.y, col.z};
+#pragma unroll
+                for (int h = 0; h < 2; ++h)  // (an infinite colour stays with its pixels)
+                    if (e[h] >= kLog2AlphaMin) D[2 * p + h] = fmaf(w[h], dot3(cc, dc[2 * p + h]), D[2 * p + h]);
+            }
+        }
+    }
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+        float t0, t1;
+        unpack2(T[p], t0, t1);
+        state[(size_t)threadIdx.x * PX + 2 * p] = make_float2(t0, D[2 * p]);
+        state[(size_t)threadIdx.x * PX + 2 * p + 1] = make_float2(t1, D[2 * p + 1]);
+    }
+}
+
+// The part of a tile's list that a backward block walks: positions [lo, hi)
+// of the list; states (null for a whole list): the segment states of the
+// tile's nseg segments, of which this is number seg.
+struct BwdSpan {
+    uint32_t lo, hi;
+    const float2* states;
+    uint32_t seg, nseg;
+};
+
+// Backward of (a span of) one tile from the stored final transmittance: each
+// pair's 9 partials at its emission slot (see BwdPixels). offsets[g]: the first
+// emission slot of Gaussian g's pairs (in a batch, of this view's). d_image and
+// target: load_dc. FINITE = true stops and returns false when a staged record
+// or a dL/dC is infinite or NaN. (The positions past a tile's last composited
+// one are walked like the others: finding that position first, from n_contrib,
+// put a load and a barrier in front of the first batch's loads.)
 template <int TS, int PX, bool FINITE>
-__device__ __forceinline__ bool bwd_tile_body(const Frame& f, int tile, uint2 range, const uint32_t* __restrict__ vals,
-                                               const float4* __restrict__ splats, const uint2* __restrict__ rect,
-                                               const uint32_t* __restrict__ offsets, const float* __restrict__ t_final,
-                                               const uint32_t* __restrict__ n_contrib,
-                                               const float* __restrict__ d_image, const float* __restrict__ target,
-                                               const PairRecords& out, BwdSmem<TS, PX, bwd_batch<TS>()>& sm) {
+__device__ __forceinline__ bool bwd_tile_body(const Frame& f, int tile, uint32_t first, const BwdSpan& span,
+                                              const uint32_t* __restrict__ vals, const float4* __restrict__ splats,
+                                              const uint2* __restrict__ rect, const uint32_t* __restrict__ offsets,
+                                              const float* __restrict__ t_final, const float* __restrict__ d_image,
+                                              const float* __restrict__ target, const PairRecords& out,
+                                              BwdSmem<TS, PX, bwd_batch<TS>()>& sm) {
     using G = TileGeom<TS, PX>;
     constexpr int BATCH = bwd_batch<TS>();
     const int tx = tile % f.TX, ty = tile / f.TX;
@@ -890,60 +993,84 @@ __device__ __forceinline__ bool bwd_tile_body(const Frame& f, int tile, uint2 ra
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const FloatSplats sp{splats};
     const auto slot_of = [offsets](uint32_t g) { return __ldg(offsets + g); };
+    // the span as batches from its front, the last one taken first
+    const uint32_t begin = first + span.lo, len = span.hi - span.lo;
+    if (len == 0) return true;
+    uint32_t at = (len - 1) / BATCH * BATCH;
+    uint32_t g0 = first_value<G, BATCH>(vals, begin + at, begin + len);
     init_null_splat(sm.rec, BATCH);
     BwdPixels<TS, PX> B;
-    uint32_t last[PX];
-    bool dc_finite = true;
+    bool dc_finite;
     {
         int ix, iy0;
         G::pixel(warp, lane, ix, iy0);
-        float tf[PX], dc[PX][3];
-        const int gx = tx * TS + ix;
+        float tf[PX], bf[PX], dc[PX][3];
+        bool inside[PX];
+        const int gx = tx * TS + ix, gy0 = ty * TS + iy0;
+        dc_finite = load_dc<PX>(f, gx, gy0, d_image, target, dc);
 #pragma unroll
         for (int k = 0; k < PX; ++k) {
-            const int gy = ty * TS + iy0 + k;
-            const bool inside = gx < f.W && gy < f.H;
-            const size_t pix = inside ? (size_t)gy * f.W + gx : 0;
-            tf[k] = inside ? t_final[pix] : 0.f;
-            last[k] = inside ? n_contrib[pix] : 0u;
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                const float g = inside ? d_image[3 * pix + c] : 0.f;
-                dc[k][c] = target && inside ? g - __ldg(target + 3 * pix + c) : g;
-                dc_finite = dc_finite && dc[k][c] * 0.f == 0.f;
+            inside[k] = gx < f.W && gy0 + k < f.H;
+            tf[k] = inside[k] ? t_final[(size_t)(gy0 + k) * f.W + gx] : 0.f;
+            bf[k] = dot3(f.bg, dc[k]);
+            if (span.states) {
+                const float2* st = span.states + (size_t)threadIdx.x * PX + k;
+                for (uint32_t s = span.nseg - 1; s > span.seg; --s) {
+                    const float2 v = __ldg(st + (size_t)s * (TS * TS));
+                    bf[k] = fmaf(v.x, bf[k], v.y);
+                }
+                if (span.seg + 1 < span.nseg) {
+                    float t = inside[k] ? 1.f : 0.f;
+                    for (uint32_t s = 0; s <= span.seg; ++s) t *= __ldg(st + (size_t)s * (TS * TS)).x;
+                    tf[k] = t;
+                }
             }
         }
-        B.init(f, lane, ix, iy0, tf, dc, sm.dC[G::sub_block(warp, lane)]);
+        B.init(lane, ix, iy0, inside, tf, bf, dc, sm.dC[G::sub_block(warp, lane)]);
     }
-    const uint32_t max_last = block_max_last<G>(last, sm.maxl, warp, lane);
-    zero_records(range, max_last, vals, rect, slot_of, tx, ty, G::THREADS, out);
-    // batches of the composited prefix [0, max_last), last batch first
-    const int nb = (int)((max_last + BATCH - 1) / BATCH);
-    for (int b = nb - 1; b >= 0; --b) {
-        const uint32_t lo = (uint32_t)b * BATCH;
-        const int cnt = (int)min((uint32_t)BATCH, max_last - lo);
+    for (;;) {
+        const int cnt = (int)min((uint32_t)BATCH, len - at);
         __syncthreads();
-        const bool ok =
-            stage_batch<G, true>(f, ox, oy, tx, ty, range.x + lo, cnt, vals, sp, rect, slot_of, sm.rec, sm.mask, sm.slot);
+        const bool ok = stage_batch<G, true>(f, ox, oy, tx, ty, begin + at, cnt, g0, vals, sp, rect, slot_of, sm.rec,
+                                             sm.mask, sm.slot);
+        const bool more = at != 0;
+        at -= more ? BATCH : 0;
+        if (more) g0 = first_value<G, BATCH>(vals, begin + at, begin + at + BATCH);
         if (!__syncthreads_and(ok && dc_finite) && FINITE) return false;
         B.template batch<FINITE>(sm, cnt, warp, lane, out);
+        if (!more) return true;
     }
-    return true;
 }
 
-template <int TS, int PX>
-__device__ __forceinline__ void blend_bwd_tile(const Frame& f, int tile, uint2 range, const uint32_t* __restrict__ vals,
-                                               const float4* __restrict__ splats, const uint2* __restrict__ rect,
-                                               const uint32_t* __restrict__ offsets, const float* __restrict__ t_final,
-                                               const uint32_t* __restrict__ n_contrib,
-                                               const float* __restrict__ d_image, const float* __restrict__ target,
-                                               const PairRecords& out, BwdSmem<TS, PX, bwd_batch<TS>()>& sm) {
-    if (bwd_tile_body<TS, PX, true>(f, tile, range, vals, splats, rect, offsets, t_final, n_contrib, d_image, target,
-                                    out, sm))
-        return;
-    __syncthreads();
-    bwd_tile_body<TS, PX, false>(f, tile, range, vals, splats, rect, offsets, t_final, n_contrib, d_image, target, out,
-                                 sm);
+// Item i of a backward: i < split.max the i-th segment of the long lists, then
+// the tiles in the order given, those with long lists left out. first: where
+// the tile's list starts. Returns false for an item that does not exist.
+__device__ __forceinline__ bool bwd_item(const TileOrder& o, const uint2* __restrict__ ranges, uint32_t i, int npix,
+                                         uint32_t& tile, uint32_t& first, BwdSpan& span) {
+    span.states = nullptr;
+    span.seg = 0;
+    span.nseg = 1;
+    const uint32_t seg_len = o.max_split ? __ldg(o.head + 1) : ~0u;
+    if (i < o.max_split) {
+        if (i >= __ldg(o.head)) return false;
+        const uint2 it = __ldg(o.split + i);
+        tile = it.x & ((1u << kSplitTileBits) - 1u);
+        const uint2 range = ranges[tile];
+        const uint32_t len = range.y - range.x;
+        first = range.x;
+        span.seg = it.x >> kSplitTileBits;
+        span.nseg = (len + seg_len - 1) / seg_len;
+        span.lo = span.seg * seg_len;
+        span.hi = min(span.lo + seg_len, len);
+        span.states = o.states + (size_t)it.y * npix;
+        return true;
+    }
+    tile = o.order ? __ldg(o.order + (i - o.max_split)) : i - o.max_split;
+    const uint2 range = ranges[tile];
+    first = range.x;
+    span.lo = 0;
+    span.hi = range.y - range.x;
+    return span.hi <= seg_len;
 }
 
 }  // namespace ws

@@ -57,6 +57,20 @@ struct FrameTable {
     int views;
 };
 
+// What launch_tile_order leaves for a backward. order: the tiles, longest list
+// first (null: as numbered). Long lists in segments (max_split > 0): head[0]
+// segments in all, of head[1] list positions each; split[i]: segment i's tile
+// | number in the tile << kSplitTileBits, and the place of the tile's first
+// segment; states: tile-side^2 (T, D) per segment.
+constexpr int kSplitTileBits = 18;
+struct TileOrder {
+    const uint32_t* order;
+    const uint32_t* head;
+    const uint2* split;
+    float2* states;
+    uint32_t max_split;
+};
+
 // The view owning global tile t (binary search over tile_off).
 __device__ __forceinline__ int view_of_tile(const uint32_t* tile_off, int views, uint32_t t) {
     int lo = 0, hi = views - 1;

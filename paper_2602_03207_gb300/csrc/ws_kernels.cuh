@@ -102,19 +102,34 @@ cudaError_t launch_render_quads(int64_t n, const float* splats, const float* dep
 
 // ---- backward
 // Tile counts for which the tiles are ordered by list length: below, every
-// block is resident at once and the order does not matter; the scratch holds
-// kOrderMax of them.
-constexpr uint32_t kOrderMin = 1024, kOrderMax = 1u << 18;
+// block is resident at once and the order does not matter (unless lists are
+// split); the scratch holds kOrderMax of them.
+constexpr uint32_t kOrderMin = 1024, kOrderMax = 1u << kSplitTileBits;
+// Long lists are split into segments where the work pays for the launch that
+// prepares them and for the blocks kept for segments that do not exist (5 us
+// together: the 720p / 500k backward call, whose longest list of 914 needs no
+// split, takes 131 us without and 137 with them): from kSplitMinCapacity keys
+// on where tiles are few (kSplitMean keys of capacity a tile: 0.9M pairs on 288
+// tiles 916 -> 257 us), from kSplitAnyCapacity whatever their number (1.9M
+// pairs of 6 uneven views, longest list 4,819: 527 -> 456 us). A segment has
+// kSplitLeast positions or more (a multiple of every tile size's staging
+// batch); kSplitStateBytes hold the states of kSplitMost at 16-pixel tiles.
+constexpr int64_t kSplitMinCapacity = 1 << 20, kSplitAnyCapacity = 3 << 20, kSplitMean = 1000;
+constexpr uint32_t kSplitLeast = 576, kSplitUnit = 192;
+constexpr size_t kSplitStateBytes = size_t(8) << 20;
+constexpr uint32_t kSplitMost = 4096;
 size_t backward_scratch_bytes(int64_t key_capacity);
-// *order: the tiles, longest list first, in the backward's scratch; null
-// where the count is outside [kOrderMin, kOrderMax].
-cudaError_t launch_tile_order(const uint32_t* ranges, uint32_t ntiles, int64_t key_capacity, void* scratch,
-                              const uint32_t** order, cudaStream_t stream);
+// Orders the tiles (side: pixels) for the blends of a training step or a
+// backward in the backward's scratch; o is all null where the tile count is
+// outside [kOrderMin, kOrderMax] (kOrderMin does not apply where lists are
+// split).
+cudaError_t launch_tile_order(const uint32_t* ranges, uint32_t ntiles, int side, int64_t key_capacity, void* scratch,
+                              TileOrder* o, cudaStream_t stream);
 // target: null, or the L2 target with the image in d_image's place.
 cudaError_t launch_backward(int64_t n, const float* means, const float* log_scales, const float* quats,
                             const float* sh, const Frame& f, const float* splats, const uint16_t* rect,
                             const uint32_t* offsets, const uint32_t* tiles_touched,
-                            const uint32_t* vals, const uint32_t* ranges, const uint32_t* order, const float* t_final,
+                            const uint32_t* vals, const uint32_t* ranges, const TileOrder& order, const float* t_final,
                             const uint32_t* n_contrib, const float* d_image, const float* target, float* d_means,
                             float* d_log_scales, float* d_quats, float* d_logits, float* d_sh,
                             int64_t key_capacity, void* scratch, cudaStream_t stream);
@@ -129,7 +144,7 @@ cudaError_t launch_rasterize_batch(const uint32_t* num_keys, const uint64_t* key
 cudaError_t launch_backward_batch(int64_t n, const float* means, const float* log_scales, const float* quats,
                                   const float* sh, const FrameTable& ft, const float* splats, const uint16_t* rect,
                                   const uint32_t* offsets, const uint32_t* tiles_touched, const uint32_t* vals,
-                                  const uint32_t* ranges, const uint32_t* order, const float* t_final,
+                                  const uint32_t* ranges, const TileOrder& order, const float* t_final,
                                   const uint32_t* n_contrib, const float* d_image, const float* target, float* d_means,
                                   float* d_log_scales, float* d_quats, float* d_logits, float* d_sh,
                                   int64_t key_capacity, bool persistent, void* scratch, cudaStream_t stream);

@@ -102,7 +102,7 @@ class Renderer:
         self.keys_alt = torch.empty(cap, dtype=torch.int64, device=d)
         self.vals_alt = torch.empty(cap, dtype=torch.int32, device=d)
         self.num_keys = torch.zeros(4, dtype=torch.int32, device=d)
-        self.ranges = torch.empty((self.tx * self.ty, 2), dtype=torch.int32, device=d)
+        self.ranges = torch.zeros((self.tx * self.ty, 2), dtype=torch.int32, device=d)  # until a call finds them
         self.image = torch.empty((height, width, 3), dtype=torch.float32, device=d)
         self.t_final = torch.empty((height, width), dtype=torch.float32, device=d)
         self.n_contrib = torch.empty((height, width), dtype=torch.int32, device=d)

@@ -65,6 +65,28 @@ def test_tile_counts_around_the_ordering(tile, width, height):
     _check(_scene(800, 3, -3.5), cam, tile, 100_000)
 
 
+@pytest.mark.parametrize("tile", [8, 16, 32])
+@pytest.mark.parametrize("n", [576, 577, 1152, 1153, 2500])
+def test_long_lists_walked_in_segments(tile, n):
+    """Lists of about n (576 to a segment) with a key capacity from which the
+    backward splits them: against the oracle, and against the unsplit walk to
+    the rounding of a product and a sum per segment."""
+    import torch
+    from paper_2602_03207_gb300 import render
+    cam = _cam(tile + 5, tile)
+    scene = _scene(n, n, -2.2)
+    scene["opacity_logits"] -= 3.0  # faint, so that the last of them still show
+    _check(scene, cam, tile, 1 << 20)
+    dev = render.scene_to_device(scene)
+    target = torch.rand(cam["height"], cam["width"], 3, generator=torch.Generator().manual_seed(4)).cuda()
+    got = []
+    for capacity in (1 << 20, 64 * n):
+        r = render.Renderer(n, cam["width"], cam["height"], tile=tile, key_capacity=capacity)
+        got.append({k: v.clone() for k, v in r.train_step_l2(dev, cam, target).items()})
+    for k in got[0]:
+        assert torch.linalg.norm(got[0][k] - got[1][k]) <= 1e-5 * torch.linalg.norm(got[1][k]), k
+
+
 @pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan])
 def test_non_finite_gradient_stays_with_its_pixel(value):
     """dL/dimage infinite or NaN at one pixel: the splats composited there get
