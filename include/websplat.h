@@ -329,6 +329,26 @@ typedef struct ws_frame_buffers {
     int64_t key_capacity;
 } ws_frame_buffers;
 
+/* One frame, a training frame or a packed frame of a scene in device memory
+ * (buf's arrays) as one call: ws_preprocess, ws_cull, the sort (ws_sort_tiles
+ * where the segmented sort applies, else ws_sort) and ws_rasterize;
+ * ws_render_train_l2 in the rasterisation's place (target and gradients as
+ * there); or the packed variants with their records (buf->splats unused).
+ * *result (host): WS_FRAME_IN_ALT when the sorted pairs are in keys_alt /
+ * vals_alt, WS_FRAME_RANGES when the sort wrote the tile ranges (pass
+ * WS_CFG_RANGES_GIVEN to later calls on the same pairs). Everything is enqueued
+ * on `stream`; results, errors and the capacity flag are those of the calls
+ * made. The paper has no counterpart. */
+#define WS_FRAME_IN_ALT 1
+#define WS_FRAME_RANGES 2
+ws_status ws_render_frame(int64_t n, const ws_camera *cam, const ws_config *cfg, const ws_frame_buffers *buf,
+                          int32_t *result, void *stream);
+ws_status ws_render_frame_packed(int64_t n, const ws_camera *cam, const ws_config *cfg, const ws_frame_buffers *buf,
+                                 float *mean2d, uint32_t *axes, uint32_t *rgba, int32_t *result, void *stream);
+ws_status ws_train_frame_l2(int64_t n, const ws_camera *cam, const ws_config *cfg, const ws_frame_buffers *buf,
+                            const float *target, float *d_means, float *d_log_scales, float *d_quats,
+                            float *d_opacity_logits, float *d_sh, int32_t *result, void *stream);
+
 /* One frame from a scene in host memory to an image in host memory, all
  * enqueued on `stream`: the five scene arrays are copied host -> device into
  * buf (cudaMemcpyAsync), then ws_preprocess, ws_cull, the sort (ws_sort_tiles

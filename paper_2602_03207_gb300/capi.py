@@ -11,6 +11,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import struct
 import threading
 
 import torch
@@ -27,6 +28,7 @@ WS_CFG_SORT_SEGMENTED = 16
 WS_CFG_PERSISTENT = 32
 WS_CFG_RANGES_GIVEN = 64
 WS_CFG_BOX_MASKS = 128
+WS_FRAME_IN_ALT, WS_FRAME_RANGES = 1, 2  # *result of the whole-frame calls
 WS_ABI_VERSION = 2
 WS_SPLAT_FLOATS = 12  # floats per splat record: centre hi/lo (4), conic (3), sigma, colour (3), axis word
 
@@ -35,7 +37,8 @@ EXPORTS = ("ws_abi_version", "ws_status_string", "ws_workspace_bytes", "ws_prepr
            "ws_rasterize_backward", "ws_read_status", "ws_batch_max_views", "ws_batch_workspace_bytes",
            "ws_preprocess_batch", "ws_cull_batch", "ws_rasterize_batch", "ws_rasterize_backward_batch",
            "ws_image_residual", "ws_sort_test_stalled_tile", "ws_render_train_l2", "ws_render_train_l2_batch",
-           "ws_sort_tiles", "ws_render_frame_host", "ws_cull_sort_tiles")
+           "ws_sort_tiles", "ws_render_frame_host", "ws_cull_sort_tiles", "ws_render_frame",
+           "ws_render_frame_packed", "ws_train_frame_l2")
 
 
 class WsError(RuntimeError):
@@ -63,17 +66,23 @@ class Config(C.Structure):
                 ("guard", C.c_float), ("flags", C.c_uint32)]
 
 
+_CAMERA = struct.Struct("=16f2i4f")  # the fields of ws_camera, in order
+
+
 def camera(cam: dict) -> Camera:
-    c = Camera()
-    vm = [float(v) for row in cam["viewmat"] for v in row] if hasattr(cam["viewmat"][0], "__len__") \
-        else [float(v) for v in cam["viewmat"]]
-    for i in range(12):
-        c.viewmat[i] = vm[i]
-    c.fx, c.fy, c.cx, c.cy = cam["fx"], cam["fy"], cam["cx"], cam["cy"]
-    c.width, c.height, c.znear = int(cam["width"]), int(cam["height"]), cam["znear"]
-    for i in range(3):
-        c.bg[i] = cam["bg"][i]
-    return c
+    vm = cam["viewmat"]
+    if hasattr(vm, "tolist"):
+        vm = vm.tolist()
+    if hasattr(vm[0], "__len__"):
+        vm = [v for row in vm for v in row]
+    bg = cam["bg"]
+    try:
+        return Camera.from_buffer_copy(_CAMERA.pack(*vm[:12], cam["fx"], cam["fy"], cam["cx"], cam["cy"],
+                                                    int(cam["width"]), int(cam["height"]), cam["znear"],
+                                                    bg[0], bg[1], bg[2]))
+    except OverflowError:  # a value past float32: infinite, as a C conversion makes it
+        return Camera((C.c_float * 12)(*vm[:12]), cam["fx"], cam["fy"], cam["cx"], cam["cy"], int(cam["width"]),
+                      int(cam["height"]), cam["znear"], (C.c_float * 3)(bg[0], bg[1], bg[2]))
 
 
 def config(tile=16, digit_bits=8, dilation=0.3, guard=1.3, flags=0) -> Config:
@@ -117,6 +126,12 @@ def lib():
             L.ws_cull_sort_tiles.restype = I32
             L.ws_render_frame_host.argtypes = [I64, P, P, P, P, P, cam_p, cfg_p, C.POINTER(FrameBuffers), P, P]
             L.ws_render_frame_host.restype = I32
+            fb_p = C.POINTER(FrameBuffers)
+            L.ws_render_frame.argtypes = [I64, cam_p, cfg_p, fb_p, C.POINTER(I32), P]
+            L.ws_render_frame_packed.argtypes = [I64, cam_p, cfg_p, fb_p, P, P, P, C.POINTER(I32), P]
+            L.ws_train_frame_l2.argtypes = [I64, cam_p, cfg_p, fb_p, P, P, P, P, P, P, C.POINTER(I32), P]
+            for name in ("ws_render_frame", "ws_render_frame_packed", "ws_train_frame_l2"):
+                getattr(L, name).restype = I32
             L.ws_sort_noalloc.argtypes = [P, I64, I32, I32, P, P, P, P, I32, C.POINTER(I32), P]
             L.ws_sort_noalloc.restype = I32
             L.ws_sort_noalloc_max_keys.restype = I64
@@ -149,13 +164,20 @@ def _ptr(t):
     if t is None:
         return None
     if isinstance(t, torch.Tensor):
-        if t.numel() and not t.is_cuda:
+        if t.is_cuda:
+            return t.data_ptr() or None
+        if t.numel():
             raise ValueError("device tensor expected")
-        return t.data_ptr() if t.numel() else None
+        return None
     return int(t)
 
 
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream):
+    if stream is None and _raw_stream is not None:
+        return C.c_void_p(_raw_stream(torch.cuda.current_device()))
     s = stream if stream is not None else torch.cuda.current_stream()
     return C.c_void_p(s.cuda_stream)
 
@@ -363,6 +385,41 @@ def ws_render_train_l2_batch(n, means, log_scales, quats, sh, cams_arr, cfg, num
         _ptr(num_keys), _ptr(keys), _ptr(vals), _ptr(splats), _ptr(rect), _ptr(offsets), _ptr(tiles_touched),
         _ptr(target), int(key_capacity), _ptr(ranges), _ptr(image), _ptr(t_final), _ptr(n_contrib), _ptr(d_means),
         _ptr(d_log_scales), _ptr(d_quats), _ptr(d_opacity_logits), _ptr(d_sh), _ptr(workspace), _stream(stream)))
+
+
+_FRAME = struct.Struct("=%dQq" % (len(FrameBuffers._fields_) - 1))
+
+
+def frame_struct(tensors, key_capacity) -> FrameBuffers:
+    """ws_frame_buffers from device tensors in field order and key_capacity."""
+    return FrameBuffers.from_buffer_copy(_FRAME.pack(*[_ptr(t) or 0 for t in tensors], int(key_capacity)))
+
+
+def ws_render_frame(n, cam, cfg, buffers, stream=None) -> int:
+    """One frame of the scene in `buffers`; the WS_FRAME_* bits of its sort."""
+    result = C.c_int32(0)
+    _check("ws_render_frame", lib().ws_render_frame(int(n), C.byref(cam), C.byref(cfg), C.byref(buffers),
+                                                    C.byref(result), _stream(stream)))
+    return result.value
+
+
+def ws_render_frame_packed(n, cam, cfg, buffers, mean2d, axes, rgba, stream=None) -> int:
+    """ws_render_frame with the packed splat record."""
+    result = C.c_int32(0)
+    _check("ws_render_frame_packed", lib().ws_render_frame_packed(
+        int(n), C.byref(cam), C.byref(cfg), C.byref(buffers), _ptr(mean2d), _ptr(axes), _ptr(rgba), C.byref(result),
+        _stream(stream)))
+    return result.value
+
+
+def ws_train_frame_l2(n, cam, cfg, buffers, target, d_means, d_log_scales, d_quats, d_opacity_logits, d_sh,
+                      stream=None) -> int:
+    """One L2 training step of the scene in `buffers`; the WS_FRAME_* bits of its sort."""
+    result = C.c_int32(0)
+    _check("ws_train_frame_l2", lib().ws_train_frame_l2(
+        int(n), C.byref(cam), C.byref(cfg), C.byref(buffers), _ptr(target), _ptr(d_means), _ptr(d_log_scales),
+        _ptr(d_quats), _ptr(d_opacity_logits), _ptr(d_sh), C.byref(result), _stream(stream)))
+    return result.value
 
 
 def frame_buffers(**ptrs) -> FrameBuffers:

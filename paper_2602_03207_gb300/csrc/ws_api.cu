@@ -343,6 +343,81 @@ ws_status ws_rasterize(const uint32_t* num_keys, const uint64_t* keys, const uin
                                             image, t_final, n_contrib, static_cast<cudaStream_t>(stream)));
 }
 
+// ws_cull and the sort of a frame: ws_sort_tiles where the segmented sort
+// applies, else ws_sort (ws_cull_sort_tiles gives the same results and, on
+// GB300, no gain over the two calls).
+static ws_status cull_and_sort(int64_t n, const ws_camera* cam, const ws_config* cfg, const ws_frame_buffers* b,
+                               int32_t* result, void* stream) {
+    ws_status st = ws_cull(n, b->tiles_touched, b->rect, b->depth, cam, cfg, b->offsets, b->keys, b->vals,
+                           b->key_capacity, b->num_keys, b->workspace, stream);
+    if (st != WS_OK) return st;
+    const int64_t tiles =
+        (int64_t)((cam->width + cfg->tile - 1) / cfg->tile) * ((cam->height + cfg->tile - 1) / cfg->tile);
+    int end_bit = 31;
+    while ((int64_t(1) << (end_bit - 31)) < tiles) ++end_bit;
+    if (end_bit == 31) end_bit = 32;
+    int32_t in_alt = 0, given = 0;
+    st = WS_ERR_UNSUPPORTED;
+    if (cfg->flags & WS_CFG_SORT_SEGMENTED) {
+        st = ws_sort_tiles(b->num_keys, b->key_capacity, end_bit, b->keys, b->vals, b->keys_alt, b->vals_alt, cfg,
+                           b->workspace, b->ranges, tiles, &in_alt, stream);
+        if (st == WS_OK) given = WS_FRAME_RANGES;
+    }
+    if (st == WS_ERR_UNSUPPORTED)
+        st = ws_sort(b->num_keys, b->key_capacity, 0, end_bit, b->keys, b->vals, b->keys_alt, b->vals_alt, cfg,
+                     b->workspace, &in_alt, stream);
+    *result = (in_alt ? WS_FRAME_IN_ALT : 0) | given;
+    return st;
+}
+
+// The configuration of the calls after the sort.
+static ws_config sorted_config(ws_config cfg, int32_t result) {
+    if (result & WS_FRAME_RANGES) cfg.flags |= WS_CFG_RANGES_GIVEN;
+    return cfg;
+}
+
+ws_status ws_render_frame(int64_t n, const ws_camera* cam, const ws_config* cfg, const ws_frame_buffers* b,
+                          int32_t* result, void* stream) {
+    if (!b || !result || !valid_camera(cam) || !valid_config(cfg)) return WS_ERR_INVALID_ARG;
+    ws_status st = ws_preprocess(n, b->means, b->log_scales, b->quats, b->opacity_logits, b->sh, cam, cfg, b->splats,
+                                 b->depth, b->rect, b->tiles_touched, stream);
+    if (st == WS_OK) st = cull_and_sort(n, cam, cfg, b, result, stream);
+    if (st != WS_OK) return st;
+    const ws_config rc = sorted_config(*cfg, *result);
+    const bool alt = *result & WS_FRAME_IN_ALT;
+    return ws_rasterize(b->num_keys, alt ? b->keys_alt : b->keys, alt ? b->vals_alt : b->vals, b->splats, cam, &rc,
+                        b->ranges, b->image, b->t_final, b->n_contrib, stream);
+}
+
+ws_status ws_render_frame_packed(int64_t n, const ws_camera* cam, const ws_config* cfg, const ws_frame_buffers* b,
+                                 float* mean2d, uint32_t* axes, uint32_t* rgba, int32_t* result, void* stream) {
+    if (!b || !result || !valid_camera(cam) || !valid_config(cfg)) return WS_ERR_INVALID_ARG;
+    ws_status st = ws_preprocess_packed(n, b->means, b->log_scales, b->quats, b->opacity_logits, b->sh, cam, cfg,
+                                        mean2d, axes, rgba, b->depth, b->rect, b->tiles_touched, stream);
+    if (st == WS_OK) st = cull_and_sort(n, cam, cfg, b, result, stream);
+    if (st != WS_OK) return st;
+    const ws_config rc = sorted_config(*cfg, *result);
+    const bool alt = *result & WS_FRAME_IN_ALT;
+    return ws_rasterize_packed(b->num_keys, alt ? b->keys_alt : b->keys, alt ? b->vals_alt : b->vals, mean2d, axes,
+                               rgba, cam, &rc, b->ranges, b->image, b->t_final, b->n_contrib, stream);
+}
+
+ws_status ws_train_frame_l2(int64_t n, const ws_camera* cam, const ws_config* cfg, const ws_frame_buffers* b,
+                            const float* target, float* d_means, float* d_log_scales, float* d_quats,
+                            float* d_opacity_logits, float* d_sh, int32_t* result, void* stream) {
+    if (!b || !result || !valid_camera(cam) || !valid_config(cfg)) return WS_ERR_INVALID_ARG;
+    ws_status st = ws_preprocess(n, b->means, b->log_scales, b->quats, b->opacity_logits, b->sh, cam, cfg, b->splats,
+                                 b->depth, b->rect, b->tiles_touched, stream);
+    if (st == WS_OK) st = cull_and_sort(n, cam, cfg, b, result, stream);
+    if (st != WS_OK) return st;
+    const ws_config rc = sorted_config(*cfg, *result);
+    const bool alt = *result & WS_FRAME_IN_ALT;
+    return ws_render_train_l2(n, b->means, b->log_scales, b->quats, b->sh, cam, &rc, b->num_keys,
+                              alt ? b->keys_alt : b->keys, alt ? b->vals_alt : b->vals, b->splats, b->rect, b->offsets,
+                              b->tiles_touched, target, b->key_capacity, b->ranges, b->image, b->t_final, b->n_contrib,
+                              d_means, d_log_scales, d_quats, d_opacity_logits, d_sh, b->workspace, stream);
+}
+
 ws_status ws_render_frame_host(int64_t n, const float* h_means, const float* h_log_scales, const float* h_quats,
                                const float* h_opacity_logits, const float* h_sh, const ws_camera* cam,
                                const ws_config* cfg, const ws_frame_buffers* b, float* h_image, void* stream) {
@@ -363,32 +438,8 @@ ws_status ws_render_frame_host(int64_t n, const float* h_means, const float* h_l
             if (cudaMemcpyAsync(c.dst, c.src, c.bytes, cudaMemcpyHostToDevice, s) != cudaSuccess) return WS_ERR_CUDA;
         }
     }
-    ws_status st = ws_preprocess(n, b->means, b->log_scales, b->quats, b->opacity_logits, b->sh, cam, cfg,
-                                 b->splats, b->depth, b->rect, b->tiles_touched, stream);
-    if (st != WS_OK) return st;
-    const int64_t tiles = (int64_t)((cam->width + cfg->tile - 1) / cfg->tile) * ((cam->height + cfg->tile - 1) / cfg->tile);
-    int end_bit = 31;
-    while ((int64_t(1) << (end_bit - 31)) < tiles) ++end_bit;
-    if (end_bit == 31) end_bit = 32;
-    // ws_cull then the sort (ws_cull_sort_tiles gives the same results and,
-    // on GB300, no gain over the two calls)
-    st = ws_cull(n, b->tiles_touched, b->rect, b->depth, cam, cfg, b->offsets, b->keys, b->vals, b->key_capacity,
-                 b->num_keys, b->workspace, stream);
-    if (st != WS_OK) return st;
-    ws_config rc = *cfg;
-    int32_t in_alt = 0;
-    st = WS_ERR_UNSUPPORTED;
-    if (cfg->flags & WS_CFG_SORT_SEGMENTED) {
-        st = ws_sort_tiles(b->num_keys, b->key_capacity, end_bit, b->keys, b->vals, b->keys_alt, b->vals_alt, cfg,
-                           b->workspace, b->ranges, tiles, &in_alt, stream);
-        if (st == WS_OK) rc.flags |= WS_CFG_RANGES_GIVEN;
-    }
-    if (st == WS_ERR_UNSUPPORTED)
-        st = ws_sort(b->num_keys, b->key_capacity, 0, end_bit, b->keys, b->vals, b->keys_alt, b->vals_alt, cfg,
-                     b->workspace, &in_alt, stream);
-    if (st != WS_OK) return st;
-    st = ws_rasterize(b->num_keys, in_alt ? b->keys_alt : b->keys, in_alt ? b->vals_alt : b->vals, b->splats, cam,
-                      &rc, b->ranges, b->image, b->t_final, b->n_contrib, stream);
+    int32_t result = 0;
+    const ws_status st = ws_render_frame(n, cam, cfg, b, &result, stream);
     if (st != WS_OK) return st;
     const size_t img = (size_t)cam->width * cam->height * 3 * sizeof(float);
     return cuda_status(cudaMemcpyAsync(h_image, b->image, img, cudaMemcpyDeviceToHost, s));

@@ -211,10 +211,32 @@ class Renderer:
         cam = capi.camera(cam_dict)
         if cam.width != self.width or cam.height != self.height:
             raise ValueError("camera resolution differs from the renderer's")
-        self.preprocess(scene, cam, stream)
-        self._cull_and_sort(cam, stream)
-        self.rasterize(cam, stream)
+        if self.fused_cull:
+            self.preprocess(scene, cam, stream)
+            self._cull_and_sort(cam, stream)
+            self.rasterize(cam, stream)
+            return self.image
+        b = self._buffers(scene, cam)
+        if self.packed:
+            done = capi.ws_render_frame_packed(self.n, cam, self.cfg, b, self.mean2d_p, self.axes, self.rgba, stream)
+        else:
+            done = capi.ws_render_frame(self.n, cam, self.cfg, b, stream)
+        self._sorted(done)
         return self.image
+
+    def _buffers(self, scene, cam):
+        """ws_frame_buffers of this frame: the scene's arrays and the
+        renderer's, taken anew for each call."""
+        self._ensure_workspace(cam)
+        return capi.frame_struct((*[scene[k] for k in SCENE_KEYS], self.splats, self.depth, self.rect,
+                                  self.tiles_touched, self.offsets, self.keys, self.keys_alt, self.vals, self.vals_alt,
+                                  self.num_keys, self.ranges, self.image, self.t_final, self.n_contrib,
+                                  self.workspace), self.key_capacity)
+
+    def _sorted(self, done):
+        """Notes where a whole-frame call left its pairs and ranges."""
+        self.sorted_in_alt = bool(done & capi.WS_FRAME_IN_ALT)
+        self.raster_cfg = with_flags(self.cfg, capi.WS_CFG_RANGES_GIVEN) if done & capi.WS_FRAME_RANGES else self.cfg
 
     def forward_quads(self, scene, cam_dict, stream=None):
         """One frame through the paper's own design (ws_render_quads: global
@@ -271,9 +293,15 @@ class Renderer:
         if self.packed:
             raise ValueError("the packed-record variant renders only (no backward)")
         cam = capi.camera(cam_dict)
-        self.preprocess(scene, cam, stream)
-        self._cull_and_sort(cam, stream)
-        return self.train_pass_l2(scene, cam_dict, target, stream)
+        if self.fused_cull:
+            self.preprocess(scene, cam, stream)
+            self._cull_and_sort(cam, stream)
+            return self.train_pass_l2(scene, cam_dict, target, stream)
+        g = self._grads()
+        done = capi.ws_train_frame_l2(self.n, cam, self.cfg, self._buffers(scene, cam), target.contiguous(),
+                                      g["means"], g["log_scales"], g["quats"], g["opacity_logits"], g["sh"], stream)
+        self._sorted(done)
+        return {k: v[:self.n] for k, v in g.items()}
 
     def train_pass_l2(self, scene, cam_dict, target, stream=None):
         """The fused pass of train_step_l2 alone (ws_render_train_l2), on the
