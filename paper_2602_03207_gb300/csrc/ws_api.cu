@@ -355,7 +355,6 @@ static ws_status cull_and_sort(int64_t n, const ws_camera* cam, const ws_config*
         (int64_t)((cam->width + cfg->tile - 1) / cfg->tile) * ((cam->height + cfg->tile - 1) / cfg->tile);
     int end_bit = 31;
     while ((int64_t(1) << (end_bit - 31)) < tiles) ++end_bit;
-    if (end_bit == 31) end_bit = 32;
     int32_t in_alt = 0, given = 0;
     st = WS_ERR_UNSUPPORTED;
     if (cfg->flags & WS_CFG_SORT_SEGMENTED) {

@@ -134,3 +134,20 @@ def test_binding_constants_match_the_header():
             assert getattr(capi, name) == value, name
             checked += 1
     assert checked >= 5, sorted(defines)
+
+
+def test_whole_frame_calls_reject_bad_arguments(lib):
+    """ws_render_frame, its packed form and ws_train_frame_l2: no buffers, no
+    result, a bad camera or configuration, and null arrays."""
+    from paper_2602_03207_gb300 import capi
+    from paper_2602_03207_gb300 import synthetic as S
+    cam, cfg, buf, done = capi.camera(S.small_forward()[1]), capi.config(), capi.FrameBuffers(), C.c_int32(0)
+    bad = capi.camera(S.small_forward()[1])
+    bad.width = 0
+    calls = [(cam, cfg, None, C.byref(done)), (cam, cfg, C.byref(buf), None), (bad, cfg, C.byref(buf), C.byref(done)),
+             (cam, capi.config(tile=12), C.byref(buf), C.byref(done)), (cam, cfg, C.byref(buf), C.byref(done))]
+    for c, g, b, r in calls:
+        c, g = C.byref(c), C.byref(g)
+        assert lib.ws_render_frame(10, c, g, b, r, None) == capi.WS_ERR_INVALID_ARG
+        assert lib.ws_render_frame_packed(10, c, g, b, None, None, None, r, None) == capi.WS_ERR_INVALID_ARG
+        assert lib.ws_train_frame_l2(10, c, g, b, *[None] * 6, r, None) == capi.WS_ERR_INVALID_ARG

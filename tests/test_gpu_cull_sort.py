@@ -126,3 +126,33 @@ def test_fused_cull_sort_past_capacity_keeps_valid_pairs():
     r.rasterize(capi.camera(cam))
     torch.cuda.synchronize()
     assert np.isfinite(r.image.cpu().numpy()).all()
+
+
+@pytest.mark.parametrize("sort", ["segmented", "lsd", "lookback"])
+@pytest.mark.parametrize("size", [(16, 16), (100, 75)], ids=["one_tile", "ragged"])
+def test_whole_frame_calls_equal_staged_calls(sort, size):
+    """A frame, a packed frame and a training step as one call against the
+    stages called one by one: the same bits, and the same ranges and pairs
+    kept for later calls."""
+    import torch
+    from paper_2602_03207_gb300 import capi, render
+    scene, cam = S.small_forward()
+    cam = dict(cam, width=size[0], height=size[1])
+    dev = render.scene_to_device(scene)
+    n = len(scene["means"])
+    target = torch.rand(size[1], size[0], 3, device="cuda")
+    for packed in (False, True):
+        a, b = (render.Renderer(n, *size, key_capacity=64 * n, packed=packed, sort=sort) for _ in range(2))
+        c = capi.camera(cam)
+        a.preprocess(dev, c)
+        a.cull(c)
+        a.sort()
+        a.rasterize(c)
+        b.forward(dev, cam)
+        assert a.sorted_in_alt == b.sorted_in_alt and a.raster_cfg.flags == b.raster_cfg.flags
+        for name in ("image", "t_final", "n_contrib", "ranges"):
+            assert torch.equal(getattr(a, name), getattr(b, name)), name
+        if not packed:
+            ga = a.train_pass_l2(dev, cam, target)
+            gb = b.train_step_l2(dev, cam, target)
+            assert all(torch.equal(ga[k], gb[k]) for k in ga) and torch.equal(a.image, b.image)
