@@ -6,7 +6,8 @@
 // tiles_touched, computed wait-free in the spirit of §3.3.2's hierarchical
 // scan: level 0 reduces fixed chunks, level 1 scans the chunk sums in one
 // block, and level 0 again scans inside each chunk and adds its chunk
-// offset. Three dispatches, no block waits for another, no global atomics.
+// offset. Three dispatches, no block waits for another, no global atomics;
+// few chunks need only one or two (kSelfSum, kSelfScan).
 //
 // Emission is balanced over pairs rather than over Gaussians: a block owns a
 // chunk of Gaussians and the contiguous slot range their pairs occupy; its
@@ -61,6 +62,18 @@ k_chunk_sums(int64_t n, const uint32_t* __restrict__ touched, uint32_t* __restri
     }
 }
 
+// What a frame's `carry` pairs in all leave: the last offset, the clamped key
+// count and the capacity flag.
+__device__ __forceinline__ void store_totals(uint64_t carry, int64_t n, uint32_t* offsets, uint32_t* num_keys,
+                                             int64_t capacity, uint32_t* status) {
+    offsets[n] = sat32(carry);
+    const bool over = carry > (uint64_t)capacity;
+    *num_keys = over ? (uint32_t)capacity : (uint32_t)carry;
+    // This frame's status words: stored outright, so no clear is needed.
+    status[0] = over ? 1u : 0u;
+    status[1] = 0u;
+}
+
 // Level 1: exclusive scan of the chunk sums in one block (64-bit running
 // total, chunk offsets stored saturated); total pairs, the clamped key count
 // and the capacity flag.
@@ -98,14 +111,7 @@ k_chunk_scan(int64_t nchunks, int64_t n, uint32_t* __restrict__ sums, uint32_t* 
         carry += s_red[32];
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        offsets[n] = sat32(carry);
-        const bool over = carry > (uint64_t)capacity;
-        *num_keys = over ? (uint32_t)capacity : (uint32_t)carry;
-        // This frame's status words: stored outright, so no clear is needed.
-        status[0] = over ? 1u : 0u;
-        status[1] = 0u;
-    }
+    if (threadIdx.x == 0) store_totals(carry, n, offsets, num_keys, capacity, status);
 }
 
 // Shared memory of a chunk's emission: the chunk's local offsets, rects and
@@ -124,12 +130,11 @@ struct ChunkSmem {
 // and, when its slots fit in shared memory, the slot -> Gaussian map (every
 // Gaussian with tiles writes its index at its first slot and a block-wide
 // running maximum fills the rest: indices increase with slots). Returns the
-// chunk's pair count; *coff = its first slot.
+// chunk's pair count; coff: its first slot.
 __device__ __forceinline__ uint32_t chunk_prologue(ChunkSmem& S, int64_t n, const uint32_t* __restrict__ touched,
                                                    const uint2* __restrict__ rect, const float* __restrict__ depth,
-                                                   const uint32_t* __restrict__ chunk_off,
-                                                   uint32_t* __restrict__ offsets, int64_t base, int cnt,
-                                                   uint32_t* coff, bool* fast) {
+                                                   uint32_t coff, uint32_t* __restrict__ offsets, int64_t base,
+                                                   int cnt, bool* fast) {
     // Blocked arrangement: thread t owns Gaussians base + t*kScanItems .. + kScanItems - 1,
     // so a thread-serial prefix plus one block scan gives the local offsets.
     uint32_t v[kScanItems];
@@ -144,12 +149,11 @@ __device__ __forceinline__ uint32_t chunk_prologue(ChunkSmem& S, int64_t n, cons
     uint32_t ex = block_exclusive_scan<kScanThreads>(acc, S.red, &total);
     // A saturated chunk offset (2^32 - 1) puts every slot of the chunk past
     // the capacity; offsets are stored saturated likewise.
-    *coff = chunk_off[blockIdx.x];
 #pragma unroll
     for (int k = 0; k < kScanItems; ++k) {
         int li = threadIdx.x * kScanItems + k;
         S.off[li] = ex;
-        if (li < cnt) offsets[base + li] = sat32((uint64_t)*coff + ex);
+        if (li < cnt) offsets[base + li] = sat32((uint64_t)coff + ex);
         ex += v[k];
     }
     if (threadIdx.x == 0) S.off[kChunk] = total;
@@ -260,21 +264,66 @@ __device__ __forceinline__ uint64_t slot_pair(const ChunkSmem& S, uint32_t s, in
     return (tile << 31) | (uint64_t)(S.depth[lo] & 0x7fffffffu);
 }
 
+// Where a chunk's emission finds its first slot. kOffScanned: the scan of
+// the chunk sums (k_chunk_scan). The others save its launch, in which one
+// block works: kOffSums, up to kSelfScan chunks, adds the sums of the earlier
+// chunks itself (8 loads a thread at most), and kOffCounts, up to kSelfSum
+// chunks, the earlier Gaussians' counts, which saves the sums' launch too; the
+// last chunk's block then stores what k_chunk_scan would. Compaction with all
+// three launches / as chosen here: 10k splats 10.4 / 7.0 us, 500k 9.8 / 8.5,
+// 1M 14.2 / 13.1; at 1,758 chunks (six views of 300k) neither is ahead.
+enum { kOffScanned, kOffSums, kOffCounts };
+constexpr int64_t kSelfScan = 2048;
+constexpr int64_t kSelfSum = 16;
+
 // Level 0 down + emission: every pair of the chunk at its slot, in slot
 // order.
-template <bool BATCH>
+template <bool BATCH, int OFF>
 __global__ void __launch_bounds__(kScanThreads)
 k_emit(int64_t n, const uint32_t* __restrict__ touched, const uint2* __restrict__ rect,
        const float* __restrict__ depth, const uint32_t* __restrict__ chunk_off, int tiles_x,
        uint32_t* __restrict__ offsets, uint64_t* __restrict__ keys, uint32_t* __restrict__ vals,
-       int64_t capacity, uint32_t per_view, const ViewGrid grid) {
+       int64_t capacity, uint32_t per_view, const ViewGrid grid, uint32_t* __restrict__ num_keys,
+       uint32_t* __restrict__ status) {
     __shared__ ChunkSmem S;
+    __shared__ uint64_t s_before[kScanThreads / 32];
     pdl_wait();
     const int64_t base = (int64_t)blockIdx.x * kChunk;
     const int cnt = (int)((n - base) < kChunk ? (n - base) : kChunk);
-    uint32_t coff;
+    uint64_t before = 0;
+    if (OFF == kOffScanned) {
+        before = chunk_off[blockIdx.x];
+    } else {
+        const uint32_t* src = OFF == kOffSums ? chunk_off : touched;
+        const int64_t m = OFF == kOffSums ? (int64_t)blockIdx.x : base;
+#pragma unroll 4
+        for (int64_t i = threadIdx.x; i < m; i += kScanThreads) before += __ldg(src + i);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(kFull, before, o);
+        if ((threadIdx.x & 31) == 0) s_before[threadIdx.x >> 5] = before;
+        __syncthreads();
+        before = 0;
+#pragma unroll
+        for (int w = 0; w < kScanThreads / 32; ++w) before += s_before[w];
+    }
+    const uint32_t coff = sat32(before);
     bool fast;
-    const uint32_t total = chunk_prologue(S, n, touched, rect, depth, chunk_off, offsets, base, cnt, &coff, &fast);
+    const uint32_t total = chunk_prologue(S, n, touched, rect, depth, coff, offsets, base, cnt, &fast);
+    if (OFF != kOffScanned && blockIdx.x == gridDim.x - 1) {
+        // the chunk's own sum in 64 bits, as the sums' kernel takes it
+        uint64_t own = 0;
+        for (int li = threadIdx.x; li < cnt; li += kScanThreads) own += __ldg(touched + base + li);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) own += __shfl_xor_sync(kFull, own, o);
+        if ((threadIdx.x & 31) == 0) s_before[threadIdx.x >> 5] = own;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            uint64_t carry = before;
+#pragma unroll
+            for (int w = 0; w < kScanThreads / 32; ++w) carry += s_before[w];
+            store_totals(carry, n, offsets, num_keys, capacity, status);
+        }
+    }
     for (uint32_t s = threadIdx.x; s < total; s += kScanThreads) {
         const int64_t slot = (int64_t)coff + s;
         if (slot >= capacity) break;
@@ -463,9 +512,9 @@ k_emit_part(int64_t n, const uint32_t* __restrict__ touched, const uint2* __rest
             tex += tv[j];
         }
     }
-    uint32_t coff;
+    const uint32_t coff = chunk_off[blockIdx.x];
     bool fast;
-    const uint32_t total = chunk_prologue(S, n, touched, rect, depth, chunk_off, offsets, base, cnt, &coff, &fast);
+    const uint32_t total = chunk_prologue(S, n, touched, rect, depth, coff, offsets, base, cnt, &fast);
     if (over) {
         for (uint32_t s = threadIdx.x; s < total; s += kScanThreads) {
             const int64_t slot = (int64_t)coff + s;
@@ -620,55 +669,53 @@ size_t cull_scratch_bytes(int64_t n) {
     return (size_t)(nchunks > 0 ? nchunks : 1) * sizeof(uint32_t);
 }
 
+// Compaction of n items (one view's Gaussians, or every view's in a batch).
+template <bool BATCH>
+static cudaError_t compact(int64_t n, const uint32_t* touched, const uint16_t* rect, const float* depth, int tiles_x,
+                           uint32_t per_view, const ViewGrid& grid, uint32_t* offsets, uint64_t* keys, uint32_t* vals,
+                           int64_t key_capacity, uint32_t* num_keys, uint32_t* status, void* scratch,
+                           cudaStream_t stream) {
+    const int64_t nchunks = (n + kChunk - 1) / kChunk;
+    uint32_t* sums = static_cast<uint32_t*>(scratch);
+    cudaError_t e = cudaSuccess;
+    if (nchunks > kSelfSum) {
+        e = launch_pdl(k_chunk_sums, dim3((unsigned)nchunks), dim3(kScanThreads), 0, stream, n, touched, sums);
+        if (e != cudaSuccess) return e;
+    }
+    if (nchunks == 0 || nchunks > kSelfScan) {
+        e = launch_pdl(k_chunk_scan, dim3(1), dim3(kTopThreads), 0, stream, nchunks, n, sums, offsets, num_keys,
+                       key_capacity, status);
+        if (e != cudaSuccess || nchunks == 0) return e;
+    }
+    auto emit = [&](auto kernel) {
+        return launch_pdl(kernel, dim3((unsigned)nchunks), dim3(kScanThreads), 0, stream, n, touched,
+                          reinterpret_cast<const uint2*>(rect), depth, (const uint32_t*)sums, tiles_x, offsets, keys,
+                          vals, key_capacity, per_view, grid, num_keys, status);
+    };
+    if (nchunks <= kSelfSum) return emit(k_emit<BATCH, kOffCounts>);
+    if (nchunks <= kSelfScan) return emit(k_emit<BATCH, kOffSums>);
+    return emit(k_emit<BATCH, kOffScanned>);
+}
+
 cudaError_t launch_cull(int64_t n, const uint32_t* tiles_touched, const uint16_t* rect,
                         const float* depth, const Frame& f, uint32_t* offsets, uint64_t* keys,
                         uint32_t* vals, int64_t key_capacity, uint32_t* num_keys,
                         uint32_t* status, void* scratch, cudaStream_t stream) {
-    const int64_t nchunks = (n + kChunk - 1) / kChunk;
-    uint32_t* sums = static_cast<uint32_t*>(scratch);
-    cudaError_t e = cudaSuccess;
-    if (nchunks > 0) {
-        e = launch_pdl(k_chunk_sums, dim3((unsigned)nchunks), dim3(kScanThreads), 0, stream, n, tiles_touched, sums);
-        if (e != cudaSuccess) return e;
-    }
-    e = launch_pdl(k_chunk_scan, dim3(1), dim3(kTopThreads), 0, stream, (int64_t)nchunks, n, sums, offsets,
-                   num_keys, key_capacity, status);
-    if (e != cudaSuccess) return e;
-    if (nchunks > 0) {
-        ViewGrid g;
-        g.views = 1;
-        g.tiles_x[0] = (uint32_t)f.TX;
-        g.tile_off[0] = 0;
-        g.tile_off[1] = (uint32_t)(f.TX * f.TY);
-        e = launch_pdl(k_emit<false>, dim3((unsigned)nchunks), dim3(kScanThreads), 0, stream, n, tiles_touched,
-                       reinterpret_cast<const uint2*>(rect), depth, (const uint32_t*)sums, (int)f.TX, offsets,
-                       keys, vals, key_capacity, (uint32_t)(n > 0 ? n : 1), g);
-    }
-    return e;
+    ViewGrid g;
+    g.views = 1;
+    g.tiles_x[0] = (uint32_t)f.TX;
+    g.tile_off[0] = 0;
+    g.tile_off[1] = (uint32_t)(f.TX * f.TY);
+    return compact<false>(n, tiles_touched, rect, depth, (int)f.TX, (uint32_t)(n > 0 ? n : 1), g, offsets, keys, vals,
+                          key_capacity, num_keys, status, scratch, stream);
 }
 
 cudaError_t launch_cull_batch(int64_t n, const ViewGrid& grid, const uint32_t* tiles_touched,
                               const uint16_t* rect, const float* depth, uint32_t* offsets, uint64_t* keys,
                               uint32_t* vals, int64_t key_capacity, uint32_t* num_keys, uint32_t* status,
                               void* scratch, cudaStream_t stream) {
-    const int64_t items = n * grid.views;
-    const int64_t nchunks = (items + kChunk - 1) / kChunk;
-    uint32_t* sums = static_cast<uint32_t*>(scratch);
-    cudaError_t e = cudaSuccess;
-    if (nchunks > 0) {
-        e = launch_pdl(k_chunk_sums, dim3((unsigned)nchunks), dim3(kScanThreads), 0, stream, items, tiles_touched,
-                       sums);
-        if (e != cudaSuccess) return e;
-    }
-    e = launch_pdl(k_chunk_scan, dim3(1), dim3(kTopThreads), 0, stream, (int64_t)nchunks, items, sums, offsets,
-                   num_keys, key_capacity, status);
-    if (e != cudaSuccess) return e;
-    if (nchunks > 0) {
-        e = launch_pdl(k_emit<true>, dim3((unsigned)nchunks), dim3(kScanThreads), 0, stream, items, tiles_touched,
-                       reinterpret_cast<const uint2*>(rect), depth, (const uint32_t*)sums, 0, offsets, keys, vals,
-                       key_capacity, (uint32_t)n, grid);
-    }
-    return e;
+    return compact<true>(n * grid.views, tiles_touched, rect, depth, 0, (uint32_t)(n > 0 ? n : 1), grid, offsets, keys,
+                         vals, key_capacity, num_keys, status, scratch, stream);
 }
 
 }  // namespace ws

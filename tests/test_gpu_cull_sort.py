@@ -128,6 +128,46 @@ def test_fused_cull_sort_past_capacity_keeps_valid_pairs():
     assert np.isfinite(r.image.cpu().numpy()).all()
 
 
+@pytest.mark.parametrize("n", [1, 16 * 1024, 16 * 1024 + 1, 2048 * 1024, 2048 * 1024 + 1])
+@pytest.mark.parametrize("room", [1.0, 0.5])
+def test_offsets_at_the_edges_of_each_scan(n, room):
+    """Each way an emission finds its first slot (the counts, the chunk sums or
+    their scan) on both sides of its limit: offsets, count, flag and pairs
+    against a cumulative sum, also where half of the pairs fit."""
+    import torch
+    from paper_2602_03207_gb300 import capi
+    rng = np.random.default_rng(n)
+    wide = rng.integers(0, 4, n)  # tiles of a one-row rectangle; 0 culls
+    rect = np.zeros((n, 4), np.uint16)
+    rect[:, 0] = rng.integers(0, 12, n)
+    rect[:, 1] = rect[:, 3] = rng.integers(0, 16, n)
+    rect[:, 2] = rect[:, 0] + np.maximum(wide, 1) - 1
+    depth = rng.uniform(1.0, 9.0, n).astype(np.float32)
+    total = int(wide.sum())
+    cap = max(1, int(total * room))
+    cam = capi.camera(dict(S.small_forward()[1], width=256, height=256))
+    cfg = capi.config()
+    dev = lambda a: torch.from_numpy(a).cuda()
+    offsets = torch.zeros(n + 4, dtype=torch.int32, device="cuda")
+    keys = torch.zeros(cap + 2, dtype=torch.int64, device="cuda")
+    vals = torch.zeros(cap + 4, dtype=torch.int32, device="cuda")
+    num = torch.zeros(4, dtype=torch.int32, device="cuda")
+    work = torch.zeros(capi.ws_workspace_bytes(n, cap, cam, cfg), dtype=torch.uint8, device="cuda")
+    capi.ws_cull(n, dev(wide.astype(np.int32)), dev(rect.view(np.int16)), dev(depth), cam, cfg, offsets, keys, vals,
+                 cap, num, work)
+    first = np.concatenate([[0], np.cumsum(wide)])
+    np.testing.assert_array_equal(offsets[:n + 1].cpu().numpy(), first)
+    kept = min(cap, total)
+    assert int(num[0]) == kept
+    assert capi.ws_read_status(work) == int(total > cap)
+    gid = np.repeat(np.arange(n), wide)[:kept]
+    tile = rect[gid, 1].astype(np.uint64) * 16 + rect[gid, 0] + (np.arange(kept) - first[gid]).astype(np.uint64)
+    np.testing.assert_array_equal(vals[:kept].cpu().numpy(), gid)
+    np.testing.assert_array_equal(keys[:kept].cpu().numpy().view(np.uint64),
+                                  (tile << np.uint64(31)) | depth[gid].view(np.uint32).astype(np.uint64))
+    assert not keys[kept:].any() and not vals[kept:].any()
+
+
 @pytest.mark.parametrize("sort", ["segmented", "lsd", "lookback"])
 @pytest.mark.parametrize("size", [(16, 16), (100, 75)], ids=["one_tile", "ragged"])
 def test_whole_frame_calls_equal_staged_calls(sort, size):
