@@ -9,26 +9,30 @@
 //   2. bounds:    start[s] = first position whose segment id is >= s, for
 //      every s in [0, 2^(end_bit - 31)], by searches of the partitioned keys.
 //   3. local:     every segment is sorted by its sub-key bits [begin_bit, 31)
-//      on chip, as 32-bit words: the sub-key's distance from the segment's
-//      smallest, cut to the leading bits that fit, above the position in the
-//      segment. The words are distinct and positions break ties, so equal
-//      sub-keys keep their input order; where bits were cut off, a check of
+//      on chip, positions breaking ties, so equal sub-keys keep their input
+//      order: a warp sorts one of at most 256 or 512 keys (alone_cap) with a
+//      bitonic network in registers, a block one of at most 2,048 (256 threads) or
+//      16,384 (1,024 threads) through buckets in shared memory or, where the
+//      sub-keys crowd together, with three 7-bit counting passes, and one of
+//      more keys with chunked 8-bit passes over global memory, ranked with warp
+//      ballots, skipping a pass whose digit is the same for every key. The
+//      network and the 7-bit passes sort 32-bit words: the sub-key's distance
+//      from the segment's smallest, cut to the leading bits that fit, above
+//      the position in the segment; where bits were cut off, a check of
 //      neighbours by the whole sub-key puts right what they would have
-//      decided (fix_order). A warp sorts a segment of at most 512 keys with a
-//      bitonic network in registers, a block one of at most 2,048 (256 threads)
-//      or 8,192 (1,024 threads) with three 7-bit counting passes in shared memory, and one of more
-//      keys with chunked 8-bit passes over global memory, ranked with warp
-//      ballots, skipping a pass whose digit is the same for every key.
+//      decided (fix_order).
 // A stable partition by the high bits followed by a stable sort of each
 // segment by the low bits orders the pairs exactly as the full-key LSD
 // sort does, ties included. There are no global atomics and no block waits
 // on another: each segment belongs to one block.
 //
-// The local sorts are bound by instruction issue: 64-bit words (the whole
+// The local sorts are bound by instruction issue where segments fill the chip
+// and by a segment's chain of dependent steps where they do not. 64-bit words (the whole
 // sub-key above the position) took the network two shuffles, a two-part
 // comparison and two selects an element and stage against a shuffle and a
-// minimum or maximum, and a block's passes four rounds of 12-byte pairs against
-// three of 4-byte words.
+// minimum or maximum.
+#include <atomic>
+
 #include "ws_common.cuh"
 #include "ws_kernels.cuh"
 
@@ -36,16 +40,17 @@ namespace ws {
 
 namespace {
 
-constexpr int kSegThreads = 256;      // a block of segments, or of one segment of at most 2,048 keys
+constexpr int kSegThreads = 256;      // a block of a warp's segments, or of one segment of at most 2,048 keys
 constexpr int kHugeThreads = 1024;     // a block of one larger segment
 constexpr int kSegWarps = kSegThreads / kWarp;
-constexpr int kSegItems = 8;
 constexpr int kWarpItems = 16;
 constexpr int kWarpCap = kWarp * kWarpItems;      // keys a warp sorts alone
 // keys that a block of THREADS sorts in shared memory, or takes at a time of a
 // larger segment
 template <int THREADS>
-__host__ __device__ constexpr int block_cap() { return THREADS * kSegItems; }
+__host__ __device__ constexpr int seg_items() { return THREADS == 1024 ? 16 : 8; }
+template <int THREADS>
+__host__ __device__ constexpr int block_cap() { return THREADS * seg_items<THREADS>(); }
 constexpr int kLocalBits = 8;
 constexpr int kLocalRadix = 1 << kLocalBits;
 constexpr int kSplitBit = 31;                     // segment id above, sub-key below
@@ -111,6 +116,7 @@ __device__ __forceinline__ uint32_t warp_or(uint32_t v) {
 
 // Rank items k < kn of this warp (input order k*32 + lane) among equal
 // digits: rnk = earlier equal digits of the warp; cnt[d] += the warp's count.
+template <int kSegItems>
 __device__ __forceinline__ void warp_rank(const uint64_t (&key)[kSegItems], int kn, int valid_base, int n,
                                           int shift, uint32_t mask, uint32_t* cnt, uint32_t (&rnk)[kSegItems]) {
     const int lane = threadIdx.x & 31;
@@ -262,6 +268,190 @@ __device__ __forceinline__ void warp_sort(const uint64_t* kin, const uint32_t* v
     }
 }
 
+// The block sorts n <= K THREADS pairs through 8 THREADS buckets in shared
+// memory: the sub-keys' range is split over the buckets, the keys stand
+// grouped by bucket after one counting pass, and each finds its place among
+// its bucket's few by comparing with them. About 50 instructions a key and a
+// dozen barriers, where the counting passes take three rounds of ballots and
+// two scans each. Comparisons are of whole sub-keys, then positions, so the
+// result is the stable order whatever order the counting's atomic additions
+// ran in. The buckets are split evenly over three intervals (see bucket_of):
+// split over the whole range alone, a few far splats left most keys of a
+// clustered scene in few buckets. Returns false, with nothing written, when a bucket
+// holds more than kBucketMost keys (sub-keys that crowd together all the same, or are
+// equal): the caller then sorts by the counting passes, whose work does not
+// depend on the distribution. 64 of them: a 417 x 473 frame of dense tiles took 65.0 us
+// for compaction and sort, 67.1 with 32, 74 with 16.
+// smem: 8 K THREADS + 16 bytes. The sorted pairs are staged there and leave in
+// full sectors; they are read a second time in input order, where gathering them in
+// sorted order read a sector for each key and each value.
+// Compaction and sort, us, by the counting passes and with blocks of up to 8,192 keys /
+// by buckets and up to 16,384: 64 views / 2M 7,460 / 6,473; 2160p / 6M 415 / 383; 288
+// tiles of 2,987 keys on average 157 / 79; the sort of 4M pairs in 8,192 segments
+// 192 / 175. The same buckets for a warp's segments lost to the network (1080p /
+// 1M 82 against 69 us): 16 keys a lane in turn through shared memory is the
+// longer chain.
+constexpr uint32_t kBucketMost = 64;
+
+__device__ __forceinline__ float warp_sum(float v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+    return v;
+}
+
+template <int THREADS, int K>
+__host__ __device__ constexpr int bucket_smem() { return 8 * K * THREADS + 16; }
+
+template <int THREADS, int K>
+__device__ __forceinline__ bool bucket_sort(const uint64_t* kin, const uint32_t* vin, uint64_t* kout, uint32_t* vout,
+                                            uint32_t b, int n, int begin_bit, unsigned char* smem, uint32_t* red) {
+    constexpr int kBuckets = 8 * THREADS;
+    constexpr int kOwn = kBuckets / THREADS;  // buckets a thread owns
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    uint32_t* s_word = reinterpret_cast<uint32_t*>(smem);             // sub-keys, grouped by bucket
+    uint16_t* s_idx = reinterpret_cast<uint16_t*>(s_word + K * THREADS);  // and their positions
+    uint16_t* s_start = s_idx + K * THREADS;  // counts, then first places; the last one is n
+    uint32_t* s_pair = reinterpret_cast<uint32_t*>(s_start);
+    const uint32_t sub_mask = (1u << (kSplitBit - begin_bit)) - 1u;
+    uint32_t v[K], at[K];
+    uint32_t least = ~0u, most = 0u;
+    float total = 0.0f;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int idx = k * THREADS + t;
+        v[k] = idx < n ? sub_key(__ldg(kin + b + idx), begin_bit, sub_mask) : 0u;
+        if (idx < n) {
+            least = min(least, v[k]);
+            most = max(most, v[k]);
+            total += (float)v[k];
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < kOwn / 2; ++k) s_pair[k * THREADS + t] = 0u;
+    least = __reduce_min_sync(kFull, least);
+    most = __reduce_max_sync(kFull, most);
+    total = warp_sum(total);
+    if (lane == 0) {
+        red[3 * warp] = least;
+        red[3 * warp + 1] = most;
+        red[3 * warp + 2] = __float_as_uint(total);
+    }
+    __syncthreads();
+    total = 0.0f;
+#pragma unroll
+    for (int w = 0; w < THREADS / kWarp; ++w) {
+        least = min(least, red[3 * w]);
+        most = max(most, red[3 * w + 1]);
+        total += __uint_as_float(red[3 * w + 2]);
+    }
+    const float mean = total / (float)n;
+    float dev = 0.0f;
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+        if (k * THREADS + t < n) dev += fabsf((float)v[k] - mean);
+    dev = warp_sum(dev);
+    constexpr int kDevs = 3 * (THREADS / kWarp);
+    if (lane == 0) red[kDevs + warp] = __float_as_uint(dev);
+    __syncthreads();
+    dev = 0.0f;
+#pragma unroll
+    for (int w = 0; w < THREADS / kWarp; ++w) dev += __uint_as_float(red[kDevs + w]);
+    dev = dev / (float)n + 1.0f;
+    // 1/2 of the buckets for mean +- 2 dev, 1/4 for +- 5 dev, 1/4 for the whole
+    // range. Every step is monotone under rounding, so the order of sub-keys is
+    // kept, which is all the buckets need.
+    const float a1 = 0.25f / dev, a2 = 0.1f / dev, a3 = 1.0f / ((float)(most - least) + 1.0f);
+    const float o1 = 0.5f - mean * a1, o2 = 0.5f - mean * a2, o3 = -(float)least * a3;
+    auto bucket_of = [&](uint32_t x) {
+        const float f = (float)x;
+        float u = 0.25f * __saturatef(fmaf(f, a3, o3));
+        u = fmaf(0.25f, __saturatef(fmaf(f, a2, o2)), u);
+        u = fmaf(0.5f, __saturatef(fmaf(f, a1, o1)), u);
+        return min((uint32_t)kBuckets - 1u, (uint32_t)(u * (float)kBuckets));
+    };
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        at[k] = 0u;
+        if (k * THREADS + t < n) {
+            const uint32_t bk = bucket_of(v[k]);
+            const uint32_t half = (bk & 1u) * 16u;
+            at[k] = bk | ((atomicAdd(s_pair + (bk >> 1), 1u << half) >> half) << 16);
+        }
+    }
+    __syncthreads();
+    // counts -> first places: thread t owns kOwn in a row
+    uint32_t c[kOwn / 2];
+    uint32_t sum = 0u, crowd = 0u;
+#pragma unroll
+    for (int k = 0; k < kOwn / 2; ++k) {
+        c[k] = s_pair[t * (kOwn / 2) + k];
+        sum += (c[k] & 0xffffu) + (c[k] >> 16);
+        crowd = max(crowd, max(c[k] & 0xffffu, c[k] >> 16));
+    }
+    if (__syncthreads_or(crowd > kBucketMost)) return false;
+    uint32_t all;
+    uint32_t first = block_exclusive_scan<THREADS>(sum, red, &all);
+#pragma unroll
+    for (int k = 0; k < kOwn / 2; ++k) {
+        const uint32_t second = first + (c[k] & 0xffffu);
+        s_pair[t * (kOwn / 2) + k] = first | (second << 16);
+        first = second + (c[k] >> 16);
+    }
+    if (t == 0) s_start[kBuckets] = (uint16_t)n;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int idx = k * THREADS + t;
+        if (idx < n) {
+            const uint32_t p = s_start[at[k] & 0xffffu] + (at[k] >> 16);
+            s_word[p] = v[k];
+            s_idx[p] = (uint16_t)idx;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int idx = k * THREADS + t;
+        if (idx < n) {
+            const uint32_t bk = at[k] & 0xffffu;
+            const uint32_t p0 = s_start[bk], p1 = s_start[bk + 1], own = p0 + (at[k] >> 16);
+            uint32_t rank = p0;
+            for (uint32_t p = p0; p < p1; ++p) {
+                const uint32_t w = s_word[p];
+                if (w < v[k]) ++rank;
+                if (w == v[k] && p != own && s_idx[p] < (uint16_t)idx) ++rank;
+            }
+            at[k] = rank;
+        }
+    }
+    __syncthreads();
+    uint64_t* s_key = reinterpret_cast<uint64_t*>(smem);
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int idx = k * THREADS + t;
+        if (idx < n) s_key[at[k]] = __ldg(kin + b + idx);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int idx = k * THREADS + t;
+        if (idx < n) kout[b + idx] = s_key[idx];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int idx = k * THREADS + t;
+        if (idx < n) s_word[at[k]] = __ldg(vin + b + idx);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int idx = k * THREADS + t;
+        if (idx < n) vout[b + idx] = s_word[idx];
+    }
+    return true;
+}
+
 // Block-wide AND / OR of one value per thread.
 template <int THREADS>
 __device__ __forceinline__ uint32_t block_varying(uint32_t a, uint32_t o, uint32_t* red) {
@@ -283,8 +473,8 @@ __device__ __forceinline__ uint32_t block_varying(uint32_t a, uint32_t o, uint32
     return ra ^ ro;
 }
 
-// The block sorts n <= 8 THREADS pairs by their sort words (log2 of that many
-// bits of position, 21 or 19 of sub-key) with three stable 7-bit LSD passes
+// The block sorts n <= block_cap pairs by their sort words (11 or 14 bits of
+// position, 21 or 18 of sub-key) with three stable 7-bit LSD passes
 // over the sub-key's part; with kn = ceil(n / THREADS), element w*32*kn + k*32
 // + lane lives in lane `lane` of warp w, item k. s_word: a word per key
 // (reused for the list of positions); s_cnt: THREADS / 32 rows of 128
@@ -296,8 +486,9 @@ template <int THREADS>
 __device__ __forceinline__ void block_sort_smem(const uint64_t* kin, const uint32_t* vin, uint64_t* kout,
                                                 uint32_t* vout, uint32_t b, int n, int begin_bit, uint32_t* s_word,
                                                 uint16_t* s_cnt, uint32_t* red) {
+    constexpr int kSegItems = seg_items<THREADS>();
     constexpr int kCap = block_cap<THREADS>();
-    constexpr int kIdxBits = THREADS == 1024 ? 13 : 11;
+    constexpr int kIdxBits = THREADS == 1024 ? 14 : 11;
     static_assert((1 << kIdxBits) == kCap && kIdxBits + 3 * kCtaDigit >= 32, "position bits and passes");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // every warp takes kn consecutive runs of 32 (input order = warp, item, lane)
@@ -423,11 +614,13 @@ template <int THREADS>
 __device__ void block_sort_global(uint64_t* kin, uint32_t* vin, uint64_t* kout, uint32_t* vout, uint32_t b,
                                   uint32_t n, int begin_bit, uint32_t (*cnt)[kLocalRadix], uint32_t* off,
                                   uint32_t* red) {
+    constexpr int kSegItems = 8;
+    constexpr uint32_t kStep = THREADS * kSegItems;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int wbase = warp * kWarp * kSegItems;
     const uint32_t sub_mask = (1u << (kSplitBit - begin_bit)) - 1u;
     uint32_t all_and = ~0u, all_or = 0u;
-    for (uint32_t c0 = 0; c0 < n; c0 += block_cap<THREADS>()) {
+    for (uint32_t c0 = 0; c0 < n; c0 += kStep) {
 #pragma unroll
         for (int k = 0; k < kSegItems; ++k) {
             const uint32_t idx = c0 + wbase + k * kWarp + lane;
@@ -451,8 +644,8 @@ __device__ void block_sort_global(uint64_t* kin, uint32_t* vin, uint64_t* kout, 
         // digit totals of the segment -> running offsets
         for (int i = threadIdx.x; i < (THREADS / kWarp) * kLocalRadix; i += THREADS) (&cnt[0][0])[i] = 0u;
         __syncthreads();
-        for (uint32_t c0 = 0; c0 < n; c0 += block_cap<THREADS>()) {
-            const int rem = (int)(n - c0 < (uint32_t)block_cap<THREADS>() ? n - c0 : (uint32_t)block_cap<THREADS>());
+        for (uint32_t c0 = 0; c0 < n; c0 += kStep) {
+            const int rem = (int)min(n - c0, kStep);
             uint64_t key[kSegItems];
             const int kn = rem > wbase ? ((rem - wbase + kWarp - 1) / kWarp < kSegItems
                                               ? (rem - wbase + kWarp - 1) / kWarp
@@ -479,8 +672,8 @@ __device__ void block_sort_global(uint64_t* kin, uint32_t* vin, uint64_t* kout, 
             if (d < kLocalRadix) off[d] = t;
         }
         __syncthreads();
-        for (uint32_t c0 = 0; c0 < n; c0 += block_cap<THREADS>()) {
-            const int rem = (int)(n - c0 < (uint32_t)block_cap<THREADS>() ? n - c0 : (uint32_t)block_cap<THREADS>());
+        for (uint32_t c0 = 0; c0 < n; c0 += kStep) {
+            const int rem = (int)min(n - c0, kStep);
             const int kn = rem > wbase ? ((rem - wbase + kWarp - 1) / kWarp < kSegItems
                                               ? (rem - wbase + kWarp - 1) / kWarp
                                               : kSegItems)
@@ -545,7 +738,9 @@ struct SegSmem {
     static constexpr int kWordBytes = block_cap<THREADS>() * 4;
     static constexpr int kBytes = kWordBytes + (THREADS / kWarp) * kCtaRadix * 2;
     static constexpr int kGlobalBytes = (THREADS / kWarp) * kLocalRadix * 4;
-    static constexpr int kRaw = kBytes > kGlobalBytes ? kBytes : kGlobalBytes;
+    static constexpr int kPassBytes = kBytes > kGlobalBytes ? kBytes : kGlobalBytes;
+    static constexpr int kBucketBytes = bucket_smem<THREADS, seg_items<THREADS>()>();
+    static constexpr int kRaw = kPassBytes > kBucketBytes ? kPassBytes : kBucketBytes;
 };
 
 // The block sorts one segment [b, b + n).
@@ -553,12 +748,22 @@ template <int THREADS>
 __device__ __forceinline__ void block_sort(uint64_t* kin, uint32_t* vin, uint64_t* kout, uint32_t* vout, uint32_t b,
                                            uint32_t n, int begin_bit, unsigned char* raw, uint32_t* off,
                                            uint32_t* red) {
-    if (n <= (uint32_t)block_cap<THREADS>())
+    if (n <= (uint32_t)block_cap<THREADS>()) {
+        bool done;
+        if (n <= 4 * THREADS)
+            done = bucket_sort<THREADS, 4>(kin, vin, kout, vout, b, (int)n, begin_bit, raw, red);
+        else if (seg_items<THREADS>() == 8 || n <= 8 * THREADS)
+            done = bucket_sort<THREADS, 8>(kin, vin, kout, vout, b, (int)n, begin_bit, raw, red);
+        else
+            done = bucket_sort<THREADS, seg_items<THREADS>()>(kin, vin, kout, vout, b, (int)n, begin_bit, raw, red);
+        if (done) return;
+        __syncthreads();  // every thread is done with the shared memory
         block_sort_smem<THREADS>(kin, vin, kout, vout, b, (int)n, begin_bit, reinterpret_cast<uint32_t*>(raw),
                                  reinterpret_cast<uint16_t*>(raw + SegSmem<THREADS>::kWordBytes), red);
-    else
+    } else {
         block_sort_global<THREADS>(kin, vin, kout, vout, b, n, begin_bit,
                                    reinterpret_cast<uint32_t (*)[kLocalRadix]>(raw), off, red);
+    }
 }
 
 // Segment s as [b, e), clamped into [0, n].
@@ -588,7 +793,20 @@ __device__ __forceinline__ void sort_own_segments(uint64_t* kin, uint32_t* vin, 
     }
 }
 
-// Blocks [0, nbig) sort the segments of more than 512 and at most `most` keys:
+// Keys a warp sorts alone: 512 where there are segments enough to fill the chip
+// several times over (the network's instructions a key bound the sort then),
+// else 256 (a warp's chain of 45 exchanges of 16 words then leaves the chip
+// waiting for the last warps, where a block of buckets is done in a third of
+// the time). Compaction and sort, 512 against 256: 2160p / 6M (32,768
+// segments of 263 keys on average) 383 against 399 us, 64 views / 2M (262,144 of
+// 460) 6.66 against 6.70 ms; 1080p / 1M (8,192 of 140) 67.4 against 65.3, 720p /
+// 500k (4,096 of 121) 47.5 against 43.2, 6 views / 300k (32,768 of 59) 153.5
+// against 147.8.
+__device__ __forceinline__ uint32_t alone_cap(uint32_t n, uint32_t nseg) {
+    return nseg > 8192u && n >= 192u * nseg ? 512u : 256u;
+}
+
+// Blocks [0, nbig) sort the segments of more than alone_cap and at most `most` keys:
 // block i those among i, i + nbig, i + 2 nbig, ..., found by one look at their
 // bounds. Blocks nbig + g, g >= 0, give warp w the segment 8g + w when it
 // holds 1 to 512 keys. The large segments come first in launch order so their
@@ -614,12 +832,13 @@ k_seg_sort(uint64_t* kin, uint32_t* vin, uint64_t* kout, uint32_t* vout, const u
     constexpr int kRaw = SegSmem<kSegThreads>::kRaw > kListBytes ? SegSmem<kSegThreads>::kRaw : kListBytes;
     __shared__ __align__(16) unsigned char s_raw[kRaw];
     __shared__ uint32_t s_off[kLocalRadix];
-    __shared__ uint32_t s_red[2 * kSegWarps + 2];
+    __shared__ uint32_t s_red[4 * kSegWarps];
     const int warp = threadIdx.x >> 5;
     pdl_wait();
     const uint32_t n_all = min(*num_keys, cap);
+    const uint32_t alone = alone_cap(n_all, nseg);
     if (blockIdx.x < nbig) {
-        sort_own_segments<kSegThreads>(kin, vin, kout, vout, start, n_all, nseg, nbig, (uint32_t)kWarpCap, most,
+        sort_own_segments<kSegThreads>(kin, vin, kout, vout, start, n_all, nseg, nbig, alone, most,
                                        begin_bit, s_raw, s_off, s_red);
         return;
     }
@@ -628,7 +847,7 @@ k_seg_sort(uint64_t* kin, uint32_t* vin, uint64_t* kout, uint32_t* vout, const u
     uint32_t b, e;
     seg_bounds(start, s, n_all, b, e);
     const int n = (int)(e - b);
-    if (n == 0 || n > kWarpCap) return;
+    if (n == 0 || n > (int)alone) return;
     uint16_t* list = reinterpret_cast<uint16_t*>(s_raw) + warp * kListLen;
     if (n <= 32)
         warp_sort<1>(kin, vin, kout, vout, b, n, begin_bit, list);
@@ -642,7 +861,7 @@ k_seg_sort(uint64_t* kin, uint32_t* vin, uint64_t* kout, uint32_t* vout, const u
         warp_sort<16>(kin, vin, kout, vout, b, n, begin_bit, list);
 }
 
-// The segments of more than 2,048 keys, 1,024 threads each (up to 8,192 keys
+// The segments of more than 2,048 keys, 1,024 threads each (up to 16,384 keys
 // in shared memory). Launched where the capacity allows such segments to be
 // common, kHugeMean keys or more a segment: the launch costs 3 us, and the
 // 256-thread blocks of k_seg_sort, which take them otherwise, 8 passes over
@@ -651,9 +870,9 @@ constexpr uint32_t kHugeMean = 600;
 __global__ void __launch_bounds__(kHugeThreads, 1)
 k_seg_sort_huge(uint64_t* kin, uint32_t* vin, uint64_t* kout, uint32_t* vout, const uint32_t* __restrict__ start,
                 const uint32_t* __restrict__ num_keys, uint32_t cap, uint32_t nseg, int begin_bit) {
-    __shared__ __align__(16) unsigned char s_raw[SegSmem<kHugeThreads>::kRaw];
+    extern __shared__ __align__(16) unsigned char s_raw[];  // SegSmem<kHugeThreads>::kRaw
     __shared__ uint32_t s_off[kLocalRadix];
-    __shared__ uint32_t s_red[2 * kHugeThreads / kWarp + 2];
+    __shared__ uint32_t s_red[4 * kHugeThreads / kWarp];
     pdl_wait();
     const uint32_t n_all = min(*num_keys, cap);
     sort_own_segments<kHugeThreads>(kin, vin, kout, vout, start, n_all, nseg, gridDim.x,
@@ -722,8 +941,20 @@ cudaError_t launch_sort_segmented(const uint32_t* num_keys, int64_t key_capacity
     const bool huge = (uint64_t)key_capacity >= (uint64_t)kHugeMean * nseg &&
                       key_capacity > (int64_t)block_cap<kSegThreads>();
     if (huge) {
+        constexpr int smem = SegSmem<kHugeThreads>::kRaw;
+        // above the default limit: set once per device
+        static std::atomic<uint64_t> configured{0};
+        int dev = 0;
+        e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        const uint64_t bit = uint64_t(1) << (dev & 63);
+        if (!(configured.load(std::memory_order_acquire) & bit)) {
+            e = cudaFuncSetAttribute(k_seg_sort_huge, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            if (e != cudaSuccess) return e;
+            configured.fetch_or(bit, std::memory_order_acq_rel);
+        }
         e = launch_pdl(k_seg_sort_huge, dim3(nseg <= 512u ? nseg : (nseg / 32u < 512u ? 512u : (nseg + 31u) / 32u)),
-                       dim3(kHugeThreads), 0, stream, pk, pv, ok, ov, (const uint32_t*)start, num_keys,
+                       dim3(kHugeThreads), (size_t)smem, stream, pk, pv, ok, ov, (const uint32_t*)start, num_keys,
                        (uint32_t)key_capacity, nseg, begin_bit);
         if (e != cudaSuccess) return e;
     }

@@ -394,3 +394,49 @@ def test_tile_ranges_of_sparse_tiles(tiles):
         t = np.sort(tile[:n]).astype(np.int64)
         want = np.stack([np.searchsorted(t, np.arange(tiles), "left"), np.searchsorted(t, np.arange(tiles), "right")], 1)
         np.testing.assert_array_equal(ranges.cpu().numpy(), want)
+
+
+def _crowded(n, most, rng):
+    """n depths spread evenly, `most` of them on one value."""
+    d = rng.permutation(np.linspace(1 << 24, 1 << 30, n)).astype(np.uint32)
+    d[rng.permutation(n)[:most]] = 1 << 29
+    return d
+
+
+@pytest.mark.parametrize("lengths", [[255, 256, 257, 1023, 1024, 1025], [2047, 2048, 2049, 4096, 4097, 8193],
+                                     [16383, 16384, 16385]])
+@pytest.mark.parametrize("most", [1, 62, 70, 10 ** 6])
+def test_segments_around_the_bucket_limits(lengths, most):
+    """Local sorts by buckets on both sides of each length they take, with
+    sub-keys that fill the buckets evenly, to just below and above the most a
+    bucket may hold, and all in one."""
+    from paper_2602_03207_gb300 import capi
+    rng = np.random.default_rng(most)
+    keys = np.concatenate([(np.uint64(s) << np.uint64(31)) | _crowded(n, min(n, most), rng).astype(np.uint64)
+                           for s, n in enumerate(lengths)])
+    keys = keys[rng.permutation(keys.size)]
+    vals = rng.permutation(keys.size).astype(np.uint32)
+    end_bit = 31 + int(np.ceil(np.log2(len(lengths))))
+    k, v = gpu_sort(keys, vals, end_bit=end_bit, capacity=max(keys.size, 700 << (end_bit - 31)),
+                    flags=capi.WS_CFG_SORT_SEGMENTED)
+    perm = np.argsort(keys, kind="stable")
+    np.testing.assert_array_equal(k, keys[perm])
+    np.testing.assert_array_equal(v, vals[perm])
+
+
+@pytest.mark.parametrize("mean", [180, 200])
+def test_many_segments_on_both_sides_of_the_warps_limit(mean):
+    """16,384 segments, lengths on both sides of 256 and 512: below and above
+    the mean length from which a warp takes 512 keys."""
+    from paper_2602_03207_gb300 import capi
+    rng = np.random.default_rng(mean)
+    nseg = 1 << 14
+    lengths = np.concatenate([[0, 1, 255, 256, 257, 511, 512, 513, 2049], rng.integers(mean - 100, mean + 101, nseg - 9)])
+    seg = np.repeat(np.arange(nseg, dtype=np.uint64), lengths)
+    keys = (seg << np.uint64(31)) | rng.integers(1 << 28, 1 << 30, seg.size, dtype=np.uint64)
+    keys = keys[rng.permutation(keys.size)]
+    vals = rng.permutation(keys.size).astype(np.uint32)
+    k, v = gpu_sort(keys, vals, end_bit=45, flags=capi.WS_CFG_SORT_SEGMENTED)
+    perm = np.argsort(keys, kind="stable")
+    np.testing.assert_array_equal(k, keys[perm])
+    np.testing.assert_array_equal(v, vals[perm])
