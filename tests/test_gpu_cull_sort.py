@@ -168,6 +168,47 @@ def test_offsets_at_the_edges_of_each_scan(n, room):
     assert not keys[kept:].any() and not vals[kept:].any()
 
 
+@pytest.mark.parametrize("kind", ["few", "many", "fits", "one_more", "large"])
+def test_emission_of_rectangles_of_every_size(kind):
+    """The slot map's ways: a thread's few pairs, a thread with more than 32, a
+    chunk of exactly 4,096 pairs and of one more, and a rectangle of more."""
+    import torch
+    from paper_2602_03207_gb300 import capi
+    rng = np.random.default_rng(len(kind))
+    n, tx = 2500, 256
+    w, h = rng.integers(1, 4, n), rng.integers(1, 3, n)
+    live = rng.random(n) < 0.6
+    if kind == "many":
+        w[::37], h[::37] = rng.integers(5, 60, n)[::37], rng.integers(1, 5, n)[::37]
+    elif kind in ("fits", "one_more"):
+        live[:1024], w[:1024], h[:1024] = True, 4, 1
+        if kind == "one_more":
+            w[500] = 5
+    elif kind == "large":
+        live[700], w[700], h[700] = True, 90, 100
+    x, y = rng.integers(0, tx - w + 1), rng.integers(0, 256 - h + 1)
+    rect = np.stack([x, y, x + w - 1, y + h - 1], 1).astype(np.uint16)
+    touched = np.where(live, w * h, 0)
+    depth = rng.uniform(1.0, 9.0, n).astype(np.float32)
+    total = int(touched.sum())
+    cam, cfg = capi.camera(dict(S.small_forward()[1], width=16 * tx, height=4096)), capi.config()
+    dev = lambda a: torch.from_numpy(a).cuda()
+    offsets = torch.zeros(n + 4, dtype=torch.int32, device="cuda")
+    keys = torch.zeros(total + 2, dtype=torch.int64, device="cuda")
+    vals = torch.zeros(total + 4, dtype=torch.int32, device="cuda")
+    num = torch.zeros(4, dtype=torch.int32, device="cuda")
+    work = torch.zeros(capi.ws_workspace_bytes(n, total, cam, cfg), dtype=torch.uint8, device="cuda")
+    capi.ws_cull(n, dev(touched.astype(np.int32)), dev(rect.view(np.int16)), dev(depth), cam, cfg, offsets, keys,
+                 vals, total, num, work)
+    gid = np.repeat(np.arange(n), touched)
+    j = np.arange(total) - np.repeat(np.cumsum(touched) - touched, touched)
+    tile = (y[gid] + j // w[gid]) * tx + x[gid] + j % w[gid]
+    assert int(num[0]) == total and capi.ws_read_status(work) == 0
+    np.testing.assert_array_equal(vals[:total].cpu().numpy(), gid)
+    np.testing.assert_array_equal(keys[:total].cpu().numpy().view(np.uint64),
+                                  (tile.astype(np.uint64) << np.uint64(31)) | depth[gid].view(np.uint32))
+
+
 @pytest.mark.parametrize("sort", ["segmented", "lsd", "lookback"])
 @pytest.mark.parametrize("size", [(16, 16), (100, 75)], ids=["one_tile", "ragged"])
 def test_whole_frame_calls_equal_staged_calls(sort, size):
