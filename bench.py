@@ -153,8 +153,18 @@ def seg_sort_bytes(keys, end_bit):
     return sort_bytes(keys, seg_partition_passes(end_bit)) + 32 * keys
 
 
-def seg_sort_launches(end_bit):
-    return 3 * seg_partition_passes(end_bit) + 2
+def seg_sort_launches(end_bit, capacity=0):
+    """Three per partition pass, the bounds, the local sort, and the large
+    segments' own launch where the capacity is 600 keys a segment or more."""
+    huge = capacity >= 600 << (end_bit - 31) and capacity > 2048
+    return 3 * seg_partition_passes(end_bit) + 2 + int(huge)
+
+
+def cull_launches(n):
+    """The emission, the chunk sums above 16 chunks of 1,024 Gaussians and
+    their scan above 2,048."""
+    chunks = (n + 1023) // 1024
+    return 1 + int(chunks > 16) + int(chunks > 2048)
 
 
 def blend_work(fetched, width, height, tile):
@@ -472,11 +482,11 @@ def run_ours(args):
     for i in range(args.warmup):
         r.forward(scene, cams[rank_pose(rank, i)])
     r.check_status()
-    # preprocess 1, cull 3, segmented sort (3 per partition pass + bounds +
-    # local), rasterize: the blend, plus the tile-range scan unless the sort
-    # wrote the ranges (ws_sort_tiles)
+    # preprocess 1, cull, segmented sort, rasterize: the blend, plus the
+    # tile-range scan unless the sort wrote the ranges (ws_sort_tiles)
     ranges_given = bool(r.raster_cfg.flags & capi.WS_CFG_RANGES_GIVEN)
-    launches_per_frame = 1 + 3 + seg_sort_launches(r.end_bit) + (1 if ranges_given else 2)
+    launches_per_frame = (1 + cull_launches(r.n) + seg_sort_launches(r.end_bit, r.key_capacity)
+                          + (1 if ranges_given else 2))
 
     ccams = [capi.camera(c) for c in cams]
 
@@ -806,7 +816,7 @@ def train_block(args, dev, min_timed_s=1.0, stage_steps=100):
     500,000-Gaussian 1280x720 scene against a U[0,1) target (the gradient
     parity workload). Timed regions of K steps as the frame metric, for the
     separate calls (ws_rasterize, ws_image_residual, ws_rasterize_backward)
-    and for the fused pass (ws_render_train_l2), which gives the same bits;
+    and for the one call (ws_render_train_l2), which gives the same bits;
     the faster is the value. Plus a per-stage split of the separate calls
     from a run with an event between stages."""
     import torch
@@ -829,7 +839,7 @@ def train_block(args, dev, min_timed_s=1.0, stage_steps=100):
         capi.ws_image_residual(tgt.numel(), r.image, tgt, d)
         r.backward(scene, cam, d)
 
-    def step_fused():  # pre-processing, compaction, sort, then the fused pass
+    def step_fused():  # pre-processing, compaction, sort, then the one call
         r.train_step_l2(scene, cam, tgt)
 
     for _ in range(max(args.warmup, 3)):
@@ -865,7 +875,7 @@ def train_block(args, dev, min_timed_s=1.0, stage_steps=100):
         e[6].record(stream)
     torch.cuda.synchronize()
     stage_ms = {nm: sum(e[j].elapsed_time(e[j + 1]) for e in ev) / stage_steps for j, nm in enumerate(names)}
-    # the fused path's split: the same three stages, then ws_render_train_l2
+    # the one call's split: the same three stages, then ws_render_train_l2
     fev = [_events(2) for _ in range(stage_steps)]
     for e in fev:
         r.preprocess(scene, ccam)
@@ -885,9 +895,9 @@ def train_block(args, dev, min_timed_s=1.0, stage_steps=100):
     peak = fp32_peak_tflops()
     if path == "fused":
         ach = (fwd_flops(evals) + bwd_flops(evals)) / (fused_ms * 1e-3) / 1e12
-        roof = {"kernel": f"k_train<{r.tile}> (timed span: ws_render_train_l2)", "bound": "alu",
+        roof = {"kernel": f"k_blend<{r.tile}> + k_blend_bwd<{r.tile}> (timed span: ws_render_train_l2)", "bound": "alu",
                 "alg_evals": int(evals), "achieved": round(ach, 3), "peak": round(peak, 2), "unit": "TFLOP/s",
-                "frac": round(ach / peak, 4), "traffic": KERNEL_TRAFFIC.get(("k_train", r.tile)),
+                "frac": round(ach / peak, 4), "traffic": KERNEL_TRAFFIC.get(("train", r.tile)),
                 "peak_source": "derived: SMs x 128 FP32 lanes x 2 x max SM clock"}
     else:
         ach = bwd_flops(evals) / (stage_ms["backward"] * 1e-3) / 1e12
@@ -907,7 +917,7 @@ def train_block(args, dev, min_timed_s=1.0, stage_steps=100):
             "step_variants": {nm: {"ms_per_step": round(v[1] / steps * 1e3, 4), "steps_s": round(steps / v[1], 2)}
                               for nm, v in timed.items()},
             "stages_ms": {k: round(v, 4) for k, v in stage_ms.items()},
-            "stages_note": "separate calls, an event between stages; the fused pass alone (ws_render_train_l2 "
+            "stages_note": "separate calls, an event between stages; the one call (ws_render_train_l2 "
                            "after the sort): " + f"{fused_ms:.4f} ms",
             "roofline": roof,
             "clocks": clk.summary()}
@@ -943,8 +953,8 @@ def batch_block(args, dev, min_timed_s=1.0, plain_min_s=0.5):
                             key_capacity=best["key_capacity"], device=dev)
     stream = torch.cuda.current_stream(dev)
     steps = max(1, min(args.steps, 5))
-    # The separate calls, the fused single pass on one block per (view, tile)
-    # and the fused pass as one persistent grid give the same bits; each is
+    # The separate calls, the one call after the sort on one block per (view,
+    # tile) and with a persistent backward grid give the same bits; each is
     # captured as a CUDA graph and timed the same way, and the fastest is the
     # value (the tuner's tile and digit width are timed on the separate calls).
     paths = [("separate", b)]
@@ -971,7 +981,7 @@ def batch_block(args, dev, min_timed_s=1.0, plain_min_s=0.5):
     pairs = b.key_count()
     variants = {nm: {"ms_per_step": round(v[1] / steps * 1e3, 3), "views_s": round(V / (v[1] / steps), 2)}
                 for nm, v in timed.items()}
-    bf = dict(paths)[path] if path != "separate" else None  # kept for the fused pass's own span
+    bf = dict(paths)[path] if path != "separate" else None  # kept for the one call's own span
     paths = None
     torch.cuda.empty_cache()
     # per-stage split of the batched step (eager launches, an event between stages)
@@ -996,7 +1006,7 @@ def batch_block(args, dev, min_timed_s=1.0, plain_min_s=0.5):
     b.check_status()
     stage_ms = {nm: sum(e[j].elapsed_time(e[j + 1]) for e in ev) / reps for j, nm in enumerate(names)}
     fused_ms = None
-    if bf is not None:  # the fused pass alone, after the same three stages
+    if bf is not None:  # the one call alone, after the same three stages
         fev = [_events(2) for _ in range(reps)]
         for e in fev:
             bf.preprocess(scene)
@@ -1032,7 +1042,7 @@ def batch_block(args, dev, min_timed_s=1.0, plain_min_s=0.5):
                             if best["tile"] in BATCH_BWD_TRAFFIC_PER_PAIR else None)}
     else:
         ach = (fwd_flops(evals) + bwd_flops(evals)) / (fused_ms * 1e-3) / 1e12
-        roof = {"kernel": f"k_train_batch<{best['tile']}> (timed span: ws_render_train_l2_batch, "
+        roof = {"kernel": f"k_blend_batch<{best['tile']}> + k_blend_bwd_batch<{best['tile']}> (timed span: ws_render_train_l2_batch, "
                           f"{'persistent grid' if path == 'fused_persistent' else 'one block per item'})",
                 "traffic": (round(BATCH_TRAIN_TRAFFIC_PER_PAIR[best["tile"]] * pairs)
                             if best["tile"] in BATCH_TRAIN_TRAFFIC_PER_PAIR and path == "fused_grid" else None)}
@@ -1050,15 +1060,15 @@ def batch_block(args, dev, min_timed_s=1.0, plain_min_s=0.5):
                    "tile": best["tile"], "digit_bits": best["digit_bits"], "pairs": pairs,
                    "path": {"separate": "ws_rasterize_batch + ws_image_residual + ws_rasterize_backward_batch",
                             "fused_grid": "ws_render_train_l2_batch, one block per (view, tile)",
-                            "fused_persistent": "ws_render_train_l2_batch, persistent grid"}[path],
+                            "fused_persistent": "ws_render_train_l2_batch, persistent backward grid"}[path],
                    "autotune": best.get("table"), "autotune_cached": best.get("cached")},
         "stages_ms": {k: round(v, 3) for k, v in stage_ms.items()},
         "stages_note": "separate calls, eager launches with an event between stages"
-                       + (f"; the fused pass alone (after the sort): {fused_ms:.3f} ms" if fused_ms else "")
+                       + (f"; the one call after the sort: {fused_ms:.3f} ms" if fused_ms else "")
                        + "; each timed step is one CUDA-graph replay",
         "step_variants": variants,
-        "step_variants_note": "the separate forward / residual / backward calls, the fused single pass per "
-                              "(view, tile) and its persistent grid give the same results; the fastest is the value",
+        "step_variants_note": "the separate forward / residual / backward calls, the one call after the sort "
+                              "and its persistent backward grid give the same results; the fastest is the value",
         "roofline": roof,
         "clocks": clk.summary(),
     }
@@ -1214,7 +1224,7 @@ def main():
     ap.add_argument("--no-ablation", action="store_true")
     ap.add_argument("--no-autotune", action="store_true", help="batch: use --tile / --digit-bits as given")
     ap.add_argument("--no-plain", action="store_true", help="batch: skip the per-view comparison")
-    ap.add_argument("--no-variants", action="store_true", help="batch: skip the fused single-pass variants")
+    ap.add_argument("--no-variants", action="store_true", help="batch: skip the one-call variants")
     ap.add_argument("--views", type=int, default=64, help="batch: the first N of the 64 seeded views")
     ap.add_argument("--no-train", action="store_true", help="skip the training-step measurement")
     ap.add_argument("--no-batch", action="store_true", help="skip the batched-views measurement")

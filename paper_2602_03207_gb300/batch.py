@@ -135,10 +135,10 @@ class BatchRenderer:
     def step(self, scene, target, stream=None):
         """One training step of 1/2 ||image - target||^2 summed over the views.
         Default: the separate calls (forward, d_image = image - target,
-        backward). fused=True (about 1.5 % faster on GB300): pre-processing,
-        compaction, sort, then ws_render_train_l2_batch (every (view, tile)
-        composited, its residual formed and its backward records written in
-        one pass; persistent=True runs that pass as one persistent grid). All
+        backward). fused=True (0.5 % faster for 64 views of 2M Gaussians):
+        pre-processing, compaction, sort, then ws_render_train_l2_batch (the
+        forward, then the backward with the residual formed as it reads the
+        image; persistent=True runs the backward as one persistent grid). All
         give the same images and gradients bit for bit."""
         if not self.fused:
             self.forward(scene, stream)
@@ -150,9 +150,9 @@ class BatchRenderer:
         return self.train_pass(scene, target, stream)
 
     def train_pass(self, scene, target, stream=None):
-        """The fused pass of a step after the sort (ws_render_train_l2_batch):
-        images, L2 residual, backward records and the per-Gaussian gradients
-        summed over the views; one persistent grid when persistent=True."""
+        """A step after the sort (ws_render_train_l2_batch): images, backward
+        records of the L2 residual and the per-Gaussian gradients summed over
+        the views; a persistent backward grid when persistent=True."""
         g = self.grads
         capi.ws_render_train_l2_batch(self.n, scene["means"], scene["log_scales"], scene["quats"], scene["sh"],
                                       self.cams_arr, self.raster_cfg, self.num_keys, self.sorted_keys, self.sorted_vals,

@@ -286,7 +286,7 @@ class Renderer:
         return {k: v[:self.n] for k, v in g.items()}
 
     def train_step_l2(self, scene, cam_dict, target, stream=None):
-        """One training step of L = 1/2 ||image - target||^2 in fused form
+        """One training step of L = 1/2 ||image - target||^2 as one call
         (ws_render_train_l2 after the pre-processing, compaction and sort):
         the same image and gradients as forward() + ws_image_residual +
         backward(), in fewer launches. Returns the gradient dict."""
@@ -304,7 +304,7 @@ class Renderer:
         return {k: v[:self.n] for k, v in g.items()}
 
     def train_pass_l2(self, scene, cam_dict, target, stream=None):
-        """The fused pass of train_step_l2 alone (ws_render_train_l2), on the
+        """train_step_l2 from the sorted pairs on (ws_render_train_l2), on the
         pairs this renderer has sorted for the same scene and camera."""
         cam = capi.camera(cam_dict)
         g = self._grads()
