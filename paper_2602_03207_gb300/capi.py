@@ -80,7 +80,9 @@ def camera(cam: dict) -> Camera:
         return Camera.from_buffer_copy(_CAMERA.pack(*vm[:12], cam["fx"], cam["fy"], cam["cx"], cam["cy"],
                                                     int(cam["width"]), int(cam["height"]), cam["znear"],
                                                     bg[0], bg[1], bg[2]))
-    except OverflowError:  # a value past float32: infinite, as a C conversion makes it
+    except (OverflowError, struct.error):  # a value past float32 (infinite) or int32, as a C conversion makes it
+        if len(vm) < 12:
+            raise IndexError("viewmat needs 12 values at least")
         return Camera((C.c_float * 12)(*vm[:12]), cam["fx"], cam["fy"], cam["cx"], cam["cy"], int(cam["width"]),
                       int(cam["height"]), cam["znear"], (C.c_float * 3)(bg[0], bg[1], bg[2]))
 

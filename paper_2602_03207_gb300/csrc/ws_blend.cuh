@@ -8,10 +8,10 @@
 // they replace (two streams of 16 lanes, one pixel per lane, a bit set per
 // 32 splats; the backward's partials summed by 12 shuffles a visit and 16
 // selects a splat), warm, at 16-pixel tiles:
-//   forward, 1080p / 1M                 80.4 -> 64.9 us (72.0M -> 51M warp instructions)
+//   forward, 1080p / 1M                 80.4 -> 62.4 us (72.0M -> 47M warp instructions)
 //   forward, 2160p / 6M                617.6 -> 448 us
 //   backward call, 720p / 500k         220.4 -> 133 us (102.6M -> 48.7M)
-//   backward call, 64 views of 2M       33.2 -> 20.6 ms
+//   backward call, 64 views of 2M       33.2 -> 20.1 ms
 #pragma once
 
 #include <type_traits>

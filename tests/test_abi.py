@@ -151,3 +151,21 @@ def test_whole_frame_calls_reject_bad_arguments(lib):
         assert lib.ws_render_frame(10, c, g, b, r, None) == capi.WS_ERR_INVALID_ARG
         assert lib.ws_render_frame_packed(10, c, g, b, None, None, None, r, None) == capi.WS_ERR_INVALID_ARG
         assert lib.ws_train_frame_l2(10, c, g, b, *[None] * 6, r, None) == capi.WS_ERR_INVALID_ARG
+
+
+def test_camera_struct_takes_what_it_always_took():
+    """Rows, flat lists and arrays of the view matrix; values past float32
+    and int32 as C conversions make them; too few values are refused."""
+    import numpy as np
+    from paper_2602_03207_gb300 import capi
+    from paper_2602_03207_gb300 import synthetic as S
+    cam = dict(S.small_forward()[1])
+    want = bytes(capi.camera(cam))
+    m = np.asarray(cam["viewmat"], np.float32)
+    for vm in (m, m.tolist(), m.reshape(-1), m.reshape(-1).tolist(), list(m), m[:3]):
+        assert bytes(capi.camera(dict(cam, viewmat=vm))) == want
+    far = capi.camera(dict(cam, znear=1e300, width=(1 << 32) + 16))
+    assert far.znear == float("inf") and far.width == 16 and list(far.viewmat) == list(m.reshape(-1)[:12])
+    for bad in (m.reshape(-1)[:11], m[:2]):
+        with pytest.raises(IndexError):
+            capi.camera(dict(cam, viewmat=bad))
