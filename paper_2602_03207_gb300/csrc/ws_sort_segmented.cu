@@ -13,14 +13,14 @@
 //      order: a warp sorts one of at most 256 or 512 keys (alone_cap) with a
 //      bitonic network in registers, a block one of at most 2,048 (256 threads) or
 //      16,384 (1,024 threads) through buckets in shared memory or, where the
-//      sub-keys crowd together, with three 7-bit counting passes, and one of
-//      more keys with chunked 8-bit passes over global memory, ranked with warp
-//      ballots, skipping a pass whose digit is the same for every key. The
-//      network and the 7-bit passes sort 32-bit words: the sub-key's distance
-//      from the segment's smallest, cut to the leading bits that fit, above
-//      the position in the segment; where bits were cut off, a check of
-//      neighbours by the whole sub-key puts right what they would have
-//      decided (fix_order).
+//      sub-keys crowd together, with counting passes over the list of their
+//      positions, and one of more keys with chunked 8-bit passes over global
+//      memory, ranked with warp ballots, skipping a pass whose digit is the
+//      same for every key. The network sorts 32-bit words: the sub-key's
+//      distance from the segment's smallest, cut to the leading bits that
+//      fit, above the position in the segment; where bits were cut off, an
+//      exchange of neighbours by the whole sub-key or two more networks put
+//      right what they would have decided (warp_sort).
 // A stable partition by the high bits followed by a stable sort of each
 // segment by the low bits orders the pairs exactly as the full-key LSD
 // sort does, ties included. There are no global atomics and no block waits
@@ -194,17 +194,18 @@ __device__ __forceinline__ void warp_bitonic(uint32_t (&v)[K]) {
 // consecutive entries of the way back fall in few banks.
 __device__ __forceinline__ int spad(int e) { return e + (e >> 4); }
 
-// Puts a list of positions right where the cut bits would have decided:
-// odd-even exchanges of neighbours by (sub-key, position) until none is out of
-// order. The list is sorted but for runs of equal sort words, so a round or
-// two will do on all but contrived inputs. any(x): the vote of `threads`
-// threads, of which this is number t, and a barrier between them.
-template <typename Order, typename Vote>
-__device__ __forceinline__ void fix_order(uint16_t* list, int n, int t, int threads, Order sub_of, Vote any) {
-    for (;;) {
+// Puts a warp's list of positions right where the cut bits would have decided:
+// odd-even exchanges of neighbours by (sub-key, position). The list is sorted
+// but for runs of equal sort words, most of them pairs, so a round or two will
+// do; returns whether kFixRounds rounds left every neighbour in order.
+constexpr int kFixRounds = 4;
+
+template <typename Order>
+__device__ __forceinline__ bool fix_order(uint16_t* list, int n, int lane, Order sub_of) {
+    for (int round = 0; round < kFixRounds; ++round) {
         bool swapped = false;
         for (int odd = 0; odd < 2; ++odd) {
-            for (int q = 2 * t + odd; q + 1 < n; q += 2 * threads) {
+            for (int q = 2 * lane + odd; q + 1 < n; q += 2 * kWarp) {
                 const uint16_t a = list[spad(q)], b = list[spad(q + 1)];
                 const uint32_t sa = sub_of(a), sb = sub_of(b);
                 if (sa > sb || (sa == sb && a > b)) {
@@ -213,25 +214,32 @@ __device__ __forceinline__ void fix_order(uint16_t* list, int n, int t, int thre
                     swapped = true;
                 }
             }
-            any(false);
+            __syncwarp();  // the exchanges before the next reads
         }
-        if (!any(swapped)) return;
+        if (!__any_sync(kFull, swapped)) return true;
     }
+    return false;
 }
 
-// One warp sorts n <= 32*K pairs [b, b + n) of (kin, vin) into (kout, vout).
+// One warp sorts n <= 32*K pairs [b, b + n) of (kin, vin) into (kout, vout): by
+// the leading bits of the sub-keys and an exchange of the few neighbours that
+// the rest decides; where many sub-keys share their leading bits (a wall seen
+// head-on behind one near splat) the network runs twice more, over the cut
+// bits and then, stably, over the leading ones.
 template <int K>
 __device__ __forceinline__ void warp_sort(const uint64_t* kin, const uint32_t* vin, uint64_t* kout, uint32_t* vout,
                                           uint32_t b, int n, int begin_bit, uint16_t* list) {
     const int lane = threadIdx.x & 31;
     const uint32_t sub_mask = (1u << (kSplitBit - begin_bit)) - 1u;
     constexpr int idx_bits = K == 1 ? 5 : (K == 2 ? 6 : (K == 4 ? 7 : (K == 8 ? 8 : 9)));
+    constexpr uint32_t kIdxMask = (1u << idx_bits) - 1u;
+    const auto sub_of = [&](uint32_t i) { return sub_key(__ldg(kin + b + i), begin_bit, sub_mask); };
     uint32_t v[K];
     uint32_t least = ~0u, most = 0u;
 #pragma unroll
     for (int k = 0; k < K; ++k) {
         const int idx = k * kWarp + lane;
-        v[k] = idx < n ? sub_key(__ldg(kin + b + idx), begin_bit, sub_mask) : 0u;
+        v[k] = idx < n ? sub_of(idx) : 0u;
         if (idx < n) {
             least = min(least, v[k]);
             most = max(most, v[k]);
@@ -246,17 +254,30 @@ __device__ __forceinline__ void warp_sort(const uint64_t* kin, const uint32_t* v
         // past the end: the largest words (the position makes them distinct)
         v[k] = idx < n ? sort_word(v[k], least, cut, idx_bits, (uint32_t)idx) : (~0u << idx_bits) | (uint32_t)idx;
     }
-    warp_bitonic<K>(v);
+    // pass 0: leading bits; 1: the cut bits; 2: leading bits over pass 1's order
+#pragma unroll 1
+    for (int pass = 0;; ++pass) {
+        warp_bitonic<K>(v);
+        if (pass == 2) {  // places in pass 1's order -> positions
 #pragma unroll
-    for (int k = 0; k < K; ++k) list[spad(lane * K + k)] = (uint16_t)(v[k] & ((1u << idx_bits) - 1u));
-    __syncwarp();
-    if (cut > 0)
-        fix_order(
-            list, n, lane, kWarp, [&](uint16_t i) { return sub_key(__ldg(kin + b + i), begin_bit, sub_mask); },
-            [](bool x) {
-                __syncwarp();  // the exchanges before the next reads
-                return __any_sync(kFull, x) != 0;
-            });
+            for (int k = 0; k < K; ++k) v[k] = list[spad((int)(v[k] & kIdxMask))];
+            __syncwarp();  // every read before the writes
+        }
+#pragma unroll
+        for (int k = 0; k < K; ++k) list[spad(lane * K + k)] = (uint16_t)(v[k] & kIdxMask);
+        __syncwarp();
+        if (pass == 2 || (pass == 0 && (cut == 0 || fix_order(list, n, lane, sub_of)))) break;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const int idx = k * kWarp + lane;
+            v[k] = (~0u << idx_bits) | (uint32_t)idx;
+            if (idx < n) {
+                const uint32_t d = sub_of(pass == 0 ? (uint32_t)idx : list[spad(idx)]) - least;
+                v[k] = ((pass == 0 ? d & ((1u << cut) - 1u) : d >> cut) << idx_bits) | (uint32_t)idx;
+            }
+        }
+        __syncwarp();
+    }
 #pragma unroll
     for (int k = 0; k < K; ++k) {
         const int p = k * kWarp + lane;
@@ -343,6 +364,13 @@ __device__ __forceinline__ bool bucket_sort(const uint64_t* kin, const uint32_t*
         least = min(least, red[3 * w]);
         most = max(most, red[3 * w + 1]);
         total += __uint_as_float(red[3 * w + 2]);
+    }
+    if (least == most) {  // in order already
+        for (int i = t; i < n; i += THREADS) {
+            kout[b + i] = __ldg(kin + b + i);
+            vout[b + i] = __ldg(vin + b + i);
+        }
+        return true;
     }
     const float mean = total / (float)n;
     float dev = 0.0f;
@@ -473,80 +501,58 @@ __device__ __forceinline__ uint32_t block_varying(uint32_t a, uint32_t o, uint32
     return ra ^ ro;
 }
 
-// The block sorts n <= block_cap pairs by their sort words (11 or 14 bits of
-// position, 21 or 18 of sub-key) with three stable 7-bit LSD passes
-// over the sub-key's part; with kn = ceil(n / THREADS), element w*32*kn + k*32
-// + lane lives in lane `lane` of warp w, item k. s_word: a word per key
-// (reused for the list of positions); s_cnt: THREADS / 32 rows of 128
-// counters.
-constexpr int kCtaDigit = 7;
+// The block sorts n <= block_cap pairs by stable 8-bit LSD passes over the list
+// of their positions, at most four, skipping those whose digit is the same
+// for every key; with kn = ceil(n / THREADS), element w*32*kn + k*32 + lane of the
+// list lives in lane `lane` of warp w, item k. s_sub: the sub-keys by position;
+// s_cnt: THREADS / 32 rows of 256 counters.
+constexpr int kCtaDigit = 8;
 constexpr int kCtaRadix = 1 << kCtaDigit;
 
 template <int THREADS>
 __device__ __forceinline__ void block_sort_smem(const uint64_t* kin, const uint32_t* vin, uint64_t* kout,
-                                                uint32_t* vout, uint32_t b, int n, int begin_bit, uint32_t* s_word,
-                                                uint16_t* s_cnt, uint32_t* red) {
+                                                uint32_t* vout, uint32_t b, int n, int begin_bit, uint32_t* s_sub,
+                                                uint16_t* s_list, uint16_t* s_cnt, uint32_t* red) {
     constexpr int kSegItems = seg_items<THREADS>();
-    constexpr int kCap = block_cap<THREADS>();
-    constexpr int kIdxBits = THREADS == 1024 ? 14 : 11;
-    static_assert((1 << kIdxBits) == kCap && kIdxBits + 3 * kCtaDigit >= 32, "position bits and passes");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // every warp takes kn consecutive runs of 32 (input order = warp, item, lane)
     const int kn = (n + THREADS - 1) / THREADS;
     const int wbase = warp * kWarp * kn;
     const uint32_t sub_mask = (1u << (kSplitBit - begin_bit)) - 1u;
-    uint32_t word[kSegItems];
-    uint32_t least = ~0u, most = 0u;
-#pragma unroll
-    for (int k = 0; k < kSegItems; ++k) {
-        word[k] = 0;
-        const int idx = wbase + k * kWarp + lane;
-        if (k < kn && idx < n) {
-            word[k] = sub_key(__ldg(kin + b + idx), begin_bit, sub_mask);
-            least = min(least, word[k]);
-            most = max(most, word[k]);
-        }
+    uint32_t all_and = ~0u, all_or = 0u;
+    for (int i = threadIdx.x; i < n; i += THREADS) {
+        const uint32_t x = sub_key(__ldg(kin + b + i), begin_bit, sub_mask);
+        s_sub[i] = x;
+        all_and &= x;
+        all_or |= x;
     }
-    least = __reduce_min_sync(kFull, least);
-    most = __reduce_max_sync(kFull, most);
-    if (lane == 0) {
-        red[2 * warp] = least;
-        red[2 * warp + 1] = most;
-    }
-    __syncthreads();
+    const uint32_t varying = block_varying<THREADS>(all_and, all_or, red);  // (its barriers publish s_sub)
+    uint32_t at[kSegItems];  // position, and the digit's count and rank in the pass
 #pragma unroll
-    for (int w = 0; w < THREADS / kWarp; ++w) {
-        least = min(least, red[2 * w]);
-        most = max(most, red[2 * w + 1]);
-    }
-    const uint32_t range = most - least;
-    const int cut = cut_bits(range, kIdxBits);
-#pragma unroll
-    for (int k = 0; k < kSegItems; ++k)
-        word[k] = sort_word(word[k], least, cut, kIdxBits, (uint32_t)(wbase + k * kWarp + lane));
-    const int top = 32 - __clz((range >> cut) | 1u);  // bits of sub-key in the words
+    for (int k = 0; k < kSegItems; ++k) at[k] = (uint32_t)(wbase + k * kWarp + lane);
     const uint32_t lt = lanemask_lt();
     uint16_t* cnt = s_cnt + warp * kCtaRadix;
-    for (int shift = kIdxBits; shift < kIdxBits + top; shift += kCtaDigit) {
-        __syncthreads();  // the last pass's reads of the words and counters
-        reinterpret_cast<uint2*>(cnt)[lane] = make_uint2(0u, 0u);
+    for (int shift = 0; shift < kSplitBit - begin_bit; shift += kCtaDigit) {
+        if (((varying >> shift) & (kCtaRadix - 1)) == 0u) continue;
+        __syncthreads();  // the last pass's reads of the list and counters
+        reinterpret_cast<uint4*>(cnt)[lane] = make_uint4(0u, 0u, 0u, 0u);
         __syncwarp();
-        uint32_t rnk[kSegItems];
+        uint16_t rnk[kSegItems];
 #pragma unroll
         for (int k = 0; k < kSegItems; ++k) {
             if (k >= kn) break;
             const bool ok = wbase + k * kWarp + lane < n;
-            const uint32_t dg = (word[k] >> shift) & (kCtaRadix - 1);
+            const uint32_t dg = ok ? (s_sub[at[k]] >> shift) & (kCtaRadix - 1) : 0u;
             const uint32_t peers = warp_match_digit<kCtaDigit>(dg, ok);
             const uint32_t prior = cnt[dg];
-            rnk[k] = prior + __popc(peers & lt);
+            rnk[k] = (uint16_t)(prior + __popc(peers & lt));
             __syncwarp();
             if (ok && (peers & lt) == 0u) cnt[dg] = (uint16_t)(prior + __popc(peers));
             __syncwarp();
         }
         __syncthreads();
         // counts -> first positions, by digit and then warp: thread t owns
-        // digit t of the first 128 threads
+        // digit t of the first 256 threads
         uint32_t run = 0;
         if (threadIdx.x < kCtaRadix)
             for (int w = 0; w < THREADS / kWarp; ++w) run += s_cnt[w * kCtaRadix + threadIdx.x];
@@ -563,33 +569,15 @@ __device__ __forceinline__ void block_sort_smem(const uint64_t* kin, const uint3
 #pragma unroll
         for (int k = 0; k < kSegItems; ++k) {
             if (k >= kn) break;
-            if (wbase + k * kWarp + lane < n) s_word[cnt[(word[k] >> shift) & (kCtaRadix - 1)] + rnk[k]] = word[k];
+            if (wbase + k * kWarp + lane < n)
+                s_list[cnt[(s_sub[at[k]] >> shift) & (kCtaRadix - 1)] + rnk[k]] = (uint16_t)at[k];
         }
         __syncthreads();
 #pragma unroll
         for (int k = 0; k < kSegItems; ++k) {
             if (k >= kn) break;
             const int idx = wbase + k * kWarp + lane;
-            if (idx < n) word[k] = s_word[idx];
-        }
-    }
-    if (cut > 0) {
-        uint16_t* list = reinterpret_cast<uint16_t*>(s_word);
-        __syncthreads();  // the words are in registers
-#pragma unroll
-        for (int k = 0; k < kSegItems; ++k) {
-            const int idx = wbase + k * kWarp + lane;
-            if (k < kn && idx < n) list[spad(idx)] = (uint16_t)(word[k] & (kCap - 1));
-        }
-        __syncthreads();
-        fix_order(
-            list, n, threadIdx.x, THREADS,
-            [&](uint16_t i) { return sub_key(__ldg(kin + b + i), begin_bit, sub_mask); },
-            [](bool x) { return __syncthreads_or(x) != 0; });
-#pragma unroll
-        for (int k = 0; k < kSegItems; ++k) {
-            const int idx = wbase + k * kWarp + lane;
-            if (k < kn && idx < n) word[k] = list[spad(idx)];
+            if (idx < n) at[k] = s_list[idx];
         }
     }
 #pragma unroll
@@ -597,9 +585,8 @@ __device__ __forceinline__ void block_sort_smem(const uint64_t* kin, const uint3
         if (k >= kn) break;
         const int idx = wbase + k * kWarp + lane;
         if (idx < n) {
-            const uint32_t src = word[k] & (kCap - 1);
-            kout[b + idx] = __ldg(kin + b + src);
-            vout[b + idx] = __ldg(vin + b + src);
+            kout[b + idx] = __ldg(kin + b + at[k]);
+            vout[b + idx] = __ldg(vin + b + at[k]);
         }
     }
 }
@@ -736,7 +723,8 @@ __device__ void block_sort_global(uint64_t* kin, uint32_t* vin, uint64_t* kout, 
 template <int THREADS>
 struct SegSmem {
     static constexpr int kWordBytes = block_cap<THREADS>() * 4;
-    static constexpr int kBytes = kWordBytes + (THREADS / kWarp) * kCtaRadix * 2;
+    static constexpr int kListBytes = block_cap<THREADS>() * 2;
+    static constexpr int kBytes = kWordBytes + kListBytes + (THREADS / kWarp) * kCtaRadix * 2;
     static constexpr int kGlobalBytes = (THREADS / kWarp) * kLocalRadix * 4;
     static constexpr int kPassBytes = kBytes > kGlobalBytes ? kBytes : kGlobalBytes;
     static constexpr int kBucketBytes = bucket_smem<THREADS, seg_items<THREADS>()>();
@@ -758,8 +746,10 @@ __device__ __forceinline__ void block_sort(uint64_t* kin, uint32_t* vin, uint64_
             done = bucket_sort<THREADS, seg_items<THREADS>()>(kin, vin, kout, vout, b, (int)n, begin_bit, raw, red);
         if (done) return;
         __syncthreads();  // every thread is done with the shared memory
+        using M = SegSmem<THREADS>;
         block_sort_smem<THREADS>(kin, vin, kout, vout, b, (int)n, begin_bit, reinterpret_cast<uint32_t*>(raw),
-                                 reinterpret_cast<uint16_t*>(raw + SegSmem<THREADS>::kWordBytes), red);
+                                 reinterpret_cast<uint16_t*>(raw + M::kWordBytes),
+                                 reinterpret_cast<uint16_t*>(raw + M::kWordBytes + M::kListBytes), red);
     } else {
         block_sort_global<THREADS>(kin, vin, kout, vout, b, n, begin_bit,
                                    reinterpret_cast<uint32_t (*)[kLocalRadix]>(raw), off, red);

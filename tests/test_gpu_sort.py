@@ -440,3 +440,30 @@ def test_many_segments_on_both_sides_of_the_warps_limit(mean):
     perm = np.argsort(keys, kind="stable")
     np.testing.assert_array_equal(k, keys[perm])
     np.testing.assert_array_equal(v, vals[perm])
+
+
+@pytest.mark.parametrize("lengths", [[20, 33, 100, 256, 500], [257, 700, 2048, 2049, 6000, 16384]])
+@pytest.mark.parametrize("kind", ["wall", "shuffled_wall", "two_walls"])
+def test_segments_whose_keys_share_their_leading_bits(lengths, kind):
+    """Most sub-keys equal, or within a few units of each other in shuffled
+    order, beside some far ones: what the leading bits leave undecided is most
+    of the order, in a warp and in a block."""
+    from paper_2602_03207_gb300 import capi
+    rng = np.random.default_rng(len(kind) + len(lengths))
+    keys = []
+    for s, n in enumerate(lengths):
+        d = np.full(n, 1 << 29) if kind == "wall" else (1 << 29) + rng.integers(0, 60, n)
+        if kind == "two_walls":
+            d = d + (rng.random(n) < 0.5) * (1 << 27)
+        far = rng.permutation(n)[:max(2, n // 20)]
+        d[far] = rng.integers(1 << 20, 1 << 30, far.size)
+        keys.append((np.uint64(s) << np.uint64(31)) | d.astype(np.uint64))
+    keys = np.concatenate(keys)
+    keys = keys[rng.permutation(keys.size)]
+    vals = rng.permutation(keys.size).astype(np.uint32)
+    end_bit = 31 + int(np.ceil(np.log2(len(lengths))))
+    k, v = gpu_sort(keys, vals, end_bit=end_bit, capacity=max(keys.size, 700 << (end_bit - 31)),
+                    flags=capi.WS_CFG_SORT_SEGMENTED)
+    perm = np.argsort(keys, kind="stable")
+    np.testing.assert_array_equal(k, keys[perm])
+    np.testing.assert_array_equal(v, vals[perm])
