@@ -34,17 +34,16 @@ WORKLOADS = {
 METRIC = "1080p frames/s at 1M splats"
 METRICS = {"hd": METRIC, "uhd": "2160p frames/s at 6M splats"}
 # DRAM bytes (read + write) per launch from one ncu capture of the current
-# kernel (k_blend on the 1080p frame; k_blend_bwd and k_train on the 720p
-# training step; the captures' summaries are kept under profiles/); to be
-# reset to None whenever that kernel changes.
-KERNEL_TRAFFIC = {("k_blend", 16): 51_944_448 + 11_329_280, ("k_blend_bwd", 16): 49_844_992 + 1_542_912,
-                  ("k_train", 16): 43_082_752 + 4_845_312}
-# k_blend_bwd_batch: DRAM bytes per (tile, splat) pair from one capture of
-# the first 8 of the 64 views (a case small enough to capture), per tile size.
-BATCH_BWD_TRAFFIC_PER_PAIR = {16: (3_824_162_000 + 986_591_232) / 17_334_892}
-# k_train_batch (the fused pass on one block per (view, tile)): the same, from
-# a capture of the same 8 views.
-BATCH_TRAIN_TRAFFIC_PER_PAIR = {16: (5_528_209_000 + 1_125_041_000) / 17_334_892}
+# kernel (k_blend on the 1080p frame; k_blend_bwd, and it and k_blend together,
+# on the 720p training step; the captures' summaries are kept under profiles/);
+# to be reset to None whenever that kernel changes.
+KERNEL_TRAFFIC = {("k_blend", 16): 53_418_240 + 8_782_336, ("k_blend_bwd", 16): 56_403_968 + 76_032,
+                  ("train", 16): 25_021_184 + 56_403_968 + 76_032}
+# k_blend_bwd_batch, and it and k_blend_batch together: DRAM bytes per (tile,
+# splat) pair from a capture of 8 views (a case small enough to capture), per
+# tile size.
+BATCH_BWD_TRAFFIC_PER_PAIR = {16: (5_589_663_232 + 1_020_721_920) / 17_053_422}
+BATCH_TRAIN_TRAFFIC_PER_PAIR = {16: (5_589_663_232 + 1_020_721_920 + 1_407_047_680 + 116_121_856) / 17_053_422}
 STAGES = ("preprocess", "cull", "sort", "rasterize")
 
 
@@ -1048,7 +1047,7 @@ def batch_block(args, dev, min_timed_s=1.0, plain_min_s=0.5):
                             if best["tile"] in BATCH_TRAIN_TRAFFIC_PER_PAIR and path == "fused_grid" else None)}
     roof.update({"bound": "alu", "alg_evals": int(evals), "achieved": round(ach, 3), "peak": round(peak, 2),
                  "unit": "TFLOP/s", "frac": round(ach / peak, 4),
-                 "traffic_note": "DRAM bytes per pair of an ncu capture of the 8-view batch (17,334,892 pairs), "
+                 "traffic_note": "DRAM bytes per pair of an ncu capture of an 8-view batch (17,053,422 pairs), "
                                  "times this step's pairs",
                  "peak_source": "derived: SMs x 128 FP32 lanes x 2 x max SM clock"})
     out = {
