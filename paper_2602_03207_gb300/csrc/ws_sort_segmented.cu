@@ -27,10 +27,10 @@
 // on another: each segment belongs to one block.
 //
 // The local sorts are bound by instruction issue where segments fill the chip
-// and by a segment's chain of dependent steps where they do not. 64-bit words (the whole
-// sub-key above the position) took the network two shuffles, a two-part
-// comparison and two selects an element and stage against a shuffle and a
-// minimum or maximum.
+// and by a segment's chain of dependent steps where they do not. 64-bit words
+// (the whole sub-key above the position) took the network two shuffles, a
+// two-part comparison and two selects an element and stage against a shuffle
+// and a minimum or maximum.
 #include <atomic>
 
 #include "ws_common.cuh"
@@ -293,25 +293,27 @@ __device__ __forceinline__ void warp_sort(const uint64_t* kin, const uint32_t* v
 // memory: the sub-keys' range is split over the buckets, the keys stand
 // grouped by bucket after one counting pass, and each finds its place among
 // its bucket's few by comparing with them. About 50 instructions a key and a
-// dozen barriers, where the counting passes take three rounds of ballots and
-// two scans each. Comparisons are of whole sub-keys, then positions, so the
-// result is the stable order whatever order the counting's atomic additions
-// ran in. The buckets are split evenly over three intervals (see bucket_of):
-// split over the whole range alone, a few far splats left most keys of a
-// clustered scene in few buckets. Returns false, with nothing written, when a bucket
-// holds more than kBucketMost keys (sub-keys that crowd together all the same, or are
-// equal): the caller then sorts by the counting passes, whose work does not
-// depend on the distribution. 64 of them: a 417 x 473 frame of dense tiles took 65.0 us
-// for compaction and sort, 67.1 with 32, 74 with 16.
-// smem: 8 K THREADS + 16 bytes. The sorted pairs are staged there and leave in
-// full sectors; they are read a second time in input order, where gathering them in
-// sorted order read a sector for each key and each value.
-// Compaction and sort, us, by the counting passes and with blocks of up to 8,192 keys /
-// by buckets and up to 16,384: 64 views / 2M 7,460 / 6,473; 2160p / 6M 415 / 383; 288
-// tiles of 2,987 keys on average 157 / 79; the sort of 4M pairs in 8,192 segments
-// 192 / 175. The same buckets for a warp's segments lost to the network (1080p /
-// 1M 82 against 69 us): 16 keys a lane in turn through shared memory is the
-// longer chain.
+// dozen barriers, where the counting passes take up to four rounds of ballots
+// and scans. Comparisons are of whole sub-keys, then positions, so the result
+// is the stable order whatever order the counting's atomic additions ran in.
+// The buckets are split evenly over three intervals (see bucket_of): split
+// over the whole range alone, a few far splats left most keys of a clustered
+// scene in few buckets. Returns false, with nothing written, when a bucket
+// holds more than kBucketMost keys (sub-keys that crowd together all the
+// same): the caller then sorts by the counting passes, whose work does not
+// depend on the distribution. 64 of them: a 417 x 473 frame of dense tiles
+// took 65.0 us for compaction and sort, 67.1 with 32, 74 with 16.
+// smem: 6 K THREADS bytes of sub-keys and positions and 16 THREADS + 2 of
+// buckets, at most bucket_smem of the block's largest K. The sorted pairs are
+// staged there (8 K THREADS) and leave in full sectors; they are read a second
+// time in input order, where gathering them in sorted order read a sector for
+// each key and each value.
+// Compaction and sort, us, by three passes over cut words and with blocks of
+// up to 8,192 keys / by buckets and up to 16,384: 64 views / 2M 7,460 / 6,473;
+// 2160p / 6M 415 / 383; 288 tiles of 2,987 keys on average 157 / 79; the sort
+// of 4M pairs in 8,192 segments 192 / 175. The same buckets for a warp's
+// segments lost to the network (1080p / 1M 82 against 69 us): 16 keys a lane
+// in turn through shared memory is the longer chain.
 constexpr uint32_t kBucketMost = 64;
 
 __device__ __forceinline__ float warp_sum(float v) {
@@ -322,6 +324,7 @@ __device__ __forceinline__ float warp_sum(float v) {
 
 template <int THREADS, int K>
 __host__ __device__ constexpr int bucket_smem() { return 8 * K * THREADS + 16; }
+static_assert(bucket_smem<1, 8>() >= 6 * 8 + 16 + 2, "sub-keys, positions and buckets of the largest K, 8 or more");
 
 template <int THREADS, int K>
 __device__ __forceinline__ bool bucket_sort(const uint64_t* kin, const uint32_t* vin, uint64_t* kout, uint32_t* vout,
