@@ -51,7 +51,7 @@ k_blend_bwd(const uint2* __restrict__ ranges, const TileOrder order, const uint3
     if (bwd_tile_body<TS, PX, true>(f, (int)t, first, span, vals, splats, rect, offsets, t_final, d_image, target, out,
                                     sm))
         return;
-    // an infinite or NaN value: the whole item again with the selecting walk
+    // an infinite, NaN or overflowing value: the whole item again with the selecting walk
     __syncthreads();
     item(t, first, span);
     bwd_tile_body<TS, PX, false>(f, (int)t, first, span, vals, splats, rect, offsets, t_final, d_image, target, out, sm);

@@ -135,7 +135,7 @@ k_blend_bwd_batch(const uint2* __restrict__ ranges, const TileOrder order, const
                 ft.f[v], (int)(t - ft.tile_off[v]), first, span, vals, splats + kSplatVec4 * vo, rect + vo,
                 offsets + vo, t_final + po, d_image + 3 * po, target ? target + 3 * po : nullptr, out, sm);
         };
-        if (!walk(std::true_type{})) {  // an infinite or NaN value: the item again with the selecting walk
+        if (!walk(std::true_type{})) {  // an infinite, NaN or overflowing value: the item again, selecting
             __syncthreads();
             walk(std::false_type{});
         }

@@ -22,6 +22,13 @@ namespace ws {
 
 constexpr int kPart = 9;  // partials of a pair: dmean x, y; dconic a, b, c; sigma dsigma; drgb r, g, b
 
+// Whether a value may enter the backward's multiplying walk (BwdPixels), where
+// a pixel that does not composite a splat adds 0 times what lies there: not
+// NaN, not infinite, and small enough that no product on the way overflows:
+// colour . dL/dC < 3 2^120, its distance from a b below 2^122 < 2^123.
+constexpr float kWalkMost = 0x1p60f, kBehindMost = 0x1p122f;
+__device__ __forceinline__ bool walkable(float x) { return fabsf(x) < kWalkMost; }
+
 // Shared-memory record of one staged splat (48 bytes):
 //   geo  = minus the tile-relative centre (-x, -y); conic premultiplied
 //          A = -log2(e) a / 2, B = -log2(e) b
@@ -472,8 +479,10 @@ struct BwdPixels {
     // A visit of this lane's stream: advances the pixels' state and stores
     // their (w, dp) in the visit's row. A pixel that does not composite the
     // splat has alpha = 0, which makes its w and dp zero and leaves T and b
-    // as they are, unless a colour or dL/dC is infinite or NaN: FINITE =
-    // false selects instead of multiplying, so that such a value reaches
+    // as they are, unless a factor is infinite or NaN: a colour, dL/dC, what
+    // lies behind (the background, the segments behind this one) or a product
+    // of them that overflows. FINITE = false, taken where any of them is not
+    // walkable, selects instead of multiplying, so that such a value reaches
     // only the pixels and splats that it belongs to.
     template <bool FINITE>
     __device__ __forceinline__ void visit(const float4& geo, const float2& g2, const float4& col, float4* row) {
@@ -508,6 +517,8 @@ struct BwdPixels {
                 unpack2(b[p], b0, b1);
                 unpack2(bn, n0, n1);
                 b[p] = pack2(al[0] > 0.f ? n0 : b0, al[1] > 0.f ? n1 : b1);
+                o.x = al[0] > 0.f ? o.x : 0.f;
+                o.y = al[1] > 0.f ? o.y : 0.f;
                 o.z = au[0] > 0.f ? o.z : 0.f;
                 o.w = au[1] > 0.f ? o.w : 0.f;
             }
@@ -764,13 +775,13 @@ __device__ __forceinline__ void sum_pair_records(const float4* __restrict__ p8, 
 // (WITH_SLOT) builds the ellipse's sub-block
 // masks, the forward's the bounding box's. g0: vals[start + threadIdx.x], which
 // the caller has loaded. Returns whether the records that this thread staged
-// are finite (WITH_SLOT).
+// are walkable (WITH_SLOT).
 template <typename G, bool WITH_SLOT, typename Splats, typename SlotBase>
 __device__ __forceinline__ bool stage_batch(const Frame& f, float ox, float oy, int tx, int ty, uint32_t start,
                                             int cnt, uint32_t g0, const uint32_t* __restrict__ vals,
                                             const Splats& sp, const uint2* __restrict__ rect, SlotBase slot_of,
                                             SplatRec* s_rec, typename G::Mask* s_mask, uint32_t* s_slot) {
-    bool finite = true;
+    bool ok = true;
     for (int j = threadIdx.x; j < cnt; j += G::THREADS) {
         const uint32_t g = j == (int)threadIdx.x ? g0 : __ldg(vals + start + j);
         typename G::Mask m;
@@ -778,15 +789,13 @@ __device__ __forceinline__ bool stage_batch(const Frame& f, float ox, float oy, 
         s_mask[j] = m;
         if (WITH_SLOT) {
             s_slot[j] = pair_slot(slot_of, rect, g, tx, ty);
-            const SplatRec& r = s_rec[j];  // 0 x is 0 for a finite x and NaN otherwise
-            float z = 0.f;
-            z = fmaf(r.geo.x, 0.f, fmaf(r.geo.y, 0.f, fmaf(r.geo.z, 0.f, fmaf(r.geo.w, 0.f, z))));
-            z = fmaf(r.geo2.x, 0.f, fmaf(r.geo2.y, 0.f, fmaf(r.geo2.z, 0.f, fmaf(r.geo2.w, 0.f, z))));
-            z = fmaf(r.col.x, 0.f, fmaf(r.col.y, 0.f, fmaf(r.col.z, 0.f, z)));
-            finite = finite && z == 0.f;
+            const SplatRec& r = s_rec[j];
+            ok = ok && walkable(r.geo.x) && walkable(r.geo.y) && walkable(r.geo.z) && walkable(r.geo.w) &&
+                 walkable(r.geo2.x) && walkable(r.geo2.y) && walkable(r.geo2.z) && walkable(r.geo2.w) &&
+                 walkable(r.col.x) && walkable(r.col.y) && walkable(r.col.z);
         }
     }
-    return finite;
+    return ok;
 }
 
 // vals[start + threadIdx.x] for the threads that stage it of a batch of the list
@@ -854,11 +863,11 @@ __device__ __forceinline__ void blend_tile(const Frame& f, int tile, uint2 range
 
 // dL/dC of this lane's pixels, zeros outside the image: d_image, or in an L2
 // training step d_image - target with the image in d_image's place. Returns
-// whether they are finite.
+// whether they are walkable.
 template <int PX>
 __device__ __forceinline__ bool load_dc(const Frame& f, int gx, int gy0, const float* __restrict__ d_image,
                                         const float* __restrict__ target, float (&dc)[PX][3]) {
-    bool finite = true;
+    bool ok = true;
 #pragma unroll
     for (int k = 0; k < PX; ++k) {
         const int gy = gy0 + k;
@@ -868,10 +877,10 @@ __device__ __forceinline__ bool load_dc(const Frame& f, int gx, int gy0, const f
         for (int c = 0; c < 3; ++c) {
             const float g = inside ? d_image[3 * pix + c] : 0.f;
             dc[k][c] = target && inside ? g - __ldg(target + 3 * pix + c) : g;
-            finite = finite && dc[k][c] * 0.f == 0.f;
+            ok = ok && walkable(dc[k][c]);
         }
     }
-    return finite;
+    return ok;
 }
 
 __device__ __forceinline__ float dot3(const float* a, const float (&d)[3]) {
@@ -975,8 +984,8 @@ struct BwdSpan {
 // Backward of (a span of) one tile from the stored final transmittance: each
 // pair's 9 partials at its emission slot (see BwdPixels). offsets[g]: the first
 // emission slot of Gaussian g's pairs (in a batch, of this view's). d_image and
-// target: load_dc. FINITE = true stops and returns false when a staged record
-// or a dL/dC is infinite or NaN. (The positions past a tile's last composited
+// target: load_dc. FINITE = true stops and returns false when a staged record,
+// a dL/dC or a pixel's state behind the span is not walkable. (The positions past a tile's last composited
 // one are walked like the others: finding that position first, from n_contrib,
 // put a load and a barrier in front of the first batch's loads.)
 template <int TS, int PX, bool FINITE>
@@ -1000,14 +1009,14 @@ __device__ __forceinline__ bool bwd_tile_body(const Frame& f, int tile, uint32_t
     uint32_t g0 = first_value<G, BATCH>(vals, begin + at, begin + len);
     init_null_splat(sm.rec, BATCH);
     BwdPixels<TS, PX> B;
-    bool dc_finite;
+    bool pixels_ok;
     {
         int ix, iy0;
         G::pixel(warp, lane, ix, iy0);
         float tf[PX], bf[PX], dc[PX][3];
         bool inside[PX];
         const int gx = tx * TS + ix, gy0 = ty * TS + iy0;
-        dc_finite = load_dc<PX>(f, gx, gy0, d_image, target, dc);
+        pixels_ok = load_dc<PX>(f, gx, gy0, d_image, target, dc);
 #pragma unroll
         for (int k = 0; k < PX; ++k) {
             inside[k] = gx < f.W && gy0 + k < f.H;
@@ -1025,6 +1034,7 @@ __device__ __forceinline__ bool bwd_tile_body(const Frame& f, int tile, uint32_t
                     tf[k] = t;
                 }
             }
+            pixels_ok = pixels_ok && fabsf(bf[k]) < kBehindMost && fabsf(tf[k]) < 2.f;
         }
         B.init(lane, ix, iy0, inside, tf, bf, dc, sm.dC[G::sub_block(warp, lane)]);
     }
@@ -1036,7 +1046,7 @@ __device__ __forceinline__ bool bwd_tile_body(const Frame& f, int tile, uint32_t
         const bool more = at != 0;
         at -= more ? BATCH : 0;
         if (more) g0 = first_value<G, BATCH>(vals, begin + at, begin + at + BATCH);
-        if (!__syncthreads_and(ok && dc_finite) && FINITE) return false;
+        if (!__syncthreads_and(ok && pixels_ok) && FINITE) return false;
         B.template batch<FINITE>(sm, cnt, warp, lane, out);
         if (!more) return true;
     }

@@ -142,3 +142,80 @@ def test_non_finite_colour_stays_with_its_splat():
     assert shared[g] and not shared.all()
     for k, v in bad.items():
         assert torch.equal(v[~shared], plain[k][~shared]), k
+
+
+def _sharing(r, scene, cam, g, bump):
+    """Which splats composite a pixel that splat g composites (one where the
+    image moves with g's colour): those whose colour a gradient of one at these
+    pixels alone reaches. Also those pixels."""
+    import torch
+    base = r.forward(scene, cam).clone()
+    sh = scene["sh"].clone()
+    scene["sh"][g, 0] += bump
+    pixels = (r.forward(scene, cam) != base).any(-1)
+    scene["sh"].copy_(sh)
+    r.forward(scene, cam)
+    one = torch.zeros_like(base)
+    one[pixels] = 1.0
+    return r.backward(scene, cam, one)["sh"].abs().sum((1, 2)) > 0, pixels
+
+
+@pytest.mark.parametrize("masked", [False, True])
+@pytest.mark.parametrize("value,scale", [(np.inf, 1.0), (1e30, 1e10)], ids=["infinite", "overflowing"])
+@pytest.mark.parametrize("tile,capacity", [(16, 1 << 20), (16, 60_000), (8, 1 << 20), (32, 1 << 20)])
+def test_non_finite_colour_stays_with_its_splat_across_segments(tile, capacity, value, scale, masked):
+    """The farthest visible splat of a list of more than 1,152 gets an infinite colour,
+    or a finite one whose product with dL/dimage overflows, where the list is
+    cut into segments and where it is not: the splats in front that share no
+    pixel with it keep the bits they have without it."""
+    import torch
+    from paper_2602_03207_gb300 import render
+    side = {8: 8, 16: 16, 32: 24}[tile]
+    n = {8: 8000, 16: 5000, 32: 3000}[tile]
+    cam = _cam(side, side)
+    s = _scene(n, 31, -3.8)
+    s["opacity_logits"] = np.random.default_rng(2).uniform(-5.2, -4.4, n).astype(np.float32)
+    scene = render.scene_to_device(s)
+    r = render.Renderer(n, side, side, tile=tile, key_capacity=capacity)
+    r.forward(scene, cam)
+    first, last = (int(x) for x in r.ranges[0])
+    assert last - first > 1152
+    for g in r.sorted_vals[first:last].flip(0).tolist():  # the farthest that covers a pixel centre
+        shared, pixels = _sharing(r, scene, cam, g, 1000.0)
+        if pixels.any():
+            break
+    live = r.tiles_touched[:n] > 0
+    assert shared[g] and (live & ~shared).sum() > 100
+    d = scale * torch.randn(side, side, 3, generator=torch.Generator().manual_seed(3)).cuda()
+    if masked:
+        d[pixels] = 0.0
+    plain = r.backward(scene, cam, d)
+    assert all(torch.isfinite(v).all() for v in plain.values())
+    scene["sh"][g, 0] = value
+    r.forward(scene, cam)
+    bad = r.backward(scene, cam, d)
+    for k, v in bad.items():
+        assert torch.equal(v[~shared], plain[k][~shared]), k
+
+
+def test_infinite_background_stays_behind_what_is_composited():
+    """An infinite background with a finite dL/dimage: colour gradients do not
+    depend on it, and splats that composite no pixel keep zero gradients."""
+    import torch
+    from paper_2602_03207_gb300 import render
+    s = _scene(500, 23, -3.0)
+    s["opacity_logits"][400:] = -5.52  # an extent of a tenth of a pixel: most cover no pixel centre
+    scene = render.scene_to_device(s)
+    grads = []
+    for bg in ((0.2, 0.4, 0.1), (float("inf"),) * 3):
+        cam = _cam(40, 37, bg=bg)
+        r = render.Renderer(500, 40, 37, key_capacity=20_000)
+        r.forward(scene, cam)
+        d = torch.randn(37, 40, 3, generator=torch.Generator().manual_seed(2)).cuda()
+        grads.append(r.backward(scene, cam, d))
+    plain, bad = grads
+    none = (plain["sh"].abs().sum((1, 2)) == 0) & (r.tiles_touched[:500] > 0)
+    assert none.sum() > 20
+    assert torch.equal(bad["sh"], plain["sh"])
+    for k, v in bad.items():
+        assert not v[none].any(), k
