@@ -113,6 +113,7 @@ class Renderer:
             self.axes = torch.empty((n1, 2), dtype=torch.int32, device=d)      # 2 x (2 binary16)
             self.rgba = torch.empty(n1, dtype=torch.int32, device=d)           # RGBA8
         self._cam_probe = None
+        self._frame = None  # (width, height) that the pairs in the buffers were binned for
         self.workspace = None
         self.sorted_in_alt = False
 
@@ -122,6 +123,24 @@ class Renderer:
             if nbytes == 0:
                 raise ValueError("ws_workspace_bytes rejected the configuration")
             self.workspace = torch.zeros(nbytes, dtype=torch.uint8, device=self.image.device)
+
+    # The C calls take the image's and the tile grid's extent from the camera.
+    def _check_camera(self, cam, binned=False):
+        """Refuses a camera whose frame does not fit this renderer's buffers;
+        binned: also one of another resolution than the pairs were binned for
+        (their tiles would be other ones)."""
+        tx, ty = tile_grid(cam.width, cam.height, self.tile)
+        if (tx * ty > self.tx * self.ty or cam.width * cam.height > self.width * self.height
+                or (binned and self._frame not in (None, (cam.width, cam.height)))):
+            raise ValueError("camera resolution differs from the renderer's")
+
+    @staticmethod
+    def _image_arg(image, cam, name):
+        """A (H, W, 3) float32 argument, contiguous."""
+        if image.dtype != torch.float32 or image.numel() < cam.width * cam.height * 3:
+            raise ValueError(f"{name} must be float32 ({cam.height}, {cam.width}, 3), got {image.dtype} "
+                             f"{tuple(image.shape)}")
+        return image.contiguous()
 
     # views of the splat record (centre hi/lo, conic, sigma, colour)
     @property
@@ -153,6 +172,7 @@ class Renderer:
 
     def cull(self, cam, stream=None):
         self._ensure_workspace(cam)
+        self._frame = (cam.width, cam.height)
         capi.ws_cull(self.n, self.tiles_touched, self.rect, self.depth, cam, self.cfg, self.offsets,
                      self.keys, self.vals, self.key_capacity, self.num_keys, self.workspace, stream)
 
@@ -173,7 +193,9 @@ class Renderer:
         pairs; on GB300 no faster than the two calls, which forward() takes
         unless the renderer was made with fused_cull=True); otherwise the
         two calls."""
+        self._check_camera(cam)
         self._ensure_workspace(cam)
+        self._frame = (cam.width, cam.height)
         if self.cfg.flags & capi.WS_CFG_SORT_SEGMENTED and getattr(self, "_fused_cull", True):
             try:
                 self.sorted_in_alt = capi.ws_cull_sort_tiles(
@@ -198,6 +220,7 @@ class Renderer:
         return self.vals_alt if self.sorted_in_alt else self.vals
 
     def rasterize(self, cam, stream=None):
+        self._check_camera(cam)
         if self.packed:
             capi.ws_rasterize_packed(self.num_keys, self.sorted_keys, self.sorted_vals, self.mean2d_p, self.axes,
                                      self.rgba, cam, self.raster_cfg, self.ranges, self.image, self.t_final,
@@ -228,6 +251,7 @@ class Renderer:
         """ws_frame_buffers of this frame: the scene's arrays and the
         renderer's, taken anew for each call."""
         self._ensure_workspace(cam)
+        self._frame = (cam.width, cam.height)
         return capi.frame_struct((*[scene[k] for k in SCENE_KEYS], self.splats, self.depth, self.rect,
                                   self.tiles_touched, self.offsets, self.keys, self.keys_alt, self.vals, self.vals_alt,
                                   self.num_keys, self.ranges, self.image, self.t_final, self.n_contrib,
@@ -245,6 +269,7 @@ class Renderer:
         if self.packed:
             raise ValueError("the quad path takes the float pre-processing outputs")
         cam = capi.camera(cam_dict)
+        self._check_camera(cam)
         self.preprocess(scene, cam, stream)
         if getattr(self, "quad_workspace", None) is None:
             nbytes = capi.ws_quads_workspace_bytes(self.n, self.key_capacity, cam, self.cfg)
@@ -269,6 +294,8 @@ class Renderer:
         if self.packed:
             raise ValueError("the packed-record variant renders only (no backward)")
         cam = capi.camera(cam_dict)
+        self._check_camera(cam, binned=True)
+        d_image = self._image_arg(d_image, cam, "d_image")
         d = self.image.device
         n1 = max(self.n, 1)
         g = {"means": torch.empty((n1, 3), dtype=torch.float32, device=d),
@@ -276,7 +303,6 @@ class Renderer:
              "quats": torch.empty((n1, 4), dtype=torch.float32, device=d),
              "opacity_logits": torch.empty(n1, dtype=torch.float32, device=d),
              "sh": torch.empty((n1, 16, 3), dtype=torch.float32, device=d)}
-        d_image = d_image.contiguous()
         capi.ws_rasterize_backward(self.n, scene["means"], scene["log_scales"], scene["quats"],
                                    scene["opacity_logits"], scene["sh"], cam, self.cfg, self.splats, self.rect,
                                    self.offsets, self.tiles_touched,
@@ -293,12 +319,14 @@ class Renderer:
         if self.packed:
             raise ValueError("the packed-record variant renders only (no backward)")
         cam = capi.camera(cam_dict)
+        self._check_camera(cam)
+        target = self._image_arg(target, cam, "target")
         if self.fused_cull:
             self.preprocess(scene, cam, stream)
             self._cull_and_sort(cam, stream)
             return self.train_pass_l2(scene, cam_dict, target, stream)
         g = self._grads()
-        done = capi.ws_train_frame_l2(self.n, cam, self.cfg, self._buffers(scene, cam), target.contiguous(),
+        done = capi.ws_train_frame_l2(self.n, cam, self.cfg, self._buffers(scene, cam), target,
                                       g["means"], g["log_scales"], g["quats"], g["opacity_logits"], g["sh"], stream)
         self._sorted(done)
         return {k: v[:self.n] for k, v in g.items()}
@@ -307,10 +335,12 @@ class Renderer:
         """train_step_l2 from the sorted pairs on (ws_render_train_l2), on the
         pairs this renderer has sorted for the same scene and camera."""
         cam = capi.camera(cam_dict)
+        self._check_camera(cam, binned=True)
+        target = self._image_arg(target, cam, "target")
         g = self._grads()
         capi.ws_render_train_l2(self.n, scene["means"], scene["log_scales"], scene["quats"], scene["sh"], cam,
                                 self.raster_cfg, self.num_keys, self.sorted_keys, self.sorted_vals, self.splats, self.rect,
-                                self.offsets, self.tiles_touched, target.contiguous(), self.key_capacity,
+                                self.offsets, self.tiles_touched, target, self.key_capacity,
                                 self.ranges, self.image, self.t_final, self.n_contrib, g["means"], g["log_scales"],
                                 g["quats"], g["opacity_logits"], g["sh"], self.workspace, stream)
         return {k: v[:self.n] for k, v in g.items()}
@@ -376,6 +406,7 @@ class FramePipeline:
         self.count += 1
         r = s["r"]
         cam = capi.camera(cam_dict)
+        r._check_camera(cam)
         if s["buf"] is None:
             r._ensure_workspace(cam)
             s["buf"] = capi.frame_buffers(

@@ -27,3 +27,46 @@ def test_config_flags():
     assert render.config_flags(capi.WS_CFG_FIXED_RADIUS, "lsd") == capi.WS_CFG_FIXED_RADIUS
     with pytest.raises(ValueError):
         render.config_flags(0, "bitonic")
+
+
+def _camera(width, height):
+    from paper_2602_03207_gb300 import synthetic as S
+    return dict(S.small_forward()[1], width=width, height=height)
+
+
+@pytest.mark.parametrize("width,height", [(65, 48), (64, 49), (640, 480), (16, 1000)])
+def test_cameras_that_do_not_fit_are_refused(width, height):
+    """The calls size the image and the tile grid by the camera: one larger
+    than the renderer is refused before anything is launched."""
+    import torch
+    r = render.Renderer(10, 64, 48, device="cpu")
+    cam, image = _camera(width, height), torch.zeros(height, width, 3)
+    calls = [lambda: r.train_step_l2({}, cam, image), lambda: r.train_pass_l2({}, cam, image),
+             lambda: r.backward({}, cam, image), lambda: r.forward_quads({}, cam), lambda: r.forward({}, cam),
+             lambda: r.rasterize(capi.camera(cam)), lambda: r.cull_sort(capi.camera(cam))]
+    for call in calls:
+        with pytest.raises(ValueError, match="camera resolution"):
+            call()
+
+
+def test_camera_of_another_frame_is_refused():
+    """A backward by another grid than the pairs were binned for."""
+    import torch
+    r = render.Renderer(10, 64, 48, device="cpu")
+    r._frame = (64, 48)
+    cam, image = _camera(48, 48), torch.zeros(48, 48, 3)
+    for call in (lambda: r.backward({}, cam, image), lambda: r.train_pass_l2({}, cam, image)):
+        with pytest.raises(ValueError, match="camera resolution"):
+            call()
+
+
+@pytest.mark.parametrize("shape,dtype", [((48, 64), "float32"), ((47, 64, 3), "float32"), ((48, 64, 3), "float16"),
+                                         ((48, 64, 3), "float64")])
+def test_images_of_another_size_or_type_are_refused(shape, dtype):
+    import torch
+    r = render.Renderer(10, 64, 48, device="cpu")
+    cam, image = _camera(64, 48), torch.zeros(shape, dtype=getattr(torch, dtype))
+    for call in (lambda: r.train_step_l2({}, cam, image), lambda: r.train_pass_l2({}, cam, image),
+                 lambda: r.backward({}, cam, image)):
+        with pytest.raises(ValueError, match="must be float32"):
+            call()
