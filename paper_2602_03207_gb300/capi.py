@@ -73,17 +73,17 @@ def camera(cam: dict) -> Camera:
     vm = cam["viewmat"]
     if hasattr(vm, "tolist"):
         vm = vm.tolist()
-    if hasattr(vm[0], "__len__"):
-        vm = [v for row in vm for v in row]
+    vm = [v for row in vm for v in row] if hasattr(vm[0], "__len__") else list(vm)
     bg = cam["bg"]
     try:
         return Camera.from_buffer_copy(_CAMERA.pack(*vm[:12], cam["fx"], cam["fy"], cam["cx"], cam["cy"],
                                                     int(cam["width"]), int(cam["height"]), cam["znear"],
                                                     bg[0], bg[1], bg[2]))
-    except (OverflowError, struct.error):  # a value past float32 (infinite) or int32, as a C conversion makes it
+    except (OverflowError, struct.error):
+        # a value past float32 (infinite) or int32, as a C conversion makes it, or a text in the view matrix
         if len(vm) < 12:
             raise IndexError("viewmat needs 12 values at least")
-        return Camera((C.c_float * 12)(*vm[:12]), cam["fx"], cam["fy"], cam["cx"], cam["cy"], int(cam["width"]),
+        return Camera((C.c_float * 12)(*[float(v) for v in vm[:12]]), cam["fx"], cam["fy"], cam["cx"], cam["cy"], int(cam["width"]),
                       int(cam["height"]), cam["znear"], (C.c_float * 3)(bg[0], bg[1], bg[2]))
 
 

@@ -169,3 +169,17 @@ def test_camera_struct_takes_what_it_always_took():
     for bad in (m.reshape(-1)[:11], m[:2]):
         with pytest.raises(IndexError):
             capi.camera(dict(cam, viewmat=bad))
+
+
+def test_camera_struct_takes_texts_and_other_sequences():
+    """A view matrix of texts (a parsed file's rows) or in a sequence without
+    slices."""
+    import collections
+    from paper_2602_03207_gb300 import capi
+    from paper_2602_03207_gb300 import synthetic as S
+    cam = dict(S.small_forward()[1])
+    want = bytes(capi.camera(cam))
+    rows = [[float(v) for v in row] for row in cam["viewmat"]]
+    flat = [v for row in rows for v in row]
+    for vm in ([[repr(v) for v in row] for row in rows], collections.deque(flat), tuple(map(tuple, rows))):
+        assert bytes(capi.camera(dict(cam, viewmat=vm))) == want
