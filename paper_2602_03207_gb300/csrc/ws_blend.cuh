@@ -476,6 +476,19 @@ struct BwdPixels {
         }
     }
 
+    // Whether what lies behind the next splats may enter the multiplying walk.
+    __device__ __forceinline__ bool walkable_state() const {
+        bool ok = true;
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            float t0, t1, b0, b1;
+            unpack2(T[p], t0, t1);
+            unpack2(b[p], b0, b1);
+            ok = ok && fabsf(t0) < 2.f && fabsf(t1) < 2.f && fabsf(b0) < kBehindMost && fabsf(b1) < kBehindMost;
+        }
+        return ok;
+    }
+
     // A visit of this lane's stream: advances the pixels' state and stores
     // their (w, dp) in the visit's row. A pixel that does not composite the
     // splat has alpha = 0, which makes its w and dp zero and leaves T and b
@@ -790,9 +803,10 @@ __device__ __forceinline__ bool stage_batch(const Frame& f, float ox, float oy, 
         if (WITH_SLOT) {
             s_slot[j] = pair_slot(slot_of, rect, g, tx, ty);
             const SplatRec& r = s_rec[j];
-            ok = ok && walkable(r.geo.x) && walkable(r.geo.y) && walkable(r.geo.z) && walkable(r.geo.w) &&
-                 walkable(r.geo2.x) && walkable(r.geo2.y) && walkable(r.geo2.z) && walkable(r.geo2.w) &&
-                 walkable(r.col.x) && walkable(r.col.y) && walkable(r.col.z);
+            // one sum of magnitudes: eleven comparisons took 1 % of a step of short lists
+            const float geo = fabsf(r.geo.x) + fabsf(r.geo.y) + fabsf(r.geo.z) + fabsf(r.geo.w);
+            const float geo2 = fabsf(r.geo2.x) + fabsf(r.geo2.y) + fabsf(r.geo2.z) + fabsf(r.geo2.w);
+            ok = ok && walkable(geo + geo2 + (fabsf(r.col.x) + fabsf(r.col.y) + fabsf(r.col.z)));
         }
     }
     return ok;
@@ -1034,7 +1048,6 @@ __device__ __forceinline__ bool bwd_tile_body(const Frame& f, int tile, uint32_t
                     tf[k] = t;
                 }
             }
-            pixels_ok = pixels_ok && fabsf(bf[k]) < kBehindMost && fabsf(tf[k]) < 2.f;
         }
         B.init(lane, ix, iy0, inside, tf, bf, dc, sm.dC[G::sub_block(warp, lane)]);
     }
@@ -1046,7 +1059,9 @@ __device__ __forceinline__ bool bwd_tile_body(const Frame& f, int tile, uint32_t
         const bool more = at != 0;
         at -= more ? BATCH : 0;
         if (more) g0 = first_value<G, BATCH>(vals, begin + at, begin + at + BATCH);
-        if (!__syncthreads_and(ok && pixels_ok) && FINITE) return false;
+        // (the state behind is looked at here and not where it is loaded: waiting
+        // for t_final there took 1.5 % of a step of short lists)
+        if (!__syncthreads_and(ok && pixels_ok && (!FINITE || B.walkable_state())) && FINITE) return false;
         B.template batch<FINITE>(sm, cnt, warp, lane, out);
         if (!more) return true;
     }
