@@ -125,20 +125,22 @@ class Renderer:
             self.workspace = torch.zeros(nbytes, dtype=torch.uint8, device=self.image.device)
 
     # The C calls take the image's and the tile grid's extent from the camera.
-    def _check_camera(self, cam, binned=False):
-        """Refuses a camera whose frame does not fit this renderer's buffers;
-        binned: also one of another resolution than the pairs were binned for
-        (their tiles would be other ones)."""
-        tx, ty = tile_grid(cam.width, cam.height, self.tile)
-        if (tx * ty > self.tx * self.ty or cam.width * cam.height > self.width * self.height
-                or (binned and self._frame not in (None, (cam.width, cam.height)))):
-            raise ValueError("camera resolution differs from the renderer's")
-
-    @staticmethod
-    def _image_arg(image, cam, name):
-        """A (H, W, 3) float32 argument, contiguous."""
-        if image.dtype != torch.float32 or image.numel() < cam.width * cam.height * 3:
-            raise ValueError(f"{name} must be float32 ({cam.height}, {cam.width}, 3), got {image.dtype} "
+    def _check(self, cam, image=None, binned=False):
+        """Refuses a camera whose frame does not fit this renderer's buffers
+        and an image argument that is not float32 of its size, which it
+        returns contiguous; binned: also a camera of another resolution than
+        the pairs were binned for (their tiles would be other ones)."""
+        w, h = cam.width, cam.height
+        if w != self.width or h != self.height:
+            tx, ty = tile_grid(w, h, self.tile)
+            if tx * ty > self.tx * self.ty or w * h > self.width * self.height:
+                raise ValueError("camera resolution differs from the renderer's")
+        if binned and self._frame not in (None, (w, h)):
+            raise ValueError("camera resolution differs from that of the pairs")
+        if image is None:
+            return None
+        if image.dtype != torch.float32 or image.numel() < 3 * w * h:
+            raise ValueError(f"the image argument must be float32 ({h}, {w}, 3), got {image.dtype} "
                              f"{tuple(image.shape)}")
         return image.contiguous()
 
@@ -193,7 +195,7 @@ class Renderer:
         pairs; on GB300 no faster than the two calls, which forward() takes
         unless the renderer was made with fused_cull=True); otherwise the
         two calls."""
-        self._check_camera(cam)
+        self._check(cam)
         self._ensure_workspace(cam)
         self._frame = (cam.width, cam.height)
         if self.cfg.flags & capi.WS_CFG_SORT_SEGMENTED and getattr(self, "_fused_cull", True):
@@ -220,7 +222,7 @@ class Renderer:
         return self.vals_alt if self.sorted_in_alt else self.vals
 
     def rasterize(self, cam, stream=None):
-        self._check_camera(cam)
+        self._check(cam)
         if self.packed:
             capi.ws_rasterize_packed(self.num_keys, self.sorted_keys, self.sorted_vals, self.mean2d_p, self.axes,
                                      self.rgba, cam, self.raster_cfg, self.ranges, self.image, self.t_final,
@@ -269,7 +271,7 @@ class Renderer:
         if self.packed:
             raise ValueError("the quad path takes the float pre-processing outputs")
         cam = capi.camera(cam_dict)
-        self._check_camera(cam)
+        self._check(cam)
         self.preprocess(scene, cam, stream)
         if getattr(self, "quad_workspace", None) is None:
             nbytes = capi.ws_quads_workspace_bytes(self.n, self.key_capacity, cam, self.cfg)
@@ -294,8 +296,7 @@ class Renderer:
         if self.packed:
             raise ValueError("the packed-record variant renders only (no backward)")
         cam = capi.camera(cam_dict)
-        self._check_camera(cam, binned=True)
-        d_image = self._image_arg(d_image, cam, "d_image")
+        d_image = self._check(cam, d_image, binned=True)
         d = self.image.device
         n1 = max(self.n, 1)
         g = {"means": torch.empty((n1, 3), dtype=torch.float32, device=d),
@@ -319,8 +320,7 @@ class Renderer:
         if self.packed:
             raise ValueError("the packed-record variant renders only (no backward)")
         cam = capi.camera(cam_dict)
-        self._check_camera(cam)
-        target = self._image_arg(target, cam, "target")
+        target = self._check(cam, target)
         if self.fused_cull:
             self.preprocess(scene, cam, stream)
             self._cull_and_sort(cam, stream)
@@ -335,8 +335,7 @@ class Renderer:
         """train_step_l2 from the sorted pairs on (ws_render_train_l2), on the
         pairs this renderer has sorted for the same scene and camera."""
         cam = capi.camera(cam_dict)
-        self._check_camera(cam, binned=True)
-        target = self._image_arg(target, cam, "target")
+        target = self._check(cam, target, binned=True)
         g = self._grads()
         capi.ws_render_train_l2(self.n, scene["means"], scene["log_scales"], scene["quats"], scene["sh"], cam,
                                 self.raster_cfg, self.num_keys, self.sorted_keys, self.sorted_vals, self.splats, self.rect,
@@ -406,7 +405,8 @@ class FramePipeline:
         self.count += 1
         r = s["r"]
         cam = capi.camera(cam_dict)
-        r._check_camera(cam)
+        r._check(cam)
+        r._frame = (cam.width, cam.height)
         if s["buf"] is None:
             r._ensure_workspace(cam)
             s["buf"] = capi.frame_buffers(
