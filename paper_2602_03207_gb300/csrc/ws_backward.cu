@@ -205,7 +205,8 @@ __device__ __forceinline__ uint32_t length_class(uint32_t len) {
 // Lists of more than head[1] positions are cut into segments of that length
 // (max_split > 0): the shortest for which max_split segments are enough, as 2
 // total / max_split positions each give at most total / head[1] + (lists cut)
-// of them.
+// of them. The total is the sum of the lengths: a caller's ranges may hold
+// anything, such as (0, 0), for an empty tile.
 __global__ void __launch_bounds__(kOrderThreads)
 k_tile_order(const uint2* __restrict__ ranges, uint32_t ntiles, uint32_t* __restrict__ order,
              uint32_t* __restrict__ head, uint2* __restrict__ split, uint32_t max_split) {
@@ -213,17 +214,17 @@ k_tile_order(const uint2* __restrict__ ranges, uint32_t ntiles, uint32_t* __rest
     __shared__ uint32_t s_cnt[W][R];
     __shared__ uint32_t s_red[W + 1];
     __shared__ uint32_t s_split;
+    __shared__ unsigned long long s_total;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < W * R; i += kOrderThreads) (&s_cnt[0][0])[i] = 0u;
-    if (threadIdx.x == 0) s_split = 0u;
+    if (threadIdx.x == 0) {
+        s_split = 0u;
+        s_total = 0ull;
+    }
     pdl_wait();
     __syncthreads();
     uint32_t seg_len = ~0u;
-    if (max_split) {
-        const uint32_t total = __ldg(ranges + ntiles - 1).y;  // pairs of all lists
-        const uint32_t need = (uint32_t)((2ull * total + max_split - 1) / max_split);
-        seg_len = max(kSplitLeast, (need + kSplitUnit - 1) / kSplitUnit * kSplitUnit);
-    }
+    unsigned long long sum = 0ull;
     const uint32_t per = (ntiles + kOrderThreads * U - 1) / (kOrderThreads * U) * (32 * U);
     const uint32_t lo = min(warp * per, ntiles), hi = min(lo + per, ntiles);
     // pass 0 counts, pass 1 places
@@ -240,6 +241,7 @@ k_tile_order(const uint2* __restrict__ ranges, uint32_t ntiles, uint32_t* __rest
             for (int u = 0; u < U; ++u) {
                 const uint32_t i = i0 + u * 32 + lane;
                 if (i >= hi) break;
+                if (!pass) sum += len[u];
                 const uint32_t at = atomicAdd(&s_cnt[warp][length_class(len[u])], 1u);
                 if (pass) order[at] = i;
                 if (pass && len[u] > seg_len) {
@@ -250,8 +252,17 @@ k_tile_order(const uint2* __restrict__ ranges, uint32_t ntiles, uint32_t* __rest
                 }
             }
         }
+        if (!pass && max_split) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
+            if (lane == 0) atomicAdd(&s_total, sum);
+        }
         __syncthreads();
         if (pass) break;
+        if (max_split) {
+            const unsigned long long need = (2ull * s_total + max_split - 1) / max_split;
+            seg_len = max(kSplitLeast, (uint32_t)min((need + kSplitUnit - 1) / kSplitUnit * kSplitUnit, 0xffffffffull));
+        }
         // counts -> first positions, by class and then warp
         static_assert(W * R == 2 * kOrderThreads, "two counters per thread");
         const int c = threadIdx.x / (W / 2), w = (threadIdx.x % (W / 2)) * 2;

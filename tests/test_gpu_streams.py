@@ -219,3 +219,45 @@ def test_infinite_background_stays_behind_what_is_composited():
     assert torch.equal(bad["sh"], plain["sh"])
     for k, v in bad.items():
         assert not v[none].any(), k
+
+
+def _spread(n, dense, width, height, tile):
+    """n splats of about two pixels spread over the image but its last tile,
+    `dense` more in one tile."""
+    rng = np.random.default_rng(n)
+    s = _scene(n + dense, 5, -4.2)
+    s["opacity_logits"] = rng.uniform(-5.2, -4.0, n + dense).astype(np.float32)
+    px, py, z = rng.uniform(0, width, n), rng.uniform(0, height, n), rng.uniform(2.5, 3.5, n + dense)
+    last = (px > width - tile - 8) & (py > height - tile - 8)
+    py[last] -= tile + 8
+    px = np.concatenate([px, rng.uniform(5 * tile + 4, 6 * tile - 4, dense)])
+    py = np.concatenate([py, rng.uniform(3 * tile + 4, 4 * tile - 4, dense)])
+    s["means"] = np.stack([(px - width / 2) * z / 64, (py - height / 2) * z / 64, z - 3], 1).astype(np.float32)
+    return s
+
+
+def test_segments_longer_than_the_shortest_and_ranges_of_empty_tiles():
+    """600 lists of about 670, one of thousands more and none in the last tile:
+    segments of more than 576 positions, against the uncut walk; and the same
+    bits when the caller's ranges hold (0, 0) for the empty tile, as when they
+    hold its place in the list."""
+    import torch
+    from paper_2602_03207_gb300 import render
+    width, height, n, dense, tile = 800, 768, 400_000, 5000, 32
+    scene = render.scene_to_device(_spread(n, dense, width, height, tile))
+    cam = _cam(width, height)
+    d = torch.randn(height, width, 3, generator=torch.Generator().manual_seed(6)).cuda()
+    got = []
+    for capacity in (1 << 20, (1 << 20) - 4):
+        r = render.Renderer(n + dense, width, height, tile=tile, key_capacity=capacity)
+        r.forward(scene, cam)
+        r.check_status()
+        length = r.ranges[:, 1] - r.ranges[:, 0]
+        assert int(length[-1]) == 0 and int((length > 576).sum()) > 512 and int(length.max()) > 4000
+        got.append(r.backward(scene, cam, d))
+        if capacity == 1 << 20:
+            r.ranges[length == 0] = 0
+            again = r.backward(scene, cam, d)
+            assert all(torch.equal(again[k], got[0][k]) for k in again)
+    for k in got[0]:
+        assert torch.linalg.norm(got[0][k] - got[1][k]) <= 1e-5 * torch.linalg.norm(got[1][k]), k
