@@ -261,3 +261,35 @@ def test_segments_longer_than_the_shortest_and_ranges_of_empty_tiles():
             assert all(torch.equal(again[k], got[0][k]) for k in again)
     for k in got[0]:
         assert torch.linalg.norm(got[0][k] - got[1][k]) <= 1e-5 * torch.linalg.norm(got[1][k]), k
+
+
+@pytest.mark.parametrize("tile", [8, 16, 32])
+def test_batched_long_lists_walked_in_segments(tile):
+    """Uneven views whose lists are cut: the separate calls, the fused step and
+    its persistent grid give the same bits, and the sum of the views' uncut
+    gradients to rounding."""
+    import torch
+    from paper_2602_03207_gb300 import batch, render
+    n = 6000
+    cams = [_cam(40, 24), _cam(24, 41, f=48.0), _cam(33, 17, f=80.0)]
+    s = _scene(n, 41, -3.8)
+    s["opacity_logits"] = np.random.default_rng(2).uniform(-5.2, -4.4, n).astype(np.float32)
+    scene = render.scene_to_device(s)
+    target = [torch.rand(c["height"], c["width"], 3, generator=torch.Generator().manual_seed(i)).cuda()
+              for i, c in enumerate(cams)]
+    grads = []
+    for kw in ({}, {"fused": True}, {"fused": True, "persistent": True}):
+        b = batch.BatchRenderer(n, cams, tile=tile, key_capacity=3 << 20, **kw)
+        grads.append({k: v.clone() for k, v in b.step(scene, b.pack(target)).items()})
+        b.check_status()
+        assert int((b.ranges[:, 1] - b.ranges[:, 0]).max()) > 1200
+    for g in grads[1:]:
+        assert all(torch.equal(g[k], grads[0][k]) for k in g)
+    want = None
+    for c, goal in zip(cams, target):
+        r = render.Renderer(n, c["width"], c["height"], tile=tile, key_capacity=1_000_000)
+        one = r.train_step_l2(scene, c, goal)
+        r.check_status()
+        want = {k: v.clone() if want is None else want[k] + v for k, v in one.items()}
+    for k in want:
+        assert torch.linalg.norm(grads[0][k] - want[k]) <= 1e-5 * torch.linalg.norm(want[k]), k
