@@ -595,9 +595,13 @@ __device__ __forceinline__ void block_sort_smem(const uint64_t* kin, const uint3
 }
 
 // The block sorts any number of pairs through global memory, 8 THREADS at a
-// time:
-// per pass a histogram sweep, then chunks in order, each scattered to its
-// digit's running offset. Ping-pongs between the two buffers' [b, b + n);
+// time: per pass a histogram sweep, then chunks in order, each scattered to its
+// digit's running offset. One block works alone, bound by its chain of loads,
+// ballots and barriers: the histogram therefore takes one addition a key, no
+// ranks, which also leaves the 256-thread block's 64 registers without spills
+// (4M pairs, a fifth of them in 20 segments of 40,000: 855-867 us, in one run of
+// four 698, with the ranks, 694-701 without; a half in 200 segments of 10,000:
+// 357-368 -> 300-335). Ping-pongs between the two buffers' [b, b + n);
 // the result ends in (kout, vout). Loads here are plain (not read-only
 // cache): the block reads what it wrote, ordered by __syncthreads.
 template <int THREADS>
@@ -631,34 +635,17 @@ __device__ void block_sort_global(uint64_t* kin, uint32_t* vin, uint64_t* kout, 
         const int bits = kSplitBit - shift < kLocalBits ? kSplitBit - shift : kLocalBits;
         const uint32_t mask = (1u << bits) - 1u;
         if (((varying >> (shift - begin_bit)) & mask) == 0u) continue;
-        // digit totals of the segment -> running offsets
-        for (int i = threadIdx.x; i < (THREADS / kWarp) * kLocalRadix; i += THREADS) (&cnt[0][0])[i] = 0u;
+        // digit totals of the segment -> running offsets (integer additions:
+        // the counts do not depend on their order)
+        if (threadIdx.x < kLocalRadix) off[threadIdx.x] = 0u;
         __syncthreads();
-        for (uint32_t c0 = 0; c0 < n; c0 += kStep) {
-            const int rem = (int)min(n - c0, kStep);
-            uint64_t key[kSegItems];
-            const int kn = rem > wbase ? ((rem - wbase + kWarp - 1) / kWarp < kSegItems
-                                              ? (rem - wbase + kWarp - 1) / kWarp
-                                              : kSegItems)
-                                       : 0;
-#pragma unroll
-            for (int k = 0; k < kSegItems; ++k) {
-                const int idx = wbase + k * kWarp + lane;
-                key[k] = (k < kn && idx < rem) ? sk[c0 + idx] : 0ull;
-            }
-            uint32_t rnk[kSegItems];
-            warp_rank(key, kn, wbase, rem, shift, mask, cnt[warp], rnk);
-        }
+#pragma unroll 8
+        for (uint32_t i = threadIdx.x; i < n; i += THREADS) atomicAdd(&off[(uint32_t)(sk[i] >> shift) & mask], 1u);
         __syncthreads();
         {
             const int d = threadIdx.x;  // the first 256 threads are the digits
-            uint32_t t = 0;
-            if (d < kLocalRadix) {
-#pragma unroll
-                for (int w = 0; w < (THREADS / kWarp); ++w) t += cnt[w][d];
-            }
             uint32_t all;
-            t = block_exclusive_scan<THREADS>(t, red, &all);
+            const uint32_t t = block_exclusive_scan<THREADS>(d < kLocalRadix ? off[d] : 0u, red, &all);
             if (d < kLocalRadix) off[d] = t;
         }
         __syncthreads();

@@ -467,3 +467,19 @@ def test_segments_whose_keys_share_their_leading_bits(lengths, kind):
     perm = np.argsort(keys, kind="stable")
     np.testing.assert_array_equal(k, keys[perm])
     np.testing.assert_array_equal(v, vals[perm])
+
+
+@pytest.mark.parametrize("kind", ["octave", "wide", "runs", "equal"])
+def test_dense_segments_among_many(kind):
+    """Segments of thousands of keys where the capacity is too small for
+    blocks of 1,024 threads: 256 threads sort them through global memory."""
+    from paper_2602_03207_gb300 import capi
+    rng = np.random.default_rng(len(kind))
+    lengths = [3, 40_000, 2049, 4096, 0, 6145] + [20] * 250
+    keys = _segments(lengths, kind, rng)
+    vals = rng.permutation(keys.size).astype(np.uint32)
+    for begin_bit in (0, 5):
+        k, v = gpu_sort(keys, vals, begin_bit=begin_bit, end_bit=31 + 8, flags=capi.WS_CFG_SORT_SEGMENTED)
+        perm = np.argsort(keys >> np.uint64(begin_bit), kind="stable")
+        np.testing.assert_array_equal(k, keys[perm])
+        np.testing.assert_array_equal(v, vals[perm])
