@@ -428,17 +428,24 @@ ws_status ws_render_quads(int64_t n, const float *splats, const float *depth, co
  * through the 0.99 alpha clamp, the Jacobian's guard-band clamp or a colour
  * channel clamped at 0.
  * Deterministic, without float atomics: each tile walks its list back to
- * front from t_final / n_contrib, reduces each pair's 9 partial derivatives
+ * front from t_final, reduces each pair's 9 partial derivatives
  * (centre 2, conic 3 in the splat's axis basis (record word 11), sigma 1
  * (times sigma), colour 3) inside the block in a fixed order
  * and writes them to the pair's emission slot offsets[g] + k in the
  * workspace; each Gaussian then sums its slots in order and applies the
- * adjoint of its pre-processing. Bitwise reproducible.
+ * adjoint of its pre-processing. Bitwise reproducible for the same arguments.
+ * From a key_capacity of 2^20 on (3 2^20, or 1,000 keys a tile) long lists are
+ * walked in segments, each from the transmittance and colour behind it, so the
+ * gradients of one frame at capacities on both sides of that line differ by
+ * rounding. An infinite or NaN d_image, colour or background, or a product of
+ * them that overflows, reaches the splats that composite its pixels and no
+ * others.
  * Inputs: the Gaussians and camera/config of the forward, the ws_preprocess
  * outputs, offsets (ws_cull), the sorted vals (ws_sort), ranges, t_final and
  * n_contrib (ws_rasterize) of the SAME frame, and the key_capacity the
  * workspace was sized with. opacity_logits may be NULL (sigma is read from
- * the splat records). */
+ * the splat records). n_contrib is checked like the others but not read: the
+ * walk finds for itself what each pixel composites. */
 ws_status ws_rasterize_backward(int64_t n, const float *means, const float *log_scales,
                                 const float *quats, const float *opacity_logits, const float *sh,
                                 const ws_camera *cam, const ws_config *cfg, const float *splats,

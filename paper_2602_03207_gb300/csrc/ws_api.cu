@@ -430,8 +430,10 @@ ws_status ws_render_frame_host(int64_t n, const float* h_means, const float* h_l
     if (n > 0) {
         const size_t nn = (size_t)n * sizeof(float);
         // The long copy first: the previous frame's image then travels back beside
-        // it and not across the short copies' boundaries (1080p / 1M, two slots:
-        // 1,161 us a frame against 1,175 with the SH records last).
+        // it and not across the short copies' boundaries (1080p / 1M, two slots, the
+        // two orders in turn, three times: 1,162-1,163 us a frame against 1,174-1,175
+        // with the SH records last; runs of one order within 0.2 %, on other days
+        // the link spreads by up to 15 %).
         const struct { void* dst; const void* src; size_t bytes; } up[] = {
             {b->sh, h_sh, 48 * nn}, {b->means, h_means, 3 * nn}, {b->log_scales, h_log_scales, 3 * nn},
             {b->quats, h_quats, 4 * nn}, {b->opacity_logits, h_opacity_logits, nn}};
@@ -542,7 +544,7 @@ ws_status ws_rasterize_backward(int64_t n, const float* means, const float* log_
     if (ws::launch_tile_order(ranges, (uint32_t)(f.TX * f.TY), f.TS, key_capacity, scratch, &order, s) != cudaSuccess)
         return WS_ERR_CUDA;
     return cuda_status(ws::launch_backward(n, means, log_scales, quats, sh, f, splats, rect, offsets, tiles_touched,
-                                           vals, ranges, order, t_final, n_contrib, d_image, nullptr, d_means,
+                                           vals, ranges, order, t_final, d_image, nullptr, d_means,
                                            d_log_scales, d_quats, d_opacity_logits, d_sh, key_capacity, scratch, s));
 }
 
@@ -635,7 +637,7 @@ ws_status ws_rasterize_backward_batch(int64_t n, const float* means, const float
         cudaSuccess)
         return WS_ERR_CUDA;
     return cuda_status(ws::launch_backward_batch(n, means, log_scales, quats, sh, ft, splats, rect, offsets,
-                                                 tiles_touched, vals, ranges, order, t_final, n_contrib, d_image,
+                                                 tiles_touched, vals, ranges, order, t_final, d_image,
                                                  nullptr, d_means, d_log_scales, d_quats, d_opacity_logits, d_sh,
                                                  key_capacity, false, scratch, s));
 }
@@ -674,7 +676,7 @@ ws_status ws_render_train_l2(int64_t n, const float* means, const float* log_sca
         e = ws::launch_rasterize(num_keys, 0, keys, vals, splats, fr, ranges, order.order, image, t_final, n_contrib, s);
     if (e != cudaSuccess) return WS_ERR_CUDA;
     return cuda_status(ws::launch_backward(n, means, log_scales, quats, sh, f, splats, rect, offsets, tiles_touched,
-                                           vals, ranges, order, t_final, n_contrib, image, target, d_means,
+                                           vals, ranges, order, t_final, image, target, d_means,
                                            d_log_scales, d_quats, d_opacity_logits, d_sh, key_capacity, scratch, s));
 }
 
@@ -711,7 +713,7 @@ ws_status ws_render_train_l2_batch(int64_t n, const float* means, const float* l
                                        n_contrib, s);
     if (e != cudaSuccess) return WS_ERR_CUDA;
     return cuda_status(ws::launch_backward_batch(n, means, log_scales, quats, sh, ft, splats, rect, offsets,
-                                                 tiles_touched, vals, ranges, order, t_final, n_contrib, image, target,
+                                                 tiles_touched, vals, ranges, order, t_final, image, target,
                                                  d_means, d_log_scales, d_quats, d_opacity_logits, d_sh, key_capacity,
                                                  (cfg->flags & WS_CFG_PERSISTENT) != 0u, scratch, s));
 }

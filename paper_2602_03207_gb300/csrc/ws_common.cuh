@@ -163,7 +163,10 @@ __device__ __forceinline__ float lg2_approx(float x) {
 }
 
 // 1/x and sqrt(x) on the special-function unit (PTX rcp.approx, sqrt.approx:
-// a few ulp). Used only where a margin absorbs the error (block masks).
+// a few ulp). Used where a margin absorbs the error (block masks), in the
+// splat's axis basis, and in the backward for 1 / (1 - alpha), the step that
+// takes T back over a splat (its few ulp a step stay within the gradients'
+// error against 64 bits).
 __device__ __forceinline__ float rcp_approx(float x) {
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));

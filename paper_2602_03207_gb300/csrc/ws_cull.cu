@@ -13,8 +13,8 @@
 // chunk of Gaussians and the contiguous slot range their pairs occupy; its
 // threads walk that slot range in order, so every key/value write is
 // coalesced no matter how many tiles one splat covers. A thread finds the
-// Gaussian of its slot by binary search over the chunk's local offsets in
-// shared memory.
+// Gaussian of its slot in a map in shared memory, or by binary search over the
+// chunk's local offsets where the chunk has more slots than the map.
 #include "ws_common.cuh"
 #include "ws_kernels.cuh"
 

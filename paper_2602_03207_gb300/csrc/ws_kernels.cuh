@@ -130,7 +130,7 @@ cudaError_t launch_backward(int64_t n, const float* means, const float* log_scal
                             const float* sh, const Frame& f, const float* splats, const uint16_t* rect,
                             const uint32_t* offsets, const uint32_t* tiles_touched,
                             const uint32_t* vals, const uint32_t* ranges, const TileOrder& order, const float* t_final,
-                            const uint32_t* n_contrib, const float* d_image, const float* target, float* d_means,
+                            const float* d_image, const float* target, float* d_means,
                             float* d_log_scales, float* d_quats, float* d_logits, float* d_sh,
                             int64_t key_capacity, void* scratch, cudaStream_t stream);
 
@@ -145,7 +145,7 @@ cudaError_t launch_backward_batch(int64_t n, const float* means, const float* lo
                                   const float* sh, const FrameTable& ft, const float* splats, const uint16_t* rect,
                                   const uint32_t* offsets, const uint32_t* tiles_touched, const uint32_t* vals,
                                   const uint32_t* ranges, const TileOrder& order, const float* t_final,
-                                  const uint32_t* n_contrib, const float* d_image, const float* target, float* d_means,
+                                  const float* d_image, const float* target, float* d_means,
                                   float* d_log_scales, float* d_quats, float* d_logits, float* d_sh,
                                   int64_t key_capacity, bool persistent, void* scratch, cudaStream_t stream);
 cudaError_t launch_residual(int64_t count, const float* image, const float* target, float* d_image,

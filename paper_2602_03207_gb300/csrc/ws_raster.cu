@@ -1,22 +1,21 @@
 // Rasterisation stage (paper §3.4 with the compositing of §2.1), re-designed
-// as a per-tile CUDA blend: one block per screen tile, one thread per pixel,
-// front to back over the tile's depth-sorted pair list.
+// as a per-tile CUDA blend: one block per screen tile, two pixels a lane (four
+// in 32-pixel tiles), front to back over the tile's depth-sorted pair list.
 //
 // Per pair:  a = min(0.99, sigma exp(-q/2)), q = d^T conic d, d = pixel
 // centre - splat centre; a < 1/255 is skipped; C += c a T; T *= 1 - a.
 //
-// The splats of a tile are staged through shared memory in batches of 256:
-// each thread gathers one splat record (value -> Gaussian index -> its
-// 48-byte record: centre, conic, opacity, colour), converts its centre to
+// The splats of a tile are staged through shared memory 128 at a time: each
+// thread gathers one splat record (value -> Gaussian index -> its 48-byte
+// record: centre, conic, opacity, colour), converts its centre to
 // tile-relative coordinates with the double-float centre (so pixel offsets
 // carry no large-magnitude rounding), folds -log2(e)/2 into the conic so the
 // exponent is one ex2 instruction, and computes the box of its
-// opacity-aware extent (§3.4). A half-warp covers a 4x4 pixel sub-block; a
-// splat whose box misses the sub-block is skipped by that half-warp, which
-// removes most of the evaluations of small splats that only graze a tile.
+// opacity-aware extent (§3.4). The lanes of a 4x4 pixel sub-block (eight, or
+// four in 32-pixel tiles) walk a list of the staged splats whose box reaches
+// it, in step with the warp's other sub-blocks (TileGeom in ws_blend.cuh).
 //
-// FP32-pipe + SFU bound: ~17 FP32 instructions and one ex2 per evaluated
-// (pixel, splat) pair.
+// Bound by instruction issue: 47M warp instructions on the 1080p / 1M frame.
 #include "ws_blend.cuh"
 #include "ws_common.cuh"
 #include "ws_kernels.cuh"

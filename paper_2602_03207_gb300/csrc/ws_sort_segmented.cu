@@ -708,8 +708,9 @@ __device__ void block_sort_global(uint64_t* kin, uint32_t* vin, uint64_t* kout, 
     }
 }
 
-// Shared memory of a block that sorts one segment: the words and counters of
-// the passes over words, or the counters of the passes over global memory.
+// Shared memory of a block that sorts one segment: the sub-keys, positions and
+// counters of the passes over positions, the counters of the passes over
+// global memory, or the buckets.
 template <int THREADS>
 struct SegSmem {
     static constexpr int kWordBytes = block_cap<THREADS>() * 4;
@@ -789,7 +790,7 @@ __device__ __forceinline__ uint32_t alone_cap(uint32_t n, uint32_t nseg) {
 // Blocks [0, nbig) sort the segments of more than alone_cap and at most `most` keys:
 // block i those among i, i + nbig, i + 2 nbig, ..., found by one look at their
 // bounds. Blocks nbig + g, g >= 0, give warp w the segment 8g + w when it
-// holds 1 to 512 keys. The large segments come first in launch order so their
+// holds 1 to alone_cap keys. The large segments come first in launch order so their
 // longer sorts start early.
 // nbig (big_blocks): every segment its own block up to 2,048 of them, then
 // 2,048 blocks and more segments each: a block that finds nothing to do still
