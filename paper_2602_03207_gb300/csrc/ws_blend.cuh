@@ -476,19 +476,6 @@ struct BwdPixels {
         }
     }
 
-    // Whether what lies behind the next splats may enter the multiplying walk.
-    __device__ __forceinline__ bool walkable_state() const {
-        bool ok = true;
-#pragma unroll
-        for (int p = 0; p < NP; ++p) {
-            float t0, t1, b0, b1;
-            unpack2(T[p], t0, t1);
-            unpack2(b[p], b0, b1);
-            ok = ok && fabsf(t0) < 2.f && fabsf(t1) < 2.f && fabsf(b0) < kBehindMost && fabsf(b1) < kBehindMost;
-        }
-        return ok;
-    }
-
     // A visit of this lane's stream: advances the pixels' state and stores
     // their (w, dp) in the visit's row. A pixel that does not composite the
     // splat has alpha = 0, which makes its w and dp zero and leaves T and b
@@ -1030,11 +1017,16 @@ __device__ __forceinline__ bool bwd_tile_body(const Frame& f, int tile, uint32_t
         float tf[PX], bf[PX], dc[PX][3];
         bool inside[PX];
         const int gx = tx * TS + ix, gy0 = ty * TS + iy0;
-        pixels_ok = load_dc<PX>(f, gx, gy0, d_image, target, dc);
+        // t_final before dL/dC: both are looked at below, and one wait serves
+        // both (behind it, a step of short lists took 358 us, not 346)
 #pragma unroll
         for (int k = 0; k < PX; ++k) {
             inside[k] = gx < f.W && gy0 + k < f.H;
             tf[k] = inside[k] ? t_final[(size_t)(gy0 + k) * f.W + gx] : 0.f;
+        }
+        pixels_ok = load_dc<PX>(f, gx, gy0, d_image, target, dc);
+#pragma unroll
+        for (int k = 0; k < PX; ++k) {
             bf[k] = dot3(f.bg, dc[k]);
             if (span.states) {
                 const float2* st = span.states + (size_t)threadIdx.x * PX + k;
@@ -1048,6 +1040,9 @@ __device__ __forceinline__ bool bwd_tile_body(const Frame& f, int tile, uint32_t
                     tf[k] = t;
                 }
             }
+            // (b stays between what lies behind and the colours projected on
+            // dL/dC, so the state is looked at only once)
+            pixels_ok = pixels_ok && fabsf(bf[k]) < kBehindMost && fabsf(tf[k]) < 2.f;
         }
         B.init(lane, ix, iy0, inside, tf, bf, dc, sm.dC[G::sub_block(warp, lane)]);
     }
@@ -1059,9 +1054,7 @@ __device__ __forceinline__ bool bwd_tile_body(const Frame& f, int tile, uint32_t
         const bool more = at != 0;
         at -= more ? BATCH : 0;
         if (more) g0 = first_value<G, BATCH>(vals, begin + at, begin + at + BATCH);
-        // (the state behind is looked at here and not where it is loaded: waiting
-        // for t_final there took 1.5 % of a step of short lists)
-        if (!__syncthreads_and(ok && pixels_ok && (!FINITE || B.walkable_state())) && FINITE) return false;
+        if (!__syncthreads_and(ok && pixels_ok) && FINITE) return false;
         B.template batch<FINITE>(sm, cnt, warp, lane, out);
         if (!more) return true;
     }
